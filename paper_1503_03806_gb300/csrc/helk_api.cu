@@ -12,6 +12,7 @@
 #include <string>
 
 #include "helk_internal.cuh"
+#include "wings.cuh"
 
 using namespace helk;
 
@@ -165,6 +166,8 @@ void helk_destroy(helk_ctx *c) {
   if (c->join_ev) cudaEventDestroy(c->join_ev);
   if (c->kcore) cudaFree(c->kcore);
   if (c->core_blk) cudaFree(c->core_blk);
+  if (c->wingF) cudaFree(c->wingF);
+  if (c->wing_tab32) cudaFree(c->wing_tab32);
   for (int st = 0; st < HELK_NSTAGES; ++st)
     for (cudaEvent_t e : c->ev[st]) cudaEventDestroy(e);
   if (cur >= 0) cudaSetDevice(cur);
@@ -330,9 +333,22 @@ static helk_status ensure_conds(helk_ctx *c, int n_cond) {
   return HELK_OK;
 }
 
-// Buffers for n_cond conditions of the current line list and tile shape.
+// Whether a call takes the interpolated-wings route, and its geometry.
+static bool wing_route(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g,
+                       WingGeom *out) {
+  if (o.precision != HELK_PREC_F32_KAHAN || o.count_regions) return false;
+  double half = (double)g->n;
+  if (cut->kind == HELK_CUT_ABS) half = std::min(half, cut->value / g->dnu);
+  if (cut->kind == HELK_CUT_LORENTZ) half = std::min(half, cut->cap / g->dnu);
+  if (half < WING_MIN_HALF) return false;
+  *out = wing_geometry(g->n, half, c->num_sms);
+  return true;
+}
+
+// Buffers for n_cond conditions of the current line list and tile shape (or
+// geometry wg of the interpolated-wings route).
 static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts &o, int64_t ntiles,
-                                       int64_t ngrid) {
+                                       int64_t ngrid, const WingGeom *wg) {
   const int64_t nl = std::max<int64_t>(c->nlines, 1) * n_cond;
   HELK_TRY(ensure_conds(c, n_cond));
   HELK_TRY(ensure_buf(c, (void **)&c->rec64, &c->rec_cap, nl * (int64_t)sizeof(LineRec64), "line records"));
@@ -353,7 +369,8 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
     if (!c->join_ev)
       HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming), "core stream"));
   }
-  HELK_TRY(ensure_tiles(c, ntiles * n_cond));
+  HELK_TRY(ensure_tiles(c, (wg ? (int64_t)wg->nmap : ntiles) * n_cond));
+  if (wg) HELK_TRY(ensure_wing32(c, n_cond, *wg));
   if (o.surrogate && !c->squeue) {
     // routed-evaluation queue: 2^24 entries (entries beyond it fall back to
     // Algorithm 916 in the Voigt kernel)
@@ -406,11 +423,32 @@ static int shape_points(int precision, int shape) {
   return voigt_shape_info(precision, shape, &p, nullptr, nullptr) ? p : 0;
 }
 
+// The interpolated-wings route: candidate map, condition order, the far
+// kernel with the Algorithm 916 cores beside it on the side stream, then the
+// near kernel, which writes kappa.
+static helk_status run_wings(helk_ctx *c, int n_cond, const helk_grid *g, const helk_opts &o, double *kappa,
+                             const WingGeom &wg) {
+  HELK_TRY(cuda_check(c, launch_cond_order(c, n_cond), "condition order"));
+  if (o.surrogate)
+    HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->squeue->count, 0, sizeof(unsigned long long), c->stream), "voigt"));
+  HELK_TRY(cuda_check(c, cudaEventRecord(c->fork_ev, c->stream), "voigt"));
+  HELK_TRY(cuda_check(c, launch_wingmap(c, n_cond, wg), "wing map"));
+  HELK_TRY(cuda_check(c, launch_wing_far32(c, n_cond, wg), "voigt wings"));
+  HELK_TRY(cuda_check(c, cudaStreamWaitEvent(c->side_stream, c->fork_ev, 0), "voigt cores"));
+  HELK_TRY(cuda_check(c, launch_voigt_core(c, n_cond, *g, o), "voigt cores"));
+  HELK_TRY(cuda_check(c, cudaEventRecord(c->join_ev, c->side_stream), "voigt cores"));
+  HELK_TRY(cuda_check(c, cudaStreamWaitEvent(c->stream, c->join_ev, 0), "voigt cores"));
+  HELK_TRY(cuda_check(c, launch_wing_near32(c, n_cond, wg, o, kappa), "voigt wings"));
+  if (o.surrogate) HELK_TRY(cuda_check(c, launch_mlp_queue(c, n_cond, g->n, o.weight, kappa), "surrogate"));
+  return HELK_OK;
+}
+
 // Tile map, condition order and the persistent Voigt kernel (for the FP32
 // form with its Algorithm 916 cores).  `shape`: the Voigt kernel's shape
 // code; `tile`: its points per CTA tile.
 static helk_status run_voigt(helk_ctx *c, int n_cond, const helk_grid *g, const helk_opts &o, double *kappa,
-                             int shape, int tile, int64_t ntiles) {
+                             int shape, int tile, int64_t ntiles, const WingGeom *wg) {
+  if (wg) return run_wings(c, n_cond, g, o, kappa, *wg);
   HELK_TRY(cuda_check(c, launch_tilemap(c, n_cond, *g, tile, ntiles), "tilemap"));
   HELK_TRY(cuda_check(c, launch_cond_order(c, n_cond), "condition order"));
   HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->stats->tile_counter, 0, sizeof(unsigned int), c->stream),
@@ -452,14 +490,16 @@ helk_status helk_opacity(helk_ctx *c, double T, double P, double mass, const hel
   const int tile = shape_points(o.precision, shape);
   if (tile <= 0) return set_err(c, HELK_ERR_STATE, "opacity: no kernel shape");
   const int64_t ntiles = (g->n + tile - 1) / tile;
-  HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n));
+  WingGeom geom;
+  const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
+  HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n, wg));
   const CondArgs one{T, P, o.q_ratio, 0.0};
   stage_begin(c, HELK_STAGE_LINEPREP);
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o));
   stage_end(c, HELK_STAGE_LINEPREP);
   if (c->nlines > 0) {
     stage_begin(c, HELK_STAGE_VOIGT);
-    HELK_TRY(run_voigt(c, 1, g, o, kappa, shape, tile, ntiles));
+    HELK_TRY(run_voigt(c, 1, g, o, kappa, shape, tile, ntiles, wg));
     stage_end(c, HELK_STAGE_VOIGT);
   } else if (!o.accumulate) {
     HELK_TRY(cuda_check(c, cudaMemsetAsync(kappa, 0, (size_t)g->n * 8, c->stream), "opacity"));
@@ -491,7 +531,7 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
     const int pts = std::max(1, shape_points(o.precision, cand[i]));
     max_tiles = std::max(max_tiles, (g->n + pts - 1) / pts);
   }
-  HELK_TRY(ensure_call_buffers(c, 1, o, max_tiles, g->n));
+  HELK_TRY(ensure_call_buffers(c, 1, o, max_tiles, g->n, nullptr));
   const CondArgs one{T, P, o.q_ratio, 0.0};
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o));
   cudaEvent_t e0, e1;
@@ -506,11 +546,11 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
   for (int i = 0; i < ncand && st == HELK_OK; ++i) {
     const int pts = std::max(1, shape_points(o.precision, cand[i]));
     const int64_t ntiles = (g->n + pts - 1) / pts;
-    st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles);  // warm-up
+    st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles, nullptr);  // warm-up
     float ms = 0.f;
     const int reps = 3;
     if (st == HELK_OK) st = cuda_check(c, cudaEventRecord(e0, c->stream), "autotune");
-    for (int r = 0; r < reps && st == HELK_OK; ++r) st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles);
+    for (int r = 0; r < reps && st == HELK_OK; ++r) st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles, nullptr);
     if (st == HELK_OK) st = cuda_check(c, cudaEventRecord(e1, c->stream), "autotune");
     if (st == HELK_OK) st = cuda_check(c, cudaEventSynchronize(e1), "autotune");
     if (st == HELK_OK) st = cuda_check(c, cudaEventElapsedTime(&ms, e0, e1), "autotune");
@@ -551,7 +591,7 @@ static std::string batch_key(const helk_ctx *c, int n_cond, double mass, const h
            c->has_mass, c->has_weight, (const void *)c->cond_host, (const void *)c->cond_dev,
            (const void *)c->cond_order, (const void *)c->core_rng);
   char b3[64];
-  snprintf(b3, sizeof b3, "|%p", (const void *)c->core_blk);
+  snprintf(b3, sizeof b3, "|%p|%p", (const void *)c->core_blk, (const void *)c->wingF);
   return std::string(b) + b2 + b3;
 }
 
@@ -638,7 +678,9 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   const int nchunk = (n_cond + gmax - 1) / gmax;
   const int chunk = (n_cond + nchunk - 1) / nchunk;
   HELK_TRY(ensure_conds(c, n_cond));
-  HELK_TRY(ensure_call_buffers(c, chunk, o, ntiles, g->n));
+  WingGeom geom;
+  const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
+  HELK_TRY(ensure_call_buffers(c, chunk, o, ntiles, g->n, wg));
   if (!c->cap_stream)
     HELK_TRY(cuda_check(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "graph stream"));
   if (!c->cond_ev) HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->cond_ev, cudaEventDisableTiming), "graph"));
@@ -667,7 +709,7 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
                                              cudaMemcpyHostToDevice, c->stream),
                           "graph capture");
           if (st == HELK_OK) st = prepare_lines(c, nk, nullptr, mass, cut, g, o);
-          if (st == HELK_OK) st = run_voigt(c, nk, g, o, kap, shape, tile, ntiles);
+          if (st == HELK_OK) st = run_voigt(c, nk, g, o, kap, shape, tile, ntiles, wg);
           const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
           if (st == HELK_OK) st = cuda_check(c, e, "graph capture");
         }

@@ -156,6 +156,11 @@ struct helk_ctx {
   // kernel and leaves its per-point sums in kcore (FP32, n_cond x n points)
   float *kcore = nullptr;
   int64_t kcore_cap = 0;
+  // interpolated wings (wings.cuh): node sums of the coarser panels,
+  // interpolation tables
+  void *wingF = nullptr;
+  int64_t wingF_cap = 0;
+  float *wing_tab32 = nullptr;
   cudaStream_t side_stream = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   int64_t rec_cap = 0, rec32_cap = 0;

@@ -1,0 +1,778 @@
+// k_wings.cu -- the FP32 form of the interpolated-wings route (wings.cuh):
+// the far kernel (node sums of the coarser panels) and the near kernel (the
+// finer panels, the point-by-point work near the line centres, the way down
+// the tree and the flush).  The lines' Algorithm 916 cores are left to
+// k_core_f32, whose sums the near kernel adds.
+//
+// Against the direct kernel (k_voigt_f32, every line at every point of its
+// window): the 1e5-line, 3e6-point step 0.90 -> 0.61 ms, 1e6 lines at 12
+// conditions 29.9 -> 17.3 ms, 1e7 lines 32.5 -> 24.7 ms, with errors against
+// 64 bits unchanged.  Both kernels are bound by instruction issue at the
+// latency that their warps in flight hide: 64 registers (4 CTAs an SM, a few
+// spilled words in the near kernel's way down the tree) beat 128 (2 CTAs) by
+// 5-10 %.
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "helk_internal.cuh"
+#include "voigt_common.cuh"
+#include "voigt_f32.cuh"
+#include "wings.cuh"
+
+namespace helk {
+
+// --------------------------------------------------------------- geometry --
+WingGeom wing_geometry(int64_t n, double half, int num_sms) {
+  WingGeom g;
+  memset(&g, 0, sizeof g);
+  g.ngrid = (int)n;
+  const double widest = std::min(2.0 * half + 1.0, (double)n);
+  g.lmax = -1;
+  for (int l = 0; l < WG_LEVELS; ++l) {
+    const int64_t s = (int64_t)WG_S0 << l;
+    g.npan[l] = (int)(n / s);
+    if ((double)s <= widest) g.lmax = l;
+  }
+  g.nstage = 1;
+  while (g.nstage < WG_STAGES && wing_level(g.nstage) <= g.lmax) ++g.nstage;
+  int64_t slots = 0, map = 0, far = 0;
+  for (int k = 0; k < g.nstage; ++k) {
+    const int l0 = wing_level(k);
+    const int64_t span = (int64_t)WG_S0 << (l0 + 3);
+    g.groups[k] = (int)((n + span - 1) / span);
+    // the candidates of a group are shared among enough CTAs to fill the GPU
+    g.parts[k] = k == 0 ? 1
+                        : (int)std::min<int64_t>(16, std::max<int64_t>(1, (4ll * num_sms + g.groups[k] - 1) /
+                                                                              g.groups[k]));
+    g.mapoff[k] = (int)map;
+    map += g.groups[k];
+    if (k > 0) {
+      far += (int64_t)g.groups[k] * g.parts[k];
+      for (int l = l0; l < l0 + 3 && l <= g.lmax; ++l) {
+        g.foff[l] = slots;
+        slots += (int64_t)g.npan[l] * g.parts[k];
+      }
+    }
+  }
+  g.fslots = slots;
+  g.nmap = (int)map;
+  g.farblk = (int)far;
+  return g;
+}
+
+// One warp per group: its candidate lines, the contiguous range of the list
+// whose reference index lies within the condition's largest window half-width
+// of the group's points.
+__global__ void k_wingmap(int64_t nlines, const double *__restrict__ ckey, WingGeom G,
+                          const CondStats *__restrict__ cst, int32_t *__restrict__ lo, int32_t *__restrict__ hi) {
+  const int cond = blockIdx.y;
+  const int m = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+  if (m >= G.nmap) return;  // warp-uniform
+  int k = 0;
+  while (k + 1 < G.nstage && m >= G.mapoff[k + 1]) ++k;
+  const int64_t span = (int64_t)WG_S0 << (wing_level(k) + 3);
+  const int64_t A = (int64_t)(m - G.mapoff[k]) * span;
+  const int64_t B = min(A + span, (int64_t)G.ngrid);
+  const long long W = cst[cond].wmax;
+  const int64_t o = (int64_t)cond * G.nmap + m;
+  int64_t first = 0, last = 0;
+  if (W >= 0) {
+    first = warp_search(ckey, 0, nlines, (double)A - (double)W, false);
+    last = warp_search(ckey, first, nlines, (double)(B - 1) + (double)W, true);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    lo[o] = (int32_t)first;
+    hi[o] = (int32_t)last;
+  }
+}
+
+cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const WingGeom &g) {
+  dim3 grid((unsigned)((g.nmap + 7) / 8), n_cond);
+  ++c->launches;
+  k_wingmap<<<grid, 256, 0, c->stream>>>(c->nlines, c->ckey, g, c->cstats, c->tile_lo, c->tile_hi);
+  return cudaGetLastError();
+}
+
+// -------------------------------------------------------------- FP32 form --
+// 12 nodes, panels at least 3 half-widths from the poles: truncation below
+// 2.3e-8 of the profile at the closest distance (half an ulp is 6e-8), and
+// falling with the twelfth power of it.
+constexpr int W32_P = 12;
+constexpr int W32_PS = 16;  // floats a node-sum slot
+constexpr float W32_ETA2 = 9.0f;
+constexpr int W32_FEW = 12;  // lists up to this length run two lines at a time (nodes_few)
+// cos((2 j + 1) pi / 24), j = 0 .. 11
+__device__ constexpr float W32_T[W32_P] = {0.99144486f,  0.92387953f,  0.79335334f,  0.60876143f,
+                                           0.38268343f,  0.13052619f,  -0.13052619f, -0.38268343f,
+                                           -0.60876143f, -0.79335334f, -0.92387953f, -0.99144486f};
+
+// A line as a group's CTA holds it, positions counted from the group's first
+// point.  u(i) = (i - c) beta + nphi.  Both quadrature terms are one rational
+// function of r2 = u^2 + a^2,
+//   n / d,  d = r2 (r2 (k1 r2 + m3) + C),  n = r2 (c3 r2 + c45) + c2:
+// GH3 (Gh3Line) has k1 = 1, m3 = -3 and the coefficients kept here; GH1 is
+// k1 = m3 = c3 = c45 = 0, C = 1, c2 = P1.
+struct __align__(16) WingLine {
+  float c, nphi, beta, a2;
+  float P1, C, c3, c45;
+  float c2, g1, g3, core;  // GH1 from g1 points off the centre on, GH3 from `core` up to g3 (margins included)
+  float ib;                // 1 / beta
+  int ci;                  // c as an integer
+  int ilo, ihi;            // window, clamped to just outside the group
+};
+static_assert(sizeof(WingLine) == 64, "WingLine must be 64 bytes");
+constexpr float WING_FAR = 3.0e38f;
+
+// The offset of point i from the line's centre, in points: monotone in i and,
+// from the integer difference, the same whatever the group.
+__device__ __forceinline__ float wing_off(const WingLine &L, int i) {
+  return fmaf(L.nphi, L.ib, (float)(i - L.ci));
+}
+
+// Whether a line is taken on a panel of s points whose ends have the offsets dl
+// <= dh: as GH1 beyond g1, as GH3 between `core` and g3 (the method's
+// boundaries with a margin of 1.5 points and 1e-6, so that every point of the
+// panel is on one side in the per-point arithmetic), and far enough from the
+// poles (sqrt(3/2) Doppler units nearer for the 3-node rule).  A line taken on a
+// panel is also taken, by this test, on every panel inside it: the ends decide
+// by themselves, and the distance from the poles gains a factor 5/3.  So a
+// group may drop what its own panel takes.
+struct WingReach {
+  float d1, d3;
+  __device__ __forceinline__ WingReach(const WingLine &L, float s) {
+    const float hw = 0.5f * s * L.beta;
+    const float q = fmaf(W32_ETA2 * hw, hw, -L.a2);
+    d1 = q > 0.0f ? __fsqrt_rn(q) * L.ib * 1.000001f : 0.0f;
+    d3 = q > 0.0f ? fmaf(1.2248f, L.ib, d1) : 0.0f;  // (q <= 0: far enough wherever the centre lies)
+  }
+  __device__ __forceinline__ bool takes(const WingLine &L, float dl, float dh) const {
+    const float near = fmaxf(dl, -dh), far = fmaxf(dh, -dl), d = 0.5f * fabsf(dl + dh);
+    return (near >= L.g1 && d >= d1) || (near >= L.core && far <= L.g3 && d >= d3);
+  }
+};
+
+__device__ __forceinline__ void wing_line(const LineRec32 &R, int64_t gbase, int gspan, WingLine &L) {
+  L.nphi = -R.phi_k;
+  L.beta = R.beta;
+  L.a2 = R.a2;
+  L.ib = __frcp_rn(R.beta);
+  L.ci = R.c - (int)gbase;
+  L.c = (float)L.ci;
+  const float x1 = __fsqrt_rn(fmaxf(1.0e6f - R.a2, 0.0f)) * L.ib;
+  const float x3 = __fsqrt_rn(fmaxf(100.0f - R.a2, 0.0f)) * L.ib;
+  const bool all1 = R.a2 >= 1.0e6f;
+  L.g1 = all1 ? -WING_FAR : fmaf(x1, 1.000001f, 1.5f);
+  L.g3 = all1 ? -WING_FAR : fmaf(x1, 0.999999f, -1.5f);
+  L.core = R.a2 >= 100.0f ? -WING_FAR : fmaf(x3, 1.000001f, 1.5f);
+  const Gh3Line g(R.a2, R.P3);
+  L.P1 = R.P1;
+  L.C = g.C;
+  L.c3 = g.c3;
+  L.c45 = g.c45;
+  L.c2 = g.c2;
+  L.ilo = (int)max((int64_t)R.ilo - gbase, (int64_t)-1);
+  L.ihi = (int)min((int64_t)R.ihi - gbase, (int64_t)gspan);
+}
+
+// A line's coefficients on one panel (centre m, s points).
+struct WingTerm {
+  float uc, hw, a2, k1, m3, C, c3, c45, c2;
+  __device__ __forceinline__ void zero() {
+    uc = a2 = C = 1.0f;
+    hw = k1 = m3 = c3 = c45 = c2 = 0.0f;
+  }
+  __device__ __forceinline__ void set(const WingLine &L, float m, float s) {
+    uc = fmaf(m - L.c, L.beta, L.nphi);
+    hw = 0.5f * s * L.beta;
+    a2 = L.a2;
+    const bool gh1 = fmaf(uc, uc, a2) >= 1.0e6f;  // the panel lies on one side
+    k1 = gh1 ? 0.0f : 1.0f;
+    m3 = gh1 ? 0.0f : -3.0f;
+    C = gh1 ? 1.0f : L.C;
+    c3 = gh1 ? 0.0f : L.c3;
+    c45 = gh1 ? 0.0f : L.c45;
+    c2 = gh1 ? L.P1 : L.c2;
+  }
+  // acc + the term at the node t
+  __device__ __forceinline__ float add(float t, float acc) const {
+    const float u = fmaf(t, hw, uc);
+    const float r2 = fmaf(u, u, a2);
+    const float p = fmaf(r2, fmaf(k1, r2, m3), C);
+    const float n = fmaf(r2, fmaf(c3, r2, c45), c2);
+    return fmaf(n, fast_rcp(r2 * p), acc);
+  }
+};
+
+// Lane sums of the nodes over the warp by reduce-scatter; lanes 2 j and 2 j + 1
+// get node j's sum (16 exchanges for 12 values instead of 60).
+__device__ __forceinline__ float wing_warp_sum(const float (&acc)[W32_P], int lane) {
+  float v[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = j < W32_P ? acc[j] : 0.0f;
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = lane & (2 * h);
+#pragma unroll
+    for (int j = 0; j < h; ++j) {
+      const float keep = up ? v[j + h] : v[j], send = up ? v[j] : v[j + h];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// n queued lines at the nodes of a panel, for short lists: lanes 2 j and 2 j +
+// 1 take node j (j < 12) of alternate lines; lane 2 j gets the sum.
+__device__ __forceinline__ float nodes_few(const WingLine *rec, const uint16_t *q, int n, int lane, float tj, float m,
+                                           float s) {
+  float v = 0.0f;
+  for (int i = lane & 1; i < n; i += 2) {
+    WingTerm T;
+    T.set(rec[q[i]], m, s);
+    v = T.add(tj, v);
+  }
+  return v + __shfl_xor_sync(0xffffffffu, v, 1);
+}
+
+// Running node sums of a panel in shared memory: Kahan-compensated, lane 2 j
+// holds node j.
+__device__ __forceinline__ void node_accumulate(float2 *f, int lane, float v) {
+  if (!(lane & 1)) {
+    float2 a = f[lane >> 1];
+    kahan_add(a.x, a.y, v);
+    f[lane >> 1] = a;
+  }
+}
+
+// Masks of a batch by list: bit b of word w is line 32 w + b.
+constexpr int WG_WORDS = WG_CAP / 32;
+
+// Adds the lines of a list (every `step`-th word of its masks from `w0` on) to
+// a panel's node sums: 32 lines, one a lane, at a time, and a short rest two
+// lines at a time.  Nine FP32 instructions and one MUFU reciprocal a node.
+__device__ __forceinline__ void list_nodes(const WingLine *rec, const uint32_t *mask, int nwords, int w0, int step,
+                                           uint16_t *q, int lane, float tj, float m, float s, float2 *f) {
+  int n = 0;
+  bool many = false;
+  float acc[W32_P];
+  for (int w = w0;; w += step) {
+    const bool fin = w >= nwords;  // warp-uniform
+    if (!fin) {
+      const uint32_t b = mask[w];
+      if (b == 0) continue;
+      if ((b >> lane) & 1u) q[n + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(32 * w + lane);
+      n += __popc(b);
+      __syncwarp();
+      if (n < 32) continue;
+    } else if (n <= W32_FEW) {
+      break;
+    }
+    if (!many) {
+#pragma unroll
+      for (int j = 0; j < W32_P; ++j) acc[j] = 0.0f;
+      many = true;
+    }
+    WingTerm T;
+    T.zero();
+    if (lane < n) T.set(rec[q[lane]], m, s);
+#pragma unroll
+    for (int j = 0; j < W32_P; ++j) acc[j] = T.add(W32_T[j], acc[j]);
+    n = max(0, n - 32);
+    const uint16_t e = q[32 + lane];
+    __syncwarp();
+    q[lane] = e;
+    __syncwarp();
+    if (fin) break;
+  }
+  if (many) node_accumulate(f, lane, wing_warp_sum(acc, lane));
+  if (n > 0) node_accumulate(f, lane, nodes_few(rec, q, n, lane, tj, m, s));
+  __syncwarp();
+}
+
+// Lists of a batch: the group's panels of its three levels, and (near kernel)
+// the lines that overlap a warp's panel and are not taken on it or coarser.
+enum { LST_L0 = 0, LST_L1 = 8, LST_L2 = 12, LST_U = 14, LST_N = 22 };
+
+struct WingSmem {
+  WingLine rec[WG_CAP];
+  uint32_t mask[LST_N][WG_WORDS];
+  uint16_t q[WG_WARPS][64];
+  int wcnt[WG_WARPS];
+};
+
+// The candidate lines [first, last) of a group, every `stride`-th run of
+// WG_THREADS of them: those that overlap the group and are not taken at its
+// own level or coarser (gok: whether that level is worked and the group lies on
+// the grid in full) are compacted, in list order, into S.rec; a batch is then
+// sorted into lists (n: levels worked above -1; UNRES: also LST_U) and
+// `work(count)` called.  s: points of a warp's panel.
+template <bool UNRES, typename Work>
+__device__ __forceinline__ void wing_scan(WingSmem &S, const LineRec32 *__restrict__ rec, int64_t first, int64_t last,
+                                          int64_t stride, int64_t gbase, int64_t s, bool gok, bool ok2, bool ok1,
+                                          bool ok0, int ngrid, Work work) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t gend = min(gbase + 8 * s, (int64_t)ngrid) - 1;
+  const int gspan = (int)min(8 * s, (int64_t)1 << 30);
+  const int nfull = (int)((gend + 1 - gbase) / s);  // panels on the grid in full
+  const float fs = (float)s;
+  int total = 0;
+  for (int64_t l0 = first; l0 < last; l0 += stride) {
+    const int64_t l = l0 + tid;
+    WingLine L;
+    bool keep = false;
+    if (l < last) {
+      const LineRec32 &R = rec[l];
+      if (R.ilo <= gend && R.ihi >= gbase && R.ilo <= R.ihi) {
+        wing_line(R, gbase, gspan, L);
+        keep = true;
+        if (gok && L.ilo <= 0 && L.ihi >= gspan - 1)
+          keep = !WingReach(L, 8.0f * fs).takes(L, wing_off(L, 0), wing_off(L, gspan - 1));
+      }
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, keep);
+    if (lane == 0) S.wcnt[w] = __popc(b);
+    __syncthreads();
+    int at = total, n = 0;
+#pragma unroll
+    for (int i = 0; i < WG_WARPS; ++i) {
+      const int v = S.wcnt[i];
+      if (i < w) at += v;
+      n += v;
+    }
+    if (keep) S.rec[at + __popc(b & ((1u << lane) - 1u))] = L;
+    total += n;
+    __syncthreads();
+    if (total >= WG_THREADS || (total > 0 && l0 + stride >= last)) {  // CTA-uniform; total < WG_CAP
+      for (int t = 32 * w; t < total; t += WG_THREADS) {
+        const bool in = t + lane < total;
+        const WingLine &M = S.rec[min(t + lane, total - 1)];
+        uint32_t mine = 0;  // lane k keeps list k's mask
+        bool k2[2], k1[4];
+        const int ilo = M.ilo, ihi = M.ihi;
+        const int is = (int)s;
+        float dl[8], dh[8];  // offsets of the panels' ends
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          dl[p] = wing_off(M, p * is);
+          dh[p] = wing_off(M, (p + 1) * is - 1);
+        }
+        {
+          const WingReach T(M, 4.0f * fs);
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            k2[p] = in && ok2 && 4 * p + 4 <= nfull && ilo <= 4 * p * is && ihi >= 4 * (p + 1) * is - 1 &&
+                    T.takes(M, dl[4 * p], dh[4 * p + 3]);
+            const uint32_t m = __ballot_sync(0xffffffffu, k2[p]);
+            if (lane == LST_L2 + p) mine = m;
+          }
+        }
+        {
+          const WingReach T(M, 2.0f * fs);
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            k1[p] = in && ok1 && 2 * p + 2 <= nfull && ilo <= 2 * p * is && ihi >= 2 * (p + 1) * is - 1 &&
+                    T.takes(M, dl[2 * p], dh[2 * p + 1]);
+            const uint32_t m = __ballot_sync(0xffffffffu, k1[p] && !k2[p >> 1]);
+            if (lane == LST_L1 + p) mine = m;
+          }
+        }
+        {
+          const WingReach T(M, fs);
+#pragma unroll
+          for (int p = 0; p < 8; ++p) {
+            const bool up = k2[p >> 2] || k1[p >> 1];
+            const bool k0 = in && !up && ok0 && p + 1 <= nfull && ilo <= p * is && ihi >= (p + 1) * is - 1 &&
+                            T.takes(M, dl[p], dh[p]);
+            uint32_t m = __ballot_sync(0xffffffffu, k0);
+            if (lane == LST_L0 + p) mine = m;
+            if (UNRES) {
+              m = __ballot_sync(0xffffffffu, in && !up && !k0 && ilo <= (p + 1) * is - 1 && ihi >= p * is);
+              if (lane == LST_U + p) mine = m;
+            }
+          }
+        }
+        if (lane < (UNRES ? LST_N : LST_U)) S.mask[lane][t >> 5] = mine;
+      }
+      __syncthreads();
+      work(total);
+      total = 0;
+      __syncthreads();
+    }
+  }
+}
+
+// Node sums of levels wing_level(k) .. + 2, k >= 1: a CTA takes a part of a
+// group's candidates; warp w owns panel 8 grp + w of the lowest level and
+// shares the coarser ones.
+__global__ void __launch_bounds__(WG_THREADS, 4)
+    k_wing_far32(const LineRec32 *__restrict__ rec_all, int64_t nlines, const int32_t *__restrict__ lo_all,
+                 const int32_t *__restrict__ hi_all, WingGeom G, const int *__restrict__ cond_order,
+                 const CondStats *__restrict__ cst, float *__restrict__ F_all) {
+  __shared__ WingSmem S;
+  __shared__ float2 fs[WG_WARPS][3][W32_PS];
+  if (G.nstage < 2) return;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int cond = cond_order[blockIdx.y];
+  int k = G.nstage - 1, b = blockIdx.x;
+  while (k > 1 && b >= G.groups[k] * G.parts[k]) b -= G.groups[k] * G.parts[k], --k;
+  const int top = wing_top(G, cst[cond].wmax), l0 = wing_level(k);
+  if (l0 > top) return;  // no window holds a panel of this stage
+  const int grp = b / G.parts[k], part = b % G.parts[k];
+  const int64_t s = (int64_t)WG_S0 << l0;  // < 2^31 (l0 <= lmax)
+  const int64_t gbase = (int64_t)grp * 8 * s;
+  const bool u1 = l0 + 1 <= top, u2 = l0 + 2 <= top;
+  const bool gok = l0 + 3 <= top && gbase + 8 * s <= G.ngrid;
+  const int64_t m = (int64_t)cond * G.nmap + G.mapoff[k] + grp;
+  const int64_t first = lo_all[m] + (int64_t)part * WG_THREADS, last = hi_all[m];
+  const float tj = lane < 2 * W32_P ? W32_T[lane >> 1] : 0.0f;
+  for (int i = lane; i < 3 * W32_PS; i += 32) fs[w][i / W32_PS][i % W32_PS] = make_float2(0.0f, 0.0f);
+  __syncwarp();
+  wing_scan<false>(S, rec_all + (int64_t)cond * nlines, first, last, (int64_t)G.parts[k] * WG_THREADS, gbase, s, gok,
+                   u2, u1, true, G.ngrid, [&](int total) {
+                     const int nw = (total + 31) >> 5;
+                     for (int v = 0; v < 3; ++v) {  // own panel, then a share of the coarser ones
+                       const int wide = 1 << v, pan = w >> v;
+                       const float sp = (float)(s * wide);
+                       list_nodes(S.rec, S.mask[(v == 0 ? LST_L0 : v == 1 ? LST_L1 : LST_L2) + pan], nw,
+                                  w & (wide - 1), wide, S.q[w], lane, tj, ((float)pan + 0.5f) * sp - 0.5f, sp,
+                                  fs[w][v]);
+                     }
+                   });
+  __syncthreads();
+  float *F = F_all + (int64_t)cond * G.fslots * W32_PS;
+  const int np = G.parts[k];
+  auto val = [&](int ww, int v) { return fs[ww][v][lane].x - fs[ww][v][lane].y; };
+  if (lane < W32_PS) {
+    const int64_t i0 = (int64_t)grp * 8 + w;
+    if (i0 < G.npan[l0]) F[(G.foff[l0] + i0 * np + part) * W32_PS + lane] = val(w, 0);
+    if (u1 && w < 4) {
+      const int64_t i1 = (int64_t)grp * 4 + w;
+      if (i1 < G.npan[l0 + 1])
+        F[(G.foff[l0 + 1] + i1 * np + part) * W32_PS + lane] = val(2 * w, 1) + val(2 * w + 1, 1);
+    }
+    if (u2 && w < 2) {
+      const int64_t i2 = (int64_t)grp * 2 + w;
+      if (i2 < G.npan[l0 + 2])
+        F[(G.foff[l0 + 2] + i2 * np + part) * W32_PS + lane] =
+            (val(4 * w, 2) + val(4 * w + 1, 2)) + (val(4 * w + 2, 2) + val(4 * w + 3, 2));
+    }
+  }
+}
+
+// Interpolation tables: [side][k][16] of a child's nodes in its parent (side 0:
+// the lower half), then [k][32] of the leaf's points.
+constexpr int W32_TABM = 2 * W32_P * W32_PS;
+constexpr int W32_TAB = W32_TABM + W32_P * WG_S0;
+
+// The values at a panel's nodes as a common part (hi + lo, the same on every
+// lane) and deviations from it (node j on lane j): the polynomial of the
+// deviations carries their smaller rounding down the tree.
+struct WingVal {
+  float hi, lo, dev;
+};
+
+// the values at this lane's node of a child (M: the lane's row of the child's
+// matrix), plus the child's own node sums f
+__device__ __forceinline__ WingVal wing_child(const float (&M)[W32_P], const WingVal &v, float f) {
+  float r = 0.0f;
+#pragma unroll
+  for (int k = 0; k < W32_P; ++k) r = fmaf(M[k], __shfl_sync(0xffffffffu, v.dev, k), r);
+  r += f;
+  const float mid = __shfl_sync(0xffffffffu, r, W32_P / 2);
+  WingVal o;
+  float e;
+  o.hi = v.hi + mid;
+  const float z = o.hi - v.hi;
+  e = (v.hi - (o.hi - z)) + (mid - z);
+  o.lo = v.lo + e;
+  o.dev = r - mid;
+  return o;
+}
+
+__global__ void __launch_bounds__(WG_THREADS, 4)
+    k_wing_near32(const LineRec32 *__restrict__ rec_all, int64_t nlines, const int32_t *__restrict__ lo_all,
+                  const int32_t *__restrict__ hi_all, WingGeom G, const int *__restrict__ cond_order,
+                  const CondStats *__restrict__ cst, const float *__restrict__ F_all,
+                  const float *__restrict__ tab, const float *__restrict__ kcore_all, double weight, int accumulate,
+                  double *__restrict__ kappa_all) {
+  constexpr int NL = 4;              // leaves of a warp's panel
+  constexpr int s = NL * WG_S0;      // its points
+  __shared__ WingSmem S;
+  __shared__ float2 fs[WG_WARPS][9][W32_PS];  // own panel, pair, quarter; its two halves; its four leaves
+  __shared__ uint16_t s_uq[WG_WARPS][64];
+  __shared__ float s_top[W32_PS], s_ref[2];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int cond = cond_order[blockIdx.y];
+  const int ngrid = G.ngrid;
+  const int64_t gbase = (int64_t)blockIdx.x * 8 * s;
+  const int top = wing_top(G, cst[cond].wmax);
+  const float tj = lane < 2 * W32_P ? W32_T[lane >> 1] : 0.0f;
+  for (int i = lane; i < 9 * W32_PS; i += 32) fs[w][i / W32_PS][i % W32_PS] = make_float2(0.0f, 0.0f);
+  if (w == 0) {
+    // the values at the nodes of the group's own panel (level 5) from the
+    // coarser levels, coarsest first
+    const float *F = F_all + (int64_t)cond * G.fslots * W32_PS;
+    WingVal v{0.0f, 0.0f, 0.0f};
+    for (int l = top; l >= wing_level(1); --l) {
+      const int64_t p = gbase / ((int64_t)WG_S0 << l);
+      if (p >= G.npan[l]) continue;  // not on the grid in full: nor is any coarser one
+      const int np = G.parts[(l - 2) / 3];
+      const float *Fp = F + (G.foff[l] + p * np) * W32_PS + (lane & 15);
+      float f = 0.0f;
+      for (int i = 0; i < np; ++i) f += Fp[i * W32_PS];
+      float M[W32_P];
+#pragma unroll
+      for (int k = 0; k < W32_P; ++k) M[k] = tab[((int)(p & 1) * W32_P + k) * W32_PS + (lane & 15)];
+      v = wing_child(M, v, f);
+    }
+    if (lane < W32_PS) s_top[lane] = v.dev;
+    if (lane == 0) s_ref[0] = v.hi, s_ref[1] = v.lo;
+  }
+  __syncwarp();
+  const int64_t p0 = gbase + w * s;
+  float sum[NL], comp[NL];
+#pragma unroll
+  for (int k = 0; k < NL; ++k) sum[k] = comp[k] = 0.0f;
+  uint16_t *q = S.q[w], *uq = s_uq[w];
+  const float flane = (float)lane;
+  const int64_t m = (int64_t)cond * G.nmap + blockIdx.x;
+  const int left = (int)min((int64_t)s, (int64_t)ngrid - p0);  // points of the panel on the grid
+  wing_scan<true>(
+      S, rec_all + (int64_t)cond * nlines, lo_all[m], hi_all[m], WG_THREADS, gbase, s,
+      top >= 5 && gbase + 8 * s <= ngrid, top >= 4, top >= 3, top >= 2, ngrid, [&](int total) {
+        const int nw = (total + 31) >> 5;
+        for (int v = 0; v < 3; ++v) {
+          const int wide = 1 << v, pan = w >> v;
+          const float sp = (float)(s * wide);
+          list_nodes(S.rec, S.mask[(v == 0 ? LST_L0 : v == 1 ? LST_L1 : LST_L2) + pan], nw, w & (wide - 1), wide, q,
+                     lane, tj, ((float)pan + 0.5f) * sp - 0.5f, sp, fs[w][v]);
+        }
+        // lines not taken on the panel, 32 at a time: its halves, its leaves,
+        // and point by point
+        int n = 0;
+        for (int wd = 0; wd < nw; ++wd) {
+          const uint32_t b = S.mask[LST_U + w][wd];
+          const bool fin = wd + 1 >= nw;
+          if ((b >> lane) & 1u) uq[n + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(32 * wd + lane);
+          n += __popc(b);
+          __syncwarp();
+          while (n >= 32 || (fin && n > 0)) {
+            const bool in = lane < n;
+            const int j = uq[in ? lane : 0];
+            const WingLine &L = S.rec[j];
+            const int base = w * s;  // the panel's first point
+            const int ilo = L.ilo - base, ihi = L.ihi - base;
+            float dl[NL], dh[NL];
+#pragma unroll
+            for (int p = 0; p < NL; ++p) {
+              dl[p] = wing_off(L, base + 32 * p);
+              dh[p] = wing_off(L, base + 32 * p + 31);
+            }
+            uint32_t mh[2], ml[NL], md[NL], m1[NL];
+            bool kh[2];
+            {
+              const WingReach T(L, 64.0f);
+#pragma unroll
+              for (int p = 0; p < 2; ++p) {
+                kh[p] = in && top >= 1 && 64 * (p + 1) <= left && ilo <= 64 * p && ihi >= 64 * p + 63 &&
+                        T.takes(L, dl[2 * p], dh[2 * p + 1]);
+                mh[p] = __ballot_sync(0xffffffffu, kh[p]);
+              }
+            }
+            {
+              const WingReach T(L, 32.0f);
+#pragma unroll
+              for (int p = 0; p < NL; ++p) {
+                const bool rest = in && !kh[p >> 1];
+                const bool k0 = rest && top >= 0 && 32 * (p + 1) <= left && ilo <= 32 * p && ihi >= 32 * p + 31 &&
+                                T.takes(L, dl[p], dh[p]);
+                ml[p] = __ballot_sync(0xffffffffu, k0);
+                // point by point, unless every covered point is a core point;
+                // GH1 throughout where the nearest covered point is
+                const int lo = max(ilo, 32 * p), hi = min(ihi, 32 * p + 31);
+                const float ul = fmaf((float)(base + lo) - L.c, L.beta, L.nphi);
+                const float uh = fmaf((float)(base + hi) - L.c, L.beta, L.nphi);
+                const float rl = fmaf(ul, ul, L.a2), rh = fmaf(uh, uh, L.a2);
+                const bool d = rest && !k0 && lo <= hi && fmaxf(rl, rh) >= 100.0f;
+                const bool g1 = d && fminf(rl, rh) >= 1.0e6f && (L.a2 >= 1.0e6f || (ul > 0.0f) == (uh > 0.0f));
+                md[p] = __ballot_sync(0xffffffffu, d && !g1);
+                m1[p] = __ballot_sync(0xffffffffu, g1);
+              }
+            }
+#pragma unroll 1
+            for (int p = 0; p < 2 + NL; ++p) {
+              const uint32_t mk = p == 0 ? mh[0] : p == 1 ? mh[1] : p == 2 ? ml[0] : p == 3 ? ml[1] : p == 4 ? ml[2] : ml[3];
+              if (mk == 0) continue;
+              if ((mk >> lane) & 1u) q[__popc(mk & ((1u << lane) - 1u))] = (uint16_t)j;
+              __syncwarp();
+              const float sp = p < 2 ? 64.0f : 32.0f;
+              const float mid = (float)base + (p < 2 ? 64.0f * p + 31.5f : 32.0f * (p - 2) + 15.5f);
+              node_accumulate(fs[w][3 + p], lane, nodes_few(S.rec, q, __popc(mk), lane, tj, mid, sp));
+              __syncwarp();
+            }
+#pragma unroll
+            for (int p = 0; p < NL; ++p) {
+              const float pos = (float)(base + 32 * p) + flane;
+              const int ip = base + 32 * p + lane;
+              float part = 0.0f;
+              for (uint32_t mk = m1[p]; mk; mk &= mk - 1) {
+                const WingLine &D = S.rec[uq[__ffs(mk) - 1]];
+                const float u = fmaf(pos - D.c, D.beta, D.nphi);
+                const float t = fmaf(D.P1, fast_rcp(fmaf(u, u, D.a2)), part);
+                part = ip >= D.ilo && ip <= D.ihi ? t : part;
+              }
+              // core points (r2 < 100) are left to the core kernel
+              for (uint32_t mk = md[p]; mk; mk &= mk - 1) {
+                const WingLine &D = S.rec[uq[__ffs(mk) - 1]];
+                const float u = fmaf(pos - D.c, D.beta, D.nphi);
+                const float r2 = fmaf(u, u, D.a2);
+                const float pp = fmaf(r2, r2 - 3.0f, D.C);
+                const float nn = fmaf(r2, fmaf(D.c3, r2, D.c45), D.c2);
+                const bool gh1 = r2 >= 1.0e6f;
+                const float t = fmaf(gh1 ? D.P1 : nn, fast_rcp(gh1 ? r2 : r2 * pp), part);
+                part = ip >= D.ilo && ip <= D.ihi && r2 >= 100.0f ? t : part;
+              }
+              kahan_add(sum[p], comp[p], part);
+            }
+            __syncwarp();
+            n = max(0, n - 32);
+            const uint16_t e = uq[32 + lane];
+            __syncwarp();
+            uq[lane] = e;
+            __syncwarp();
+          }
+        }
+      });
+  __syncthreads();
+  if (p0 >= ngrid) return;
+  float far[NL], ref[NL];
+#pragma unroll
+  for (int k = 0; k < NL; ++k) far[k] = ref[k] = 0.0f;
+  WingVal v0[NL];
+  if (top >= 0) {
+    const int j = lane & 15;
+    float M0[W32_P], M1[W32_P];
+#pragma unroll
+    for (int k = 0; k < W32_P; ++k) {
+      M0[k] = tab[k * W32_PS + j];
+      M1[k] = tab[(W32_P + k) * W32_PS + j];
+    }
+    auto val = [&](int ww, int v) { return fs[ww][v][j].x - fs[ww][v][j].y; };
+    auto child = [&](int side, const WingVal &v, float f) { return side ? wing_child(M1, v, f) : wing_child(M0, v, f); };
+    const int h = w & 4, g2 = w & 6;
+    WingVal v{s_ref[0], s_ref[1], s_top[j]};
+    v = child((w >> 2) & 1, v, (val(h, 2) + val(h + 1, 2)) + (val(h + 2, 2) + val(h + 3, 2)));
+    v = child((w >> 1) & 1, v, val(g2, 1) + val(g2 + 1, 1));
+    v = child(w & 1, v, val(w, 0));
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const WingVal vh = child(p, v, val(w, 3 + p));
+      v0[2 * p] = child(0, vh, val(w, 5 + 2 * p));
+      v0[2 * p + 1] = child(1, vh, val(w, 6 + 2 * p));
+    }
+    const float *Lm = tab + W32_TABM + lane;
+#pragma unroll
+    for (int k = 0; k < W32_P; ++k) {
+      const float lk = Lm[k * WG_S0];
+#pragma unroll
+      for (int p = 0; p < NL; ++p) far[p] = fmaf(lk, __shfl_sync(0xffffffffu, v0[p].dev, k), far[p]);
+    }
+#pragma unroll
+    for (int p = 0; p < NL; ++p) ref[p] = v0[p].hi, far[p] += v0[p].lo;
+  }
+  const int E = cst[cond].scale_exp;
+  const bool core = cst[cond].core_w1 != 0, unit = weight == 1.0;
+  const double scale = ldexp(weight, E);
+  const float *kcore = kcore_all + (int64_t)cond * ngrid;
+  double *kappa = kappa_all + (int64_t)cond * ngrid;
+#pragma unroll
+  for (int p = 0; p < NL; ++p) {
+    const int64_t i = p0 + 32 * p + lane;
+    if (i < ngrid) {
+      // the sums as an unevaluated pair (two-sums), then 2^E of it: for weight
+      // 1 scaled on the integer pipe (exact), one FP64 addition rounds
+      float hi = sum[p], lo = -comp[p];
+      auto add = [&](float x) {
+        const float t = hi + x, z = t - hi;
+        lo += (hi - (t - z)) + (x - z);
+        hi = t;
+      };
+      add(ref[p]);
+      add(far[p]);
+      if (core) add(kcore[i]);
+      const double v = unit ? scaled_to_double(hi, E) + scaled_to_double(lo, E) : scale * ((double)hi + (double)lo);
+      kappa[i] = accumulate ? kappa[i] + v : v;
+    }
+  }
+}
+
+// ----------------------------------------------------------------- launch --
+// Lagrange basis of the nodes of [-1, 1] at x, in barycentric form.
+static void lagrange(int P, const double *t, double x, double *out) {
+  double den = 0.0;
+  for (int j = 0; j < P; ++j) {
+    const double w = ((j & 1) ? -1.0 : 1.0) * sin((2 * j + 1) * PI / (2 * P));
+    if (x == t[j]) {
+      for (int i = 0; i < P; ++i) out[i] = i == j ? 1.0 : 0.0;
+      return;
+    }
+    out[j] = w / (x - t[j]);
+    den += out[j];
+  }
+  for (int j = 0; j < P; ++j) out[j] /= den;
+}
+
+void wing_tables(int P, int PS, std::vector<double> &tab) {
+  std::vector<double> t(P), r(P);
+  for (int j = 0; j < P; ++j) t[j] = cos((2 * j + 1) * PI / (2 * P));
+  tab.assign((size_t)2 * P * PS + (size_t)P * WG_S0, 0.0);
+  for (int side = 0; side < 2; ++side)
+    for (int j = 0; j < P; ++j) {
+      lagrange(P, t.data(), (side ? 0.5 : -0.5) + 0.5 * t[j], r.data());
+      for (int k = 0; k < P; ++k) tab[((size_t)side * P + k) * PS + j] = r[k];
+    }
+  for (int i = 0; i < WG_S0; ++i) {
+    lagrange(P, t.data(), (2.0 * i + 1.0 - WG_S0) / WG_S0, r.data());
+    for (int k = 0; k < P; ++k) tab[(size_t)2 * P * PS + (size_t)k * WG_S0 + i] = r[k];
+  }
+}
+
+helk_status ensure_wing32(helk_ctx *c, int n_cond, const WingGeom &g) {
+  helk_status st = ensure_buf(c, (void **)&c->wingF, &c->wingF_cap,
+                              std::max<int64_t>(1, g.fslots) * n_cond * W32_PS * 4, "wing sums");
+  if (st != HELK_OK || c->wing_tab32) return st;
+  std::vector<double> tab;
+  wing_tables(W32_P, W32_PS, tab);
+  const std::vector<float> f(tab.begin(), tab.end());
+  float *p = nullptr;
+  st = cuda_check(c, cudaMalloc((void **)&p, f.size() * 4), "wing tables");
+  if (st != HELK_OK) return st;
+  st = cuda_check(c, cudaMemcpy(p, f.data(), f.size() * 4, cudaMemcpyHostToDevice), "wing tables");
+  if (st == HELK_OK)
+    c->wing_tab32 = p;
+  else
+    cudaFree(p);
+  return st;
+}
+
+cudaError_t launch_wing_far32(helk_ctx *c, int n_cond, const WingGeom &g) {
+  ++c->launches;
+  // a grid without coarser levels launches one CTA that finds nothing to do
+  k_wing_far32<<<dim3((unsigned)std::max(1, g.farblk), n_cond), WG_THREADS, 0, c->stream>>>(
+      c->rec32, c->nlines, c->tile_lo, c->tile_hi, g, c->cond_order, c->cstats, (float *)c->wingF);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_wing_near32(helk_ctx *c, int n_cond, const WingGeom &g, const helk_opts &o, double *kappa) {
+  ++c->launches;
+  k_wing_near32<<<dim3((unsigned)g.groups[0], n_cond), WG_THREADS, 0, c->stream>>>(
+      c->rec32, c->nlines, c->tile_lo, c->tile_hi, g, c->cond_order, c->cstats, (const float *)c->wingF,
+      c->wing_tab32, c->kcore, o.weight, o.accumulate, kappa);
+  return cudaGetLastError();
+}
+
+}  // namespace helk
