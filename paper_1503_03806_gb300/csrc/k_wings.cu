@@ -104,7 +104,6 @@ cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const WingGeom &g) {
 constexpr int W32_P = 12;
 constexpr int W32_PS = 16;  // floats a node-sum slot
 constexpr float W32_ETA2 = 9.0f;
-constexpr int W32_FEW = 12;  // lists up to this length run two lines at a time (nodes_few)
 // cos((2 j + 1) pi / 24), j = 0 .. 11
 __device__ constexpr float W32_T[W32_P] = {0.99144486f,  0.92387953f,  0.79335334f,  0.60876143f,
                                            0.38268343f,  0.13052619f,  -0.13052619f, -0.38268343f,
@@ -114,23 +113,22 @@ __device__ constexpr float W32_T[W32_P] = {0.99144486f,  0.92387953f,  0.7933533
 // point.  u(i) = (i - c) beta + nphi.  Both quadrature terms are one rational
 // function of r2 = u^2 + a^2,
 //   n / d,  d = r2 (r2 (k1 r2 + m3) + C),  n = r2 (c3 r2 + c45) + c2:
-// GH3 (Gh3Line) has k1 = 1, m3 = -3 and the coefficients kept here; GH1 is
-// k1 = m3 = c3 = c45 = 0, C = 1, c2 = P1.
+// GH3 (Gh3Line) has k1 = 1, m3 = -3, C = 9/4 + 6 a^2, c45 = -3/2 c3, c2 = c3 (4 a^2
+// + 3/2); GH1 is k1 = m3 = c3 = c45 = 0, C = 1, c2 = P1.
 struct __align__(16) WingLine {
-  float c, nphi, beta, a2;
-  float P1, C, c3, c45;
-  float c2, g1, g3, core;  // GH1 from g1 points off the centre on, GH3 from `core` up to g3 (margins included)
-  float ib;                // 1 / beta
-  int ci;                  // c as an integer
-  int ilo, ihi;            // window, clamped to just outside the group
+  int c;
+  float nphi, beta, a2;
+  float P1, c3, g1, g3;   // GH1 from g1 points off the centre on, GH3 from `core` up to g3 (margins included)
+  float core, ib;         // ib: 1 / beta
+  int ilo, ihi;           // window, clamped to just outside the group
 };
-static_assert(sizeof(WingLine) == 64, "WingLine must be 64 bytes");
+static_assert(sizeof(WingLine) == 48, "WingLine must be 48 bytes");
 constexpr float WING_FAR = 3.0e38f;
 
 // The offset of point i from the line's centre, in points: monotone in i and,
 // from the integer difference, the same whatever the group.
 __device__ __forceinline__ float wing_off(const WingLine &L, int i) {
-  return fmaf(L.nphi, L.ib, (float)(i - L.ci));
+  return fmaf(L.nphi, L.ib, (float)(i - L.c));
 }
 
 // Whether a line is taken on a panel of s points whose ends have the offsets dl
@@ -156,24 +154,19 @@ struct WingReach {
 };
 
 __device__ __forceinline__ void wing_line(const LineRec32 &R, int64_t gbase, int gspan, WingLine &L) {
+  L.c = R.c - (int)gbase;
   L.nphi = -R.phi_k;
   L.beta = R.beta;
   L.a2 = R.a2;
   L.ib = __frcp_rn(R.beta);
-  L.ci = R.c - (int)gbase;
-  L.c = (float)L.ci;
   const float x1 = __fsqrt_rn(fmaxf(1.0e6f - R.a2, 0.0f)) * L.ib;
   const float x3 = __fsqrt_rn(fmaxf(100.0f - R.a2, 0.0f)) * L.ib;
   const bool all1 = R.a2 >= 1.0e6f;
   L.g1 = all1 ? -WING_FAR : fmaf(x1, 1.000001f, 1.5f);
   L.g3 = all1 ? -WING_FAR : fmaf(x1, 0.999999f, -1.5f);
   L.core = R.a2 >= 100.0f ? -WING_FAR : fmaf(x3, 1.000001f, 1.5f);
-  const Gh3Line g(R.a2, R.P3);
   L.P1 = R.P1;
-  L.C = g.C;
-  L.c3 = g.c3;
-  L.c45 = g.c45;
-  L.c2 = g.c2;
+  L.c3 = 6.0f * R.P3;
   L.ilo = (int)max((int64_t)R.ilo - gbase, (int64_t)-1);
   L.ihi = (int)min((int64_t)R.ihi - gbase, (int64_t)gspan);
 }
@@ -186,16 +179,16 @@ struct WingTerm {
     hw = k1 = m3 = c3 = c45 = c2 = 0.0f;
   }
   __device__ __forceinline__ void set(const WingLine &L, float m, float s) {
-    uc = fmaf(m - L.c, L.beta, L.nphi);
+    uc = fmaf(m - (float)L.c, L.beta, L.nphi);
     hw = 0.5f * s * L.beta;
     a2 = L.a2;
     const bool gh1 = fmaf(uc, uc, a2) >= 1.0e6f;  // the panel lies on one side
     k1 = gh1 ? 0.0f : 1.0f;
     m3 = gh1 ? 0.0f : -3.0f;
-    C = gh1 ? 1.0f : L.C;
+    C = gh1 ? 1.0f : fmaf(6.0f, a2, 2.25f);
     c3 = gh1 ? 0.0f : L.c3;
-    c45 = gh1 ? 0.0f : L.c45;
-    c2 = gh1 ? L.P1 : L.c2;
+    c45 = -1.5f * c3;
+    c2 = gh1 ? L.P1 : L.c3 * fmaf(4.0f, a2, 1.5f);
   }
   // acc + the term at the node t
   __device__ __forceinline__ float add(float t, float acc) const {
@@ -207,89 +200,77 @@ struct WingTerm {
   }
 };
 
-// Lane sums of the nodes over the warp by reduce-scatter; lanes 2 j and 2 j + 1
-// get node j's sum (16 exchanges for 12 values instead of 60).
-__device__ __forceinline__ float wing_warp_sum(const float (&acc)[W32_P], int lane) {
-  float v[16];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = j < W32_P ? acc[j] : 0.0f;
-#pragma unroll
-  for (int h = 8; h >= 1; h >>= 1) {
-    const bool up = lane & (2 * h);
-#pragma unroll
-    for (int j = 0; j < h; ++j) {
-      const float keep = up ? v[j + h] : v[j], send = up ? v[j] : v[j + h];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
-    }
-  }
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
-// n queued lines at the nodes of a panel, for short lists: lanes 2 j and 2 j +
-// 1 take node j (j < 12) of alternate lines; lane 2 j gets the sum.
-__device__ __forceinline__ float nodes_few(const WingLine *rec, const uint16_t *q, int n, int lane, float tj, float m,
-                                           float s) {
-  float v = 0.0f;
-  for (int i = lane & 1; i < n; i += 2) {
-    WingTerm T;
-    T.set(rec[q[i]], m, s);
-    v = T.add(tj, v);
-  }
-  return v + __shfl_xor_sync(0xffffffffu, v, 1);
-}
-
-// Running node sums of a panel in shared memory: Kahan-compensated, lane 2 j
-// holds node j.
-__device__ __forceinline__ void node_accumulate(float2 *f, int lane, float v) {
-  if (!(lane & 1)) {
-    float2 a = f[lane >> 1];
-    kahan_add(a.x, a.y, v);
-    f[lane >> 1] = a;
-  }
-}
-
 // Masks of a batch by list: bit b of word w is line 32 w + b.
 constexpr int WG_WORDS = WG_CAP / 32;
 
-// Adds the lines of a list (every `step`-th word of its masks from `w0` on) to
-// a panel's node sums: 32 lines, one a lane, at a time, and a short rest two
-// lines at a time.  Nine FP32 instructions and one MUFU reciprocal a node.
-__device__ __forceinline__ void list_nodes(const WingLine *rec, const uint32_t *mask, int nwords, int w0, int step,
-                                           uint16_t *q, int lane, float tj, float m, float s, float2 *f) {
+// Adds the lines of a list (every `step`-th word of its masks from `w0` on;
+// bit b of word w is line 32 w + b, or idx[32 w + b]) to a panel's node sums f
+// (Kahan-compensated, in shared memory).  M lines at a time, one a lane of each
+// of 32 / M groups of lanes, which share the nodes: nodes 12 M / 32 (lane / M)
+// on; nine FP32 instructions and one MUFU reciprocal a node.  M = 8 suits the
+// lists of the near kernel (a handful to some tens of lines), M = 32 (every
+// node on a lane, no repeated coefficients) the longer ones of the far kernel.
+template <int M>
+__device__ __forceinline__ void list_nodes(const WingLine *rec, const uint32_t *mask, const uint16_t *idx, int nwords,
+                                           int w0, int step, uint16_t *q, int lane, const float *T, float m, float s,
+                                           float2 *f) {
+  constexpr int NPL = W32_P * M / 32;  // nodes a lane
+  const int grp = lane / M, at = lane % M;
+  float acc[NPL], tn[NPL];
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    acc[j] = 0.0f;
+    tn[j] = M == 32 ? W32_T[j] : T[grp * NPL + j];
+  }
   int n = 0;
-  bool many = false;
-  float acc[W32_P];
+  bool any = false;
   for (int w = w0;; w += step) {
     const bool fin = w >= nwords;  // warp-uniform
     if (!fin) {
       const uint32_t b = mask[w];
       if (b == 0) continue;
-      if ((b >> lane) & 1u) q[n + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(32 * w + lane);
+      if ((b >> lane) & 1u) {
+        const int j = 32 * w + lane;
+        q[n + __popc(b & ((1u << lane) - 1u))] = idx ? idx[j] : (uint16_t)j;
+      }
       n += __popc(b);
       __syncwarp();
       if (n < 32) continue;
-    } else if (n <= W32_FEW) {
+    } else if (n == 0) {
       break;
     }
-    if (!many) {
+    any = true;
+    const int take = min(n, 32);
+#pragma unroll 1
+    for (int i = 0; i < take; i += M) {
+      WingTerm W;
+      W.zero();
+      if (i + at < take) W.set(rec[q[i + at]], m, s);
 #pragma unroll
-      for (int j = 0; j < W32_P; ++j) acc[j] = 0.0f;
-      many = true;
+      for (int j = 0; j < NPL; ++j) acc[j] = W.add(tn[j], acc[j]);
     }
-    WingTerm T;
-    T.zero();
-    if (lane < n) T.set(rec[q[lane]], m, s);
-#pragma unroll
-    for (int j = 0; j < W32_P; ++j) acc[j] = T.add(W32_T[j], acc[j]);
-    n = max(0, n - 32);
+    if (fin) break;
+    n -= 32;
     const uint16_t e = q[32 + lane];
     __syncwarp();
     q[lane] = e;
     __syncwarp();
-    if (fin) break;
   }
-  if (many) node_accumulate(f, lane, wing_warp_sum(acc, lane));
-  if (n > 0) node_accumulate(f, lane, nodes_few(rec, q, n, lane, tj, m, s));
+  if (any) {
+    // sums over the M lanes of a group
+    float v = 0.0f;
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+#pragma unroll
+      for (int o = M / 2; o >= 1; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+      v = at == j ? acc[j] : v;
+    }
+    if (at < NPL) {
+      float2 a = f[grp * NPL + at];
+      kahan_add(a.x, a.y, v);
+      f[grp * NPL + at] = a;
+    }
+  }
   __syncwarp();
 }
 
@@ -326,7 +307,10 @@ __device__ __forceinline__ void wing_scan(WingSmem &S, const LineRec32 *__restri
     bool keep = false;
     if (l < last) {
       const LineRec32 &R = rec[l];
-      if (R.ilo <= gend && R.ihi >= gbase && R.ilo <= R.ihi) {
+      // lines whose whole window is core are the core kernel's
+      const float ul = fmaf((float)(R.ilo - R.c), R.beta, -R.phi_k), uh = fmaf((float)(R.ihi - R.c), R.beta, -R.phi_k);
+      if (R.ilo <= gend && R.ihi >= gbase && R.ilo <= R.ihi &&
+          fmaxf(fmaf(ul, ul, R.a2), fmaf(uh, uh, R.a2)) >= 100.0f) {
         wing_line(R, gbase, gspan, L);
         keep = true;
         if (gok && L.ilo <= 0 && L.ihi >= gspan - 1)
@@ -346,7 +330,7 @@ __device__ __forceinline__ void wing_scan(WingSmem &S, const LineRec32 *__restri
     if (keep) S.rec[at + __popc(b & ((1u << lane) - 1u))] = L;
     total += n;
     __syncthreads();
-    if (total >= WG_THREADS || (total > 0 && l0 + stride >= last)) {  // CTA-uniform; total < WG_CAP
+    if (total > WG_CAP - WG_THREADS || (total > 0 && l0 + stride >= last)) {  // CTA-uniform; total <= WG_CAP
       for (int t = 32 * w; t < total; t += WG_THREADS) {
         const bool in = t + lane < total;
         const WingLine &M = S.rec[min(t + lane, total - 1)];
@@ -408,12 +392,12 @@ __device__ __forceinline__ void wing_scan(WingSmem &S, const LineRec32 *__restri
 // Node sums of levels wing_level(k) .. + 2, k >= 1: a CTA takes a part of a
 // group's candidates; warp w owns panel 8 grp + w of the lowest level and
 // shares the coarser ones.
-__global__ void __launch_bounds__(WG_THREADS, 4)
+__global__ void __launch_bounds__(WG_THREADS, 3)
     k_wing_far32(const LineRec32 *__restrict__ rec_all, int64_t nlines, const int32_t *__restrict__ lo_all,
                  const int32_t *__restrict__ hi_all, WingGeom G, const int *__restrict__ cond_order,
                  const CondStats *__restrict__ cst, float *__restrict__ F_all) {
   __shared__ WingSmem S;
-  __shared__ float2 fs[WG_WARPS][3][W32_PS];
+  __shared__ float2 fs[WG_WARPS][3][W32_P];
   if (G.nstage < 2) return;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int cond = cond_order[blockIdx.y];
@@ -428,24 +412,25 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
   const bool gok = l0 + 3 <= top && gbase + 8 * s <= G.ngrid;
   const int64_t m = (int64_t)cond * G.nmap + G.mapoff[k] + grp;
   const int64_t first = lo_all[m] + (int64_t)part * WG_THREADS, last = hi_all[m];
-  const float tj = lane < 2 * W32_P ? W32_T[lane >> 1] : 0.0f;
-  for (int i = lane; i < 3 * W32_PS; i += 32) fs[w][i / W32_PS][i % W32_PS] = make_float2(0.0f, 0.0f);
+  if (lane < W32_P)
+    for (int v = 0; v < 3; ++v) fs[w][v][lane] = make_float2(0.0f, 0.0f);
   __syncwarp();
   wing_scan<false>(S, rec_all + (int64_t)cond * nlines, first, last, (int64_t)G.parts[k] * WG_THREADS, gbase, s, gok,
                    u2, u1, true, G.ngrid, [&](int total) {
                      const int nw = (total + 31) >> 5;
+#pragma unroll 1
                      for (int v = 0; v < 3; ++v) {  // own panel, then a share of the coarser ones
                        const int wide = 1 << v, pan = w >> v;
                        const float sp = (float)(s * wide);
-                       list_nodes(S.rec, S.mask[(v == 0 ? LST_L0 : v == 1 ? LST_L1 : LST_L2) + pan], nw,
-                                  w & (wide - 1), wide, S.q[w], lane, tj, ((float)pan + 0.5f) * sp - 0.5f, sp,
-                                  fs[w][v]);
+                       list_nodes<32>(S.rec, S.mask[(v == 0 ? LST_L0 : v == 1 ? LST_L1 : LST_L2) + pan], nullptr, nw,
+                                      w & (wide - 1), wide, S.q[w], lane, nullptr, ((float)pan + 0.5f) * sp - 0.5f,
+                                      sp, fs[w][v]);
                      }
                    });
   __syncthreads();
   float *F = F_all + (int64_t)cond * G.fslots * W32_PS;
   const int np = G.parts[k];
-  auto val = [&](int ww, int v) { return fs[ww][v][lane].x - fs[ww][v][lane].y; };
+  auto val = [&](int ww, int v) { return lane < W32_P ? fs[ww][v][lane].x - fs[ww][v][lane].y : 0.0f; };
   if (lane < W32_PS) {
     const int64_t i0 = (int64_t)grp * 8 + w;
     if (i0 < G.npan[l0]) F[(G.foff[l0] + i0 * np + part) * W32_PS + lane] = val(w, 0);
@@ -464,34 +449,49 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
 }
 
 // Interpolation tables: [side][k][16] of a child's nodes in its parent (side 0:
-// the lower half), then [k][32] of the leaf's points.
+// the lower half), [k][32] of the leaf's points, the nodes.
 constexpr int W32_TABM = 2 * W32_P * W32_PS;
-constexpr int W32_TAB = W32_TABM + W32_P * WG_S0;
+constexpr int W32_TABT = W32_TABM + W32_P * WG_S0;
 
-// The values at a panel's nodes as a common part (hi + lo, the same on every
-// lane) and deviations from it (node j on lane j): the polynomial of the
-// deviations carries their smaller rounding down the tree.
-struct WingVal {
-  float hi, lo, dev;
+// The values at a panel's nodes: a common part (hi + lo) and deviations from
+// it.  The polynomial of the deviations carries their smaller rounding down
+// the tree.
+struct __align__(16) WingVal {
+  float dev[W32_P];
+  float hi, lo, pad[2];
 };
 
-// the values at this lane's node of a child (M: the lane's row of the child's
-// matrix), plus the child's own node sums f
-__device__ __forceinline__ WingVal wing_child(const float (&M)[W32_P], const WingVal &v, float f) {
+// Both children of a panel at once: lanes 0 .. 11 the nodes of the lower half,
+// lanes 16 .. 27 those of the upper (M: the lane's row of its child's matrix),
+// plus the children's own node sums f.  The side `side` (or both, side < 0) is
+// written to out[0] / out[1] (out + side for one side).
+__device__ __forceinline__ void wing_children(const float (&M)[W32_P], const WingVal &v, float f, int lane, int side,
+                                              WingVal *out) {
+  const float vh = v.hi, vl = v.lo;  // `out` may be v itself
   float r = 0.0f;
 #pragma unroll
-  for (int k = 0; k < W32_P; ++k) r = fmaf(M[k], __shfl_sync(0xffffffffu, v.dev, k), r);
+  for (int k = 0; k < W32_P; ++k) r = fmaf(M[k], v.dev[k], r);
   r += f;
-  const float mid = __shfl_sync(0xffffffffu, r, W32_P / 2);
-  WingVal o;
-  float e;
-  o.hi = v.hi + mid;
-  const float z = o.hi - v.hi;
-  e = (v.hi - (o.hi - z)) + (mid - z);
-  o.lo = v.lo + e;
-  o.dev = r - mid;
-  return o;
+  const float mid = __shfl_sync(0xffffffffu, r, (lane & 16) + W32_P / 2);
+  const int j = lane & 15;
+  if (side < 0 || (lane >> 4) == side) {
+    WingVal &o = out[side < 0 ? lane >> 4 : 0];
+    if (j < W32_P) o.dev[j] = r - mid;
+    if (j == 15) {
+      const float h = vh + mid, z = h - vh;
+      o.hi = h;
+      o.lo = vl + ((vh - (h - z)) + (mid - z));
+    }
+  }
+  __syncwarp();
 }
+
+// Lists of a warp's own lines: its panel's halves and leaves, and point by point
+// on the leaves (GH1 throughout, or per point).
+enum { SUB_H = 0, SUB_L = 2, SUB_G1 = 6, SUB_D = 10, SUB_N = 14 };
+// Leaf lists up to this length are run point by point: at one point a lane that
+// costs a line no more than a short list's nodes.
+constexpr int W32_LEAF_MIN = 6;
 
 __global__ void __launch_bounds__(WG_THREADS, 4)
     k_wing_near32(const LineRec32 *__restrict__ rec_all, int64_t nlines, const int32_t *__restrict__ lo_all,
@@ -501,192 +501,197 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
                   double *__restrict__ kappa_all) {
   constexpr int NL = 4;              // leaves of a warp's panel
   constexpr int s = NL * WG_S0;      // its points
+  constexpr int NV = 9;              // node sums of a warp: own panel, pair, quarter; two halves; four leaves
   __shared__ WingSmem S;
-  __shared__ float2 fs[WG_WARPS][9][W32_PS];  // own panel, pair, quarter; its two halves; its four leaves
-  __shared__ uint16_t s_uq[WG_WARPS][64];
-  __shared__ float s_top[W32_PS], s_ref[2];
+  __shared__ float2 fs[WG_WARPS][NV][W32_P];
+  __shared__ uint16_t s_uq[WG_WARPS][WG_CAP];  // lines not taken on the warp's panel or coarser
+  __shared__ uint32_t s_sub[WG_WARPS][SUB_N][WG_WORDS];
+  __shared__ WingVal s_top;
+  __shared__ float s_T[W32_P];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int cond = cond_order[blockIdx.y];
   const int ngrid = G.ngrid;
   const int64_t gbase = (int64_t)blockIdx.x * 8 * s;
   const int top = wing_top(G, cst[cond].wmax);
-  const float tj = lane < 2 * W32_P ? W32_T[lane >> 1] : 0.0f;
-  for (int i = lane; i < 9 * W32_PS; i += 32) fs[w][i / W32_PS][i % W32_PS] = make_float2(0.0f, 0.0f);
-  if (w == 0) {
-    // the values at the nodes of the group's own panel (level 5) from the
-    // coarser levels, coarsest first
-    const float *F = F_all + (int64_t)cond * G.fslots * W32_PS;
-    WingVal v{0.0f, 0.0f, 0.0f};
-    for (int l = top; l >= wing_level(1); --l) {
-      const int64_t p = gbase / ((int64_t)WG_S0 << l);
-      if (p >= G.npan[l]) continue;  // not on the grid in full: nor is any coarser one
-      const int np = G.parts[(l - 2) / 3];
-      const float *Fp = F + (G.foff[l] + p * np) * W32_PS + (lane & 15);
-      float f = 0.0f;
-      for (int i = 0; i < np; ++i) f += Fp[i * W32_PS];
-      float M[W32_P];
-#pragma unroll
-      for (int k = 0; k < W32_P; ++k) M[k] = tab[((int)(p & 1) * W32_P + k) * W32_PS + (lane & 15)];
-      v = wing_child(M, v, f);
-    }
-    if (lane < W32_PS) s_top[lane] = v.dev;
-    if (lane == 0) s_ref[0] = v.hi, s_ref[1] = v.lo;
-  }
+  if (lane < W32_P)
+    for (int v = 0; v < NV; ++v) fs[w][v][lane] = make_float2(0.0f, 0.0f);
+  if (tid < W32_P) s_T[tid] = tab[W32_TABT + tid];
   __syncwarp();
   const int64_t p0 = gbase + w * s;
   float sum[NL], comp[NL];
 #pragma unroll
   for (int k = 0; k < NL; ++k) sum[k] = comp[k] = 0.0f;
   uint16_t *q = S.q[w], *uq = s_uq[w];
-  const float flane = (float)lane;
+  uint32_t *sub = s_sub[w][0];
   const int64_t m = (int64_t)cond * G.nmap + blockIdx.x;
   const int left = (int)min((int64_t)s, (int64_t)ngrid - p0);  // points of the panel on the grid
+  const int base = w * s;                                      // the panel's first point in the group
   wing_scan<true>(
       S, rec_all + (int64_t)cond * nlines, lo_all[m], hi_all[m], WG_THREADS, gbase, s,
       top >= 5 && gbase + 8 * s <= ngrid, top >= 4, top >= 3, top >= 2, ngrid, [&](int total) {
         const int nw = (total + 31) >> 5;
-        for (int v = 0; v < 3; ++v) {
-          const int wide = 1 << v, pan = w >> v;
-          const float sp = (float)(s * wide);
-          list_nodes(S.rec, S.mask[(v == 0 ? LST_L0 : v == 1 ? LST_L1 : LST_L2) + pan], nw, w & (wide - 1), wide, q,
-                     lane, tj, ((float)pan + 0.5f) * sp - 0.5f, sp, fs[w][v]);
-        }
-        // lines not taken on the panel, 32 at a time: its halves, its leaves,
-        // and point by point
+        // lines not taken on the panel: its halves, its leaves, point by point
         int n = 0;
         for (int wd = 0; wd < nw; ++wd) {
           const uint32_t b = S.mask[LST_U + w][wd];
-          const bool fin = wd + 1 >= nw;
           if ((b >> lane) & 1u) uq[n + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(32 * wd + lane);
           n += __popc(b);
-          __syncwarp();
-          while (n >= 32 || (fin && n > 0)) {
-            const bool in = lane < n;
-            const int j = uq[in ? lane : 0];
-            const WingLine &L = S.rec[j];
-            const int base = w * s;  // the panel's first point
-            const int ilo = L.ilo - base, ihi = L.ihi - base;
-            float dl[NL], dh[NL];
+        }
+        __syncwarp();
+        const int nu = (n + 31) >> 5;
+        int nleaf[NL];
 #pragma unroll
-            for (int p = 0; p < NL; ++p) {
-              dl[p] = wing_off(L, base + 32 * p);
-              dh[p] = wing_off(L, base + 32 * p + 31);
-            }
-            uint32_t mh[2], ml[NL], md[NL], m1[NL];
-            bool kh[2];
-            {
-              const WingReach T(L, 64.0f);
-#pragma unroll
-              for (int p = 0; p < 2; ++p) {
-                kh[p] = in && top >= 1 && 64 * (p + 1) <= left && ilo <= 64 * p && ihi >= 64 * p + 63 &&
-                        T.takes(L, dl[2 * p], dh[2 * p + 1]);
-                mh[p] = __ballot_sync(0xffffffffu, kh[p]);
-              }
-            }
-            {
-              const WingReach T(L, 32.0f);
-#pragma unroll
-              for (int p = 0; p < NL; ++p) {
-                const bool rest = in && !kh[p >> 1];
-                const bool k0 = rest && top >= 0 && 32 * (p + 1) <= left && ilo <= 32 * p && ihi >= 32 * p + 31 &&
-                                T.takes(L, dl[p], dh[p]);
-                ml[p] = __ballot_sync(0xffffffffu, k0);
-                // point by point, unless every covered point is a core point;
-                // GH1 throughout where the nearest covered point is
-                const int lo = max(ilo, 32 * p), hi = min(ihi, 32 * p + 31);
-                const float ul = fmaf((float)(base + lo) - L.c, L.beta, L.nphi);
-                const float uh = fmaf((float)(base + hi) - L.c, L.beta, L.nphi);
-                const float rl = fmaf(ul, ul, L.a2), rh = fmaf(uh, uh, L.a2);
-                const bool d = rest && !k0 && lo <= hi && fmaxf(rl, rh) >= 100.0f;
-                const bool g1 = d && fminf(rl, rh) >= 1.0e6f && (L.a2 >= 1.0e6f || (ul > 0.0f) == (uh > 0.0f));
-                md[p] = __ballot_sync(0xffffffffu, d && !g1);
-                m1[p] = __ballot_sync(0xffffffffu, g1);
-              }
-            }
+        for (int p = 0; p < NL; ++p) nleaf[p] = 0;
 #pragma unroll 1
-            for (int p = 0; p < 2 + NL; ++p) {
-              const uint32_t mk = p == 0 ? mh[0] : p == 1 ? mh[1] : p == 2 ? ml[0] : p == 3 ? ml[1] : p == 4 ? ml[2] : ml[3];
-              if (mk == 0) continue;
-              if ((mk >> lane) & 1u) q[__popc(mk & ((1u << lane) - 1u))] = (uint16_t)j;
-              __syncwarp();
-              const float sp = p < 2 ? 64.0f : 32.0f;
-              const float mid = (float)base + (p < 2 ? 64.0f * p + 31.5f : 32.0f * (p - 2) + 15.5f);
-              node_accumulate(fs[w][3 + p], lane, nodes_few(S.rec, q, __popc(mk), lane, tj, mid, sp));
-              __syncwarp();
+        for (int t = 0; t < nu; ++t) {
+          const bool in = 32 * t + lane < n;
+          const WingLine L = S.rec[uq[in ? 32 * t + lane : 0]];
+          const int ilo = L.ilo - base, ihi = L.ihi - base;
+          uint32_t mine = 0;  // lane k keeps list k's mask
+          float dl[NL], dh[NL];
+#pragma unroll
+          for (int p = 0; p < NL; ++p) {
+            dl[p] = wing_off(L, base + 32 * p);
+            dh[p] = wing_off(L, base + 32 * p + 31);
+          }
+          const WingReach T1(L, 64.0f), T0(L, 32.0f);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const bool kh = in && top >= 1 && 64 * (h + 1) <= left && ilo <= 64 * h && ihi >= 64 * h + 63 &&
+                            T1.takes(L, dl[2 * h], dh[2 * h + 1]);
+            uint32_t m = __ballot_sync(0xffffffffu, kh);
+            if (lane == SUB_H + h) mine = m;
+#pragma unroll
+            for (int p = 2 * h; p < 2 * h + 2; ++p) {
+              const bool rest = in && !kh;
+              const bool k0 = rest && top >= 0 && 32 * (p + 1) <= left && ilo <= 32 * p && ihi >= 32 * p + 31 &&
+                              T0.takes(L, dl[p], dh[p]);
+              m = __ballot_sync(0xffffffffu, k0);
+              if (lane == SUB_L + p) mine = m;
+              nleaf[p] += __popc(m);
+              // point by point, unless every covered point is a core point;
+              // GH1 throughout where the nearest covered point is
+              const int lo = max(ilo, 32 * p), hi = min(ihi, 32 * p + 31);
+              const float ul = fmaf((float)(base + lo - L.c), L.beta, L.nphi);
+              const float uh = fmaf((float)(base + hi - L.c), L.beta, L.nphi);
+              const float rl = fmaf(ul, ul, L.a2), rh = fmaf(uh, uh, L.a2);
+              const bool d = rest && !k0 && lo <= hi && fmaxf(rl, rh) >= 100.0f;
+              const bool g1 = d && fminf(rl, rh) >= 1.0e6f && (L.a2 >= 1.0e6f || (ul > 0.0f) == (uh > 0.0f));
+              m = __ballot_sync(0xffffffffu, g1);
+              if (lane == SUB_G1 + p) mine = m;
+              m = __ballot_sync(0xffffffffu, d && !g1);
+              if (lane == SUB_D + p) mine = m;
+            }
+          }
+          if (lane < SUB_N) sub[lane * WG_WORDS + t] = mine;
+        }
+        __syncwarp();
+        // the panels' node sums: own, pair, quarter (shared with the other
+        // warps), halves, leaves
+#pragma unroll 1
+        for (int v = 0; v < NV; ++v) {
+          if (v >= 5) {
+            const int nl = v == 5 ? nleaf[0] : v == 6 ? nleaf[1] : v == 7 ? nleaf[2] : nleaf[3];
+            if (nl <= W32_LEAF_MIN) continue;
+          }
+          const bool out = v < 3;
+          const int wide = out ? 1 << v : 1, pan = w >> v;
+          const float sp = out ? (float)(s * wide) : v < 5 ? 64.0f : 32.0f;
+          const float mid = out ? ((float)pan + 0.5f) * sp - 0.5f
+                                : (float)base + ((float)(v < 5 ? v - 3 : v - 5) + 0.5f) * sp - 0.5f;
+          const uint32_t *mk = out ? S.mask[(v == 0 ? LST_L0 : v == 1 ? LST_L1 : LST_L2) + pan]
+                                   : sub + (v < 5 ? SUB_H + v - 3 : SUB_L + v - 5) * WG_WORDS;
+          list_nodes<8>(S.rec, mk, out ? nullptr : uq, out ? nw : nu, out ? w & (wide - 1) : 0, wide, q, lane, s_T, mid,
+                        sp, fs[w][v]);
+        }
+#pragma unroll 1
+        for (int p = 0; p < NL; ++p) {
+          const int ip = base + 32 * p + lane;
+          const bool few = (p == 0 ? nleaf[0] : p == 1 ? nleaf[1] : p == 2 ? nleaf[2] : nleaf[3]) <= W32_LEAF_MIN;
+#pragma unroll 1
+          for (int t = 0; t < nu; ++t) {
+            const uint32_t m1 = sub[(SUB_G1 + p) * WG_WORDS + t];
+            const uint32_t md = sub[(SUB_D + p) * WG_WORDS + t] | (few ? sub[(SUB_L + p) * WG_WORDS + t] : 0u);
+            if ((m1 | md) == 0) continue;
+            // the word's lines in order: first those GH1 throughout
+            const int n1 = __popc(m1), nd = __popc(md);
+            const uint32_t lt = (1u << lane) - 1u;
+            if ((m1 >> lane) & 1u) q[__popc(m1 & lt)] = uq[32 * t + lane];
+            if ((md >> lane) & 1u) q[n1 + __popc(md & lt)] = uq[32 * t + lane];
+            __syncwarp();
+            float part = 0.0f;
+#pragma unroll 2
+            for (int i = 0; i < n1; ++i) {
+              const WingLine &D = S.rec[q[i]];
+              const float u = fmaf((float)(ip - D.c), D.beta, D.nphi);
+              const float v = fmaf(D.P1, fast_rcp(fmaf(u, u, D.a2)), part);
+              part = ip >= D.ilo && ip <= D.ihi ? v : part;
+            }
+            // core points (r2 < 100) are left to the core kernel
+#pragma unroll 2
+            for (int i = n1; i < n1 + nd; ++i) {
+              const WingLine &D = S.rec[q[i]];
+              const float a2 = D.a2, c3 = D.c3;
+              const float u = fmaf((float)(ip - D.c), D.beta, D.nphi);
+              const float r2 = fmaf(u, u, a2);
+              const float pp = fmaf(r2, r2 - 3.0f, fmaf(6.0f, a2, 2.25f));
+              const float nn = c3 * fmaf(r2, r2 - 1.5f, fmaf(4.0f, a2, 1.5f));
+              const bool gh1 = r2 >= 1.0e6f;
+              const float v = fmaf(gh1 ? D.P1 : nn, fast_rcp(gh1 ? r2 : r2 * pp), part);
+              part = ip >= D.ilo && ip <= D.ihi && r2 >= 100.0f ? v : part;
             }
 #pragma unroll
-            for (int p = 0; p < NL; ++p) {
-              const float pos = (float)(base + 32 * p) + flane;
-              const int ip = base + 32 * p + lane;
-              float part = 0.0f;
-              for (uint32_t mk = m1[p]; mk; mk &= mk - 1) {
-                const WingLine &D = S.rec[uq[__ffs(mk) - 1]];
-                const float u = fmaf(pos - D.c, D.beta, D.nphi);
-                const float t = fmaf(D.P1, fast_rcp(fmaf(u, u, D.a2)), part);
-                part = ip >= D.ilo && ip <= D.ihi ? t : part;
-              }
-              // core points (r2 < 100) are left to the core kernel
-              for (uint32_t mk = md[p]; mk; mk &= mk - 1) {
-                const WingLine &D = S.rec[uq[__ffs(mk) - 1]];
-                const float u = fmaf(pos - D.c, D.beta, D.nphi);
-                const float r2 = fmaf(u, u, D.a2);
-                const float pp = fmaf(r2, r2 - 3.0f, D.C);
-                const float nn = fmaf(r2, fmaf(D.c3, r2, D.c45), D.c2);
-                const bool gh1 = r2 >= 1.0e6f;
-                const float t = fmaf(gh1 ? D.P1 : nn, fast_rcp(gh1 ? r2 : r2 * pp), part);
-                part = ip >= D.ilo && ip <= D.ihi && r2 >= 100.0f ? t : part;
-              }
-              kahan_add(sum[p], comp[p], part);
-            }
-            __syncwarp();
-            n = max(0, n - 32);
-            const uint16_t e = uq[32 + lane];
-            __syncwarp();
-            uq[lane] = e;
+            for (int k = 0; k < NL; ++k)
+              if (k == p) kahan_add(sum[k], comp[k], part);
             __syncwarp();
           }
         }
       });
+  __syncthreads();  // the batch's shared memory is free
+  WingVal *tv = reinterpret_cast<WingVal *>(S.rec) + w * 10;
+  float M[W32_P];
+  if (top >= 0) {
+#pragma unroll
+    for (int k = 0; k < W32_P; ++k) M[k] = tab[((lane >> 4) * W32_P + k) * W32_PS + (lane & 15)];
+    if (w == 0) {
+      // the values at the nodes of the group's own panel (level 5) from the
+      // coarser levels, coarsest first
+      const float *F = F_all + (int64_t)cond * G.fslots * W32_PS;
+      if (lane < 16) reinterpret_cast<float *>(&s_top)[lane] = 0.0f;
+      __syncwarp();
+      for (int l = top; l >= wing_level(1); --l) {
+        const int64_t p = gbase / ((int64_t)WG_S0 << l);
+        if (p >= G.npan[l]) continue;  // not on the grid in full: nor is any coarser one
+        const int np = G.parts[(l - 2) / 3];
+        const float *Fp = F + (G.foff[l] + p * np) * W32_PS + (lane & 15);
+        float f = 0.0f;
+        for (int i = 0; i < np; ++i) f += Fp[i * W32_PS];
+        wing_children(M, s_top, f, lane, (int)(p & 1), &s_top);
+      }
+    }
+  }
   __syncthreads();
   if (p0 >= ngrid) return;
-  float far[NL], ref[NL];
-#pragma unroll
-  for (int k = 0; k < NL; ++k) far[k] = ref[k] = 0.0f;
-  WingVal v0[NL];
   if (top >= 0) {
-    const int j = lane & 15;
-    float M0[W32_P], M1[W32_P];
-#pragma unroll
-    for (int k = 0; k < W32_P; ++k) {
-      M0[k] = tab[k * W32_PS + j];
-      M1[k] = tab[(W32_P + k) * W32_PS + j];
-    }
+    // down the tree: the quarter, the pair, the warp's panel, its halves, its leaves
+    const int j = min(lane & 15, W32_P - 1), h4 = w & 4, h2 = w & 6, side = lane >> 4;
     auto val = [&](int ww, int v) { return fs[ww][v][j].x - fs[ww][v][j].y; };
-    auto child = [&](int side, const WingVal &v, float f) { return side ? wing_child(M1, v, f) : wing_child(M0, v, f); };
-    const int h = w & 4, g2 = w & 6;
-    WingVal v{s_ref[0], s_ref[1], s_top[j]};
-    v = child((w >> 2) & 1, v, (val(h, 2) + val(h + 1, 2)) + (val(h + 2, 2) + val(h + 3, 2)));
-    v = child((w >> 1) & 1, v, val(g2, 1) + val(g2 + 1, 1));
-    v = child(w & 1, v, val(w, 0));
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const WingVal vh = child(p, v, val(w, 3 + p));
-      v0[2 * p] = child(0, vh, val(w, 5 + 2 * p));
-      v0[2 * p + 1] = child(1, vh, val(w, 6 + 2 * p));
-    }
-    const float *Lm = tab + W32_TABM + lane;
-#pragma unroll
-    for (int k = 0; k < W32_P; ++k) {
-      const float lk = Lm[k * WG_S0];
-#pragma unroll
-      for (int p = 0; p < NL; ++p) far[p] = fmaf(lk, __shfl_sync(0xffffffffu, v0[p].dev, k), far[p]);
+#pragma unroll 1
+    for (int t = 0; t < 6; ++t) {
+      const float f = t == 0 ? (val(h4, 2) + val(h4 + 1, 2)) + (val(h4 + 2, 2) + val(h4 + 3, 2))
+                      : t == 1 ? val(h2, 1) + val(h2 + 1, 1)
+                      : t == 2 ? val(w, 0)
+                               : val(w, t == 3 ? 3 + side : t == 4 ? 5 + side : 7 + side);
+      // tv[0 .. 2]: quarter, pair, own; 3, 4: halves; 5 .. 8: leaves
+      const WingVal &v = t == 0 ? s_top : tv[t - 1];
+      wing_children(M, v, f, lane, t == 0 ? (w >> 2) & 1 : t == 1 ? (w >> 1) & 1 : t == 2 ? w & 1 : -1,
+                    t < 3 ? tv + t : t == 3 ? tv + 3 : t == 4 ? tv + 5 : tv + 7);
     }
 #pragma unroll
-    for (int p = 0; p < NL; ++p) ref[p] = v0[p].hi, far[p] += v0[p].lo;
+    for (int k = 0; k < W32_P; ++k) M[k] = tab[W32_TABM + k * WG_S0 + lane];
   }
   const int E = cst[cond].scale_exp;
   const bool core = cst[cond].core_w1 != 0, unit = weight == 1.0;
-  const double scale = ldexp(weight, E);
   const float *kcore = kcore_all + (int64_t)cond * ngrid;
   double *kappa = kappa_all + (int64_t)cond * ngrid;
 #pragma unroll
@@ -701,10 +706,18 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
         lo += (hi - (t - z)) + (x - z);
         hi = t;
       };
-      add(ref[p]);
-      add(far[p]);
+      if (top >= 0) {
+        const WingVal &v = tv[5 + p];
+        float far = 0.0f;
+#pragma unroll
+        for (int k = 0; k < W32_P; ++k) far = fmaf(M[k], v.dev[k], far);
+        add(v.hi);
+        add(far);
+        lo += v.lo;
+      }
       if (core) add(kcore[i]);
-      const double v = unit ? scaled_to_double(hi, E) + scaled_to_double(lo, E) : scale * ((double)hi + (double)lo);
+      const double v = unit ? scaled_to_double(hi, E) + scaled_to_double(lo, E)
+                            : ldexp(weight, E) * ((double)hi + (double)lo);
       kappa[i] = accumulate ? kappa[i] + v : v;
     }
   }
@@ -729,7 +742,8 @@ static void lagrange(int P, const double *t, double x, double *out) {
 void wing_tables(int P, int PS, std::vector<double> &tab) {
   std::vector<double> t(P), r(P);
   for (int j = 0; j < P; ++j) t[j] = cos((2 * j + 1) * PI / (2 * P));
-  tab.assign((size_t)2 * P * PS + (size_t)P * WG_S0, 0.0);
+  tab.assign((size_t)2 * P * PS + (size_t)P * WG_S0 + P, 0.0);
+  for (int j = 0; j < P; ++j) tab[(size_t)2 * P * PS + (size_t)P * WG_S0 + j] = t[j];
   for (int side = 0; side < 2; ++side)
     for (int j = 0; j < P; ++j) {
       lagrange(P, t.data(), (side ? 0.5 : -0.5) + 0.5 * t[j], r.data());

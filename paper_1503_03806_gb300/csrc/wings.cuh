@@ -42,7 +42,7 @@ constexpr int WG_LEVELS = 23;               // the coarsest panels have 2^27 poi
 constexpr int WG_STAGES = 7;
 constexpr int WG_WARPS = 8;                 // panels (warps) a group
 constexpr int WG_THREADS = 32 * WG_WARPS;
-constexpr int WG_CAP = 2 * WG_THREADS;      // lines of a batch in shared memory
+constexpr int WG_CAP = 480;                // lines of a batch in shared memory (32 * 15)
 
 // The lowest level of a stage's groups (one panel a warp).
 __host__ __device__ inline int wing_level(int stage) { return 3 * stage + 2; }
