@@ -51,23 +51,19 @@ __device__ __forceinline__ unsigned long long surr_reserve(SurrQueue *sq) {
   return g.shfl(base, 0) + g.thread_rank();
 }
 
-// One core evaluation (x^2 + y^2 < 100): S' K by Algorithm 916, or 0 after
-// appending the point to the surrogate's queue when its cell is validated
-// (the queue's kernel adds it later).
-__device__ __forceinline__ float core_point(const LineRec32 &L, float x, int i, int srow, SurrQueue *sq,
-                                         int cond, const float *w) {
-  if (srow >= 0 && surr_route(sq, srow, x)) {
-    const unsigned long long slot = surr_reserve(sq);
-    if (slot < sq->cap) {
-      sq->idx[slot] = i;
-      sq->cond[slot] = cond;
-      sq->w[slot] = L.Sp;
-      sq->x[slot] = x;
-      sq->y[slot] = L.a;
-      return 0.0f;
-    }
-  }
-  return L.Sp * k916_f32(x, L.a, L.erfcx_a, L.sig1, w);
+// Appends one core evaluation (x^2 + y^2 < 100) to the surrogate's queue when
+// its cell is validated (the queue's kernel adds it later); false when it has
+// to be evaluated here.
+__device__ __forceinline__ bool core_routed(float Sp, float a, float x, int i, int srow, SurrQueue *sq, int cond) {
+  if (srow < 0 || !surr_route(sq, srow, x)) return false;
+  const unsigned long long slot = surr_reserve(sq);
+  if (slot >= sq->cap) return false;
+  sq->idx[slot] = i;
+  sq->cond[slot] = cond;
+  sq->w[slot] = Sp;
+  sq->x[slot] = x;
+  sq->y[slot] = a;
+  return true;
 }
 
 // ---- FP32 line pipeline: a ring of F32_STAGES chunks of candidate lines,
@@ -290,33 +286,43 @@ __global__ void __launch_bounds__(BLOCK, MINB)
 
 // ------------------------------------------------- Algorithm 916 cores --
 // The points of every line's core (fma(u, u, a^2) < 100 in the FP32
-// arithmetic of k_voigt_f32, which skips exactly these points), one thread
-// per grid point: the candidate lines of a warp's 32 points are those whose
+// arithmetic of the wing kernels, which skip exactly these points), one thread
+// per grid point.  The candidate lines of a warp's 32 points are those whose
 // reference index lies within the condition's core reach of them (found by
-// the warp's own search), screened by each line's core range from the pack;
-// each thread adds S' K(|u|, a) of the lines whose core holds its point, in
-// list order (deterministic), or appends the point to the surrogate's queue
-// when routed.  The per-point sums go to kcore (every point written), so the
-// kernel can run beside k_voigt_f32; k_core_add then adds them into kappa,
-// rescaled like the main kernel's sums.  Few lines' cores overlap at a point
-// (~4 at the medium workload), so the plain FP32 sum loses < 1e-7 relative.
+// the warp's own search); the lanes screen 32 of them at a time by their core
+// ranges and prepare those that reach the warp, one a lane, in shared memory;
+// the warp then takes them in list order (deterministic): it fills the line's
+// table of series weights and Gauss-Hermite constants, and each lane whose
+// point lies in the core adds S' K(|u|, a) by one of the two forms of
+// voigt_core.cuh (or appends the point to the surrogate's queue when routed).
+// The per-point sums go to kcore (every point written), so the kernel can run
+// beside others; they are added into kappa rescaled like the main sums.
+// Kahan-compensated: hundreds of cores can overlap at a point.
 constexpr int CORE_BLOCK = 128;
+
+struct __align__(16) CoreLine {
+  float c, beta, nphi, a2;  // c: reference index from the warp's first point
+  float y, A, D, Sp;
+  float xc2;                // core_inner(y)
+  int lo, hi, pad;          // core points
+};
 
 template <bool COUNT>
 __global__ void __launch_bounds__(CORE_BLOCK)
     k_core_f32(const LineRec32 *__restrict__ rec_all, const int2 *__restrict__ core_all, int64_t nlines,
                const int32_t *__restrict__ ckey, int ngrid, float *__restrict__ kcore_all, CondStats *cst,
                SurrQueue *sq, const int *__restrict__ core_blk_all) {
-  // per warp: the series weights of the line being evaluated
-  __shared__ float s_w[CORE_BLOCK / 32][32];
+  constexpr int NW = CORE_BLOCK / 32;
+  __shared__ CoreLine s_line[NW][32];
+  __shared__ __align__(16) float s_c[NW][24];
+  __shared__ float4 s_g[NW][4];
   const int cond = blockIdx.y;
   const int cw1 = cst[cond].core_w1;
-  if (cw1 == 0) return;  // no line of the condition has a core (k_core_add skips it too)
+  if (cw1 == 0) return;  // no line of the condition has a core (its sums are not read)
   // each warp finds its own 32 points' candidate lines: no CTA barrier
   const int64_t A = (int64_t)blockIdx.x * CORE_BLOCK + (threadIdx.x & ~31);
   if (A >= ngrid) return;  // warp-uniform
-  const int lane = threadIdx.x & 31;
-  float *w = s_w[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t B = min(A + 32, (int64_t)ngrid);
   // The candidate window: the condition's largest core reach, or, when that
   // is below a block, the largest reach of the lines whose reference index
@@ -339,34 +345,86 @@ __global__ void __launch_bounds__(CORE_BLOCK)
   const LineRec32 *rec = rec_all + (int64_t)cond * nlines;
   const int2 *core = core_all + (int64_t)cond * nlines;
   const int i = (int)(A + lane);
-  float v = 0.0f;
+  // the lane's part of a line's tables: series term n = lane + 1, and the
+  // Gauss-Hermite pair lane & 3
+  float gauss = 0.0f;
+  if (lane < CORE_TERMS) {
+    const int n = lane + 1;
+    gauss = n < A916_TERMS_F32 ? ldexpf(A916_GAUSS_F32[n], 4 * n) : A916_GAUSS_HIGH[n - A916_TERMS_F32];
+    gauss *= 0.15915494f;  // h / pi
+  }
+  const float n2 = 0.25f * (float)((lane + 1) * (lane + 1));
+  // nodes t^2 and weights 2 w / pi of the 8-node rule
+  const int j = lane & 3;
+  const float t2 = j == 0 ? 0.14530352f : j == 1 ? 1.33909729f : j == 2 ? 3.9269635f : 8.58863569f;
+  const float w2 = j == 0 ? 0.420899261f : j == 1 ? 0.132291069f : j == 2 ? 1.08721817e-2f : 1.27071899e-4f;
+  CoreLine *sl = s_line[wid];
+  float *sc = s_c[wid];
+  float4 *sg = s_g[wid];
+  const float flane = (float)lane;
+  float v = 0.0f, vc = 0.0f;
   unsigned long long n916 = 0, nterm = 0;
-  // the line loop is warp-uniform: each line's weight table is built by the
-  // whole warp when any lane's point lies in its core
-  for (int64_t l = first; l < last; ++l) {
-    const int2 cr = core[l];  // the line's core points, a superset of r^2 < 100
-    bool in = i < ngrid && i >= cr.x && i <= cr.y;
-    float u = 0.0f;
-    const LineRec32 &L = rec[l];
-    if (in) {
-      u = fmaf((float)(i - L.c), L.beta, -L.phi_k);
-      in = fmaf(u, u, L.a2) < 100.0f;
-    }
-    if (!__any_sync(0xffffffffu, in)) continue;
-    w[lane] = a916_weight_f32(lane + 1, L.a2);
+  for (int64_t l0 = first; l0 < last; l0 += 32) {
+    const int64_t l = l0 + lane;
+    int2 cr = make_int2(1, 0);
+    if (l < last) cr = core[l];
+    uint32_t todo = __ballot_sync(0xffffffffu, cr.x <= cr.y && cr.x < B && cr.y >= A);
+    if (todo == 0) continue;
     __syncwarp();
-    if (in) {
-      v += core_point(L, fabsf(u), i, surr_row(sq, L.a), sq, cond, w);
-      if (COUNT) {
+    if ((todo >> lane) & 1u) {
+      const LineRec32 L = rec[l];
+      CoreLine q;
+      q.c = (float)(L.c - (int)A);  // within 2^23 points of a core point: exact
+      q.beta = L.beta;
+      q.nphi = -L.phi_k;
+      q.a2 = L.a2;
+      q.y = L.a;
+      q.A = fmaf(-0.318309886f * L.a, L.sig1, L.erfcx_a);
+      q.D = (L.a > 1.0e-15f ? __fdividef(0.318309886f, L.a) : 0.0f) - 2.0f * q.A;
+      q.Sp = L.Sp;
+      q.xc2 = core_inner(L.a);
+      q.lo = cr.x;
+      q.hi = cr.y;
+      sl[lane] = q;
+    }
+    __syncwarp();
+    for (; todo; todo &= todo - 1) {
+      const CoreLine &L = sl[__ffs(todo) - 1];
+      const float u = fmaf(flane - L.c, L.beta, L.nphi);
+      const float y = L.y, y2 = L.a2, xc2 = L.xc2;
+      bool in = i < ngrid && i >= L.lo && i <= L.hi && fmaf(u, u, y2) < 100.0f;
+      const float x = fabsf(u), x2 = x * x;
+      if (COUNT && in) {
         int n0, n1;
-        a916_range_f32(fabsf(u), n0, n1);
+        a916_range_f32(x, n0, n1);
         ++n916;
         nterm += (unsigned long long)(n1 - n0 + 1);
       }
+      if (sq && in) in = !core_routed(L.Sp, y, x, i, surr_row(sq, y), sq, cond);
+      const bool inner = in && x2 < xc2;
+      const unsigned bi = __ballot_sync(0xffffffffu, inner);
+      const unsigned bo = __ballot_sync(0xffffffffu, in && !inner);
+      if (bi) {
+        if (lane < 24) sc[lane] = gauss * y * core_rcp(n2 + y2);
+      }
+      if (bo) {
+        if (lane < 4) {
+          const float al = w2 * y;
+          sg[lane] = make_float4(y2 - t2, al, al * (t2 + t2), 4.0f * y2 * t2);
+        }
+      }
+      __syncwarp();
+      float K = 0.0f;
+      if (bi && inner) K = k916_inner(x, x2, y, L.A, L.D, sc);
+      if (bo && in && !inner) {
+        K = k916_outer(x2, sg);
+        if (y < 1.0e-8f) K += core_gauss(x, x2);
+      }
+      if (in) kahan_add(v, vc, L.Sp * K);
+      __syncwarp();  // the tables are rebuilt for the next line
     }
-    __syncwarp();  // the table is rebuilt for the next line
   }
-  if (i < ngrid) kcore_all[(int64_t)cond * ngrid + i] = v;
+  if (i < ngrid) kcore_all[(int64_t)cond * ngrid + i] = v - vc;
   if (COUNT) {
     for (int o = 16; o > 0; o >>= 1) {
       n916 += __shfl_down_sync(0xffffffffu, n916, o);
