@@ -168,6 +168,9 @@ void helk_destroy(helk_ctx *c) {
   if (c->core_blk) cudaFree(c->core_blk);
   if (c->wingF) cudaFree(c->wingF);
   if (c->wing_tab32) cudaFree(c->wing_tab32);
+  if (c->wing_tab64) cudaFree(c->wing_tab64);
+  if (c->ext64) cudaFree(c->ext64);
+  if (c->kcore64) cudaFree(c->kcore64);
   for (int st = 0; st < HELK_NSTAGES; ++st)
     for (cudaEvent_t e : c->ev[st]) cudaEventDestroy(e);
   if (cur >= 0) cudaSetDevice(cur);
@@ -336,7 +339,7 @@ static helk_status ensure_conds(helk_ctx *c, int n_cond) {
 // Whether a call takes the interpolated-wings route, and its geometry.
 static bool wing_route(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g,
                        WingGeom *out) {
-  if (o.precision != HELK_PREC_F32_KAHAN || o.count_regions) return false;
+  if (o.count_regions) return false;
   double half = (double)g->n;
   if (cut->kind == HELK_CUT_ABS) half = std::min(half, cut->value / g->dnu);
   if (cut->kind == HELK_CUT_LORENTZ) half = std::min(half, cut->cap / g->dnu);
@@ -370,7 +373,8 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
       HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming), "core stream"));
   }
   HELK_TRY(ensure_tiles(c, (wg ? (int64_t)wg->nmap : ntiles) * n_cond));
-  if (wg) HELK_TRY(ensure_wing32(c, n_cond, *wg));
+  if (wg)
+    HELK_TRY(o.precision == HELK_PREC_F32_KAHAN ? ensure_wing32(c, n_cond, *wg) : ensure_wing64(c, n_cond, *wg));
   if (o.surrogate && !c->squeue) {
     // routed-evaluation queue: 2^24 entries (entries beyond it fall back to
     // Algorithm 916 in the Voigt kernel)
@@ -399,13 +403,16 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
 // conditions: single != NULL passes the one condition by value, otherwise
 // they are read from c->cond_dev.
 static helk_status prepare_lines(helk_ctx *c, int n_cond, const CondArgs *single, double mass,
-                                 const helk_cutoff *cut, const helk_grid *g, const helk_opts &o) {
+                                 const helk_cutoff *cut, const helk_grid *g, const helk_opts &o, bool wings) {
   HELK_TRY(cuda_check(c, cudaMemsetAsync(c->cstats, 0, n_cond * sizeof(CondStats), c->stream), "stats"));
   for (int k = 0; k < n_cond; ++k)
     HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->cstats[k].wmax, 0xFF, sizeof(long long), c->stream), "stats"));
   if (c->nlines > 0) {
-    HELK_TRY(cuda_check(c, launch_lineprep(c, n_cond, single, mass, *cut, *g, o.precision != HELK_PREC_F32_KAHAN),
-                        "lineprep"));
+    const bool f64 = o.precision != HELK_PREC_F32_KAHAN;
+    if (f64 && wings)
+      HELK_TRY(cuda_check(c, cudaMemsetAsync(c->core_blk, 0, (size_t)core_blocks(g->n) * n_cond * 4, c->stream),
+                          "lineprep"));
+    HELK_TRY(cuda_check(c, launch_lineprep(c, n_cond, single, mass, *cut, *g, f64, f64 && wings), "lineprep"));
     if (o.precision == HELK_PREC_F32_KAHAN) {
       HELK_TRY(cuda_check(c, cudaMemsetAsync(c->core_blk, 0, (size_t)core_blocks(g->n) * n_cond * 4, c->stream),
                           "pack32"));
@@ -425,9 +432,15 @@ static int shape_points(int precision, int shape) {
 
 // The interpolated-wings route: candidate map, condition order, the far
 // kernel with the Algorithm 916 cores beside it on the side stream, then the
-// near kernel, which writes kappa.
+// near kernel, which writes kappa.  FP64 form: the cores share the far
+// kernel's launch.
 static helk_status run_wings(helk_ctx *c, int n_cond, const helk_grid *g, const helk_opts &o, double *kappa,
                              const WingGeom &wg) {
+  if (o.precision != HELK_PREC_F32_KAHAN) {
+    HELK_TRY(cuda_check(c, launch_wingmap(c, n_cond, wg), "wing map"));
+    HELK_TRY(cuda_check(c, launch_wing_far64(c, n_cond, wg, *g), "voigt wings"));
+    return cuda_check(c, launch_wing_near64(c, n_cond, wg, *g, o, kappa), "voigt wings");
+  }
   HELK_TRY(cuda_check(c, launch_cond_order(c, n_cond), "condition order"));
   if (o.surrogate)
     HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->squeue->count, 0, sizeof(unsigned long long), c->stream), "voigt"));
@@ -495,7 +508,7 @@ helk_status helk_opacity(helk_ctx *c, double T, double P, double mass, const hel
   HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n, wg));
   const CondArgs one{T, P, o.q_ratio, 0.0};
   stage_begin(c, HELK_STAGE_LINEPREP);
-  HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o));
+  HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, wg != nullptr));
   stage_end(c, HELK_STAGE_LINEPREP);
   if (c->nlines > 0) {
     stage_begin(c, HELK_STAGE_VOIGT);
@@ -533,7 +546,7 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
   }
   HELK_TRY(ensure_call_buffers(c, 1, o, max_tiles, g->n, nullptr));
   const CondArgs one{T, P, o.q_ratio, 0.0};
-  HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o));
+  HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, false));
   cudaEvent_t e0, e1;
   HELK_TRY(cuda_check(c, cudaEventCreate(&e0), "autotune"));
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -590,8 +603,9 @@ static std::string batch_key(const helk_ctx *c, int n_cond, double mass, const h
   snprintf(b2, sizeof b2, "|%d%d%d%d%d%d|%p|%p|%p|%p", c->has_E, c->has_gself, c->has_ncoll, c->has_delta,
            c->has_mass, c->has_weight, (const void *)c->cond_host, (const void *)c->cond_dev,
            (const void *)c->cond_order, (const void *)c->core_rng);
-  char b3[64];
-  snprintf(b3, sizeof b3, "|%p|%p", (const void *)c->core_blk, (const void *)c->wingF);
+  char b3[128];
+  snprintf(b3, sizeof b3, "|%p|%p|%p|%p|%p", (const void *)c->core_blk, (const void *)c->wingF, (const void *)c->ext64,
+           (const void *)c->kcore64, (const void *)c->ckey32);
   return std::string(b) + b2 + b3;
 }
 
@@ -670,16 +684,17 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   // record budget (one chunk unless the list is very long), each chunk one
   // captured graph; the chunks share the record, tile-map and core buffers
   // and follow each other on the stream.
+  WingGeom geom;
+  const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
   const int64_t rec_line =
       (int64_t)sizeof(LineRec64) +
-      (o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2)) : 0);
+      (o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2))
+                                          : wg ? (int64_t)sizeof(WingExt64) : 0);
   const int64_t per_cond = std::max<int64_t>(c->nlines, 1) * rec_line;
   const int gmax = (int)std::max<int64_t>(1, std::min<int64_t>(n_cond, c->batch_budget / per_cond));
   const int nchunk = (n_cond + gmax - 1) / gmax;
   const int chunk = (n_cond + nchunk - 1) / nchunk;
   HELK_TRY(ensure_conds(c, n_cond));
-  WingGeom geom;
-  const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
   HELK_TRY(ensure_call_buffers(c, chunk, o, ntiles, g->n, wg));
   if (!c->cap_stream)
     HELK_TRY(cuda_check(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "graph stream"));
@@ -708,7 +723,7 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
           st = cuda_check(c, cudaMemcpyAsync(c->cond_dev, c->cond_host, nk * sizeof(CondArgs),
                                              cudaMemcpyHostToDevice, c->stream),
                           "graph capture");
-          if (st == HELK_OK) st = prepare_lines(c, nk, nullptr, mass, cut, g, o);
+          if (st == HELK_OK) st = prepare_lines(c, nk, nullptr, mass, cut, g, o, wg != nullptr);
           if (st == HELK_OK) st = run_voigt(c, nk, g, o, kap, shape, tile, ntiles, wg);
           const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
           if (st == HELK_OK) st = cuda_check(c, e, "graph capture");

@@ -59,6 +59,18 @@ struct __align__(16) LineRec64 {
 };
 static_assert(sizeof(LineRec64) == 64, "LineRec64 must be 64 bytes");
 
+// Beside a LineRec64 on the interpolated-wings route: the grid indices at which
+// the method changes, by the FP64 definition of r^2 at a point (Sec. 2.4):
+// GH1 for i <= g1l and i >= g1r, the core (Algorithm 916) for g3l < i < g3r, GH3
+// between; the centre as the nearest grid index c (clamped to the grid) plus
+// frac, and, in grid steps, gamma = a / ku and the outer node sqrt(3/2) / ku.
+struct __align__(16) WingExt64 {
+  int32_t g1l, g1r, g3l, g3r;
+  int32_t c;
+  float frac, gamma, node;
+};
+static_assert(sizeof(WingExt64) == 32, "WingExt64 must be 32 bytes");
+
 struct __align__(16) LineRec32 {
   int32_t c;       // reference grid index near the shifted centre
   int32_t ilo, ihi;
@@ -161,6 +173,11 @@ struct helk_ctx {
   void *wingF = nullptr;
   int64_t wingF_cap = 0;
   float *wing_tab32 = nullptr;
+  double *wing_tab64 = nullptr;
+  helk::WingExt64 *ext64 = nullptr;  // FP64 form: per line and condition
+  int64_t ext64_cap = 0;
+  double *kcore64 = nullptr;         // FP64 form: core sums (n_cond x n points)
+  int64_t kcore64_cap = 0;
   cudaStream_t side_stream = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   int64_t rec_cap = 0, rec32_cap = 0;
@@ -329,9 +346,10 @@ cudaError_t launch_sort_lines(helk_ctx *c, int64_t n);  // orders SoA by nu0
 // the one condition passed by value.  Records of condition k start at
 // k * nlines; tile maps at k * ntiles.
 // a916_f64: also the FP64 Algorithm 916 per-line factors (erfcx(a), S1(a)),
-// which only the FP64 form reads.
+// which only the FP64 form reads.  wings: also the WingExt64 and the core reach
+// of the FP64 interpolated-wings route.
 cudaError_t launch_lineprep(helk_ctx *c, int n_cond, const CondArgs *single, double mass,
-                            const helk_cutoff &cut, const helk_grid &g, bool a916_f64);
+                            const helk_cutoff &cut, const helk_grid &g, bool a916_f64, bool wings);
 cudaError_t launch_pack32(helk_ctx *c, int n_cond, const helk_grid &g);
 cudaError_t launch_tilemap(helk_ctx *c, int n_cond, const helk_grid &g, int tile, int64_t ntiles);
 // Conditions ordered by decreasing evaluation count (largest work first).

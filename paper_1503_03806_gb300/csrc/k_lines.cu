@@ -6,6 +6,7 @@
 // evaluates a point (a, ku) must be the correctly rounded results of the
 // operations written here, with no contraction into FMA.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -255,6 +256,53 @@ struct PrepArgs {
 //   a = sqrt(ln2) Gamma_L / Gamma_D, ku = sqrt(ln2)/Gamma_D,
 //   S' = S sqrt(ln2/pi) / Gamma_D, window from the cutoff   (Sec. 2.4)
 // blockIdx.y is the condition; records of condition k start at k * n.
+// r^2 >= R at grid index i, by the FP64 definition (each operation rounded)
+__device__ __forceinline__ bool prep_beyond(const PrepArgs &A, double i, double nu0p, double ku, double a2, double R) {
+  const double u = ((A.nu_min + i * A.dnu) - nu0p) * ku;
+  return u * u + a2 >= R;
+}
+
+// The grid indices around a line's centre at which r^2 crosses R: the last one
+// on the left with r^2 >= R (-1: none on the grid) and the first on the right (n:
+// none).  r^2 is monotone on either side of the centre (cf: the index nearest to
+// it, unclamped), so an estimate (w: the crossing's distance in steps) is moved
+// until the definition holds; past a few steps by bisection.
+__device__ __forceinline__ void prep_cross(const PrepArgs &A, double cf, double w, double nu0p, double ku, double a2,
+                                           double R, int &left, int &right) {
+  const double n = (double)A.ngrid;
+  // left: the largest i in [-1, cf] with r^2 >= R (index -1 stands for "none")
+  double hi = fmin(cf, n - 1.0), i = fmin(fmax(floor(cf - w), -1.0), hi);
+  int step = 0;
+  while (i >= 0.0 && step < 6 && !prep_beyond(A, i, nu0p, ku, a2, R)) i -= 1.0, ++step;
+  while (i + 1.0 <= hi && step < 6 && prep_beyond(A, i + 1.0, nu0p, ku, a2, R)) i += 1.0, ++step;
+  if (step >= 6) {
+    double lo = -1.0;  // beyond at lo (or lo = -1), not beyond past hi
+    while (lo < hi) {
+      const double m = floor(0.5 * (lo + hi + 1.0));
+      if (prep_beyond(A, m, nu0p, ku, a2, R)) lo = m;
+      else hi = m - 1.0;
+    }
+    i = lo;
+  }
+  left = (int)fmax(i, -1.0);
+  // right: the smallest i in [cf, n] with r^2 >= R (index n stands for "none")
+  double lo = fmax(cf, 0.0);
+  i = fmax(fmin(ceil(cf + w), n), lo);
+  step = 0;
+  while (i < n && step < 6 && !prep_beyond(A, i, nu0p, ku, a2, R)) i += 1.0, ++step;
+  while (i - 1.0 >= lo && step < 6 && prep_beyond(A, i - 1.0, nu0p, ku, a2, R)) i -= 1.0, ++step;
+  if (step >= 6) {
+    double h = n;
+    while (lo < h) {
+      const double m = floor(0.5 * (lo + h));
+      if (prep_beyond(A, m, nu0p, ku, a2, R)) h = m;
+      else lo = m + 1.0;
+    }
+    i = h;
+  }
+  right = (int)fmin(i, n);
+}
+
 __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const double *__restrict__ S0,
                            const double *__restrict__ El, const double *__restrict__ gair,
                            const double *__restrict__ gself, const double *__restrict__ ncoll,
@@ -262,7 +310,8 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
                            const double *__restrict__ lweight, PrepArgs A,
                            const CondArgs *__restrict__ conds, CondArgs single,
                            LineRec64 *__restrict__ rec_all, double *__restrict__ ckey,
-                           CondStats *cst_all, int a916_f64) {
+                           CondStats *cst_all, int a916_f64, WingExt64 *__restrict__ ext_all,
+                           int32_t *__restrict__ ckey32, int *__restrict__ core_blk_all, int nblk) {
   const int cond = blockIdx.y;
   const CondArgs C = conds ? conds[cond] : single;
   LineRec64 *rec = rec_all + (int64_t)cond * n;
@@ -270,6 +319,7 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
   unsigned long long evals = 0;
   long long wmax = -1;
   unsigned long long spmax = 0;
+  int cw1 = 0;
   const double vth = sqrt(2.0 * LN2 * KB * C.T / (A.mass * AMU)) / CLIGHT;
   const double tfac_half = sqrt(T0 / C.T);  // (T0/T)^n for the usual n = 1/2
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
@@ -351,6 +401,42 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
     if (ck < -4.0e15) ck = -4.0e15;
     if (ck > 4.0e15) ck = 4.0e15;
     if (cond == 0) ckey[l] = ck;
+    if (ext_all) {
+      WingExt64 x;
+      const double idnu = 1.0 / A.dnu, pos = (nu0p - A.nu_min) * idnu;
+      const double cf = rint(pos), cc = fmin(fmax(cf, 0.0), (double)(A.ngrid - 1));
+      const float step = (float)(1.0 / (ku * A.dnu));  // a Doppler unit in grid steps
+      x.c = (int)cc;
+      x.frac = (float)(pos - cc);
+      x.gamma = (float)a * step;
+      x.node = 1.2248f * step;
+      if (r.a2 >= R2_GH1) {
+        x.g1l = x.g3l = INT_MAX;
+        x.g1r = x.g3r = INT_MIN;
+      } else {
+        prep_cross(A, cf, (double)(sqrtf((float)(R2_GH1 - r.a2)) * step), nu0p, ku, r.a2, R2_GH1, x.g1l, x.g1r);
+        if (r.a2 >= R2_GH3) {
+          x.g3l = INT_MAX;
+          x.g3r = INT_MIN;
+        } else {
+          prep_cross(A, cf, (double)(sqrtf((float)(R2_GH3 - r.a2)) * step), nu0p, ku, r.a2, R2_GH3, x.g3l, x.g3r);
+        }
+      }
+      ext_all[(int64_t)cond * n + l] = x;
+      // the core reach, as k_pack32 keeps it for the FP32 form
+      const long long key = (long long)ck;
+      const int k32 = (int)min(max(key, -2147483647ll), 2147483647ll);
+      if (cond == 0) ckey32[l] = k32;
+      const int clo = r.a2 >= R2_GH3 ? 1 : max(r.ilo, x.g3l + 1), chi = r.a2 >= R2_GH3 ? 0 : min(r.ihi, x.g3r - 1);
+      int w1 = 0;
+      if (clo <= chi) w1 = (int)min(max(key - clo, chi - key) + 1, 2000000000ll);
+      cw1 = max(cw1, w1);
+      const int blk = min(max(k32 >> 12, 0), nblk - 1);  // CORE_BLK_PTS = 2^12
+      const unsigned peers = __match_any_sync(__activemask(), blk);
+      const int wblk = __reduce_max_sync(peers, w1);
+      if ((int)(threadIdx.x & 31) == __ffs(peers) - 1 && wblk > 0)
+        atomicMax(&core_blk_all[(int64_t)cond * nblk + blk], wblk);
+    }
     if (r.ihi >= r.ilo) {
       evals += (unsigned long long)(r.ihi - r.ilo + 1);
       long long c0 = (long long)ck;
@@ -368,11 +454,13 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
     if (w2 > wmax) wmax = w2;
     unsigned long long s2 = __shfl_down_sync(0xffffffffu, spmax, o);
     if (s2 > spmax) spmax = s2;
+    cw1 = max(cw1, __shfl_down_sync(0xffffffffu, cw1, o));
   }
   if ((threadIdx.x & 31) == 0) {
     if (evals) atomicAdd(&cst->evals, evals);
     if (wmax >= 0) atomicMax(&cst->wmax, wmax);
     if (spmax) atomicMax(&cst->spmax_bits, spmax);
+    if (cw1 > 0) atomicMax(&cst->core_w1, cw1);
   }
 }
 
@@ -384,7 +472,7 @@ static int line_blocks(helk_ctx *c, int64_t n, int n_cond) {
 }
 
 cudaError_t launch_lineprep(helk_ctx *c, int n_cond, const CondArgs *single, double mass,
-                            const helk_cutoff &cut, const helk_grid &g, bool a916_f64) {
+                            const helk_cutoff &cut, const helk_grid &g, bool a916_f64, bool wings) {
   const int64_t n = c->nlines;
   if (n <= 0) return cudaSuccess;
   PrepArgs A{mass, cut.kind, cut.value, cut.cap, g.nu_min, g.dnu, g.n};
@@ -395,7 +483,8 @@ cudaError_t launch_lineprep(helk_ctx *c, int n_cond, const CondArgs *single, dou
       n, c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair, c->has_gself ? c->gself : nullptr,
       c->has_ncoll ? c->ncoll : nullptr, c->has_delta ? c->delta : nullptr,
       c->has_mass ? c->lmass : nullptr, c->has_weight ? c->lweight : nullptr, A,
-      single ? nullptr : c->cond_dev, one, c->rec64, c->ckey, c->cstats, a916_f64 ? 1 : 0);
+      single ? nullptr : c->cond_dev, one, c->rec64, c->ckey, c->cstats, a916_f64 ? 1 : 0,
+      wings ? c->ext64 : nullptr, wings ? c->ckey32 : nullptr, wings ? c->core_blk : nullptr, core_blocks(g.n));
   return cudaGetLastError();
 }
 

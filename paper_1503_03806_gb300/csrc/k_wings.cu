@@ -30,6 +30,7 @@ WingGeom wing_geometry(int64_t n, double half, int num_sms) {
   WingGeom g;
   memset(&g, 0, sizeof g);
   g.ngrid = (int)n;
+  g.lvl0 = n < (int64_t)2 * num_sms * WG_WARPS * (WG_S0 << 2) ? 0 : 2;
   const double widest = std::min(2.0 * half + 1.0, (double)n);
   g.lmax = -1;
   for (int l = 0; l < WG_LEVELS; ++l) {
@@ -38,10 +39,10 @@ WingGeom wing_geometry(int64_t n, double half, int num_sms) {
     if ((double)s <= widest) g.lmax = l;
   }
   g.nstage = 1;
-  while (g.nstage < WG_STAGES && wing_level(g.nstage) <= g.lmax) ++g.nstage;
+  while (g.nstage < WG_STAGES && wing_level(g, g.nstage) <= g.lmax) ++g.nstage;
   int64_t slots = 0, map = 0, far = 0;
   for (int k = 0; k < g.nstage; ++k) {
-    const int l0 = wing_level(k);
+    const int l0 = wing_level(g, k);
     const int64_t span = (int64_t)WG_S0 << (l0 + 3);
     g.groups[k] = (int)((n + span - 1) / span);
     // the candidates of a group are shared among enough CTAs to fill the GPU
@@ -74,7 +75,7 @@ __global__ void k_wingmap(int64_t nlines, const double *__restrict__ ckey, WingG
   if (m >= G.nmap) return;  // warp-uniform
   int k = 0;
   while (k + 1 < G.nstage && m >= G.mapoff[k + 1]) ++k;
-  const int64_t span = (int64_t)WG_S0 << (wing_level(k) + 3);
+  const int64_t span = (int64_t)WG_S0 << (wing_level(G, k) + 3);
   const int64_t A = (int64_t)(m - G.mapoff[k]) * span;
   const int64_t B = min(A + span, (int64_t)G.ngrid);
   const long long W = cst[cond].wmax;
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(WG_THREADS, 3)
   const int cond = cond_order[blockIdx.y];
   int k = G.nstage - 1, b = blockIdx.x;
   while (k > 1 && b >= G.groups[k] * G.parts[k]) b -= G.groups[k] * G.parts[k], --k;
-  const int top = wing_top(G, cst[cond].wmax), l0 = wing_level(k);
+  const int top = wing_top(G, cst[cond].wmax), l0 = wing_level(G, k);
   if (l0 > top) return;  // no window holds a panel of this stage
   const int grp = b / G.parts[k], part = b % G.parts[k];
   const int64_t s = (int64_t)WG_S0 << l0;  // < 2^31 (l0 <= lmax)
@@ -493,15 +494,17 @@ enum { SUB_H = 0, SUB_L = 2, SUB_G1 = 6, SUB_D = 10, SUB_N = 14 };
 // costs a line no more than a short list's nodes.
 constexpr int W32_LEAF_MIN = 6;
 
+// NL: leaves of a warp's panel, 4 or 1 (WingGeom::lvl0 2 or 0).
+template <int NL>
 __global__ void __launch_bounds__(WG_THREADS, 4)
     k_wing_near32(const LineRec32 *__restrict__ rec_all, int64_t nlines, const int32_t *__restrict__ lo_all,
                   const int32_t *__restrict__ hi_all, WingGeom G, const int *__restrict__ cond_order,
                   const CondStats *__restrict__ cst, const float *__restrict__ F_all,
                   const float *__restrict__ tab, const float *__restrict__ kcore_all, double weight, int accumulate,
                   double *__restrict__ kappa_all) {
-  constexpr int NL = 4;              // leaves of a warp's panel
-  constexpr int s = NL * WG_S0;      // its points
-  constexpr int NV = 9;              // node sums of a warp: own panel, pair, quarter; two halves; four leaves
+  constexpr int s = NL * WG_S0;          // points of a warp's panel
+  constexpr int NH = NL / 2;             // its halves
+  constexpr int NV = NL == 1 ? 3 : 9;    // node sums of a warp: own panel, pair, quarter; halves; leaves
   __shared__ WingSmem S;
   __shared__ float2 fs[WG_WARPS][NV][W32_P];
   __shared__ uint16_t s_uq[WG_WARPS][WG_CAP];  // lines not taken on the warp's panel or coarser
@@ -528,7 +531,8 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
   const int base = w * s;                                      // the panel's first point in the group
   wing_scan<true>(
       S, rec_all + (int64_t)cond * nlines, lo_all[m], hi_all[m], WG_THREADS, gbase, s,
-      top >= 5 && gbase + 8 * s <= ngrid, top >= 4, top >= 3, top >= 2, ngrid, [&](int total) {
+      top >= G.lvl0 + 3 && gbase + 8 * s <= ngrid, top >= G.lvl0 + 2, top >= G.lvl0 + 1, top >= G.lvl0, ngrid,
+      [&](int total) {
         const int nw = (total + 31) >> 5;
         // lines not taken on the panel: its halves, its leaves, point by point
         int n = 0;
@@ -555,33 +559,37 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
             dh[p] = wing_off(L, base + 32 * p + 31);
           }
           const WingReach T1(L, 64.0f), T0(L, 32.0f);
+          bool kh[2] = {false, false};
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const bool kh = in && top >= 1 && 64 * (h + 1) <= left && ilo <= 64 * h && ihi >= 64 * h + 63 &&
-                            T1.takes(L, dl[2 * h], dh[2 * h + 1]);
-            uint32_t m = __ballot_sync(0xffffffffu, kh);
+          for (int h = 0; h < NH; ++h) {
+            kh[h] = in && top >= 1 && 64 * (h + 1) <= left && ilo <= 64 * h && ihi >= 64 * h + 63 &&
+                    T1.takes(L, dl[2 * h], dh[2 * h + 1]);
+            const uint32_t m = __ballot_sync(0xffffffffu, kh[h]);
             if (lane == SUB_H + h) mine = m;
+          }
 #pragma unroll
-            for (int p = 2 * h; p < 2 * h + 2; ++p) {
-              const bool rest = in && !kh;
-              const bool k0 = rest && top >= 0 && 32 * (p + 1) <= left && ilo <= 32 * p && ihi >= 32 * p + 31 &&
-                              T0.takes(L, dl[p], dh[p]);
-              m = __ballot_sync(0xffffffffu, k0);
+          for (int p = 0; p < NL; ++p) {
+            const bool rest = in && !kh[p >> 1];
+            bool k0 = false;
+            if (NL > 1) {
+              k0 = rest && top >= 0 && 32 * (p + 1) <= left && ilo <= 32 * p && ihi >= 32 * p + 31 &&
+                   T0.takes(L, dl[p], dh[p]);
+              const uint32_t m = __ballot_sync(0xffffffffu, k0);
               if (lane == SUB_L + p) mine = m;
               nleaf[p] += __popc(m);
-              // point by point, unless every covered point is a core point;
-              // GH1 throughout where the nearest covered point is
-              const int lo = max(ilo, 32 * p), hi = min(ihi, 32 * p + 31);
-              const float ul = fmaf((float)(base + lo - L.c), L.beta, L.nphi);
-              const float uh = fmaf((float)(base + hi - L.c), L.beta, L.nphi);
-              const float rl = fmaf(ul, ul, L.a2), rh = fmaf(uh, uh, L.a2);
-              const bool d = rest && !k0 && lo <= hi && fmaxf(rl, rh) >= 100.0f;
-              const bool g1 = d && fminf(rl, rh) >= 1.0e6f && (L.a2 >= 1.0e6f || (ul > 0.0f) == (uh > 0.0f));
-              m = __ballot_sync(0xffffffffu, g1);
-              if (lane == SUB_G1 + p) mine = m;
-              m = __ballot_sync(0xffffffffu, d && !g1);
-              if (lane == SUB_D + p) mine = m;
             }
+            // point by point, unless every covered point is a core point;
+            // GH1 throughout where the nearest covered point is
+            const int lo = max(ilo, 32 * p), hi = min(ihi, 32 * p + 31);
+            const float ul = fmaf((float)(base + lo - L.c), L.beta, L.nphi);
+            const float uh = fmaf((float)(base + hi - L.c), L.beta, L.nphi);
+            const float rl = fmaf(ul, ul, L.a2), rh = fmaf(uh, uh, L.a2);
+            const bool d = rest && !k0 && lo <= hi && fmaxf(rl, rh) >= 100.0f;
+            const bool g1 = d && fminf(rl, rh) >= 1.0e6f && (L.a2 >= 1.0e6f || (ul > 0.0f) == (uh > 0.0f));
+            uint32_t m = __ballot_sync(0xffffffffu, g1);
+            if (lane == SUB_G1 + p) mine = m;
+            m = __ballot_sync(0xffffffffu, d && !g1);
+            if (lane == SUB_D + p) mine = m;
           }
           if (lane < SUB_N) sub[lane * WG_WORDS + t] = mine;
         }
@@ -591,7 +599,7 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
 #pragma unroll 1
         for (int v = 0; v < NV; ++v) {
           if (v >= 5) {
-            const int nl = v == 5 ? nleaf[0] : v == 6 ? nleaf[1] : v == 7 ? nleaf[2] : nleaf[3];
+            const int nl = v == 5 ? nleaf[0] : v == 6 ? nleaf[1 % NL] : v == 7 ? nleaf[2 % NL] : nleaf[3 % NL];
             if (nl <= W32_LEAF_MIN) continue;
           }
           const bool out = v < 3;
@@ -607,7 +615,8 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
 #pragma unroll 1
         for (int p = 0; p < NL; ++p) {
           const int ip = base + 32 * p + lane;
-          const bool few = (p == 0 ? nleaf[0] : p == 1 ? nleaf[1] : p == 2 ? nleaf[2] : nleaf[3]) <= W32_LEAF_MIN;
+          const bool few =
+              NL > 1 && (p == 0 ? nleaf[0] : p == 1 ? nleaf[1 % NL] : p == 2 ? nleaf[2 % NL] : nleaf[3 % NL]) <= W32_LEAF_MIN;
 #pragma unroll 1
           for (int t = 0; t < nu; ++t) {
             const uint32_t m1 = sub[(SUB_G1 + p) * WG_WORDS + t];
@@ -654,15 +663,15 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
 #pragma unroll
     for (int k = 0; k < W32_P; ++k) M[k] = tab[((lane >> 4) * W32_P + k) * W32_PS + (lane & 15)];
     if (w == 0) {
-      // the values at the nodes of the group's own panel (level 5) from the
+      // the values at the nodes of the group's own panel from the
       // coarser levels, coarsest first
       const float *F = F_all + (int64_t)cond * G.fslots * W32_PS;
       if (lane < 16) reinterpret_cast<float *>(&s_top)[lane] = 0.0f;
       __syncwarp();
-      for (int l = top; l >= wing_level(1); --l) {
+      for (int l = top; l >= wing_level(G, 1); --l) {
         const int64_t p = gbase / ((int64_t)WG_S0 << l);
         if (p >= G.npan[l]) continue;  // not on the grid in full: nor is any coarser one
-        const int np = G.parts[(l - 2) / 3];
+        const int np = G.parts[(l - G.lvl0) / 3];
         const float *Fp = F + (G.foff[l] + p * np) * W32_PS + (lane & 15);
         float f = 0.0f;
         for (int i = 0; i < np; ++i) f += Fp[i * W32_PS];
@@ -677,11 +686,11 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
     const int j = min(lane & 15, W32_P - 1), h4 = w & 4, h2 = w & 6, side = lane >> 4;
     auto val = [&](int ww, int v) { return fs[ww][v][j].x - fs[ww][v][j].y; };
 #pragma unroll 1
-    for (int t = 0; t < 6; ++t) {
+    for (int t = 0; t < (NL == 1 ? 3 : 6); ++t) {
       const float f = t == 0 ? (val(h4, 2) + val(h4 + 1, 2)) + (val(h4 + 2, 2) + val(h4 + 3, 2))
                       : t == 1 ? val(h2, 1) + val(h2 + 1, 1)
                       : t == 2 ? val(w, 0)
-                               : val(w, t == 3 ? 3 + side : t == 4 ? 5 + side : 7 + side);
+                               : val(w, (t == 3 ? 3 + side : t == 4 ? 5 + side : 7 + side) % NV);
       // tv[0 .. 2]: quarter, pair, own; 3, 4: halves; 5 .. 8: leaves
       const WingVal &v = t == 0 ? s_top : tv[t - 1];
       wing_children(M, v, f, lane, t == 0 ? (w >> 2) & 1 : t == 1 ? (w >> 1) & 1 : t == 2 ? w & 1 : -1,
@@ -707,7 +716,7 @@ __global__ void __launch_bounds__(WG_THREADS, 4)
         hi = t;
       };
       if (top >= 0) {
-        const WingVal &v = tv[5 + p];
+        const WingVal &v = tv[NL == 1 ? 2 : 5 + p];
         float far = 0.0f;
 #pragma unroll
         for (int k = 0; k < W32_P; ++k) far = fmaf(M[k], v.dev[k], far);
@@ -783,7 +792,8 @@ cudaError_t launch_wing_far32(helk_ctx *c, int n_cond, const WingGeom &g) {
 
 cudaError_t launch_wing_near32(helk_ctx *c, int n_cond, const WingGeom &g, const helk_opts &o, double *kappa) {
   ++c->launches;
-  k_wing_near32<<<dim3((unsigned)g.groups[0], n_cond), WG_THREADS, 0, c->stream>>>(
+  auto near = g.lvl0 == 2 ? k_wing_near32<4> : k_wing_near32<1>;
+  near<<<dim3((unsigned)g.groups[0], n_cond), WG_THREADS, 0, c->stream>>>(
       c->rec32, c->nlines, c->tile_lo, c->tile_hi, g, c->cond_order, c->cstats, (const float *)c->wingF,
       c->wing_tab32, c->kcore, o.weight, o.accumulate, kappa);
   return cudaGetLastError();

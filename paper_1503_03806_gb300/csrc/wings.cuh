@@ -21,15 +21,19 @@
 // within the grid's range.
 //
 // A CTA works a group of 8 panels of one level, one a warp, and the two levels
-// above it: the near kernel (stage 0) takes the 128-point panels of level 2,
-// with levels 3 and 4 shared by its warps and levels 1 and 0 and the
-// point-by-point work below; the far kernel (stage k >= 1) levels 3k + 2 ..
-// 3k + 4.  A group scans its candidate lines once; lines taken at the group's
-// own level (3k + 5) or coarser are dropped at once.
+// above it: the near kernel (stage 0) takes the panels of level lvl0, with the
+// next two levels shared by its warps and any finer ones and the
+// point-by-point work below; the far kernel (stage k >= 1) levels lvl0 + 3k and
+// the next two.  A group scans its candidate lines once; lines taken at the
+// group's own level (lvl0 + 3k + 3) or coarser are dropped at once.  lvl0 is 2
+// (128 points a warp, 1024 a CTA), or 0 (32 and 256) on grids too short to give
+// every SM two CTAs of the former.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <vector>
 
 #include "helk_internal.cuh"
 
@@ -44,15 +48,13 @@ constexpr int WG_WARPS = 8;                 // panels (warps) a group
 constexpr int WG_THREADS = 32 * WG_WARPS;
 constexpr int WG_CAP = 480;                // lines of a batch in shared memory (32 * 15)
 
-// The lowest level of a stage's groups (one panel a warp).
-__host__ __device__ inline int wing_level(int stage) { return 3 * stage + 2; }
-
 struct WingGeom {
   int ngrid;
+  int lvl0;                     // level of the near kernel's panels (one a warp)
   int lmax;                     // coarsest level (-1: no panel of any level)
   int nstage;                   // stages with levels <= lmax (at least 1)
   int npan[WG_LEVELS];          // panels of a level that lie on the grid in full
-  int64_t foff[WG_LEVELS];      // node-sum slots: first of a level (levels >= 5)
+  int64_t foff[WG_LEVELS];      // node-sum slots: first of a level (of the far stages)
   int64_t fslots;               // node-sum slots of a condition
   int groups[WG_STAGES];        // groups of a stage
   int parts[WG_STAGES];         // CTAs that share a group's candidate lines
@@ -60,6 +62,9 @@ struct WingGeom {
   int nmap;                     // candidate-map entries of a condition
   int farblk;                   // CTAs of the far kernel, coarsest stage first
 };
+
+// The lowest level of a stage's groups (one panel a warp).
+__host__ __device__ inline int wing_level(const WingGeom &g, int stage) { return g.lvl0 + 3 * stage; }
 
 // The coarsest level worth working for windows of at most wmax points on
 // either side: a panel must lie inside a window.  Both kernels use it, so a
@@ -81,5 +86,15 @@ cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const WingGeom &g);
 helk_status ensure_wing32(helk_ctx *c, int n_cond, const WingGeom &g);
 cudaError_t launch_wing_far32(helk_ctx *c, int n_cond, const WingGeom &g);
 cudaError_t launch_wing_near32(helk_ctx *c, int n_cond, const WingGeom &g, const helk_opts &o, double *kappa);
+
+// the interpolation tables for P nodes, rows padded to PS (FP64, on the host):
+// [side][k][PS], [k][WG_S0], the nodes
+void wing_tables(int P, int PS, std::vector<double> &tab);
+
+// k_wings64.cu: the FP64 form (the far launch also takes the core sums)
+helk_status ensure_wing64(helk_ctx *c, int n_cond, const WingGeom &g);
+cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const WingGeom &g, const helk_grid &grid);
+cudaError_t launch_wing_near64(helk_ctx *c, int n_cond, const WingGeom &g, const helk_grid &grid, const helk_opts &o,
+                               double *kappa);
 
 }  // namespace helk

@@ -4,9 +4,9 @@ point sums: grids at the edges of leaves (32 points), warp panels (128),
 groups (1024) and coarser levels, windows from narrower than a panel to the
 whole grid, broad and narrow lines, centres on and off the grid.
 
-FP32 form: the stated bar of the form, 1e-5 where the opacity exceeds 1e-8 of
-the maximum (a line lost or taken twice on one panel is off by the order of
-its own share).
+FP64 form: 1e-9 at every point.  FP32 form: the stated bar of the form, 1e-5
+where the opacity exceeds 1e-8 of the maximum.  A line lost or taken twice on
+one panel is off by the order of its own share.
 """
 import numpy as np
 import pytest
@@ -34,6 +34,7 @@ def check(ctx, lines, case):
     from paper_1503_03806_gb300 import helk
     ctx.upload(lines)
     ko, _, _ = oracle.opacity(lines, case.oracle_cond(), nthreads=NTHREADS)
+    assert_rel(case.gpu(ctx).cpu().numpy(), ko, 1e-9, "FP64")
     k32 = case.gpu(ctx, precision=helk.HELK_PREC_F32_KAHAN).cpu().numpy()
     ctx.sync()
     sel = ko > 1e-8 * ko.max()
@@ -60,6 +61,14 @@ def test_dense_list_takes_several_batches(ctx):
     # more lines than a group's batch in shared memory, all of them near
     lines = synth.random_lines(6000, 78, 500.0, 520.0)
     check(ctx, lines, Case(700.0, 0.5, 18.0, (500.0, 0.01, 2000), ("abs", 8.0)))
+
+
+@pytest.mark.parametrize("dnu,nu", [(1e-6, 800.0), (5.0, 1.0)])
+def test_method_boundaries_on_extreme_grids(ctx, dnu, nu):
+    # thousands of grid points in a Doppler unit, and thousands of Doppler units
+    # between two points (a method changes from one point to the next)
+    lines = synth.random_lines(40, 80, nu, nu + 3000 * dnu, extra_fields=True)
+    check(ctx, lines, Case(1500.0, 0.1, 18.0, (nu - 20 * dnu, dnu, 3000), ("none",)))
 
 
 def test_accumulate_and_weight(ctx):

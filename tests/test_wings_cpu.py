@@ -21,7 +21,7 @@ def basis(P, x):
     return t, L / L.sum(1, keepdims=True)
 
 
-@pytest.mark.parametrize("P,eta,bound", [(12, 3.0, 2.4e-8)])
+@pytest.mark.parametrize("P,eta,bound", [(12, 3.0, 2.4e-8), (16, 5.0, 6e-15)])
 def test_truncation_bound(P, eta, bound):
     x = np.linspace(-1.0, 1.0, 801)
     t, L = basis(P, x)
