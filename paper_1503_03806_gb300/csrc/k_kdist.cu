@@ -1506,24 +1506,141 @@ __global__ void __launch_bounds__(TR_THREADS)
   if (threadIdx.x == 0) bins[b] = TrBin{k0, ldexp(1.0, F), s_jz, s_ju, 1, 0};
 }
 
-// The sum of the terms of one (bin, m) over the CTA, in a fixed order.
-__device__ __forceinline__ double tr_block_sum(double v, double *red) {
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < TR_THREADS / 32; ++w) t += red[w];
-  return t;  // on thread 0
+// ---- blocks of neighbouring values --------------------------------------
+// The sorted differences of a bin vary slowly, so a block of TR_BLK of them is
+// summed at once for every column mass at which it is narrow: with c a value
+// inside the block, R the power of two above max |D_j - c| and z = R M <= 1,
+//   sum_j e^{-D_j M} = e^{-c M} sum_p a_p (-z)^p,  a_p = sum_j ((D_j - c)/R)^p / p!,
+// p <= 17 (the first term left out is below 1 / 18! = 1.6e-16 of the block), p <=
+// 10 as float-float pairs and the rest, below 2.5e-8 of the sum, in FP32.  One
+// exponential and 18 terms instead of 64 exponentials.  Wider blocks (large m)
+// are summed value by value, beyond d = 32 (1.3e-14 a term against a sum >= 1)
+// in plain FP32.
+constexpr int TR_BLK = 64;
+constexpr int TR_P = 18;        // coefficients
+constexpr int TR_PP = 11;       // of them pairs
+constexpr int TR_ROWS = 2 + 2 * TR_PP + (TR_P - TR_PP);  // floats a block: c, R, pairs (high then low), the rest
+constexpr float TR_D32 = 32.0f;
+
+__host__ __device__ __forceinline__ int64_t tr_nblk(int64_t nb) { return (nb + TR_BLK - 1) / TR_BLK; }
+
+// 1 / p! as pairs
+__device__ constexpr float TR_IFACT[TR_P][2] = {
+    {1.0f, 0.0f}, {1.0f, 0.0f}, {0.5f, 0.0f},
+    {(float)(1.0 / 6.0), (float)(1.0 / 6.0 - (double)(float)(1.0 / 6.0))},
+    {(float)(1.0 / 24.0), (float)(1.0 / 24.0 - (double)(float)(1.0 / 24.0))},
+    {(float)(1.0 / 120.0), (float)(1.0 / 120.0 - (double)(float)(1.0 / 120.0))},
+    {(float)(1.0 / 720.0), (float)(1.0 / 720.0 - (double)(float)(1.0 / 720.0))},
+    {(float)(1.0 / 5040.0), (float)(1.0 / 5040.0 - (double)(float)(1.0 / 5040.0))},
+    {(float)(1.0 / 40320.0), (float)(1.0 / 40320.0 - (double)(float)(1.0 / 40320.0))},
+    {(float)(1.0 / 362880.0), (float)(1.0 / 362880.0 - (double)(float)(1.0 / 362880.0))},
+    {(float)(1.0 / 3628800.0), (float)(1.0 / 3628800.0 - (double)(float)(1.0 / 3628800.0))},
+    {(float)(1.0 / 39916800.0), 0.0f}, {(float)(1.0 / 479001600.0), 0.0f}, {(float)(1.0 / 6227020800.0), 0.0f},
+    {(float)(1.0 / 87178291200.0), 0.0f}, {(float)(1.0 / 1307674368000.0), 0.0f},
+    {(float)(1.0 / 20922789888000.0), 0.0f}, {(float)(1.0 / 355687428096000.0), 0.0f}};
+
+// The coefficients of one block of at most TR_BLK pairs (a warp; each lane
+// gives two, have: which of them exist), to out[row * stride].
+__device__ __forceinline__ void tr_block(float2 d0, float2 d1, bool have0, bool have1, int n, float *out,
+                                         int64_t stride) {
+  const int lane = threadIdx.x & 31;
+  float c = (have0 ? d0.x : 0.0f) / (float)n + (have1 ? d1.x : 0.0f) / (float)n;
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);  // about the mean
+  auto off = [&](float2 d) {
+    float s, e;
+    two_sum_f(d.x, -c, s, e);
+    e += d.y;
+    const float h = s + e;
+    return make_float2(h, e - (h - s));
+  };
+  float2 q0 = have0 ? off(d0) : make_float2(0.0f, 0.0f), q1 = have1 ? off(d1) : make_float2(0.0f, 0.0f);
+  float mx = fmaxf(fabsf(q0.x), fabsf(q1.x));
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  float R = 0.0f, ri = 0.0f;
+  if (mx > 0.0f) {
+    const int e = ((__float_as_int(mx) >> 23) & 0xFF) + 1;  // R = 2^(e - 127) > mx
+    // differences this small beside their values' scale: never narrow
+    R = e < 40 ? INFINITY : __int_as_float(e << 23);
+    ri = e < 40 ? 0.0f : __int_as_float((254 - e) << 23);
+  }
+  q0 = make_float2(q0.x * ri, q0.y * ri);
+  q1 = make_float2(q1.x * ri, q1.y * ri);
+  if (lane == 0) {
+    out[0] = c;
+    out[stride] = R;
+  }
+  float2 w0 = make_float2(have0 ? 1.0f : 0.0f, 0.0f), w1 = make_float2(have1 ? 1.0f : 0.0f, 0.0f);
+#pragma unroll
+  for (int g = 0; g < 3; ++g) {
+    float2 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      v[i] = ff_add(w0, w1);
+      w0 = ff_mul(w0, q0);
+      w1 = ff_mul(w1, q1);
+    }
+    const float2 r = ff_warp_sum8(v, lane);
+    const int p = 8 * g + (lane >> 2);
+    if ((lane & 3) == 0 && p < TR_P) {
+      const float2 a = ff_mul(r, make_float2(TR_IFACT[p][0], TR_IFACT[p][1]));
+      if (p < TR_PP) {
+        out[(2 + p) * stride] = a.x;
+        out[(2 + TR_PP + p) * stride] = a.y;
+      } else {
+        out[(2 + TR_PP + p) * stride] = a.x;
+      }
+    }
+  }
 }
 
-// One warp per (bin, column mass): a CTA takes one bin and TR_THREADS/32 of
-// its column masses at a time (no CTA barrier); each warp finds its range of
-// terms by a 32-ary search and sums them in a fixed order.
+// Coefficients of a bin's blocks (from its first pair on), rows [TR_ROWS][nblk].
+__global__ void __launch_bounds__(TR_THREADS)
+    k_trans_blocks(int64_t nb, const float2 *__restrict__ D, const TrBin *__restrict__ bins, float *__restrict__ blk) {
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
+  const TrBin B = bins[b];
+  if (!B.ok) return;
+  const int64_t nblk = tr_nblk(nb);
+  const float2 *Db = D + (int64_t)b * nb;
+  for (int64_t q = blockIdx.y * (TR_THREADS / 32) + (threadIdx.x >> 5); B.ju + q * TR_BLK < nb;
+       q += gridDim.y * (TR_THREADS / 32)) {
+    const int64_t j = B.ju + q * TR_BLK + lane;
+    const bool h0 = j < nb, h1 = j + 32 < nb;
+    const float2 z = make_float2(0.0f, 0.0f);
+    tr_block(h0 ? Db[j] : z, h1 ? Db[j + 32] : z, h0, h1, (int)min((int64_t)TR_BLK, nb - B.ju - q * TR_BLK),
+             blk + (int64_t)b * TR_ROWS * nblk + q, nblk);
+  }
+}
+
+// sum_p a_p (-z)^p of a block for z = R M (rows at a[row * stride])
+__device__ __forceinline__ float2 tr_poly(const float *a, int64_t stride, float R, float2 M) {
+  const float2 z = make_float2(-R * M.x, -R * M.y);  // exact
+  float f = a[(2 + TR_PP + TR_P - 1) * stride];
+#pragma unroll
+  for (int p = TR_P - 2; p >= TR_PP; --p) f = fmaf(f, z.x, a[(2 + TR_PP + p) * stride]);
+  float2 s = make_float2(f * z.x, 0.0f);
+#pragma unroll
+  for (int p = TR_PP - 1; p >= 0; --p) {
+    // s <- a_p + s z for p < TR_PP - 1; the first step adds the FP32 tail
+    if (p < TR_PP - 1) {
+      const float h = s.x * z.x;
+      const float e = fmaf(s.x, z.y, fmaf(s.y, z.x, fmaf(s.x, z.x, -h)));
+      s = make_float2(h, e);
+    }
+    float t, e;
+    two_sum_f(a[(2 + p) * stride], s.x, t, e);
+    s = make_float2(t, e + (a[(2 + TR_PP + p) * stride] + s.y));
+  }
+  const float h = s.x + s.y;
+  return make_float2(h, s.y - (h - s.x));
+}
+
+// A warp takes `per` (a power of two up to 32) column masses of a bin: the lanes
+// prepare one each (the FP64 work), then the warp runs through them, the lanes
+// sharing the bin's blocks.
 __global__ void __launch_bounds__(TR_THREADS)
     k_trans_direct(const double *__restrict__ sorted, int64_t nb, int nm, const double *__restrict__ m,
-                   const float2 *__restrict__ D, const TrBin *__restrict__ bins, TrConsts L,
-                   double *__restrict__ out) {
+                   const float2 *__restrict__ D, const TrBin *__restrict__ bins, const float *__restrict__ blk,
+                   TrConsts L, int per, double *__restrict__ out) {
   __shared__ float2 tab[TR_TAB];
   tr_table(tab);
   __syncthreads();
@@ -1531,67 +1648,84 @@ __global__ void __launch_bounds__(TR_THREADS)
   const double *k = sorted + (int64_t)b * nb;
   const float2 *Db = D + (int64_t)b * nb;
   const TrBin B = bins[b];
-  constexpr int WPB = TR_THREADS / 32;
-  for (int i = blockIdx.y * WPB + (threadIdx.x >> 5); i < nm; i += gridDim.y * WPB) {  // warp-uniform
-    const double mi = m[i];
-    double res = 0.0;
-    if (!B.ok) {  // the plain FP64 sum
-      double s = 0.0;
-      for (int64_t j = lane; j < nb; j += 32) s += exp(-k[j] * mi);
-      res = warp_sum(s) / (double)nb;
-    } else {
-      const double E0 = exp(-(B.k0 * mi));
-      if (E0 > 0.0) {  // else every term underflows, as e^{-k_0 m} does
-        // jmax: the first j >= ju with (k_j - k_0) m >= 87 (nb if none), the
-        // lanes probing 32 evenly spaced places of [lo, hi) a round
-        int64_t lo = B.ju, hi = nb;
-        while (hi > lo) {
-          const int64_t span = hi - lo;
-          const int64_t step = (span + 31) >> 5;
-          const int64_t p = lo + (int64_t)lane * step;
-          const bool past = p < hi && (k[p] - B.k0) * mi >= TR_DMAX;
-          const unsigned bal = __ballot_sync(0xffffffffu, past);
-          if (step == 1) {  // every place probed: the first past one, or hi
-            hi = bal ? lo + __ffs(bal) - 1 : hi;
-            break;
-          }
-          // the first lane past (the probes increase, so all later valid ones are past too);
-          // none past: the answer lies after the last valid probe
-          const int64_t last = (span - 1) / step;  // lanes 0..last probe inside [lo, hi)
-          if (bal) {
-            const int f = __ffs(bal) - 1;
-            const int64_t nhi = lo + (int64_t)f * step;
-            lo = f > 0 ? lo + (int64_t)(f - 1) * step + 1 : lo;
-            hi = nhi;
-          } else {
-            lo = lo + last * step + 1;
-          }
+  const int64_t nblk = tr_nblk(nb);
+  const int used = (int)((nb - B.ju + TR_BLK - 1) / TR_BLK);
+  const float *Bk = blk + (int64_t)b * TR_ROWS * nblk;
+  const int i = (blockIdx.y * (TR_THREADS / 32) + (threadIdx.x >> 5)) * per + lane;
+  if (i - lane >= nm) return;  // warp-uniform
+  const bool have = lane < per && i < nm;
+  const double mi = have ? m[i] : 0.0;
+  if (!B.ok) {  // the plain FP64 sum
+    for (int s = 0; s < per && i - lane + s < nm; ++s) {
+      const double ms = __shfl_sync(0xffffffffu, mi, s);
+      double t = 0.0;
+      for (int64_t j = lane; j < nb; j += 32) t += exp(-k[j] * ms);
+      t = warp_sum(t);
+      if (lane == 0) out[(int64_t)b * nm + i + s] = t / (double)nb;
+    }
+    return;
+  }
+  const double E0 = exp(-(B.k0 * mi));  // 0: every term underflows, as e^{-k_0 m} does
+  const double Md = mi * B.scale;
+  const bool pairs = Md < 0x1p107;  // else every pair has d >= 128
+  const float2 M = split_pair(pairs ? Md : 0.0);
+  const uint32_t run = __ballot_sync(0xffffffffu, have && E0 > 0.0 && pairs);
+  float2 mine = make_float2(0.0f, 0.0f);
+  double pd = 0.0;
+  if (B.ju > B.jz) {  // tiny differences, FP64
+    for (int64_t j = B.jz; j < B.ju; ++j) {
+      const double d = (k[j] - B.k0) * mi;
+      if (d < TR_DMAX) pd += exp(-d);
+    }
+  }
+  for (uint32_t left = run; left; left &= left - 1) {
+    const int s = __ffs(left) - 1;
+    const float2 Ms = make_float2(__shfl_sync(0xffffffffu, M.x, s), __shfl_sync(0xffffffffu, M.y, s));
+    float sh = 0.0f, sl = 0.0f, sf = 0.0f;
+    for (int q0 = 0; q0 < used; q0 += 32) {
+      const int q = q0 + lane;
+      float c = 0.0f, R = 0.0f;
+      if (q < used) {
+        c = Bk[q];
+        R = Bk[nblk + q];
+      }
+      const float low = isinf(R) ? 0.0f : (c - R) * Ms.x;
+      const bool use = q < used && low < (float)TR_DMAX;
+      const bool narrow = use && R * Ms.x <= 1.0f;
+      if (!__any_sync(0xffffffffu, use)) {
+        // later blocks hold larger values still
+        if (__all_sync(0xffffffffu, q >= used || !isinf(R))) break;
+      }
+      if (narrow) {
+        const float2 S = tr_poly(Bk + q, nblk, R, Ms);
+        const float2 d = ff_prod(make_float2(c, 0.0f), Ms);
+        tr_acc(sh, sl, ff_mul(ff_exp_neg(d.x, d.y, tab, L), S));
+      }
+      for (uint32_t wide = __ballot_sync(0xffffffffu, use && !narrow); wide; wide &= wide - 1) {
+        const int o = __ffs(wide) - 1;
+        const float lo = __shfl_sync(0xffffffffu, low, o);
+        const int64_t j = B.ju + (int64_t)(q0 + o) * TR_BLK + lane;
+        if (lo > TR_D32) {
+          const float d0 = j < nb ? Db[j].x * Ms.x : 1.0e3f, d1 = j + 32 < nb ? Db[j + 32].x * Ms.x : 1.0e3f;
+          if (d0 < (float)TR_DMAX) sf += expf(-d0);
+          if (d1 < (float)TR_DMAX) sf += expf(-d1);
+        } else {
+          const float2 far = make_float2(INFINITY, 0.0f);
+          const float2 d0 = j < nb ? ff_prod(Db[j], Ms) : far, d1 = j + 32 < nb ? ff_prod(Db[j + 32], Ms) : far;
+          const float2 e0 = ff_exp_neg(fminf(d0.x, 86.0f), d0.y, tab, L);
+          const float2 e1 = ff_exp_neg(fminf(d1.x, 86.0f), d1.y, tab, L);
+          if (d0.x < (float)TR_DMAX) tr_acc(sh, sl, e0);
+          if (d1.x < (float)TR_DMAX) tr_acc(sh, sl, e1);
         }
-        const int64_t jmax = hi;
-        double pd = 0.0;  // tiny differences, FP64
-        for (int64_t j = B.jz + lane; j < min((int64_t)B.ju, jmax); j += 32) pd += exp(-((k[j] - B.k0) * mi));
-        float sh = 0.0f, sl = 0.0f;
-        if (jmax > B.ju) {  // then m 2^F < 87 2^100 (a pair)
-          const float2 M = split_pair(mi * B.scale);
-          // two terms a lane per pass (independent exponentials side by side)
-          int64_t j = B.ju + lane;
-          for (; j + 32 < jmax; j += 64) {
-            const float2 d0 = ff_prod(Db[j], M), d1 = ff_prod(Db[j + 32], M);
-            const float2 e0 = ff_exp_neg(fminf(d0.x, 86.0f), d0.y, tab, L);
-            const float2 e1 = ff_exp_neg(fminf(d1.x, 86.0f), d1.y, tab, L);
-            if (d0.x < (float)TR_DMAX) tr_acc(sh, sl, e0);
-            if (d1.x < (float)TR_DMAX) tr_acc(sh, sl, e1);
-          }
-          if (j < jmax) {
-            const float2 d = ff_prod(Db[j], M);
-            if (d.x < (float)TR_DMAX) tr_acc(sh, sl, ff_exp_neg(d.x, d.y, tab, L));
-          }
-        }
-        const double t = warp_sum((double)sh + (double)sl + pd);
-        res = E0 * ((double)B.jz + t) / (double)nb;
       }
     }
-    if (lane == 0) out[(int64_t)b * nm + i] = res;
+    float2 t = make_float2(sh, sl + sf);
+    for (int o = 16; o > 0; o >>= 1) t = ff_add(t, shfl_xor_f2(t, o));
+    if (lane == s) mine = t;
+  }
+  if (have) {
+    const double t = (double)B.jz + pd + ((double)mine.x + (double)mine.y);
+    out[(int64_t)b * nm + i] = E0 > 0.0 ? E0 * t / (double)nb : 0.0;
   }
 }
 
@@ -1609,18 +1743,26 @@ __device__ __forceinline__ double tr_kfit(const double *c, int ncheb, int j, int
   return exp(v);
 }
 
-// One CTA per (bin, block of column masses), one column mass a thread, the
-// fit's ng values of k (and their pairs) in shared memory.  The values are
-// not sorted, so every point is visited; terms with d >= 87 are skipped.
+// CTAs of one bin, one column mass to each group of P threads (a power of two up
+// to a warp; they share the blocks), the fit's ng values of k, their
+// pairs and the coefficients of blocks of `len` neighbouring points in shared
+// memory (k(g) is smooth in g, sorted or not).  A block whose spread is narrow for
+// a thread's mass is one exponential and a polynomial, any other point by point
+// (terms with d >= 87 skipped).  len is 16 while shared memory holds that; longer
+// blocks for the largest ng, past TR_BLK points without coefficients.
+constexpr int TRF_ROW = 36;  // floats a block: TR_ROWS, the smallest d, padding
+static_assert(TR_ROWS < TRF_ROW && TRF_ROW % 4 == 0, "block rows");
+
 __global__ void __launch_bounds__(TR_THREADS)
     k_trans_fit(const double *__restrict__ coef, int ncheb, int ng, int nm, const double *__restrict__ m,
-                TrConsts L, double *__restrict__ out) {
-  extern __shared__ double kfit[];  // ng values, then ng pairs (a negative pair: FP64 term)
+                TrConsts L, int P, int len, double *__restrict__ out) {
+  extern __shared__ __align__(16) double kfit[];  // ng values, ng pairs (a negative pair: FP64 term), the blocks
   float2 *Dg = reinterpret_cast<float2 *>(kfit + ng);
+  float *blk = reinterpret_cast<float *>(kfit + 2 * ng);  // 16 ng bytes in: 16-byte aligned
   __shared__ float2 tab[TR_TAB];
   __shared__ double rmin[TR_THREADS / 32], rmax[TR_THREADS / 32];
   tr_table(tab);
-  const int b = blockIdx.x;
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
   const double *c = coef + (int64_t)b * ncheb;
   double vmin = INFINITY, vmax = 0.0;
   bool bad = false;
@@ -1635,7 +1777,7 @@ __global__ void __launch_bounds__(TR_THREADS)
     vmin = fmin(vmin, __shfl_down_sync(0xffffffffu, vmin, o));
     vmax = fmax(vmax, __shfl_down_sync(0xffffffffu, vmax, o));
   }
-  if ((threadIdx.x & 31) == 0) {
+  if (lane == 0) {
     rmin[threadIdx.x >> 5] = vmin;
     rmax[threadIdx.x >> 5] = vmax;
   }
@@ -1655,37 +1797,83 @@ __global__ void __launch_bounds__(TR_THREADS)
       Dg[j] = (dj == 0.0 || dj >= tiny) ? split_pair(dj * inv) : make_float2(-1.0f, 0.0f);
     }
   __syncthreads();
-  for (int i = blockIdx.y * TR_THREADS + threadIdx.x; i < nm; i += gridDim.y * TR_THREADS) {
-    const double mi = m[i];
-    double res;
+  const int nblk = (ng + len - 1) / len;
+  if (!bad)
+    for (int q = threadIdx.x >> 5; q < nblk; q += TR_THREADS / 32) {  // one warp a block
+      const int j0 = q * len, n = min(len, ng - j0);
+      float lo = INFINITY;
+      bool odd = len > TR_BLK;
+      for (int j = lane; j < n; j += 32) {
+        lo = fminf(lo, Dg[j0 + j].x);
+        odd |= Dg[j0 + j].x < 0.0f;  // holds an FP64 term: point by point
+      }
+      odd = __any_sync(0xffffffffu, odd);
+      for (int o = 16; o > 0; o >>= 1) lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      if (!odd) {
+        const float2 z = make_float2(0.0f, 0.0f);
+        tr_block(lane < n ? Dg[j0 + lane] : z, lane + 32 < n ? Dg[j0 + lane + 32] : z, lane < n, lane + 32 < n, n,
+                 blk + q * TRF_ROW, 1);
+      } else if (lane == 0) {
+        blk[q * TRF_ROW + 1] = INFINITY;
+      }
+      if (lane == 0) blk[q * TRF_ROW + TR_ROWS] = fmaxf(lo, 0.0f);
+    }
+  __syncthreads();
+  const int part = lane & (P - 1), step = gridDim.y * (TR_THREADS / P);
+  for (int i0 = blockIdx.y * (TR_THREADS / P) + (threadIdx.x & ~31) / P; i0 < nm; i0 += step) {  // warp-uniform
+    const int i = i0 + lane / P;
+    const bool have = i < nm;
+    const double mi = have ? m[i] : 0.0;
+    float sh = 0.0f, sl = 0.0f;
+    double pd = 0.0, E0 = 0.0;
     if (bad) {  // the plain FP64 sum
-      double s = 0.0;
-      for (int j = 0; j < ng; ++j) s += exp(-kfit[j] * mi);
-      res = s / (double)ng;
+      if (have)
+        for (int j = part; j < ng; j += P) pd += exp(-kfit[j] * mi);
+      E0 = 1.0;
     } else {
-      const double E0 = exp(-(vmin * mi));
-      res = 0.0;
-      if (E0 > 0.0) {
+      E0 = exp(-(vmin * mi));
+      if (have && E0 > 0.0) {
         const double Md = mi * scale;
         const bool pairs = Md < 0x1p107;  // else every pair term has d >= 128
         const float2 M = split_pair(pairs ? Md : 0.0);
-        float sh = 0.0f, sl = 0.0f;
-        double pd = 0.0;
-        for (int j = 0; j < ng; ++j) {
-          const float2 Dj = Dg[j];
-          if (Dj.x < 0.0f) {
-            pd += exp(-((kfit[j] - vmin) * mi));
-          } else if (pairs) {
-            const float2 d = ff_prod(Dj, M);
-            if (d.x < (float)TR_DMAX) {
-              tr_acc(sh, sl, ff_exp_neg(d.x, d.y, tab, L));
+        for (int q = part; q < nblk; q += P) {
+          const float *bk = blk + q * TRF_ROW;
+          const float R = bk[1], low = bk[TR_ROWS] * M.x;
+          if (low >= (float)TR_DMAX) continue;
+          if (pairs && R * M.x <= 1.0f) {
+            float a[TRF_ROW];
+#pragma unroll
+            for (int r = 0; r < TRF_ROW / 4; ++r) {
+              const float4 v = reinterpret_cast<const float4 *>(bk)[r];
+              a[4 * r] = v.x, a[4 * r + 1] = v.y, a[4 * r + 2] = v.z, a[4 * r + 3] = v.w;
+            }
+            const float2 S = tr_poly(a, 1, R, M);
+            const float2 d = ff_prod(make_float2(a[0], 0.0f), M);
+            tr_acc(sh, sl, ff_mul(ff_exp_neg(d.x, d.y, tab, L), S));
+            continue;
+          }
+          const int j1 = min(ng, (q + 1) * len);
+          for (int j = q * len; j < j1; ++j) {
+            const float2 Dj = Dg[j];
+            if (Dj.x < 0.0f) {
+              pd += exp(-((kfit[j] - vmin) * mi));
+            } else if (pairs) {
+              const float2 d = ff_prod(Dj, M);
+              if (d.x >= (float)TR_DMAX) continue;
+              if (low > TR_D32) sl += expf(-d.x);
+              else tr_acc(sh, sl, ff_exp_neg(d.x, d.y, tab, L));
             }
           }
         }
-        res = E0 * ((double)sh + (double)sl + pd) / (double)ng;
       }
     }
-    out[(int64_t)b * nm + i] = res;
+    float2 t = make_float2(sh, sl);
+    const bool any = __any_sync(0xffffffffu, pd != 0.0);
+    for (int o = P >> 1; o > 0; o >>= 1) {
+      t = ff_add(t, shfl_xor_f2(t, o));
+      if (any) pd += __shfl_xor_sync(0xffffffffu, pd, o);
+    }
+    if (have && part == 0) out[(int64_t)b * nm + i] = E0 * (((double)t.x + (double)t.y) + pd) / (double)ng;
   }
 }
 
@@ -1732,7 +1920,10 @@ static TrConsts tr_consts() {
   return TrConsts{l1, l2, l3};
 }
 
-size_t trans_pair_bytes(int nbins, int64_t nb) { return (size_t)nbins * (size_t)nb * sizeof(float2); }
+// the pairs, then the blocks' coefficients
+size_t trans_pair_bytes(int nbins, int64_t nb) {
+  return (size_t)nbins * ((size_t)nb * sizeof(float2) + (size_t)tr_nblk(nb) * TR_ROWS * sizeof(float));
+}
 size_t trans_bin_bytes(int nbins) { return (size_t)nbins * sizeof(TrBin); }
 
 cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double *sorted,
@@ -1746,22 +1937,41 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
     k_trans_prep<<<nbins, TR_THREADS, 0, c->stream>>>(sorted, nb, D, bins);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 grid(nbins, std::max(1, std::min(8, (nm + TR_THREADS / 32 - 1) / (TR_THREADS / 32))));
+    float *blk = reinterpret_cast<float *>(D + (int64_t)nbins * nb);
     ++c->launches;
-    k_trans_direct<<<grid, TR_THREADS, 0, c->stream>>>(sorted, nb, nm, m_dev, D, bins, L, direct);
+    const int wpc = TR_THREADS / 32;
+    const int64_t nblk = tr_nblk(nb);
+    k_trans_blocks<<<dim3(nbins, (unsigned)std::min<int64_t>((nblk + wpc - 1) / wpc, 64)), TR_THREADS, 0, c->stream>>>(
+        nb, D, bins, blk);
+    // as many masses a warp (their FP64 exponentials cost one) as leave 16 warps an SM
+    int per = 32;
+    while (per > 1 && (int64_t)nbins * ((nm + per - 1) / per) < 16ll * c->num_sms) per >>= 1;
+    dim3 grid(nbins, ((nm + per - 1) / per + wpc - 1) / wpc);
+    ++c->launches;
+    k_trans_direct<<<grid, TR_THREADS, 0, c->stream>>>(sorted, nb, nm, m_dev, D, bins, blk, L, per, direct);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   if (coef && fit) {
-    dim3 grid(nbins, (nm + TR_THREADS - 1) / TR_THREADS);
-    const size_t smem = (size_t)ng * (sizeof(double) + sizeof(float2));
-    if (smem + 2048 <= (size_t)c->max_smem_optin) {
+    // threads that share a mass: as many as give every SM 512 threads; the values
+    // of k cost each CTA ng FP64 exponentials: as few CTAs a bin as leave two an SM
+    int P = 1;
+    while (P < 32 && (int64_t)nbins * nm * P < 512ll * c->num_sms) P <<= 1;
+    const int most = (int)(((int64_t)nm * P + TR_THREADS - 1) / TR_THREADS);
+    dim3 grid(nbins, std::min(most, std::max(1, (2 * c->num_sms + nbins - 1) / nbins)));
+    int len = 16;
+    auto fit_smem = [&](int n) {
+      return (size_t)ng * (sizeof(double) + sizeof(float2)) + (size_t)((ng + n - 1) / n) * TRF_ROW * sizeof(float);
+    };
+    while (len < 16384 && fit_smem(len) + 2304 > (size_t)c->max_smem_optin) len <<= 1;
+    const size_t smem = fit_smem(len);
+    if (smem + 2304 <= (size_t)c->max_smem_optin) {
       if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_trans_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
       }
       ++c->launches;
-      k_trans_fit<<<grid, TR_THREADS, smem, c->stream>>>(coef, ncheb, ng, nm, m_dev, L, fit);
+      k_trans_fit<<<grid, TR_THREADS, smem, c->stream>>>(coef, ncheb, ng, nm, m_dev, L, P, len, fit);
     } else {
       const size_t smem64 = (size_t)ng * sizeof(double);
       if (smem64 > 48 * 1024) {
@@ -1770,7 +1980,8 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
         if (e != cudaSuccess) return e;
       }
       ++c->launches;
-      k_trans_fit64<<<grid, TR_THREADS, smem64, c->stream>>>(coef, ncheb, ng, nm, m_dev, fit);
+      k_trans_fit64<<<dim3(nbins, (nm + TR_THREADS - 1) / TR_THREADS), TR_THREADS, smem64, c->stream>>>(coef, ncheb, ng,
+                                                                                                    nm, m_dev, fit);
     }
     return cudaGetLastError();
   }
