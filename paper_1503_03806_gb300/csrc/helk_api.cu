@@ -149,7 +149,7 @@ void helk_destroy(helk_ctx *c) {
   void *bufs[] = {c->nu0,  c->S0,     c->El,    c->gair,   c->gself,  c->ncoll,
                   c->delta, c->lmass, c->lweight, c->rec64, c->rec32, c->core_rng, c->ckey, c->ckey32, c->tile_lo, c->tile_hi,
                   c->stats, c->kappa, c->sort_a, c->sort_b, c->pinv,  c->coef_dev,
-                  c->mean_dev, c->tmp, c->kd_fold, c->kd_part, c->kd_done, c->tr_pairs, c->tr_bins};
+                  c->mean_dev, c->tmp, c->kd_fold, c->kd_part, c->kd_done, c->kd_split, c->tr_pairs, c->tr_bins};
   for (void *p : bufs)
     if (p) cudaFree(p);
   if (c->stats_host) cudaFreeHost(c->stats_host);
@@ -820,6 +820,7 @@ helk_status helk_kdist(helk_ctx *c, const double *kappa, int64_t n, int32_t nbin
       c->sort_cap = n * 8;
     }
   }
+  HELK_TRY(ensure_buf(c, &c->kd_split, &c->kd_split_cap, kdist_split_bytes(nbins), "kdist scratch"));
   HELK_TRY(ensure_buf(c, &c->kd_fold, &c->kd_fold_cap, kdist_fold_bytes(n, nbins), "kdist scratch"));
   HELK_TRY(ensure_buf(c, &c->kd_part, &c->kd_part_cap, kdist_part_bytes(c, n, nbins), "kdist scratch"));
   if (kdist_done_bytes(nbins) > c->kd_done_cap) {

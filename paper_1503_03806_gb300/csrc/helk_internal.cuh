@@ -212,6 +212,8 @@ struct helk_ctx {
   // fit stage: logarithm pairs, partial sums, per-row counts of finished
   // CTAs (zero between calls)
   void *kd_fold = nullptr, *kd_part = nullptr, *kd_done = nullptr;
+  void *kd_split = nullptr;  // cuts of the bins split by value, their flags
+  int64_t kd_split_cap = 0;
   int64_t kd_fold_cap = 0, kd_part_cap = 0, kd_done_cap = 0;
   double *coef_dev = nullptr, *mean_dev = nullptr;
   int64_t coef_cap = 0, mean_cap = 0;
@@ -394,6 +396,7 @@ int64_t kdist_smem_max_points(helk_ctx *c);
 int64_t kdist_fold_bytes(int64_t n, int nbins);
 int64_t kdist_part_bytes(helk_ctx *c, int64_t n, int nbins);
 int64_t kdist_done_bytes(int nbins);
+int64_t kdist_split_bytes(int nbins);
 size_t trans_pair_bytes(int nbins, int64_t nb);
 size_t trans_bin_bytes(int nbins);
 // k_mlp.cu

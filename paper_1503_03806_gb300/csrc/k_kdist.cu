@@ -671,8 +671,9 @@ __global__ void __launch_bounds__(KD_THREADS)
     k_kdist_bin(const double *__restrict__ kappa, int nb, int ncheb, double kappa_floor,
                 const float2 *__restrict__ P, const float2 *__restrict__ lntab, unsigned long long *gA,
                 unsigned long long *gB, double *__restrict__ coef, double *__restrict__ mean,
-                double *__restrict__ kg_out, float4 *__restrict__ Lf) {
+                double *__restrict__ kg_out, float4 *__restrict__ Lf, const int *__restrict__ only) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  if (only && !only[blockIdx.x]) return;  // left to the part kernels
   __shared__ uint32_t hist[KD_HIST];
   __shared__ uint32_t wtot[32];
   __shared__ unsigned long long red_and[KD_WARPS], red_or[KD_WARPS], red_min[KD_WARPS], red_max[KD_WARPS];
@@ -1136,6 +1137,307 @@ __global__ void __launch_bounds__(KD_THREADS, 2)
   }
 }
 
+// ------------------------------------------------- bins split by value --
+// Bins too large for shared memory are split by value into parts of about
+// KP_KEYS keys: k_kdist_split (a CTA a bin) counts the keys in 4096 buckets over
+// the bin's range and cuts the range at bucket bounds; k_kdist_part (a CTA a part,
+// two CTAs an SM) reads the bin once, keeps the keys of its part in shared memory
+// and sorts them there as k_kdist_rank does, in 4096 buckets over the part's own
+// range, writing each key to its sorted place; k_kdist_logs takes the bin mean and
+// the folded logarithms from the sorted values.  Keys equal to the bin's smallest
+// (a spectrum's zeros) are counted, not stored.  A bin with a part that does not
+// fit (many keys in one bucket) is flagged and left to k_kdist_bin.
+// 1000 bins of 30000 points: 3.16 ms in k_kdist_bin (every pass through global
+// memory, one CTA a bin).
+constexpr int KP_KEYS = 7168;
+constexpr int KP_CAP = 10000;  // keys a part can hold: 10 B each, two CTAs an SM
+constexpr int KP_MAXP = 8;     // parts: every part reads the whole bin
+
+struct KdPart {
+  unsigned long long lo, hi;  // keys in [lo, hi)
+  int start, count;           // its first sorted place past the smallest keys', its keys
+};
+struct KdSplit {
+  unsigned long long vmin;
+  int n0, pad;  // keys equal to vmin
+  KdPart part[KP_MAXP];
+};
+
+static int kd_parts(int64_t nb) {
+  const int64_t p = (nb + KP_KEYS - 1) / KP_KEYS;
+  return p <= KP_MAXP ? (int)p : 0;
+}
+int64_t kdist_split_bytes(int nbins) { return (int64_t)nbins * ((int64_t)sizeof(KdSplit) + 4); }
+
+__global__ void __launch_bounds__(KD_THREADS)
+    k_kdist_split(const double *__restrict__ kappa, int nb, int np, KdSplit *__restrict__ split, int *__restrict__ flag) {
+  __shared__ uint32_t hist[KD_HIST];
+  __shared__ uint32_t wtot[32];
+  __shared__ unsigned long long red[2][KD_WARPS];
+  __shared__ int s_n0;
+  __shared__ int s_cut[KP_MAXP + 1], s_start[KP_MAXP + 1];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const unsigned long long *K = reinterpret_cast<const unsigned long long *>(kappa + (int64_t)blockIdx.x * nb);
+  unsigned long long vmin = ~0ull, vmax = 0ull;
+  for (int j0 = tid; j0 < nb; j0 += KR_UNROLL * KD_THREADS) {
+    unsigned long long kq[KR_UNROLL];
+#pragma unroll
+    for (int q = 0; q < KR_UNROLL; ++q) {
+      const int j = j0 + q * KD_THREADS;
+      kq[q] = K[j < nb ? j : j0];
+    }
+#pragma unroll
+    for (int q = 0; q < KR_UNROLL; ++q) {
+      vmin = min(vmin, kq[q]);
+      vmax = max(vmax, kq[q]);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    vmin = min(vmin, __shfl_down_sync(0xffffffffu, vmin, o));
+    vmax = max(vmax, __shfl_down_sync(0xffffffffu, vmax, o));
+  }
+  if (lane == 0) {
+    red[0][w] = vmin;
+    red[1][w] = vmax;
+  }
+  for (int i = tid; i < KD_HIST; i += KD_THREADS) hist[i] = 0;
+  if (tid == 0) s_n0 = 0;
+  __syncthreads();
+  for (int i = 0; i < KD_WARPS; ++i) {
+    vmin = i ? min(vmin, red[0][i]) : red[0][0];
+    vmax = i ? max(vmax, red[1][i]) : red[1][0];
+  }
+  const int sh = max(0, 64 - __clzll((long long)(vmax - vmin)) - 12);
+  const int pt = (tid * 97) & (KD_THREADS - 1);  // lanes 97 apart: mostly different counters
+  int n0 = 0;
+  for (int j0 = pt; j0 < nb; j0 += KR_UNROLL * KD_THREADS) {
+    unsigned long long kq[KR_UNROLL];
+#pragma unroll
+    for (int q = 0; q < KR_UNROLL; ++q) {
+      const int j = j0 + q * KD_THREADS;
+      kq[q] = j < nb ? K[j] : vmin;
+      n0 += j < nb && kq[q] == vmin;
+    }
+#pragma unroll
+    for (int q = 0; q < KR_UNROLL; ++q)
+      if (kq[q] != vmin) atomicAdd(&hist[hpad((int)((kq[q] - vmin) >> sh))], 1u);
+  }
+  n0 = __reduce_add_sync(0xffffffffu, n0);
+  if (lane == 0 && n0) atomicAdd(&s_n0, n0);
+  __syncthreads();
+  block_exscan_4096(hist, wtot);  // bucket starts
+  n0 = s_n0;
+  const int N = nb - n0, T = max(1, (N + np - 1) / np);
+  if (tid <= np) {  // parts without keys keep the bin's end
+    s_cut[tid] = tid == 0 ? 0 : KD_NBUCKET;
+    s_start[tid] = tid == 0 ? 0 : N;
+  }
+  __syncthreads();
+  for (int b = 1 + tid; b < KD_NBUCKET; b += KD_THREADS) {
+    // part r > 0 begins at the first bucket whose start reaches r T
+    const int s0 = (int)hist[hpad(b - 1)], s1 = (int)hist[hpad(b)];
+    if (s1 != s0)
+      for (int r = s0 / T + 1; r < np && r * T <= s1; ++r) {
+        s_cut[r] = b;
+        s_start[r] = s1;
+      }
+  }
+  __syncthreads();
+  KdSplit &S = split[blockIdx.x];
+  bool over = false;
+  if (tid < np) {
+    KdPart P;
+    P.lo = vmin + ((unsigned long long)s_cut[tid] << sh);
+    P.hi = s_cut[tid + 1] >= KD_NBUCKET ? ~0ull : vmin + ((unsigned long long)s_cut[tid + 1] << sh);
+    P.start = s_start[tid];
+    P.count = s_start[tid + 1] - P.start;
+    if (s_cut[tid] >= KD_NBUCKET) P.lo = ~0ull, P.count = 0;
+    over = P.count > KP_CAP;
+    S.part[tid] = P;
+  }
+  over = __syncthreads_or(over);
+  if (tid == 0) {
+    S.vmin = vmin;
+    S.n0 = n0;
+    flag[blockIdx.x] = over;
+  }
+}
+
+__global__ void __launch_bounds__(KD_THREADS, 2)
+    k_kdist_part(const double *__restrict__ kappa, int nb, const KdSplit *__restrict__ split, int *__restrict__ flag,
+                 double *__restrict__ sorted) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ uint32_t hw[KR_HWORDS];
+  __shared__ uint32_t wtot[32];
+  __shared__ unsigned long long red[2][KD_WARPS];
+  __shared__ int s_n;
+  unsigned long long *B = reinterpret_cast<unsigned long long *>(dsm);       // the part's keys, any order
+  uint16_t *Q = reinterpret_cast<uint16_t *>(dsm + (size_t)KP_CAP * 8);      // their places in B by bucket
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t off = (int64_t)blockIdx.x * nb;
+  if (flag[blockIdx.x] == 1) return;
+  const KdSplit &S = split[blockIdx.x];
+  const KdPart P = S.part[blockIdx.y];
+  const unsigned long long vmin = S.vmin;
+  const int n0 = S.n0;
+  if (blockIdx.y == 0)
+    for (int j = tid; j < n0; j += KD_THREADS) sorted[off + j] = __longlong_as_double((long long)vmin);
+  if (P.count == 0) return;
+  const unsigned long long *K = reinterpret_cast<const unsigned long long *>(kappa + off);
+  if (tid == 0) s_n = 0;
+  for (int i = tid; i < KR_HWORDS; i += KD_THREADS) hw[i] = 0;
+  __syncthreads();
+  unsigned long long kmin = ~0ull, kmax = 0ull;
+  constexpr int U = 8;
+  for (int j0 = 0; j0 < nb; j0 += U * KD_THREADS) {
+    unsigned long long kq[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int j = j0 + q * KD_THREADS + tid;
+      kq[q] = j < nb ? K[j] : vmin;
+    }
+    uint32_t bal[U];
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const bool in = kq[q] >= P.lo && (kq[q] < P.hi || P.hi == ~0ull) && kq[q] != vmin;
+      bal[q] = __ballot_sync(0xffffffffu, in);
+      n += __popc(bal[q]);
+      if (in) {
+        kmin = min(kmin, kq[q]);
+        kmax = max(kmax, kq[q]);
+      }
+    }
+    int at = 0;
+    if (lane == 0 && n) at = atomicAdd(&s_n, n);
+    at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int p = at + __popc(bal[q] & lanemask_lt_kd());
+      if (((bal[q] >> lane) & 1u) && p < KP_CAP) B[p] = kq[q];
+      at += __popc(bal[q]);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    kmin = min(kmin, __shfl_down_sync(0xffffffffu, kmin, o));
+    kmax = max(kmax, __shfl_down_sync(0xffffffffu, kmax, o));
+  }
+  if (lane == 0) {
+    red[0][w] = kmin;
+    red[1][w] = kmax;
+  }
+  __syncthreads();
+  const int n = s_n;
+  if (n != P.count || n > KP_CAP) {  // (keys that are not opacities: the general sort)
+    if (tid == 0) flag[blockIdx.x] = 2;
+    return;
+  }
+  for (int i = 0; i < KD_WARPS; ++i) {
+    kmin = i ? min(kmin, red[0][i]) : red[0][0];
+    kmax = i ? max(kmax, red[1][i]) : red[1][0];
+  }
+  const int sh = max(0, 64 - __clzll((long long)(kmax - kmin)) - 12);
+  for (int p = tid; p < n; p += KD_THREADS) hw_inc(hw, (int)((B[p] - kmin) >> sh));
+  __syncthreads();
+  uint32_t mx = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) mx = max(mx, hw_get(hw, tid * 8 + i));
+  const bool big = __syncthreads_or(mx > (uint32_t)KD_BUCKET_MAX);
+  block_exscan_4096_u16(hw, wtot);  // bucket starts
+  for (int p = tid; p < n; p += KD_THREADS) Q[hw_inc(hw, (int)((B[p] - kmin) >> sh))] = (uint16_t)p;
+  __syncthreads();  // hw now holds each bucket's end
+  if (big) {
+    // is every bucket over KD_BUCKET_MAX keys a run of one value?
+    bool mixed = false;
+    for (int p = tid; p < n; p += KD_THREADS) {
+      const unsigned long long k = B[Q[p]];
+      const int b = (int)((k - kmin) >> sh);
+      const int lo = b > 0 ? (int)hw_get(hw, b - 1) : 0, hi = (int)hw_get(hw, b);
+      mixed |= hi - lo > KD_BUCKET_MAX && k != B[Q[lo]];
+    }
+    if (__syncthreads_or(mixed)) {
+      if (tid == 0) flag[blockIdx.x] = 2;
+      return;
+    }
+  }
+  double *out = sorted + off + n0 + P.start;
+  for (int p = tid; p < n; p += KD_THREADS) {
+    const unsigned long long k = B[Q[p]];
+    const int b = (int)((k - kmin) >> sh);
+    const int lo = b > 0 ? (int)hw_get(hw, b - 1) : 0, hi = (int)hw_get(hw, b);
+    int r = lo;
+    if (hi - lo > KD_BUCKET_MAX) {
+      r = p;
+    } else {
+      for (int i = lo; i < hi; ++i) {
+        const unsigned long long x = B[Q[i]];
+        r += (x < k) || (x == k && i < p);
+      }
+    }
+    out[r] = __longlong_as_double((long long)k);
+  }
+}
+
+// The bin mean and the folded logarithms of sorted bins.
+__global__ void __launch_bounds__(KD_THREADS)
+    k_kdist_logs(const double *__restrict__ sorted, int nb, int npad, double kappa_floor,
+                 const float2 *__restrict__ lntab, const int *__restrict__ flag, double *__restrict__ mean,
+                 float4 *__restrict__ X) {
+  __shared__ float2 s_lnc[128], s_invc[128];
+  __shared__ unsigned long long red_fx[KD_WARPS][2];
+  if (flag[blockIdx.x]) return;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (tid < KD_LNTAB) {
+    const float2 t = lntab[tid];
+    if (tid < 128)
+      s_lnc[tid] = t;
+    else
+      s_invc[tid - 128] = t;
+  }
+  __syncthreads();
+  const unsigned long long *S = reinterpret_cast<const unsigned long long *>(sorted + (int64_t)blockIdx.x * nb);
+  const int nh = (nb + 1) >> 1;
+  float4 *Xb = X + (int64_t)blockIdx.x * npad;
+  for (int jj = nh + tid; jj < npad; jj += KD_THREADS) Xb[jj] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const unsigned long long kmax = S[nb - 1];
+  const int emax = max((int)(kmax >> 52), 1);
+  const int fxb = 74 - (nb > 1 ? 32 - __clz(nb - 1) : 0);
+  const BinOut o{s_lnc, s_invc, (unsigned long long)__double_as_longlong(kappa_floor), nullptr, Xb, nb, emax, fxb};
+  unsigned long long fx_lo = 0, fx_hi = 0;
+  constexpr int U = 4;  // places a thread has in flight
+  for (int j0 = tid; j0 < nh; j0 += U * KD_THREADS) {
+    unsigned long long ka[U], kb[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int j = min(j0 + q * KD_THREADS, nh - 1);
+      ka[q] = S[j];
+      kb[q] = S[nb - 1 - j];
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+      if (j0 + q * KD_THREADS < nh) pair_out(o, j0 + q * KD_THREADS, ka[q], kb[q], fx_lo, fx_hi);
+  }
+  fx_warp_sum(fx_lo, fx_hi);
+  if (lane == 0) {
+    red_fx[w][0] = fx_lo;
+    red_fx[w][1] = fx_hi;
+  }
+  __syncthreads();
+  if (tid == 0 && mean) {
+    unsigned long long lo = 0, hi = 0;
+    for (int i = 0; i < KD_WARPS; ++i) {
+      lo += red_fx[i][0];
+      hi += red_fx[i][1] + (lo < red_fx[i][0]);
+    }
+    double m;
+    if ((kmax >> 52) >= 0x7FF)  // infinite or NaN largest value (or a negative one)
+      m = (kmax >> 63) ? __longlong_as_double(0x7FF8000000000000ll) : __longlong_as_double((long long)kmax);
+    else
+      m = ldexp(fma((double)hi, 0x1p64, (double)lo), emax - 1075 - fxb) / (double)nb;
+    mean[blockIdx.x] = m;
+  }
+}
+
 // --------------------------------------------------------------- the fit --
 // c = P L for many bins at once: a CTA takes KF_BINS bins (one warp each)
 // and one group of P's column blocks, and streams them through shared
@@ -1320,9 +1622,27 @@ cudaError_t launch_kdist_bins(helk_ctx *c, const double *kappa, int64_t n, int n
     k_kdist_rank<<<nbins, KD_THREADS, smem, c->stream>>>(kappa, nb, npad, kappa_floor, lntab, c->sort_a,
                                                          c->sort_b, mean, kg_out, Lf);
   } else {
+    // (the parts of a bin write while others still read: not onto kappa itself)
+    const bool apart = !kg_out || kg_out >= kappa + n || kappa >= kg_out + n;
+    const int np = apart ? kd_parts(nb) : 0;
+    int *flag = nullptr;
+    if (np > 0) {
+      KdSplit *split = reinterpret_cast<KdSplit *>(c->kd_split);
+      flag = reinterpret_cast<int *>(split + nbins);
+      double *sorted = kg_out ? kg_out : reinterpret_cast<double *>(c->sort_a);
+      const int smem = KP_CAP * 10;
+      cudaError_t e = cudaFuncSetAttribute(k_kdist_part, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e != cudaSuccess) return e;
+      ++c->launches;
+      k_kdist_split<<<nbins, KD_THREADS, 0, c->stream>>>(kappa, nb, np, split, flag);
+      ++c->launches;
+      k_kdist_part<<<dim3(nbins, np), KD_THREADS, smem, c->stream>>>(kappa, nb, split, flag, sorted);
+      ++c->launches;
+      k_kdist_logs<<<nbins, KD_THREADS, 0, c->stream>>>(sorted, nb, npad, kappa_floor, lntab, flag, mean, Lf);
+    }
     ++c->launches;
-    k_kdist_bin<1, false><<<nbins, KD_THREADS, 0, c->stream>>>(kappa, nb, ncheb, kappa_floor, P, lntab,
-                                                               c->sort_a, c->sort_b, coef, mean, kg_out, Lf);
+    k_kdist_bin<1, false><<<nbins, KD_THREADS, 0, c->stream>>>(kappa, nb, ncheb, kappa_floor, P, lntab, c->sort_a,
+                                                               c->sort_b, coef, mean, kg_out, Lf, flag);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -2062,6 +2382,6 @@ extern "C" helk_status helk_kdist_static(const double *kappa, int64_t n, int32_t
   k_kdist_bin<0, true><<<nbins, KD_THREADS, smem, st>>>(kappa, (int)nb, ncheb, kappa_floor,
                                                   reinterpret_cast<const float2 *>(ptr),
                                                   reinterpret_cast<const float2 *>(ptr + 2 * KDIST_STATIC_PINV),
-                                                  nullptr, nullptr, coeffs, mean, kg_out, nullptr);
+                                                  nullptr, nullptr, coeffs, mean, kg_out, nullptr, nullptr);
   return cudaGetLastError() == cudaSuccess ? HELK_OK : HELK_ERR_CUDA;
 }
