@@ -117,12 +117,18 @@ __device__ __forceinline__ float2 log_ff(unsigned long long b, const float2 *lnc
 __host__ __device__ __forceinline__ int64_t pinv_index(int k, int64_t j, int ncheb) {
   return ((j >> 5) * ncheb + k) * 32 + (j & 31);
 }
-constexpr int PINV_MIN_COLS = 64;  // buffers hold max(N_b, 64) columns
+constexpr int PINV_MIN_COLS = 64;  // buffers hold at least 64 columns
 // The design matrix A_jk = T_k(t_j), t_j = (2j+1)/N_b - 1, is the same for
-// every bin, so its pseudo-inverse P = R^{-1} Q_1^T (Householder QR, A = QR)
-// is computed once per (N_b, n_cheb) and each bin's coefficients are
-// c = P L.  One CTA; A is built column-major in `work` (n_cheb columns of
-// N_b), Q_1 is formed in `P` and turned into P column by column.
+// every bin, so its pseudo-inverse P is computed once per (N_b, n_cheb) and each
+// bin's coefficients are c = P L.  The abscissae are symmetric, t_{nb-1-j} =
+// -t_j, and T_k(-t) = (-1)^k T_k(t): the even and the odd columns are orthogonal,
+// and each is a least-squares problem of half the columns on half the points
+// (weight 2 for a pair, 1 for the middle point of an odd N_b) -- a quarter of
+// the work of the whole one together, one CTA each (blockIdx.x: the parity).
+// By Householder QR, A = QR, P = R^{-1} Q_1^T; A and then the reflectors
+// column-major in `work` (nh = ceil(N_b / 2) rows), Q_1 behind them.  FP64-unit
+// bound: 8.3 ms at 10000 points and 20 coefficients for the whole problem in one
+// CTA.
 constexpr int PI_THREADS = 512;
 
 __device__ double block_sum_pi(double v, double *red) {
@@ -131,46 +137,56 @@ __device__ double block_sum_pi(double v, double *red) {
   __syncthreads();
   if (lane == 0) red[w] = v;
   __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < PI_THREADS / 32; ++i) s += red[i];
-  return s;
+  if (w == 0) {
+    double s = lane < PI_THREADS / 32 ? red[lane] : 0.0;
+    s = warp_sum(s);
+    if (lane == 0) red[0] = s;
+  }
+  __syncthreads();
+  return red[0];
 }
 
-// `tag` (optional, device): the (N_b, n_cheb) whose pseudo-inverse P
-// already holds; the kernel returns at once when they equal this call's and
-// records them when it has rebuilt P.
-__global__ void __launch_bounds__(PI_THREADS) k_pinv(int64_t nb, int ncheb, double *work,
-                                                     double *vtv_out, double *P, float2 *lntab,
+// `tag` (optional, device): per parity, the sizes whose half of the
+// pseudo-inverse P already holds; the CTA returns at once when they equal this
+// call's and records them when it has rebuilt its half.
+__global__ void __launch_bounds__(PI_THREADS) k_pinv(int64_t nb, int ncheb, double *work, double *P, float2 *lntab,
                                                      long long *tag) {
   __shared__ double red[PI_THREADS / 32];
-  __shared__ double R[NCHEB_MAX * NCHEB_MAX];
-  __shared__ double vtv[NCHEB_MAX];
+  constexpr int NK = NCHEB_MAX / 2;
+  __shared__ double R[NK * NK];
+  __shared__ double vtv[NK];
   __shared__ int s_current;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, par = blockIdx.x;
+  const long long sizes = (long long)nb * 64 + ncheb;
   if (tag) {
-    if (tid == 0) s_current = tag[0] == (long long)nb && tag[1] == (long long)ncheb;
+    if (tid == 0) s_current = tag[par] == sizes;
     __syncthreads();
     if (s_current) return;
   }
-  // A, column-major
-  for (int64_t j = tid; j < nb; j += PI_THREADS) {
+  const int64_t nh = (nb + 1) / 2;
+  const int even = (ncheb + 1) / 2, nk = par ? ncheb / 2 : even;
+  double *V = work + (par ? (int64_t)even * nh : 0), *Q = V + (int64_t)ncheb * nh;
+  // A's columns of this parity, rows by the square root of their weight
+  const double rt2 = 1.4142135623730950488;
+  for (int64_t j = tid; j < nh; j += PI_THREADS) {
     const double t = (double)(2 * j + 1) / (double)nb - 1.0;
+    const double wt = 2 * j + 1 == nb ? 1.0 : rt2;
     double tkm1 = 1.0, tk = t;
-    work[j] = 1.0;
-    if (ncheb > 1) work[nb + j] = t;
+    if (!par) V[j] = wt;
+    else if (nk > 0) V[j] = wt * t;
     for (int k = 2; k < ncheb; ++k) {
       const double tn = 2.0 * t * tk - tkm1;
       tkm1 = tk;
       tk = tn;
-      work[(int64_t)k * nb + j] = tn;
+      if ((k & 1) == par) V[(int64_t)(k >> 1) * nh + j] = wt * tn;
     }
   }
   __syncthreads();
-  // Householder QR: column c becomes the reflector v_c (rows c..nb-1)
-  for (int c = 0; c < ncheb; ++c) {
-    double *col = work + (int64_t)c * nb;
+  // Householder QR: column c becomes the reflector v_c (rows c .. nh - 1)
+  for (int c = 0; c < nk; ++c) {
+    double *col = V + (int64_t)c * nh;
     double s = 0.0;
-    for (int64_t j = c + tid; j < nb; j += PI_THREADS) s += col[j] * col[j];
+    for (int64_t j = c + tid; j < nh; j += PI_THREADS) s += col[j] * col[j];
     const double norm = sqrt(block_sum_pi(s, red));
     const double x0 = col[c];
     const double alpha = x0 > 0.0 ? -norm : norm;
@@ -178,93 +194,72 @@ __global__ void __launch_bounds__(PI_THREADS) k_pinv(int64_t nb, int ncheb, doub
     if (tid == 0) col[c] = x0 - alpha;
     __syncthreads();
     s = 0.0;
-    for (int64_t j = c + tid; j < nb; j += PI_THREADS) s += col[j] * col[j];
+    for (int64_t j = c + tid; j < nh; j += PI_THREADS) s += col[j] * col[j];
     const double vv = block_sum_pi(s, red);
     if (tid == 0) {
       vtv[c] = vv;
-      R[c * NCHEB_MAX + c] = alpha;
+      R[c * NK + c] = alpha;
     }
-    for (int cc = c + 1; cc < ncheb; ++cc) {
-      double *oc = work + (int64_t)cc * nb;
+    for (int cc = c + 1; cc < nk; ++cc) {
+      double *oc = V + (int64_t)cc * nh;
       s = 0.0;
-      for (int64_t j = c + tid; j < nb; j += PI_THREADS) s += col[j] * oc[j];
+      for (int64_t j = c + tid; j < nh; j += PI_THREADS) s += col[j] * oc[j];
       const double f = 2.0 * block_sum_pi(s, red) / vv;
-      for (int64_t j = c + tid; j < nb; j += PI_THREADS) oc[j] -= f * col[j];
+      for (int64_t j = c + tid; j < nh; j += PI_THREADS) oc[j] -= f * col[j];
       __syncthreads();
-      if (tid == 0) R[c * NCHEB_MAX + cc] = oc[c];
+      if (tid == 0) R[c * NK + cc] = oc[c];
     }
     __syncthreads();
   }
-  // Q_1 = H_0 H_1 ... H_{n-1} [I; 0], column-major in P
-  for (int k = 0; k < ncheb; ++k)
-    for (int64_t j = tid; j < nb; j += PI_THREADS) P[(int64_t)k * nb + j] = (j == k) ? 1.0 : 0.0;
+  // Q_1 = H_0 H_1 ... H_{n-1} [I; 0]
+  for (int k = 0; k < nk; ++k)
+    for (int64_t j = tid; j < nh; j += PI_THREADS) Q[(int64_t)k * nh + j] = (j == k) ? 1.0 : 0.0;
   __syncthreads();
-  for (int c = ncheb - 1; c >= 0; --c) {
-    const double *v = work + (int64_t)c * nb;
-    for (int k = 0; k < ncheb; ++k) {
-      double *e = P + (int64_t)k * nb;
+  for (int c = nk - 1; c >= 0; --c) {
+    const double *v = V + (int64_t)c * nh;
+    for (int k = c; k < nk; ++k) {  // columns before c are still zero past row c
+      double *e = Q + (int64_t)k * nh;
       double s = 0.0;
-      for (int64_t j = c + tid; j < nb; j += PI_THREADS) s += v[j] * e[j];
+      for (int64_t j = c + tid; j < nh; j += PI_THREADS) s += v[j] * e[j];
       const double f = 2.0 * block_sum_pi(s, red) / vtv[c];
-      for (int64_t j = c + tid; j < nb; j += PI_THREADS) e[j] -= f * v[j];
+      for (int64_t j = c + tid; j < nh; j += PI_THREADS) e[j] -= f * v[j];
       __syncthreads();
     }
   }
-  // P[:, j] = R^{-1} Q_1[j, :]^T, k-major (P[k*nb + j])
-  for (int64_t j = tid; j < nb; j += PI_THREADS) {
-    double p[NCHEB_MAX];
-    for (int k = ncheb - 1; k >= 0; --k) {
-      double v = P[(int64_t)k * nb + j];
-      for (int m = k + 1; m < ncheb; ++m) v -= R[k * NCHEB_MAX + m] * p[m];
-      p[k] = v / R[k * NCHEB_MAX + k];
-    }
-    for (int k = 0; k < ncheb; ++k) P[(int64_t)k * nb + j] = p[k];
-  }
-  __syncthreads();
-  // The abscissae are symmetric, t_{nb-1-j} = -t_j, and T_k(-t) = (-1)^k T_k(t),
-  // so P[k][nb-1-j] = (-1)^k P[k][j]: only the symmetrized first half,
-  // j < nh = ceil(nb/2), is kept, as FP32 (high, low) pairs in blocks of 32
-  // columns, [j / 32][k][j % 32] (pinv_index; columns past nh are zero), so
-  // that any run of whole blocks is one contiguous copy; built in `work` and
-  // then moved to the front of P.
-  const int64_t nh = (nb + 1) / 2;
+  // P[:, j] = R^{-1} Q_1[j, :]^T, times what the row's weight leaves for the sum
+  // (or difference) of a pair of logarithms; as FP32 (high, low) pairs in blocks
+  // of 32 columns, [j / 32][k][j % 32] (pinv_index; columns past nh are zero), so
+  // that any run of whole blocks is one contiguous copy.
   const int64_t npad = ((nh + 31) / 32) * 32;
-  float2 *W = reinterpret_cast<float2 *>(work);
-  for (int64_t e = tid; e < (int64_t)ncheb * npad; e += PI_THREADS) {
-    const int k = (int)(e / npad);
-    const int64_t j = e % npad;
-    float2 v2 = make_float2(0.0f, 0.0f);
-    if (j < nh) {
-      const double v =
-          0.5 * (P[(int64_t)k * nb + j] + ((k & 1) ? -1.0 : 1.0) * P[(int64_t)k * nb + (nb - 1 - j)]);
-      const float hi = (float)v;
-      v2 = make_float2(hi, (float)(v - (double)hi));
-    }
-    W[pinv_index(k, j, ncheb)] = v2;
-  }
-  __syncthreads();
   float2 *Ps = reinterpret_cast<float2 *>(P);
-  for (int64_t e = tid; e < (int64_t)ncheb * npad; e += PI_THREADS) Ps[e] = W[e];
-  if (tid == 0 && vtv_out) vtv_out[0] = vtv[0];
+  for (int64_t j = tid; j < npad; j += PI_THREADS) {
+    double p[NK];
+    const double wt = 2 * j + 1 == nb ? 1.0 : 1.0 / rt2;
+    for (int k = nk - 1; k >= 0; --k) {
+      double v = j < nh ? Q[(int64_t)k * nh + j] : 0.0;
+      for (int m = k + 1; m < nk; ++m) v -= R[k * NK + m] * p[m];
+      p[k] = v / R[k * NK + k];
+      const double x = p[k] * wt;
+      const float hi = (float)x;
+      Ps[pinv_index(2 * k + par, j, ncheb)] = make_float2(hi, (float)(x - (double)hi));
+    }
+  }
   // the logarithm's table, ln c_j and 1/c_j (c_j = 1 + j/128) as FP32
   // (high, low) pairs, computed here once instead of in every bin's CTA
-  if (tid < 128) {
+  if (par == 0 && tid < 128) {
     const double cj = 1.0 + tid / 128.0, l = log(cj), ic = 1.0 / cj;
     const float lh = (float)l, ih = (float)ic;
     lntab[tid] = make_float2(lh, (float)(l - (double)lh));
     lntab[128 + tid] = make_float2(ih, (float)(ic - (double)ih));
   }
-  if (tid == 0 && tag) {  // read by later launches only (stream order)
-    tag[0] = (long long)nb;
-    tag[1] = (long long)ncheb;
-  }
+  if (tid == 0 && tag) tag[par] = sizes;  // read by later launches only (stream order)
 }
 
-// The pseudo-inverse buffer: max(nb, 64) ncheb doubles of work space (the
-// blocked symmetrized half of P at its front when done; it takes at most
-// ncheb (ceil(nb/2) + 31) FP32 pairs), then the logarithm's table.  The
-// Householder work array k_pinv is given has the same size.
-int64_t pinv_work_doubles(int64_t nb, int ncheb) { return std::max<int64_t>(nb, PINV_MIN_COLS) * ncheb; }
+// The pseudo-inverse buffer: the blocked half of P (ncheb (ceil(nb/2) + 31) FP32
+// pairs at most), then, past max(nb, 64) + 1 rows of ncheb doubles, the
+// logarithm's table.  The work array k_pinv is given (the reflectors and Q_1,
+// ceil(nb/2) rows each) has the same size.
+int64_t pinv_work_doubles(int64_t nb, int ncheb) { return (std::max<int64_t>(nb, PINV_MIN_COLS) + 1) * ncheb; }
 int64_t pinv_bytes(int64_t nb, int ncheb) { return (pinv_work_doubles(nb, ncheb) + KD_LNTAB) * 8; }
 
 static float2 *pinv_lntab(helk_ctx *c, int64_t nb, int ncheb) {
@@ -273,8 +268,7 @@ static float2 *pinv_lntab(helk_ctx *c, int64_t nb, int ncheb) {
 
 cudaError_t launch_pinv(helk_ctx *c, int64_t nb, int ncheb, double *work) {
   ++c->launches;
-  k_pinv<<<1, PI_THREADS, 0, c->stream>>>(nb, ncheb, work, nullptr, c->pinv, pinv_lntab(c, nb, ncheb),
-                                        nullptr);
+  k_pinv<<<2, PI_THREADS, 0, c->stream>>>(nb, ncheb, work, c->pinv, pinv_lntab(c, nb, ncheb), nullptr);
   return cudaGetLastError();
 }
 
@@ -2370,7 +2364,7 @@ extern "C" helk_status helk_kdist_static(const double *kappa, int64_t n, int32_t
   // The pseudo-inverse for these sizes: rebuilt on the device only when the
   // sizes recorded in the array differ (the check runs in stream order, so
   // it sees what earlier calls on the stream left there).
-  k_pinv<<<1, PI_THREADS, 0, st>>>(nb, ncheb, ptr + KDIST_STATIC_PINV, nullptr, ptr,
+  k_pinv<<<2, PI_THREADS, 0, st>>>(nb, ncheb, ptr + KDIST_STATIC_PINV, ptr,
                                    reinterpret_cast<float2 *>(ptr + 2 * KDIST_STATIC_PINV),
                                    reinterpret_cast<long long *>(ptr + KDIST_STATIC_TAG));
   if (cudaGetLastError() != cudaSuccess) return HELK_ERR_CUDA;
