@@ -101,12 +101,13 @@ __device__ __forceinline__ void wing_line64(const LineRec64 &R, const WingExt64 
   L.g3r = clamp_to((int64_t)X.g3r - gbase, gspan);
 }
 
-// The two quadrature terms as n / d of r2 (Sec. 2.4): GH1 P1 / r2; GH3 P1 (r2 (r2
-// - 3/2) + 4 a^2 + 3/2) / (r2 (r2 (r2 - 3) + 9/4 + 6 a^2)).
-__device__ __forceinline__ double gh3_term(double r2, double a2, double P1) {
-  const double p = fma(r2, r2 - 3.0, fma(6.0, a2, 2.25));
-  const double n = fma(r2, r2 - 1.5, fma(4.0, a2, 1.5));
-  return P1 * n * rcp_f64(r2 * p);
+// The quadrature terms (Sec. 2.4) of r2: GH1 P1 / r2; GH3 P1 n / (r2 p), with w = r2 -
+// 3/2: p = r2 (r2 - 3) + 9/4 + 6 a^2 = w^2 + 6 a^2, n = r2 (r2 - 3/2) + 4 a^2 + 3/2 = p + 3/2
+// w + 3/2 - 2 a^2.  a6 = 6 a^2, kn = 3/2 - 2 a^2.
+__device__ __forceinline__ void gh3_nd(double r2, double a6, double kn, double &n, double &d) {
+  const double w = r2 - 1.5, p = fma(w, w, a6);
+  n = p + fma(1.5, w, kn);
+  d = r2 * p;
 }
 
 // Adds the lines of a list to a panel's node sums: M lines at a time, one a lane
@@ -146,25 +147,28 @@ __device__ __forceinline__ void list_nodes64(const WingLine64 *rec, const uint32
     const int take = min(n, 32);
 #pragma unroll 1
     for (int i = 0; i < take; i += M) {
-      if (i + at < take) {
-        const WingLine64 &L = rec[q[i + at]];
-        const double ku = L.ku, a2 = L.a2, P1 = L.P1;
-        const double uc = ((ph - L.xh) + (pl - (double)L.xl)) * ku, hw = hstep * ku;
-        if (m <= L.g1l || m >= L.g1r) {  // the panel lies on one side: its middle point decides
+      const bool have = i + at < take;
+      const WingLine64 &L = rec[q[have ? i + at : 0]];
+      const double ku = L.ku, a2 = L.a2, P1 = have ? L.P1 : 0.0;
+      const double uc = ((ph - L.xh) + (pl - (double)L.xl)) * ku, hw = hstep * ku;
+      const bool gh1 = m <= L.g1l || m >= L.g1r;  // the panel lies on one side: its middle point decides
+      if (__any_sync(0xffffffffu, have && !gh1)) {
+        // one reciprocal for either method: lanes of both share the pass
+        const double a6 = 6.0 * a2, kn = fma(-2.0, a2, 1.5);
 #pragma unroll
-          for (int j = 0; j < NPL; ++j) {
-            const double u = fma(tn[j], hw, uc);
-            acc[j] = fma(P1, rcp_f64(fma(u, u, a2)), acc[j]);
-          }
-        } else {
+        for (int j = 0; j < NPL; ++j) {
+          const double u = fma(tn[j], hw, uc), r2 = fma(u, u, a2);
+          double nn, dd;
+          gh3_nd(r2, a6, kn, nn, dd);
+          acc[j] = fma(gh1 ? P1 : P1 * nn, rcp_f64(gh1 ? r2 : dd), acc[j]);
+        }
+      } else {
 #pragma unroll
-          for (int j = 0; j < NPL; ++j) {
-            const double u = fma(tn[j], hw, uc);
-            acc[j] += gh3_term(fma(u, u, a2), a2, P1);
-          }
+        for (int j = 0; j < NPL; ++j) {
+          const double u = fma(tn[j], hw, uc);
+          acc[j] = fma(P1, rcp_f64(fma(u, u, a2)), acc[j]);
         }
       }
-      __syncwarp();
     }
     if (fin) break;
     n -= 32;
@@ -677,9 +681,9 @@ __global__ void __launch_bounds__(WG_THREADS, 3)
               const bool core = ip > D.g3l && ip < D.g3r;  // left to the core sums
               double nn = 1.0, dd = r2;
               if (__any_sync(0xffffffffu, in && !gh1 && !core)) {
-                const double pp = fma(r2, r2 - 3.0, fma(6.0, a2, 2.25));
-                nn = gh1 ? 1.0 : fma(r2, r2 - 1.5, fma(4.0, a2, 1.5));
-                dd = gh1 ? r2 : r2 * pp;
+                gh3_nd(r2, 6.0 * a2, fma(-2.0, a2, 1.5), nn, dd);
+                nn = gh1 ? 1.0 : nn;
+                dd = gh1 ? r2 : dd;
               }
               const double v = fma(P1 * nn, rcp_f64(dd), part);
               part = in && !core ? v : part;
