@@ -354,7 +354,8 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
                                        int64_t ngrid, const WingGeom *wg) {
   const int64_t nl = std::max<int64_t>(c->nlines, 1) * n_cond;
   HELK_TRY(ensure_conds(c, n_cond));
-  HELK_TRY(ensure_buf(c, (void **)&c->rec64, &c->rec_cap, nl * (int64_t)sizeof(LineRec64), "line records"));
+  if (o.precision != HELK_PREC_F32_KAHAN)
+    HELK_TRY(ensure_buf(c, (void **)&c->rec64, &c->rec_cap, nl * (int64_t)sizeof(LineRec64), "line records"));
   HELK_TRY(ensure_buf(c, (void **)&c->ckey, &c->ckey_cap, std::max<int64_t>(c->nlines, 1) * 8, "line keys"));
   if (o.precision == HELK_PREC_F32_KAHAN) {
     HELK_TRY(ensure_buf(c, (void **)&c->rec32, &c->rec32_cap, nl * (int64_t)sizeof(LineRec32),
@@ -399,6 +400,11 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
   return HELK_OK;
 }
 
+static CondArgs make_cond(const helk_ctx *c, double T, double P, double q_ratio, double mass) {
+  const double vth = sqrt(2.0 * LN2 * KB * T / ((c->has_mass ? 1.0 : mass) * AMU)) / CLIGHT;
+  return CondArgs{T, P, q_ratio, sqrt(T0 / T), C2 / T0 - C2 / T, C2 / T, SQRTLN2 / vth, log(T0 / T)};
+}
+
 // Statistics reset and line preparation (and the FP32 records) of n_cond
 // conditions: single != NULL passes the one condition by value, otherwise
 // they are read from c->cond_dev.
@@ -412,7 +418,10 @@ static helk_status prepare_lines(helk_ctx *c, int n_cond, const CondArgs *single
     if (f64 && wings)
       HELK_TRY(cuda_check(c, cudaMemsetAsync(c->core_blk, 0, (size_t)core_blocks(g->n) * n_cond * 4, c->stream),
                           "lineprep"));
-    HELK_TRY(cuda_check(c, launch_lineprep(c, n_cond, single, mass, *cut, *g, f64, f64 && wings), "lineprep"));
+    if (f64)
+      HELK_TRY(cuda_check(c, launch_lineprep(c, n_cond, single, mass, *cut, *g, wings), "lineprep"));
+    else
+      HELK_TRY(cuda_check(c, launch_prep32(c, n_cond, single, mass, *cut, *g), "lineprep"));
     if (o.precision == HELK_PREC_F32_KAHAN) {
       HELK_TRY(cuda_check(c, cudaMemsetAsync(c->core_blk, 0, (size_t)core_blocks(g->n) * n_cond * 4, c->stream),
                           "pack32"));
@@ -506,7 +515,7 @@ helk_status helk_opacity(helk_ctx *c, double T, double P, double mass, const hel
   WingGeom geom;
   const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
   HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n, wg));
-  const CondArgs one{T, P, o.q_ratio, 0.0};
+  const CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
   stage_begin(c, HELK_STAGE_LINEPREP);
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, wg != nullptr));
   stage_end(c, HELK_STAGE_LINEPREP);
@@ -545,7 +554,7 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
     max_tiles = std::max(max_tiles, (g->n + pts - 1) / pts);
   }
   HELK_TRY(ensure_call_buffers(c, 1, o, max_tiles, g->n, nullptr));
-  const CondArgs one{T, P, o.q_ratio, 0.0};
+  const CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, false));
   cudaEvent_t e0, e1;
   HELK_TRY(cuda_check(c, cudaEventCreate(&e0), "autotune"));
@@ -687,9 +696,8 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   WingGeom geom;
   const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
   const int64_t rec_line =
-      (int64_t)sizeof(LineRec64) +
-      (o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2))
-                                          : wg ? (int64_t)sizeof(WingExt64) : 0);
+      o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2))
+                                         : (int64_t)(sizeof(LineRec64) + (wg ? sizeof(WingExt64) : 0));
   const int64_t per_cond = std::max<int64_t>(c->nlines, 1) * rec_line;
   const int gmax = (int)std::max<int64_t>(1, std::min<int64_t>(n_cond, c->batch_budget / per_cond));
   const int nchunk = (n_cond + gmax - 1) / gmax;
@@ -701,7 +709,8 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   if (!c->cond_ev) HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->cond_ev, cudaEventDisableTiming), "graph"));
   // the previous batch must have read the staging buffer before it changes
   HELK_TRY(cuda_check(c, cudaEventSynchronize(c->cond_ev), "opacity_batch"));
-  for (int k = 0; k < n_cond; ++k) c->cond_host[k] = CondArgs{T[k], P[k], q_ratio ? q_ratio[k] : o.q_ratio, 0.0};
+  for (int k = 0; k < n_cond; ++k) 
+    c->cond_host[k] = make_cond(c, T[k], P[k], q_ratio ? q_ratio[k] : o.q_ratio, mass);
   stage_begin(c, HELK_STAGE_VOIGT);
   for (int j = 0; j < nchunk; ++j) {
     const int k0 = j * chunk, nk = std::min(chunk, n_cond - k0);

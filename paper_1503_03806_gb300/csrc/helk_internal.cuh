@@ -108,7 +108,11 @@ struct SurrQueue {
 
 // One (T, P) condition of a call.
 struct CondArgs {
-  double T, P, q_ratio, pad;
+  double T, P, q_ratio;
+  // from them, on the host: (T0/T)^{1/2}; c2 (1/T0 - 1/T); c2 / T; sqrt(ln2) nu /
+  // Gamma_D for the call's mass (1 amu where the lines carry masses)
+  double tfac, kE, cT, kc;
+  double lnT;  // ln(T0 / T)
 };
 
 // Per-condition results of line preparation and of the Voigt kernel.
@@ -347,11 +351,13 @@ cudaError_t launch_sort_lines(helk_ctx *c, int64_t n);  // orders SoA by nu0
 // n_cond conditions: from c->cond_dev, or (n_cond == 1 and single != NULL)
 // the one condition passed by value.  Records of condition k start at
 // k * nlines; tile maps at k * ntiles.
-// a916_f64: also the FP64 Algorithm 916 per-line factors (erfcx(a), S1(a)),
-// which only the FP64 form reads.  wings: also the WingExt64 and the core reach
+// The FP64 form's records.  wings: also the WingExt64 and the core reach
 // of the FP64 interpolated-wings route.
 cudaError_t launch_lineprep(helk_ctx *c, int n_cond, const CondArgs *single, double mass,
-                            const helk_cutoff &cut, const helk_grid &g, bool a916_f64, bool wings);
+                            const helk_cutoff &cut, const helk_grid &g, bool wings);
+// FP32 form: its records, in two steps (k_pack32 needs the largest strength)
+cudaError_t launch_prep32(helk_ctx *c, int n_cond, const CondArgs *single, double mass, const helk_cutoff &cut,
+                          const helk_grid &g);
 cudaError_t launch_pack32(helk_ctx *c, int n_cond, const helk_grid &g);
 cudaError_t launch_tilemap(helk_ctx *c, int n_cond, const helk_grid &g, int tile, int64_t ntiles);
 // Conditions ordered by decreasing evaluation count (largest work first).

@@ -243,7 +243,7 @@ struct PrepArgs {
   double mass;
   int cut_kind;
   double cut_value, cut_cap;
-  double nu_min, dnu;
+  double nu_min, dnu, idnu;  // idnu = 1 / dnu
   int64_t ngrid;
 };
 
@@ -310,7 +310,7 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
                            const double *__restrict__ lweight, PrepArgs A,
                            const CondArgs *__restrict__ conds, CondArgs single,
                            LineRec64 *__restrict__ rec_all, double *__restrict__ ckey,
-                           CondStats *cst_all, int a916_f64, WingExt64 *__restrict__ ext_all,
+                           CondStats *cst_all, WingExt64 *__restrict__ ext_all,
                            int32_t *__restrict__ ckey32, int *__restrict__ core_blk_all, int nblk) {
   const int cond = blockIdx.y;
   const CondArgs C = conds ? conds[cond] : single;
@@ -342,21 +342,11 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
     const double pself = 0.5 * C.P;
     const double gL = tfac * (ga * (C.P - pself) + gs * pself);
     const double gD = nu0p * (lmass ? sqrt(2.0 * LN2 * KB * C.T / (lmass[l] * AMU)) / CLIGHT : vth);
-    // The FP64 form divides (a and k_u are then the correctly rounded results
-    // the oracle computes, so every method choice matches it); the FP32 form
-    // rounds them to FP32 anyway and multiplies by one reciprocal (FP64
-    // divisions are long sequences on the scarce FP64 unit).
-    double a, ku, Sp;
-    if (a916_f64) {
-      a = SQRTLN2 * gL / gD;
-      ku = SQRTLN2 / gD;
-      Sp = S * SQRTLN2PI / gD;
-    } else {
-      const double igD = 1.0 / gD;
-      a = SQRTLN2 * gL * igD;
-      ku = SQRTLN2 * igD;
-      Sp = S * SQRTLN2PI * igD;
-    }
+    // divisions: a and k_u are the correctly rounded results the definition gives,
+    // so every method choice matches it
+    const double a = SQRTLN2 * gL / gD;
+    const double ku = SQRTLN2 / gD;
+    const double Sp = S * SQRTLN2PI / gD;
     double cut;
     if (A.cut_kind == HELK_CUT_ABS) cut = A.cut_value;
     else if (A.cut_kind == HELK_CUT_LORENTZ) cut = fmin(A.cut_value * gL, A.cut_cap);
@@ -381,9 +371,8 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
     r.Sp = Sp;
     r.ilo = (int32_t)lo;
     r.ihi = (int32_t)hi;
-    // Algorithm 916 per-line factors (only reachable when a < 10); the FP32
-    // form takes them in FP32 when packing its records
-    if (a916_f64 && a < 10.0) {
+    // Algorithm 916 per-line factors (only reachable when a < 10)
+    if (a < 10.0) {
       r.erfcx_a = erfcx(a);
       double s1 = 0.0;
       for (int k = 0; k < A916_S1_TERMS; ++k) {
@@ -472,76 +461,326 @@ static int line_blocks(helk_ctx *c, int64_t n, int n_cond) {
 }
 
 cudaError_t launch_lineprep(helk_ctx *c, int n_cond, const CondArgs *single, double mass,
-                            const helk_cutoff &cut, const helk_grid &g, bool a916_f64, bool wings) {
+                            const helk_cutoff &cut, const helk_grid &g, bool wings) {
   const int64_t n = c->nlines;
   if (n <= 0) return cudaSuccess;
-  PrepArgs A{mass, cut.kind, cut.value, cut.cap, g.nu_min, g.dnu, g.n};
-  const CondArgs one = single ? *single : CondArgs{0, 0, 0, 0};
+  PrepArgs A{mass, cut.kind, cut.value, cut.cap, g.nu_min, g.dnu, 1.0 / g.dnu, g.n};
+  const CondArgs one = single ? *single : CondArgs{};
   dim3 grid(line_blocks(c, n, n_cond), n_cond);
   ++c->launches;
   k_lineprep<<<grid, 256, 0, c->stream>>>(
       n, c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair, c->has_gself ? c->gself : nullptr,
       c->has_ncoll ? c->ncoll : nullptr, c->has_delta ? c->delta : nullptr,
       c->has_mass ? c->lmass : nullptr, c->has_weight ? c->lweight : nullptr, A,
-      single ? nullptr : c->cond_dev, one, c->rec64, c->ckey, c->cstats, a916_f64 ? 1 : 0,
+      single ? nullptr : c->cond_dev, one, c->rec64, c->ckey, c->cstats,
       wings ? c->ext64 : nullptr, wings ? c->ckey32 : nullptr, wings ? c->core_blk : nullptr, core_blocks(g.n));
   return cudaGetLastError();
 }
 
 // ----------------------------------------------------- FP32 line records --
-// From the FP64 records: strengths scaled by 2^-E (E from the largest S' of
-// the condition, so every scaled term is <= 1 and the FP32 range covers 38
-// decades below it); the centre as the integer grid index c plus the FP32
-// offset phi = (nu0' - nu_c) ku, so that u_i = (i - c) beta - phi keeps full
-// relative precision near the line centre.
-// the 3-node GH factor over S' a: (sqrt(pi)/6)/pi, as one constant (one FP64
-// multiplication a line instead of a division)
-constexpr double P3_FACTOR = SQRTPI / 6.0 / PI;
+// The FP32 form's records straight from the line list.  The FP64 unit (1/64 of the
+// FP32 rate) bounds the preparation, so FP64 is kept for what decides the
+// windows -- the shifted centre, Gamma_L, the cutoff bounds -- and the rest runs on
+// FP32 (high, low) pairs: the strength with its two kinds of exponential
+// (relative error ~1e-10) and k_u, a and their products (~1e-13), each rounded to
+// FP32 once.  The divisions by the grid step are products by 1 / dnu where no
+// integer lies within their rounding.  What is left is ~30 FP64 operations a line
+// and condition, still the bound: 1e6 lines, 12 conditions take 0.85 ms and 0.21 ms
+// to finish the records, against 3.5 + 0.6 ms with the FP64 form's records and a
+// packing pass; 1e7 lines, one condition 0.70 + 0.21 against 3.0 + 0.5 ms.
+struct F2 {
+  float h, l;
+};
+__device__ __forceinline__ F2 f2_norm(float h, float l) {
+  const float s = h + l;
+  return F2{s, l - (s - h)};
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  const float p = a.h * b.h;
+  return f2_norm(p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p))));
+}
+__device__ __forceinline__ F2 f2_div(F2 a, F2 b) {
+  const float r = __frcp_rn(b.h), q = a.h * r;
+  const float rem = fmaf(-q, b.l, fmaf(-q, b.h, a.h) + a.l);
+  return f2_norm(q, rem * r);
+}
+// v as a pair, from its bits (no FP64 instruction for 2^-70 < |v| < 2^127 and 0)
+__device__ __forceinline__ F2 f2_of(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7FF) - 1023;
+  if (e > -70 && e < 127) {
+    const unsigned sign = hi & 0x80000000u;
+    const float h = __uint_as_float(sign | (unsigned)(e + 127) << 23 | (hi & 0xFFFFFu) << 3 | lo >> 29);
+    const float l = (float)(lo & 0x1FFFFFFFu) * __int_as_float((e - 52 + 127) << 23);
+    return F2{h, sign ? -l : l};
+  }
+  if (e == -1023) return F2{0.0f, 0.0f};
+  const float h = (float)v;
+  return F2{h, e < 127 ? (float)(v - (double)h) : 0.0f};
+}
+// v = (h + l) 2^e with 1 <= |h| < 2, from the bits (a normal v)
+__device__ __forceinline__ F2 f2_mant(double v, int &e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  e = (int)((b >> 52) & 0x7FF) - 1023;
+  const unsigned sign = (unsigned)(b >> 63) << 31;
+  const float h = __uint_as_float(sign | 0x3F800000u | (unsigned)((b >> 29) & 0x7FFFFFu));
+  const float l = (float)(unsigned)(b & 0x1FFFFFFFu) * 0x1p-52f;
+  return f2_norm(h, sign ? -l : l);
+}
+__device__ __forceinline__ F2 prep_mant(double v, int &e) {  // also a subnormal v
+  if (__double2hiint(v) >= 23 << 20) return f2_mant(v, e);
+  const F2 r = f2_mant(v * 0x1p200, e);
+  e -= 200;
+  return r;
+}
+__device__ __forceinline__ float f_pow2(int e) {  // 2^e, clamped to the FP32 normal range
+  return __int_as_float((min(max(e, -126), 127) + 127) << 23);
+}
 
-__global__ void k_pack32(int64_t n, const LineRec64 *__restrict__ r64_all, double nu_min, double dnu, int64_t ngrid,
-                         const double *__restrict__ ckey, CondStats *cst_all, LineRec32 *__restrict__ r32_all,
-                         int2 *__restrict__ core_all, int32_t *__restrict__ ckey32, int *err_flags,
-                         int *__restrict__ core_blk_all, int nblk) {
+// 2^{j/32}, j = 0 .. 31
+__device__ constexpr float PREP_POW[32][2] = {
+    {0x1.0000000000000p+0f, 0x0.0p+0f}, {0x1.059b0e0000000p+0f, -0x1.9d4f520000000p-25f}, {0x1.0b55860000000p+0f, 0x1.9f31220000000p-25f},
+    {0x1.11301e0000000p+0f, -0x1.fdb4960000000p-25f}, {0x1.172b840000000p+0f, -0x1.c157420000000p-27f}, {0x1.1d48740000000p+0f, -0x1.d2e8ca0000000p-25f},
+    {0x1.2387a60000000p+0f, 0x1.ceac480000000p-25f}, {0x1.29e9e00000000p+0f, -0x1.5c04240000000p-25f}, {0x1.306fe00000000p+0f, 0x1.4636e20000000p-25f},
+    {0x1.371a740000000p+0f, -0x1.18aac60000000p-25f}, {0x1.3dea640000000p+0f, 0x1.8246840000000p-25f}, {0x1.44e0860000000p+0f, 0x1.8624b40000000p-30f},
+    {0x1.4bfdae0000000p+0f, -0x1.593abc0000000p-25f}, {0x1.5342b60000000p+0f, -0x1.2c56100000000p-25f}, {0x1.5ab07e0000000p+0f, -0x1.5bd5ec0000000p-27f},
+    {0x1.6247ec0000000p+0f, -0x1.f8b5500000000p-25f}, {0x1.6a09e60000000p+0f, 0x1.9fcef40000000p-26f}, {0x1.71f75e0000000p+0f, 0x1.1d8bee0000000p-25f},
+    {0x1.7a11480000000p+0f, -0x1.829fd00000000p-25f}, {0x1.82589a0000000p+0f, -0x1.accc7c0000000p-26f}, {0x1.8ace540000000p+0f, 0x1.15506e0000000p-27f},
+    {0x1.93737c0000000p+0f, -0x1.e647440000000p-25f}, {0x1.9c49180000000p+0f, 0x1.51f8480000000p-27f}, {0x1.a5503c0000000p+0f, -0x1.b83b540000000p-25f},
+    {0x1.ae89fa0000000p+0f, -0x1.a94b140000000p-26f}, {0x1.b7f7700000000p+0f, -0x1.a094380000000p-25f}, {0x1.c199be0000000p+0f, -0x1.3d56b20000000p-27f},
+    {0x1.cb720e0000000p+0f, -0x1.8837cc0000000p-27f}, {0x1.d5818e0000000p+0f, -0x1.822dbc0000000p-27f}, {0x1.dfc9740000000p+0f, -0x1.908c940000000p-25f},
+    {0x1.ea4afa0000000p+0f, 0x1.52486c0000000p-27f}, {0x1.f507660000000p+0f, -0x1.246eb00000000p-26f}};
+
+// e^z as v 2^m, z a pair (clamped to +-80000: 2^m is then far out of range): z = (32 m + j) ln2 / 32 + r, |r| <= ln2 / 64,
+// 2^{j/32} from the table and e^r - 1 by its Taylor polynomial to r^4 (1.3e-12).
+// small: e^z - 1 itself where m = j = 0 (no cancellation), else v 2^m - 1.
+__device__ __forceinline__ F2 prep_exp(F2 z, int &m, bool minus1) {
+  if (fabsf(z.h) > 80000.0f) z = F2{copysignf(80000.0f, z.h), 0.0f};
+  const float g = fmaf(z.h, 0x1.715476p+5f, 12582912.0f), n = g - 12582912.0f;
+  const int k = __float_as_int(g) - 0x4B400000;
+  const float p = n * 0x1.62e4300000000p-6f, pe = fmaf(n, 0x1.62e4300000000p-6f, -p);
+  const F2 r = f2_norm(z.h - p, fmaf(-n, -0x1.05c6100000000p-34f, z.l - pe));
+  const float q = r.h * r.h * fmaf(r.h, fmaf(r.h, 1.0f / 24.0f, 1.0f / 6.0f), 0.5f);
+  const F2 e1 = f2_norm(r.h, fmaf(r.h, r.l, q) + r.l);  // e^r - 1
+  m = k >> 5;
+  if (minus1 && k == 0) return e1;
+  const float th = PREP_POW[k & 31][0], tl = PREP_POW[k & 31][1];
+  const F2 t = f2_mul(F2{th, tl}, e1);
+  const float s = th + t.h;  // |t| < |th|
+  F2 v = f2_norm(s, (t.h - (s - th)) + (tl + t.l));
+  if (minus1) {  // z <= 0: m <= 0
+    const float sc = m < -100 ? 0.0f : f_pow2(m);
+    v = F2{v.h * sc, v.l * sc};
+    const float d = v.h - 1.0f, bb = d - v.h;
+    v = f2_norm(d, ((v.h - (d - bb)) + (-1.0f - bb)) + v.l);
+    m = 0;
+  }
+  return v;
+}
+
+// q = v / dnu rounded up (UP) or down to an integer, clamped to [-2^30, 2^31 - 1]:
+// from v (1 / dnu) where no integer lies within the rounding of that or of the
+// division (2^-46 |q|; both err by < 2^-51 |q|), else by the division itself.
+// Adding 1.5 2^52 leaves the nearest integer in the low word; comparisons are made
+// on the high words, so the common path is a product and three additions.
+constexpr double PREP_MAGIC = 6755399441055744.0;
+__device__ __noinline__ int prep_index_div(double v, double dnu, bool up) {
+  const double q = v / dnu;
+  if (q <= -1073741824.0) return -1073741824;
+  return (int)fmin(up ? ceil(q) : floor(q), 2147483647.0);
+}
+template <bool UP>
+__device__ __forceinline__ int prep_index(double v, double dnu, double idnu) {
+  const double q = v * idnu, t = q + PREP_MAGIC, d = q - (t - PREP_MAGIC);
+  const int hq = __double2hiint(q) & 0x7FFFFFFF, hd = __double2hiint(d), r = __double2loint(t);
+  if (hq >= 0x41D00000 || hq - (hd & 0x7FFFFFFF) >= 46 << 20) return prep_index_div(v, dnu, UP);
+  return UP ? r + (hd >= 0 ? 1 : 0) : r - (hd < 0 ? 1 : 0);
+}
+
+// The FP32 records with strengths as a mantissa in [1, 2) -- Sp, and P1 and P3 from
+// it -- and its binary exponent in erfcx_a's place; sig1's place: the centre was
+// clamped to the grid.  k_pack32 finishes them.
+__global__ void __launch_bounds__(256)
+    k_prep32(int64_t n, const double *__restrict__ nu0, const double *__restrict__ S0, const double *__restrict__ El,
+             const double *__restrict__ gair, const double *__restrict__ gself, const double *__restrict__ ncoll,
+             const double *__restrict__ delta, const double *__restrict__ lmass, const double *__restrict__ lweight,
+             PrepArgs A, const CondArgs *__restrict__ conds, CondArgs single, LineRec32 *__restrict__ rec_all,
+             double *__restrict__ ckey, CondStats *cst_all) {
   const int cond = blockIdx.y;
-  const LineRec64 *r64 = r64_all + (int64_t)cond * n;
+  const CondArgs C = conds ? conds[cond] : single;
+  LineRec32 *rec = rec_all + (int64_t)cond * n;
+  CondStats *cst = cst_all + cond;
+  unsigned long long evals = 0;
+  long long wmax = -1;
+  unsigned long long spmax = 0;
+  const double idnu = A.idnu, pself = 0.5 * C.P, pair_p = C.P - pself;
+  const F2 kE = f2_of(C.kE), cT = f2_of(C.cT), cT0 = f2_of(C2 / T0), kc = f2_of(C.kc), dnu2 = f2_of(A.dnu);
+  const F2 lnT = f2_of(C.lnT);
+  int eq;
+  const F2 qr = prep_mant(C.q_ratio, eq);
+  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
+       l += (int64_t)gridDim.x * blockDim.x) {
+    const double v0 = nu0[l], ga = gair[l];
+    const double gs = gself ? gself[l] : ga;
+    const double nc = ncoll ? ncoll[l] : 0.5;
+    const double nu0p = delta ? v0 + delta[l] * C.P : v0;
+    // Gamma_L: in FP64 where it decides the window, as k_lineprep rounds it
+    const double gP = ga * pair_p + gs * pself;
+    double gL = C.tfac * gP;
+    F2 gL2;
+    if (nc != 0.5 && A.cut_kind != HELK_CUT_LORENTZ) {
+      int m;
+      const F2 t = prep_exp(f2_mul(f2_of(nc), lnT), m, false);
+      const float sc = f_pow2(m);
+      gL2 = f2_mul(F2{t.h * sc, t.l * sc}, f2_of(gP));
+    } else {
+      if (nc != 0.5) gL = pow(T0 / C.T, nc) * gP;
+      gL2 = f2_of(gL);
+    }
+    LineRec32 q;
+    if (A.cut_kind == HELK_CUT_NONE) {
+      q.ilo = 0;
+      q.ihi = (int)(A.ngrid - 1);
+    } else {
+      const double cut = A.cut_kind == HELK_CUT_ABS ? A.cut_value : fmin(A.cut_value * gL, A.cut_cap);
+      q.ilo = min(max(prep_index<true>(nu0p - cut - A.nu_min, A.dnu, idnu), 0), (int)A.ngrid);
+      q.ihi = max(min(prep_index<false>(nu0p + cut - A.nu_min, A.dnu, idnu), (int)(A.ngrid - 1)), -1);
+    }
+    // k_u, a and the centre
+    const F2 nup = f2_of(nu0p);
+    F2 k = kc;  // sqrt(ln2) nu0' / Gamma_D, for this line's mass
+    if (lmass) {
+      const F2 mm = f2_of(lmass[l]);
+      const float rs = rsqrtf(mm.h), s = mm.h * rs;
+      k = f2_mul(k, f2_norm(s, 0.5f * rs * (fmaf(-s, s, mm.h) + mm.l)));
+    }
+    const F2 ku = f2_div(k, nup);
+    const F2 a = f2_mul(gL2, ku);
+    const F2 beta = f2_mul(dnu2, ku);
+    q.beta = beta.h;
+    q.a = a.h;
+    q.a2 = fmaf(a.h, a.h, 2.0f * a.h * a.l);
+    const double pos = (nu0p - A.nu_min) * idnu, pt = pos + PREP_MAGIC;
+    double cf = pt - PREP_MAGIC;
+    q.c = __double2loint(pt);
+    const int hp = __double2hiint(pos);
+    const bool big = (hp & 0x7FFFFFFF) >= 0x41D00000;
+    const bool below = big ? hp < 0 : q.c < 0, above = big ? hp >= 0 : q.c > A.ngrid - 1;
+    if (below || above) {
+      q.c = below ? 0 : (int)(A.ngrid - 1);
+      cf = (double)q.c;
+    }
+    q.phi_k = f2_mul(f2_of(nu0p - (A.nu_min + cf * A.dnu)), ku).h;
+    // S' = S ku / sqrt(pi), as a pair of order one times 2^e
+    int e = 0;
+    F2 S{0.0f, 0.0f};
+    const double s0 = S0[l], wt = lweight ? lweight[l] : 1.0;
+    if (__double_as_longlong(s0) > 0 && __double_as_longlong(wt) > 0) {
+      int e1;
+      S = prep_mant(s0, e);
+      if (El) {
+        const double E = El[l];
+        const F2 vv = f2_of(v0);
+        S = f2_mul(S, prep_exp(f2_mul(f2_of(E), kE), e1, false));
+        e += e1 + eq;
+        S = f2_mul(S, qr);
+        const F2 x = f2_mul(vv, cT), y = f2_mul(vv, cT0);
+        S = f2_mul(S, vv.h < 1e-12f  // the limit T0 / T, to 1e-14
+                          ? f2_div(cT, cT0)
+                          : f2_div(prep_exp(F2{-x.h, -x.l}, e1, true), prep_exp(F2{-y.h, -y.l}, e1, true)));
+      }
+      if (lweight) {
+        S = f2_mul(S, prep_mant(wt, e1));
+        e += e1;
+      }
+      S = f2_mul(f2_mul(S, ku), F2{0x1.20dd760000000p-1f, -0x1.f7ac920000000p-26f});
+      // mantissa to [1, 2)
+      const int ex = ((__float_as_int(S.h) >> 23) & 0xFF) - 127;
+      const float sc = f_pow2(-ex);
+      S = F2{S.h * sc, S.l * sc};
+      e += ex;
+    }
+    q.Sp = S.h;
+    const F2 Sa = f2_mul(S, a);
+    q.P1 = f2_mul(Sa, F2{0x1.20dd760000000p-1f, -0x1.f7ac920000000p-26f}).h;
+    q.P3 = f2_mul(Sa, F2{0x1.8127460000000p-4f, 0x1.606f3c0000000p-29f}).h;
+    q.erfcx_a = __int_as_float(e);
+    q.sig1 = below || above ? 1.0f : 0.0f;
+    rec[l] = q;
+    // reference index of the unshifted centre: non-decreasing in list order
+    long long c0 = prep_index<false>(v0 - A.nu_min, A.dnu, idnu);
+    if (c0 <= -1073741824 || c0 >= 2147483647) {
+      double ck = floor((v0 - A.nu_min) / A.dnu);
+      ck = fmin(fmax(ck, -4.0e15), 4.0e15);
+      c0 = (long long)ck;
+    }
+    if (cond == 0) ckey[l] = (double)c0;
+    if (q.ihi >= q.ilo) {
+      evals += (unsigned long long)(q.ihi - q.ilo + 1);
+      wmax = max(wmax, max(c0 - q.ilo, (long long)q.ihi - c0));
+      // the bits of S' as a double (its largest gives the common scale)
+      if (S.h > 0.0f && e > -1023 && e < 1024) {
+        const unsigned long long sb =
+            ((unsigned long long)(e + 1023) << 52) | ((unsigned long long)(__float_as_uint(S.h) & 0x7FFFFFu) << 29);
+        spmax = max(spmax, sb);
+      }
+    }
+  }
+  // warp-aggregate then one atomic per warp
+  for (int o = 16; o > 0; o >>= 1) {
+    evals += __shfl_down_sync(0xffffffffu, evals, o);
+    wmax = max(wmax, __shfl_down_sync(0xffffffffu, wmax, o));
+    spmax = max(spmax, __shfl_down_sync(0xffffffffu, spmax, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (evals) atomicAdd(&cst->evals, evals);
+    if (wmax >= 0) atomicMax(&cst->wmax, wmax);
+    if (spmax) atomicMax(&cst->spmax_bits, spmax);
+  }
+}
+
+cudaError_t launch_prep32(helk_ctx *c, int n_cond, const CondArgs *single, double mass, const helk_cutoff &cut,
+                          const helk_grid &g) {
+  const int64_t n = c->nlines;
+  if (n <= 0) return cudaSuccess;
+  PrepArgs A{mass, cut.kind, cut.value, cut.cap, g.nu_min, g.dnu, 1.0 / g.dnu, g.n};
+  const CondArgs one = single ? *single : CondArgs{};
+  ++c->launches;
+  k_prep32<<<dim3(line_blocks(c, n, n_cond), n_cond), 256, 0, c->stream>>>(
+      n, c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair, c->has_gself ? c->gself : nullptr,
+      c->has_ncoll ? c->ncoll : nullptr, c->has_delta ? c->delta : nullptr, c->has_mass ? c->lmass : nullptr,
+      c->has_weight ? c->lweight : nullptr, A, single ? nullptr : c->cond_dev, one, c->rec32, c->ckey, c->cstats);
+  return cudaGetLastError();
+}
+
+// The records finished: strengths scaled by 2^-E (E from the largest S' of the
+// condition, so every scaled term is <= 1 and the FP32 range covers 38 decades
+// below it; a power of two, so exact), the Algorithm 916 factors, the core range.
+__global__ void k_pack32(int64_t n, int64_t ngrid, const double *__restrict__ ckey, CondStats *cst_all,
+                         LineRec32 *__restrict__ r32_all, int2 *__restrict__ core_all, int32_t *__restrict__ ckey32,
+                         int *err_flags, int *__restrict__ core_blk_all, int nblk) {
+  const int cond = blockIdx.y;
   LineRec32 *r32 = r32_all + (int64_t)cond * n;
   CondStats *cst = cst_all + cond;
-  const double spmax = __longlong_as_double((long long)cst->spmax_bits);
-  const int E = spmax > 0.0 ? ilogb(spmax) + 1 : 0;
+  const unsigned long long sb = cst->spmax_bits;
+  const int E = sb ? (int)(sb >> 52) - 1022 : 0;  // ilogb + 1
   if (blockIdx.x == 0 && threadIdx.x == 0) cst->scale_exp = E;
-  const double pow2mE = ldexp(1.0, -E);  // exact: S' 2^-E by one multiplication
-  const double idnu = 1.0 / dnu;
   int cw1 = 0;
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
        l += (int64_t)gridDim.x * blockDim.x) {
-    const LineRec64 r = r64[l];
-    // the reference index is an integer below 2^53 in magnitude: integer
-    // operations from here on (the FP64 unit bounds this kernel)
     const long long key = (long long)ckey[l];
     const int k32 = (int)min(max(key, -2147483647ll), 2147483647ll);
     if (cond == 0) ckey32[l] = k32;
-    LineRec32 q;
-    // any integer within a step of the centre serves as c (phi takes the
-    // rest), so a product by 1/dnu replaces the division
-    // (clamped to the grid, [0, ngrid - 1]: exact for every centre on the
-    // grid, and i - c then fits in 32 bits for every grid index i; a centre
-    // off the grid leaves its offset in phi, which has the sign of i - c, so
-    // u = (i - c) beta - phi takes no cancellation)
-    double cf = rint((r.nu0p - nu_min) * idnu);
-    const bool clamped = cf < 0.0 || cf > (double)(ngrid - 1);
-    if (cf < 0.0) cf = 0.0;
-    if (cf > (double)(ngrid - 1)) cf = (double)(ngrid - 1);
-    q.c = (int32_t)cf;
-    q.ilo = r.ilo;
-    q.ihi = r.ihi;
-    q.phi_k = (float)((r.nu0p - (nu_min + cf * dnu)) * r.ku);
-    q.beta = (float)(dnu * r.ku);
-    q.a = (float)r.a;
-    q.a2 = (float)r.a2;
-    const double sp = r.Sp * pow2mE;
-    q.P1 = (float)(sp * r.a * INV_SQRTPI);
-    q.P3 = (float)(sp * r.a * P3_FACTOR);
-    q.Sp = (float)sp;
+    LineRec32 q = r32[l];
+    const bool clamped = q.sig1 != 0.0f;
+    {
+      // 2^(e - E) in two factors: the first step stays normal
+      const int d = min(max(__float_as_int(q.erfcx_a) - E, -250), 120);
+      const float f1 = f_pow2(d / 2), f2 = f_pow2(d - d / 2);
+      q.Sp = q.Sp * f1 * f2;
+      q.P1 = q.P1 * f1 * f2;
+      q.P3 = q.P3 * f1 * f2;
+    }
     if (q.a < 10.0f) {  // Algorithm 916 per-line factors, in FP32
       q.erfcx_a = erfcxf(q.a);
       float s1 = 0.0f;
@@ -606,7 +845,7 @@ cudaError_t launch_pack32(helk_ctx *c, int n_cond, const helk_grid &g) {
   if (n <= 0) return cudaSuccess;
   dim3 grid(line_blocks(c, n, n_cond), n_cond);
   ++c->launches;
-  k_pack32<<<grid, 256, 0, c->stream>>>(n, c->rec64, g.nu_min, g.dnu, g.n, c->ckey, c->cstats, c->rec32,
+  k_pack32<<<grid, 256, 0, c->stream>>>(n, g.n, c->ckey, c->cstats, c->rec32,
                                         c->core_rng, c->ckey32, &c->stats->err_flags, c->core_blk,
                                         core_blocks(g.n));
   return cudaGetLastError();
