@@ -405,6 +405,15 @@ static CondArgs make_cond(const helk_ctx *c, double T, double P, double q_ratio,
   return CondArgs{T, P, q_ratio, sqrt(T0 / T), C2 / T0 - C2 / T, C2 / T, SQRTLN2 / vth, log(T0 / T)};
 }
 
+// Which core kernel (FP32 form): the one with nodes if a line of a condition can have
+// beta <= CORE_NODE_BETA on the grid (a factor of 2 for centres beyond its end and
+// for shifts).  If none can, the plain kernel gives the same sums.
+static void choose_core_nodes(helk_ctx *c, const CondArgs *conds, int n_cond, const helk_grid &g) {
+  const double top = std::max(fabs(g.nu_min), fabs(g.nu_min + g.dnu * (double)g.n));
+  c->core_nodes = c->has_mass;
+  for (int k = 0; k < n_cond; ++k) c->core_nodes |= g.dnu * conds[k].kc <= 2.0 * CORE_NODE_BETA * top;
+}
+
 // Statistics reset and line preparation (and the FP32 records) of n_cond
 // conditions: single != NULL passes the one condition by value, otherwise
 // they are read from c->cond_dev.
@@ -516,6 +525,7 @@ helk_status helk_opacity(helk_ctx *c, double T, double P, double mass, const hel
   const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
   HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n, wg));
   const CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
+  choose_core_nodes(c, &one, 1, *g);
   stage_begin(c, HELK_STAGE_LINEPREP);
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, wg != nullptr));
   stage_end(c, HELK_STAGE_LINEPREP);
@@ -555,6 +565,7 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
   }
   HELK_TRY(ensure_call_buffers(c, 1, o, max_tiles, g->n, nullptr));
   const CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
+  choose_core_nodes(c, &one, 1, *g);
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, false));
   cudaEvent_t e0, e1;
   HELK_TRY(cuda_check(c, cudaEventCreate(&e0), "autotune"));
@@ -613,7 +624,7 @@ static std::string batch_key(const helk_ctx *c, int n_cond, double mass, const h
            c->has_mass, c->has_weight, (const void *)c->cond_host, (const void *)c->cond_dev,
            (const void *)c->cond_order, (const void *)c->core_rng);
   char b3[128];
-  snprintf(b3, sizeof b3, "|%p|%p|%p|%p|%p", (const void *)c->core_blk, (const void *)c->wingF, (const void *)c->ext64,
+  snprintf(b3, sizeof b3, "|%d|%p|%p|%p|%p|%p", c->core_nodes, (const void *)c->core_blk, (const void *)c->wingF, (const void *)c->ext64,
            (const void *)c->kcore64, (const void *)c->ckey32);
   return std::string(b) + b2 + b3;
 }
@@ -709,8 +720,9 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   if (!c->cond_ev) HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->cond_ev, cudaEventDisableTiming), "graph"));
   // the previous batch must have read the staging buffer before it changes
   HELK_TRY(cuda_check(c, cudaEventSynchronize(c->cond_ev), "opacity_batch"));
-  for (int k = 0; k < n_cond; ++k) 
+  for (int k = 0; k < n_cond; ++k)
     c->cond_host[k] = make_cond(c, T[k], P[k], q_ratio ? q_ratio[k] : o.q_ratio, mass);
+  choose_core_nodes(c, c->cond_host, n_cond, *g);
   stage_begin(c, HELK_STAGE_VOIGT);
   for (int j = 0; j < nchunk; ++j) {
     const int k0 = j * chunk, nk = std::min(chunk, n_cond - k0);

@@ -190,6 +190,7 @@ struct helk_ctx {
   helk::DevStats *stats = nullptr;      // device
   helk::DevStats *stats_host = nullptr; // pinned
   // conditions of the current call
+  bool core_nodes = false;  // this call's choice of core kernel
   helk::CondArgs *cond_dev = nullptr, *cond_host = nullptr;  // host side pinned
   helk::CondStats *cstats = nullptr, *cstats_host = nullptr; // host side pinned
   int *cond_order = nullptr;
@@ -381,6 +382,8 @@ cudaError_t launch_voigt(helk_ctx *c, int n_cond, const helk_grid &g, const helk
                          double *kappa, int shape, int64_t ntiles);
 // FP32 form: the Algorithm 916 cores that k_voigt_f32 leaves out, added into
 // kappa (launched after launch_voigt; no-op for the FP64 form).
+// largest beta of a line whose cores are taken through nodes
+constexpr double CORE_NODE_BETA = 0.3 / 16.0;
 cudaError_t launch_voigt_core(helk_ctx *c, int n_cond, const helk_grid &g, const helk_opts &o);
 cudaError_t launch_core_add(helk_ctx *c, int n_cond, const helk_grid &g, const helk_opts &o, double *kappa);
 // k_voigt64.cu: the FP64 form (called by the dispatch above) and the
