@@ -252,7 +252,8 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
                    "lines_upload: " + std::to_string(c->stats_host->bad_lines) +
                        " lines with non-finite or negative values");
   if (c->stats_host->unsorted) {
-    HELK_TRY(cuda_check(c, launch_sort_lines(c, n), "sort lines"));
+    HELK_TRY(cuda_check(c, launch_sort_lines(c, n, c->stats_host->unsorted, c->stats_host->run_end),
+                        "sort lines"));
     HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "sort lines"));
   }
   c->nlines = n;

@@ -87,11 +87,15 @@ struct __align__(16) LineRec32 {
 static_assert(sizeof(LineRec32) == 48, "LineRec32 must be 48 bytes");
 
 // Device-side error flags and upload checks.
+// Upload: lists of at most this many ordered runs are merged, others sorted.
+constexpr int SORT_RUNS = 16;
+
 struct DevStats {
   int err_flags;                    // ERRF_*
   int bad_lines;                    // validation failures at upload
-  int unsorted;                     // upload: nu0 not ordered
+  int unsorted;                     // upload: descents of nu0, counted to SORT_RUNS or a few more
   unsigned int tile_counter;        // next (condition, tile) item of the persistent Voigt kernel
+  int run_end[SORT_RUNS];           // upload: where the first of them are (in no order)
 };
 
 // Core evaluations routed to the surrogate by the FP32 Voigt kernel: the
@@ -348,7 +352,8 @@ __device__ __forceinline__ void tma_load_1d(uint32_t dst_smem, const void *src, 
 // ---------------------------------------------------------- launchers ---
 // k_lines.cu
 cudaError_t launch_validate_lines(helk_ctx *c, int64_t n);
-cudaError_t launch_sort_lines(helk_ctx *c, int64_t n);  // orders SoA by nu0
+// descents, run_end: DevStats::unsorted and its run ends
+cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end);  // orders SoA by nu0
 // n_cond conditions: from c->cond_dev, or (n_cond == 1 and single != NULL)
 // the one condition passed by value.  Records of condition k start at
 // k * nlines; tile maps at k * ntiles.

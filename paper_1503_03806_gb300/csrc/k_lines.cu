@@ -33,7 +33,7 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
                            const double *__restrict__ gself, const double *__restrict__ ncoll,
                            const double *__restrict__ delta, const double *__restrict__ lmass,
                            const double *__restrict__ lweight, DevStats *st) {
-  int bad = 0, unsorted = 0;
+  int bad = 0;
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
        l += (int64_t)gridDim.x * blockDim.x) {
     double v = nu0[l];
@@ -46,10 +46,12 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
     if (lmass) ok = ok && isfinite(lmass[l]) && lmass[l] > 0.0;
     if (lweight) ok = ok && isfinite(lweight[l]) && lweight[l] >= 0.0;
     bad += !ok;
-    if (l + 1 < n && nu0[l + 1] < v) unsorted = 1;
+    if (l + 1 < n && nu0[l + 1] < v && *(volatile int *)&st->unsorted < SORT_RUNS) {
+      const int q = atomicAdd(&st->unsorted, 1);
+      if (q < SORT_RUNS) st->run_end[q] = (int)(l + 1);
+    }
   }
   if (bad) atomicAdd(&st->bad_lines, bad);
-  if (unsorted) atomicOr(&st->unsorted, 1);
 }
 
 cudaError_t launch_validate_lines(helk_ctx *c, int64_t n) {
@@ -187,21 +189,108 @@ __global__ void k_line_keys(int64_t n, const double *__restrict__ nu0, unsigned 
   }
 }
 
-__global__ void k_gather(int64_t n, const uint32_t *__restrict__ perm, const double *__restrict__ src,
-                         double *__restrict__ dst) {
-  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
-       l += (int64_t)gridDim.x * blockDim.x)
-    dst[l] = src[perm[l]];
+// The order of a list that is a few ordered runs one after the other (one species
+// or file each): an element's place is its place in its run plus, in every other
+// run, the number of elements before it (equal centres: earlier runs first, so the
+// order is stable), by bisection, a chain of dependent loads.  2e5 lines in 4 runs:
+// 48 us, against 320 us for the radix passes.
+struct SortRuns {
+  int n, end[SORT_RUNS + 1];
+};
+__global__ void k_merge_runs(SortRuns R, const double *__restrict__ nu0, uint32_t *__restrict__ perm) {
+  const int n = R.end[R.n - 1];
+  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < n; l += gridDim.x * blockDim.x) {
+    const double v = nu0[l];
+    int at = 0, b = 0;
+    for (int r = 0; r < R.n; ++r) {
+      const int e = R.end[r];
+      if (l >= b && l < e) {
+        at += l - b;
+      } else {
+        int lo = b, hi = e;
+        const bool before = e <= l;
+        while (lo < hi) {
+          const int m = (lo + hi) >> 1;
+          const double w = nu0[m];
+          if (before ? w <= v : w < v) lo = m + 1;
+          else hi = m;
+        }
+        at += lo - b;
+      }
+      b = e;
+    }
+    perm[at] = (uint32_t)l;
+  }
 }
 
-cudaError_t launch_sort_lines(helk_ctx *c, int64_t n) {
+// Up to four fields a launch: into the order of perm, and back to their places.
+constexpr int GATHER_FIELDS = 4;
+struct GatherSet {
+  int m;
+  double *field[GATHER_FIELDS], *tmp[GATHER_FIELDS];
+};
+__global__ void k_gather(int64_t n, const uint32_t *__restrict__ perm, GatherSet G) {
+  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
+       l += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t p = perm[l];
+    for (int f = 0; f < G.m; ++f) G.tmp[f][l] = G.field[f][p];
+  }
+}
+__global__ void k_gather_back(int64_t n, GatherSet G) {
+  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
+       l += (int64_t)gridDim.x * blockDim.x)
+    for (int f = 0; f < G.m; ++f) G.field[f][l] = G.tmp[f][l];
+}
+
+// All fields into the order of perm, as many at a time as there are scratch arrays.
+static cudaError_t reorder_fields(helk_ctx *c, int64_t n, const uint32_t *perm, double *const *tmp, int ntmp) {
+  double *fields[9] = {c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair,
+                       c->has_gself ? c->gself : nullptr, c->has_ncoll ? c->ncoll : nullptr,
+                       c->has_delta ? c->delta : nullptr, c->has_mass ? c->lmass : nullptr,
+                       c->has_weight ? c->lweight : nullptr};
+  const int gb = (int)std::min<int64_t>((n + 255) / 256, (int64_t)c->num_sms * 16);
+  GatherSet G{};
+  for (int f = 0; f <= 9; ++f) {
+    if (f < 9 && fields[f]) {
+      G.field[G.m] = fields[f];
+      G.tmp[G.m] = tmp[G.m];
+      ++G.m;
+    }
+    if (G.m == ntmp || (f == 9 && G.m > 0)) {
+      c->launches += 2;
+      k_gather<<<gb, 256, 0, c->stream>>>(n, perm, G);
+      k_gather_back<<<gb, 256, 0, c->stream>>>(n, G);
+      G.m = 0;
+    }
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end) {
   if (n <= 1) return cudaSuccess;
   const int nblk = (int)((n + RS_TILE - 1) / RS_TILE);
   // scratch: 2 key arrays, 2 value arrays, counts, one double array
   int64_t need = 2 * n * 8 + 2 * n * 4 + (int64_t)256 * nblk * 4 + n * 8 + 64;
+  const bool merge = descents < SORT_RUNS;
+  if (merge) need = (int64_t)GATHER_FIELDS * n * 8 + n * 4;
   helk_status st = ensure_buf(c, &c->tmp, &c->tmp_cap, need, "line sort scratch");
   if (st != HELK_OK) return cudaErrorMemoryAllocation;
   char *p = (char *)c->tmp;
+  int gb = (int)((n + 255) / 256);
+  if (gb > c->num_sms * 16) gb = c->num_sms * 16;
+  if (merge) {
+    double *tmp[GATHER_FIELDS];
+    for (int f = 0; f < GATHER_FIELDS; ++f, p += n * 8) tmp[f] = (double *)p;
+    uint32_t *perm = (uint32_t *)p;
+    SortRuns R{};
+    R.n = descents + 1;
+    for (int r = 0; r < descents; ++r) R.end[r] = run_end[r];
+    std::sort(R.end, R.end + descents);
+    R.end[descents] = (int)n;
+    ++c->launches;
+    k_merge_runs<<<gb, 256, 0, c->stream>>>(R, c->nu0, perm);
+    return reorder_fields(c, n, perm, tmp, GATHER_FIELDS);
+  }
   unsigned long long *ka = (unsigned long long *)p;  p += n * 8;
   unsigned long long *kb = (unsigned long long *)p;  p += n * 8;
   uint32_t *va = (uint32_t *)p;                      p += n * 4;
@@ -209,8 +298,6 @@ cudaError_t launch_sort_lines(helk_ctx *c, int64_t n) {
   uint32_t *counts = (uint32_t *)p;                  p += (int64_t)256 * nblk * 4;
   p = (char *)(((uintptr_t)p + 15) & ~(uintptr_t)15);
   double *dtmp = (double *)p;
-  int gb = (int)((n + 255) / 256);
-  if (gb > c->num_sms * 16) gb = c->num_sms * 16;
   ++c->launches;
   k_line_keys<<<gb, 256, 0, c->stream>>>(n, c->nu0, ka, va);
   for (int pass = 0; pass < 8; ++pass) {
@@ -224,18 +311,8 @@ cudaError_t launch_sort_lines(helk_ctx *c, int64_t n) {
     unsigned long long *tk = ka; ka = kb; kb = tk;
     uint32_t *tv = va; va = vb; vb = tv;
   }
-  double *fields[9] = {c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair,
-                       c->has_gself ? c->gself : nullptr, c->has_ncoll ? c->ncoll : nullptr,
-                       c->has_delta ? c->delta : nullptr, c->has_mass ? c->lmass : nullptr,
-                       c->has_weight ? c->lweight : nullptr};
-  for (int f = 0; f < 9; ++f) {
-    if (!fields[f]) continue;
-    ++c->launches;
-    k_gather<<<gb, 256, 0, c->stream>>>(n, va, fields[f], dtmp);
-    cudaError_t e = cudaMemcpyAsync(fields[f], dtmp, n * 8, cudaMemcpyDeviceToDevice, c->stream);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  double *const tmp[3] = {(double *)ka, (double *)kb, dtmp};  // the keys are done with
+  return reorder_fields(c, n, va, tmp, 3);
 }
 
 // ------------------------------------------------------- line preparation --
