@@ -710,7 +710,9 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   const int64_t rec_line =
       o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2))
                                          : (int64_t)(sizeof(LineRec64) + (wg ? sizeof(WingExt64) : 0));
-  const int64_t per_cond = std::max<int64_t>(c->nlines, 1) * rec_line;
+  // the FP64 wings route also keeps a core sum a point
+  const int64_t rec_grid = wg && o.precision != HELK_PREC_F32_KAHAN ? g->n * 8 : 0;
+  const int64_t per_cond = std::max<int64_t>(c->nlines, 1) * rec_line + rec_grid;
   const int gmax = (int)std::max<int64_t>(1, std::min<int64_t>(n_cond, c->batch_budget / per_cond));
   const int nchunk = (n_cond + gmax - 1) / gmax;
   const int chunk = (n_cond + nchunk - 1) / nchunk;

@@ -774,7 +774,9 @@ helk_status ensure_wing32(helk_ctx *c, int n_cond, const WingGeom &g) {
   float *p = nullptr;
   st = cuda_check(c, cudaMalloc((void **)&p, f.size() * 4), "wing tables");
   if (st != HELK_OK) return st;
-  st = cuda_check(c, cudaMemcpy(p, f.data(), f.size() * 4, cudaMemcpyHostToDevice), "wing tables");
+  // on the context's stream and waited for, so that every stream finds it complete
+  st = cuda_check(c, cudaMemcpyAsync(p, f.data(), f.size() * 4, cudaMemcpyHostToDevice, c->stream), "wing tables");
+  if (st == HELK_OK) st = cuda_check(c, cudaStreamSynchronize(c->stream), "wing tables");
   if (st == HELK_OK)
     c->wing_tab32 = p;
   else

@@ -799,7 +799,9 @@ helk_status ensure_wing64(helk_ctx *c, int n_cond, const WingGeom &g) {
   double *p = nullptr;
   st = cuda_check(c, cudaMalloc((void **)&p, tab.size() * 8), "wing tables");
   if (st != HELK_OK) return st;
-  st = cuda_check(c, cudaMemcpy(p, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice), "wing tables");
+  // on the context's stream and waited for, so that every stream finds it complete
+  st = cuda_check(c, cudaMemcpyAsync(p, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, c->stream), "wing tables");
+  if (st == HELK_OK) st = cuda_check(c, cudaStreamSynchronize(c->stream), "wing tables");
   if (st == HELK_OK)
     c->wing_tab64 = p;
   else
