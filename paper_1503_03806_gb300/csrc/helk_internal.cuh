@@ -45,6 +45,14 @@ constexpr double R2_GH1 = 1.0e6;
 constexpr double A916_H = 0.5;
 constexpr double A916_TAIL = 6.2;
 constexpr int A916_S1_TERMS = 13;  // e^{-(nh)^2} < 1e-18 beyond n = 13
+// e^{-(nh)^2}, h = 1/2, n = 1 .. 13: weights of the S1 series of Algorithm 916 (of the
+// line's damping only, so it is summed once per line)
+__constant__ constexpr double A916_EXP_NH2[A916_S1_TERMS] = {
+    0.77880078307140486825,  0.3678794411714423216,   0.10539922456186433678,
+    0.018315638888734180294, 0.0019304541362277092422, 0.0001234098040866795495,
+    4.7851173921290090896e-6, 1.1253517471925911451e-7, 1.6052280551856116087e-9,
+    1.3887943864964020595e-11, 7.2877240958196924193e-14, 2.3195228302435693883e-16,
+    4.477732441718301199e-19};
 
 // ------------------------------------------------------------ records ---
 struct __align__(16) LineRec64 {

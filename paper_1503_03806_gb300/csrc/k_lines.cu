@@ -17,16 +17,6 @@
 
 namespace helk {
 
-// e^{-(n h)^2}, h = 1/2, n = 1..13: weights of the S1 series of
-// Algorithm 916 (depends on the line's damping only, so it is summed once
-// per line).
-__constant__ double c_exp_nh2[A916_S1_TERMS] = {
-    0.77880078307140486825,  0.3678794411714423216,   0.10539922456186433678,
-    0.018315638888734180294, 0.0019304541362277092422, 0.0001234098040866795495,
-    4.7851173921290090896e-6, 1.1253517471925911451e-7, 1.6052280551856116087e-9,
-    1.3887943864964020595e-11, 7.2877240958196924193e-14, 2.3195228302435693883e-16,
-    4.477732441718301199e-19};
-
 // -------------------------------------------------------- validation ---
 __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const double *__restrict__ S0,
                            const double *__restrict__ El, const double *__restrict__ gair,
@@ -454,7 +444,7 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
       double s1 = 0.0;
       for (int k = 0; k < A916_S1_TERMS; ++k) {
         double nh = (double)(k + 1) * A916_H;
-        s1 += c_exp_nh2[k] / (nh * nh + a * a);
+        s1 += A916_EXP_NH2[k] / (nh * nh + a * a);
       }
       r.sig1 = s1;
     } else {
@@ -741,7 +731,7 @@ __global__ void __launch_bounds__(256)
     double cf = pt - PREP_MAGIC;
     q.c = __double2loint(pt);
     const int hp = __double2hiint(pos);
-    const bool big = (hp & 0x7FFFFFFF) >= 0x41D00000;
+    const bool big = (hp & 0x7FFFFFFF) >= 0x41DFFFFF;  // |pos| >= 2^31 - 1024: beyond any grid
     const bool below = big ? hp < 0 : q.c < 0, above = big ? hp >= 0 : q.c > A.ngrid - 1;
     if (below || above) {
       q.c = below ? 0 : (int)(A.ngrid - 1);
@@ -863,7 +853,7 @@ __global__ void k_pack32(int64_t n, int64_t ngrid, const double *__restrict__ ck
       float s1 = 0.0f;
       for (int k = 0; k < A916_S1_TERMS; ++k) {
         const float nh = (float)(k + 1) * (float)A916_H;
-        s1 += (float)c_exp_nh2[k] / (nh * nh + q.a2);
+        s1 += (float)A916_EXP_NH2[k] / (nh * nh + q.a2);
       }
       q.sig1 = s1;
     } else {

@@ -435,11 +435,13 @@ __device__ __forceinline__ double u01(uint64_t seed, uint64_t i, uint64_t k) {
   return (double)(z >> 11) * (1.0 / 9007199254740992.0);
 }
 
+// S1(y), with the e^{-(nh)^2} from a table (2.6e5 samples: 616 -> 499 us against
+// 13 FP64 exponentials a sample; the FP64 unit bounds what is left).
 __device__ double sig1_of(double y) {
   double s = 0.0;
   for (int k = 1; k <= A916_S1_TERMS; ++k) {
     const double nh = k * A916_H;
-    s += exp(-nh * nh) / (nh * nh + y * y);
+    s += A916_EXP_NH2[k - 1] / (nh * nh + y * y);
   }
   return s;
 }
