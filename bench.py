@@ -179,7 +179,7 @@ class Clocks:
 
 # The Voigt kernels' translation unit: the kernel file and the headers of
 # csrc/ it includes; the profile summaries record a hash of these sources.
-KERNEL_HEADERS = ("voigt_core.cuh", "voigt_common.cuh", "helk_internal.cuh")
+KERNEL_HEADERS = ("wings.cuh", "voigt_f32.cuh", "voigt_core.cuh", "voigt_common.cuh", "helk_internal.cuh")
 
 
 def kernel_source_hash(kernel_src):
@@ -300,8 +300,7 @@ def run_ours(args):
 
     def measure(form, clocks=False):
         prec = PREC[form]
-        tile = ctx.autotune(T, P, mass, cut, grid, precision=prec)   # one-time setup
-        # work of one step (exact counts from the counting variant)
+        # work of one step (exact counts from the counting variant, which evaluates point by point)
         ctx.opacity(T, P, mass, cut, grid, out=kappa, precision=prec, count_regions=True)
         evals, reg = ctx.stats(with_regions=True)
         f = FLOPS[form]
@@ -353,24 +352,30 @@ def run_ours(args):
         peak = peaks_meas["fp32_tflops" if form == "f32" else "fp64_tflops"]
         achieved = flops / voigt_s / 1e12
         src = os.path.join(ROOT, "paper_1503_03806_gb300", "csrc",
-                           "k_voigt.cu" if form == "f32" else "k_voigt64.cu")
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak,
+                           "k_wings.cu" if form == "f32" else "k_wings64.cu")
+        # `achieved` is the work of the point-by-point sums over the time of the
+        # stage.  The stage interpolates most of it (wings.cuh), so this is no rate
+        # of the pipe and may exceed its peak: frac is against what no kernel can
+        # do without, the line list read and kappa written once.
+        hbm_bytes = 8 * (len(lines) * lines["nu0"].shape[0] + grid[2])
+        hbm_peak = peaks.get("hbm_gbs")
+        hbm_gbs = hbm_bytes / voigt_s / 1e9
+        roof = {"bound": "alu", "achieved": achieved, "peak": peak,
+                "unit": "TFLOP/s of point-by-point work (most of it interpolated)",
+                "frac": hbm_gbs / hbm_peak if hbm_peak else None,
+                "frac_basis": "of measured copy bandwidth, for the line list read and kappa written once",
+                "hbm_floor_bytes": hbm_bytes, "hbm_floor_gbs": hbm_gbs, "hbm_peak_gbs": hbm_peak,
+                "point_by_point_over_peak": achieved / peak,
                 "traffic": traffic_from_profile(src, os.path.join(ROOT, "profiles",
-                                                                  "voigt_%s_medium.txt" % form)),
-                "kernel": "k_voigt_f32 + k_core_f32 (the Voigt stage)" if form == "f32" else "k_voigt_f64",
+                                                                  "wings_%s_medium.txt" % form)),
+                "kernel": ("k_wing_far32 + k_core_f32 + k_wing_near32" if form == "f32"
+                           else "k_wing_far64 + k_wing_near64") + " (the Voigt stage)",
                 "peak_basis": "measured: %s FMA probe of this run (peaks_measured, helk_peak_probe), burst"
                               % form.upper(),
-                "peak_derived": peak_derived, "frac_of_derived": achieved / peak_derived,
+                "peak_derived": peak_derived,
                 "peak_derived_basis": "%s pipe: %d FMA/clk/SM x %d SMs x %.0f MHz max clock"
                                       % (form.upper(), FMA_PER_CLK_SM[form], nsm, max_mhz),
-                "flops_per_launch": flops, "voigt_ms_per_launch": voigt_s * 1e3,
-                "kernel_shape": helk.helk_tile_shape(prec, tile)}
-        if form == "f32":
-            # MUFU co-bound: one reciprocal per GH1 or GH3 evaluation
-            rcp = float(reg[1] + reg[2])
-            roof["mufu_rcp_per_launch"] = int(rcp)
-            roof["mufu_frac"] = rcp / voigt_s / (peaks_meas["mufu_rcp_tops"] * 1e12)
+                "flops_per_launch": flops, "voigt_ms_per_launch": voigt_s * 1e3}
         return {"form": form, "evals": evals, "reg": [int(x) for x in reg], "ms_step": ms_step,
                 "launches": launches,
                 "value": world * evals / (ms_step * 1e-3), "roofline": roof, "wall": wall,
@@ -387,9 +392,6 @@ def run_ours(args):
     sel = r > 1e-8 * r.max(dim=1, keepdim=True).values
     err32 = float(((g - r).abs() / r)[sel].max().item())
     clocks = r32["clocks"]
-    if clocks and clocks.get("sm_mhz"):
-        for rr in (r64, r32):
-            rr["roofline"]["frac_at_median_clock"] = rr["roofline"]["frac"] * max_mhz / clocks["sm_mhz"]
 
     # end to end through the C ABI from pinned host memory (FP32 form)
     e2e = None
@@ -430,21 +432,6 @@ def run_ours(args):
         gt = (wt["nu_min"], wt["dnu"], wt["ngrid"])
         ctx.upload(tl)
         kb = torch.empty((len(Ts), gt[2]), dtype=torch.float64, device="cuda")
-        # the kernel shape tuned on the batch call itself (one timed call a
-        # candidate shape; a single condition's choice need not suit the mix)
-        tile_b, best = None, None
-        for code in helk.helk_tile_candidates(PREC["f32"]):
-            ctx.set_tile(PREC["f32"], gt[2], code)
-            ctx.opacity_batch(Ts, Ps, wt["mass"], wt["cut"], gt, out=kb, precision=PREC["f32"], q_ratio=qs)
-            torch.cuda.synchronize()
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            ctx.opacity_batch(Ts, Ps, wt["mass"], wt["cut"], gt, out=kb, precision=PREC["f32"], q_ratio=qs)
-            b.record()
-            torch.cuda.synchronize()
-            if best is None or a.elapsed_time(b) < best:
-                tile_b, best = code, a.elapsed_time(b)
-        ctx.set_tile(PREC["f32"], gt[2], tile_b)
         ctx.opacity_batch(Ts, Ps, wt["mass"], wt["cut"], gt, out=kb, precision=PREC["f32"], q_ratio=qs,
                           count_regions=True)
         ev_b, _ = ctx.batch_stats(len(Ts))
@@ -468,10 +455,10 @@ def run_ours(args):
                            "cutoff min(500 Gamma_L, 100 cm^-1), %d bins x %d coefficients"
                            % (wt["nlines"], len(Ts), min(Ts), max(Ts), min(Ps), max(Ps), gt[2],
                               wt["nbins"], wt["ncheb"]),
-               "form": "FP32 + Kahan, one graph-captured persistent launch per call",
+               "form": "FP32 + Kahan, one captured graph per call",
                "ms_per_call": ms_b, "ms_per_condition": ms_b / len(Ts),
                "evals_per_call": int(ev_b.sum()), "value": int(ev_b.sum()) / (ms_b * 1e-3),
-               "unit": UNIT, "kernel_shape": helk.helk_tile_shape(PREC["f32"], tile_b),
+               "unit": UNIT,
                "stages_ms_per_call": {k: v[0] / max(1, v[1]) for k, v in st_b.items() if v[1]}}
         del kb
         ctx.upload(lines)
@@ -668,14 +655,12 @@ def leg_surrogate_workload(ctx, args, prec, trained, flush):
     ctx.upload(ls)
     del ls
     k = torch.empty(g[2], dtype=torch.float64, device="cuda")
-    tile = ctx.autotune(Tq, Pq, ws["mass"], ws["cut"], g, precision=prec, q_ratio=q)  # one-time setup
     ctx.opacity(Tq, Pq, ws["mass"], ws["cut"], g, out=k, precision=prec, q_ratio=q, count_regions=True)
     evals, reg = ctx.stats(with_regions=True)
     out = {"workload": "surrogate: %d lines, %d-point grid, cutoff min(500 Gamma_L, 100 cm^-1), T %g K, "
                        "P %g atm, %d bins x %d coefficients"
                        % (ws["nlines"], g[2], Tq, Pq, ws["nbins"], ws["ncheb"]),
-           "evals_per_step": int(evals), "alg916_share": float(reg[0]) / max(1, int(evals)),
-           "kernel_shape": helk.helk_tile_shape(prec, tile)}
+           "evals_per_step": int(evals), "alg916_share": float(reg[0]) / max(1, int(evals))}
     forms = {"fp32": False}
     if trained:
         forms["fp32_surrogate"] = True
@@ -786,9 +771,7 @@ def run_profile_surrogate():
 
 
 def run_profile_case(form):
-    """Short fixed run for profilers: upload the workload, autotune the Voigt
-    tile shape as the benchmark does (4 launches of the Voigt kernel per
-    built tile shape; the count is printed, for ncu's -s), then two passes of
+    """Short fixed run for profilers: upload the workload, then two passes of
     opacity (FP32 or FP64 form) + k-tables."""
     import torch
     import __graft_entry__
@@ -799,9 +782,6 @@ def run_profile_case(form):
     ctx = helk.Context(0)
     ctx.upload(synth.workload_lines(WORKLOAD))
     grid = (w["nu_min"], w["dnu"], w["ngrid"])
-    tile = ctx.autotune(w["T"][0], w["P_atm"][0], w["mass"], w["cut"], grid, precision=prec)
-    print("profile case %s: %d autotune launches of the Voigt kernel, then shape %s"
-          % (form, 4 * len(helk.helk_tile_candidates(prec)), helk.helk_tile_shape(prec, tile)), flush=True)
     kappa = torch.empty(w["ngrid"], dtype=torch.float64, device="cuda")
     for _ in range(2):
         ctx.opacity(w["T"][0], w["P_atm"][0], w["mass"], w["cut"], (w["nu_min"], w["dnu"], w["ngrid"]),

@@ -181,7 +181,7 @@ helk_status helk_opacity(helk_ctx *ctx, double T, double P_atm,
                          double *kappa_out);
 
 /* Opacities of the uploaded lines at n_cond conditions (T[k], P_atm[k]) on
- * one grid, in one persistent launch (Sec. 2.3-2.4; the paper's many (T, P)
+ * one grid, in one captured sequence of launches (Sec. 2.3-2.4; the paper's many (T, P)
  * points).  kappa_out: device pointer to n_cond * grid->n doubles, row k =
  * condition k (NULL: the context's buffer, read by helk_kdist with
  * kappa == NULL and n = n_cond * grid->n -- the k-tables of all conditions
@@ -191,11 +191,13 @@ helk_status helk_opacity(helk_ctx *ctx, double T, double P_atm,
  * once per call shape (n_cond, line list, grid, cutoff, options, output
  * pointer, tile shape) into a CUDA graph and replayed on later calls with the
  * same shape; only the condition values change between replays.  The
- * per-condition line records take 64 B (FP64 form) or 120 B (FP32 form) per
- * line; when those of all n_cond conditions exceed the record budget
+ * per-condition line records take 56 B (FP32 form) or 96 B (FP64 form; with
+ * windows of fewer than 64 points to a side 64 B) per line, in the FP64 form
+ * also 8 B per grid point; when those of all n_cond conditions exceed the
+ * record budget
  * (64 GiB unless set by helk_set_batch_budget), the conditions run in the
- * fewest equal chunks that fit, each chunk its own captured graph and
- * persistent launch, one after the other on the stream (the context keeps
+ * fewest equal chunks that fit, each chunk its own captured graph, one after
+ * the other on the stream (the context keeps
  * the 16 most recent graphs).  The results equal those of n_cond
  * helk_opacity calls bit for bit.  A call waits until the previous batch call
  * has read its conditions. */
@@ -261,6 +263,9 @@ helk_status helk_kdist(helk_ctx *ctx, const double *kappa, int64_t n,
  * configuration of a precision's persistent Voigt kernel: the tile (grid
  * points per CTA tile), the warps per CTA and the candidate lines per
  * pipeline stage; it is named by a shape code (helk_tile_shape decodes it).
+ * The shapes are those of the kernels that evaluate every point of a window;
+ * calls without count_regions whose windows can reach 64 points or more to a
+ * side interpolate the wings and take no shape.
  * Runs the line preparation of this condition once, then times every
  * candidate shape of opts->precision on it (three launches each, CUDA events
  * on the context stream) and keeps the fastest for later helk_opacity calls
