@@ -192,7 +192,7 @@ helk_status helk_opacity(helk_ctx *ctx, double T, double P_atm,
  * pointer, tile shape) into a CUDA graph and replayed on later calls with the
  * same shape; only the condition values change between replays.  The
  * per-condition line records take 56 B (FP32 form) or 96 B (FP64 form; with
- * windows of fewer than 64 points to a side 64 B) per line, in the FP64 form
+ * windows of fewer than 24 points to a side 64 B) per line, in the FP64 form
  * also 8 B per grid point; when those of all n_cond conditions exceed the
  * record budget
  * (64 GiB unless set by helk_set_batch_budget), the conditions run in the
@@ -264,8 +264,9 @@ helk_status helk_kdist(helk_ctx *ctx, const double *kappa, int64_t n,
  * points per CTA tile), the warps per CTA and the candidate lines per
  * pipeline stage; it is named by a shape code (helk_tile_shape decodes it).
  * The shapes are those of the kernels that evaluate every point of a window;
- * calls without count_regions whose windows can reach 64 points or more to a
- * side interpolate the wings and take no shape.
+ * calls without count_regions whose windows can reach 24 points to a side in
+ * the FP64 form, or 64 and ~40 lines to a point in the FP32 form, interpolate
+ * the wings and take no shape.
  * Runs the line preparation of this condition once, then times every
  * candidate shape of opts->precision on it (three launches each, CUDA events
  * on the context stream) and keeps the fastest for later helk_opacity calls

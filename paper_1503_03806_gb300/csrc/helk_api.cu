@@ -344,7 +344,12 @@ static bool wing_route(const helk_ctx *c, const helk_opts &o, const helk_cutoff 
   double half = (double)g->n;
   if (cut->kind == HELK_CUT_ABS) half = std::min(half, cut->value / g->dnu);
   if (cut->kind == HELK_CUT_LORENTZ) half = std::min(half, cut->cap / g->dnu);
-  if (half < WING_MIN_HALF) return false;
+  if (o.precision != HELK_PREC_F32_KAHAN) {
+    if (half < WING64_MIN_HALF) return false;
+  } else {
+    const bool sparse = 2.0 * half * (double)c->nlines < WING32_MIN_LINES * (double)g->n;
+    if (half < WING32_MIN_HALF || (sparse && g->n > (int64_t)c->num_sms * 512)) return false;
+  }
   *out = wing_geometry(g->n, half, c->num_sms);
   return true;
 }
