@@ -740,7 +740,7 @@ def leg_mixed(ctx, prec, device_index, peaks):
            "kdist_hbm": {"bytes": 8 * n_all, "achieved": kd_gbs, "unit": "GB/s",
                          "peak": peaks.get("hbm_gbs"),
                          "frac": kd_gbs / peaks["hbm_gbs"] if peaks.get("hbm_gbs") else None,
-                         "note": "bins of 30000 points: bucket-sorted through global ping-pong buffers; the "
+                         "note": "bins of 30000 points: split by value into parts sorted in shared memory; the "
                                  "one-time pseudo-inverse of this bin size is built before the timing"},
            "stages_ms": {k: v[0] for k, v in st.items() if v[1]},
            "clocks": clk.summary(), "timed_calls": 1}

@@ -2,7 +2,7 @@
 //
 // One CTA per bin: the bin's opacities (non-negative doubles, ordered as
 // their IEEE bit patterns) are sorted in shared memory when they fit (larger bins
-// by value in two to four parts that do, else in a global ping-pong buffer), then the same CTA computes
+// by value in up to eight parts that do, else in a global ping-pong buffer), then the same CTA computes
 // L_j = ln max(k_j, kappa_floor) on g_j = (j + 1/2)/N_b and the least-squares
 // Chebyshev coefficients c = P L, where P is the pseudo-inverse of the design
 // matrix (shared by all bins of one size; computed once by k_pinv).

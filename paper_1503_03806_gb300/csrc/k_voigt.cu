@@ -299,6 +299,9 @@ __global__ void __launch_bounds__(BLOCK, MINB)
 // The per-point sums go to kcore (every point written), so the kernel can run
 // beside others; they are added into kappa rescaled like the main sums.
 // Kahan-compensated: hundreds of cores can overlap at a point.
+// Bound by instruction issue (81 % of the slots, ~150 a line and warp): 1e5 lines, 3e6
+// points 129 us, 12 conditions of 1e6 lines 3.38 ms (141 us and 4.53 ms with a
+// recurrence over the series terms of each point).
 constexpr int CORE_BLOCK = 128;
 
 struct __align__(16) CoreLine {

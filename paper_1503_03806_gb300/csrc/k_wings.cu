@@ -5,9 +5,10 @@
 // k_core_f32, whose sums the near kernel adds.
 //
 // Against the direct kernel (k_voigt_f32, every line at every point of its
-// window): the 1e5-line, 3e6-point step 0.90 -> 0.61 ms, 1e6 lines at 12
-// conditions 29.9 -> 17.3 ms, 1e7 lines 32.5 -> 24.7 ms, with errors against
-// 64 bits unchanged.  Both kernels are bound by instruction issue at the
+// window), far + near: 1e5 lines, 3e6 points 702 -> 259 us (69 % of the issue
+// slots in near, 55 % in far), 1e6 lines at 12 conditions 21.0 -> 6.3 ms, 1e7
+// lines 21.3 -> 9.2 ms, with errors against 64 bits no larger.
+// Both kernels are bound by instruction issue at the
 // latency that their warps in flight hide: 64 registers (4 CTAs an SM, a few
 // spilled words in the near kernel's way down the tree) beat 128 (2 CTAs) by
 // 5-10 %.
@@ -491,7 +492,8 @@ __device__ __forceinline__ void wing_children(const float (&M)[W32_P], const Win
 // on the leaves (GH1 throughout, or per point).
 enum { SUB_H = 0, SUB_L = 2, SUB_G1 = 6, SUB_D = 10, SUB_N = 14 };
 // Leaf lists up to this length are run point by point: at one point a lane that
-// costs a line no more than a short list's nodes.
+// costs a line no more than a short list's nodes (1e5 lines, 3e6 points: near
+// 211 us, 428 us with every leaf list through nodes).
 constexpr int W32_LEAF_MIN = 6;
 
 // NL: leaves of a warp's panel, 4 or 1 (WingGeom::lvl0 2 or 0).

@@ -7,7 +7,9 @@
 //
 // The FP64 unit (2 lanes a clock per SM, 1/64 of the FP32 rate) bounds all of
 // it, so classes and lists are integer and FP32 work and a node or point costs
-// 9 (GH1) to 15 (GH3) FP64 instructions.
+// 9 (GH1) to 15 (GH3) FP64 instructions.  1e5 lines, 3e6 points: far and cores
+// 3.88 ms, near 4.09 ms, both at 86-87 % of the unit's issue rate, against 97.2 ms
+// for every line at every point; 1e4 lines, 3e5 points 0.17 + 0.39 against 2.85 ms.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
