@@ -649,7 +649,9 @@ __device__ __forceinline__ F2 prep_exp(F2 z, int &m, bool minus1) {
 // from v (1 / dnu) where no integer lies within the rounding of that or of the
 // division (2^-46 |q|; both err by < 2^-51 |q|), else by the division itself.
 // Adding 1.5 2^52 leaves the nearest integer in the low word; comparisons are made
-// on the high words, so the common path is a product and three additions.
+// on the high words, so the common path is a product and three additions.  Zero
+// (a window that begins on the grid's first point) is an integer too, but has no
+// exponent for that comparison: it has its own test.
 constexpr double PREP_MAGIC = 6755399441055744.0;
 __device__ __noinline__ int prep_index_div(double v, double dnu, bool up) {
   const double q = v / dnu;
@@ -660,7 +662,8 @@ template <bool UP>
 __device__ __forceinline__ int prep_index(double v, double dnu, double idnu) {
   const double q = v * idnu, t = q + PREP_MAGIC, d = q - (t - PREP_MAGIC);
   const int hq = __double2hiint(q) & 0x7FFFFFFF, hd = __double2hiint(d), r = __double2loint(t);
-  if (hq >= 0x41D00000 || hq - (hd & 0x7FFFFFFF) >= 46 << 20) return prep_index_div(v, dnu, UP);
+  const int ad = hd & 0x7FFFFFFF;
+  if (hq >= 0x41D00000 || ad == 0 || hq - ad >= 46 << 20) return prep_index_div(v, dnu, UP);
   return UP ? r + (hd >= 0 ? 1 : 0) : r - (hd < 0 ? 1 : 0);
 }
 
