@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/helk.h"
+#include "sort_runs.cuh"
 
 // Line-record budget of one chunk of helk_opacity_batch (64 GiB).
 constexpr int64_t HELK_DEFAULT_BATCH_BUDGET = (int64_t)64 << 30;
@@ -95,9 +96,6 @@ struct __align__(16) LineRec32 {
 static_assert(sizeof(LineRec32) == 48, "LineRec32 must be 48 bytes");
 
 // Device-side error flags and upload checks.
-// Upload: lists of at most this many ordered runs are merged, others sorted.
-constexpr int SORT_RUNS = 16;
-
 struct DevStats {
   int err_flags;                    // ERRF_*
   int bad_lines;                    // validation failures at upload

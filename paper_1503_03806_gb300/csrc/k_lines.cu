@@ -179,38 +179,12 @@ __global__ void k_line_keys(int64_t n, const double *__restrict__ nu0, unsigned 
   }
 }
 
-// The order of a list that is a few ordered runs one after the other (one species
-// or file each): an element's place is its place in its run plus, in every other
-// run, the number of elements before it (equal centres: earlier runs first, so the
-// order is stable), by bisection, a chain of dependent loads.  2e5 lines in 4 runs:
-// 48 us, against 320 us for the radix passes.
-struct SortRuns {
-  int n, end[SORT_RUNS + 1];
-};
+// The order of a list that is a few ordered runs (sort_runs.cuh).  2e5 lines in 4
+// runs: 48 us, against 320 us for the radix passes.
 __global__ void k_merge_runs(SortRuns R, const double *__restrict__ nu0, uint32_t *__restrict__ perm) {
-  const int n = R.end[R.n - 1];
-  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < n; l += gridDim.x * blockDim.x) {
-    const double v = nu0[l];
-    int at = 0, b = 0;
-    for (int r = 0; r < R.n; ++r) {
-      const int e = R.end[r];
-      if (l >= b && l < e) {
-        at += l - b;
-      } else {
-        int lo = b, hi = e;
-        const bool before = e <= l;
-        while (lo < hi) {
-          const int m = (lo + hi) >> 1;
-          const double w = nu0[m];
-          if (before ? w <= v : w < v) lo = m + 1;
-          else hi = m;
-        }
-        at += lo - b;
-      }
-      b = e;
-    }
-    perm[at] = (uint32_t)l;
-  }
+  const int64_t n = R.end[R.n - 1];
+  for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n; l += (int64_t)gridDim.x * blockDim.x)
+    perm[merged_place(R, l, [=](int64_t i) { return nu0[i]; })] = (uint32_t)l;
 }
 
 // Up to four fields a launch: into the order of perm, and back to their places.
