@@ -615,24 +615,30 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
 // (condition upload from pinned staging, statistics reset, line preparation,
 // FP32 records, tile maps, condition order, Voigt kernel) is captured once
 // into a CUDA graph per call shape and replayed.
+// The key of a captured sequence: its shape, and the address of every buffer that it
+// reads or writes and that a later call may move (all of them: a list that grows and
+// shrinks again can move some and leave others where they were).
 static std::string batch_key(const helk_ctx *c, int n_cond, double mass, const helk_cutoff *cut,
                              const helk_grid *g, const helk_opts &o, const double *kappa, int shape) {
-  char b[512];
-  snprintf(b, sizeof b, "%d|%lld|%p|%a|%d|%a|%a|%a|%a|%lld|%d|%d|%a|%d|%d|%p|%d|%p|%p|%p|%p|%p|%p", n_cond,
-           (long long)c->nlines, (const void *)c->nu0, mass, cut->kind, cut->value, cut->cap, g->nu_min,
-           g->dnu, (long long)g->n, o.precision, o.accumulate, o.weight, o.count_regions, o.surrogate,
-           (const void *)kappa, shape, (const void *)c->rec64, (const void *)c->rec32,
-           (const void *)c->tile_lo, (const void *)c->cstats, (const void *)c->squeue, (const void *)c->kcore);
-  // the line fields present (absent ones are passed to line preparation as
-  // null pointers) and the per-condition arrays of the chunk
-  char b2[192];
-  snprintf(b2, sizeof b2, "|%d%d%d%d%d%d|%p|%p|%p|%p", c->has_E, c->has_gself, c->has_ncoll, c->has_delta,
-           c->has_mass, c->has_weight, (const void *)c->cond_host, (const void *)c->cond_dev,
-           (const void *)c->cond_order, (const void *)c->core_rng);
-  char b3[128];
-  snprintf(b3, sizeof b3, "|%d|%p|%p|%p|%p|%p", c->core_nodes, (const void *)c->core_blk, (const void *)c->wingF, (const void *)c->ext64,
-           (const void *)c->kcore64, (const void *)c->ckey32);
-  return std::string(b) + b2 + b3;
+  char b[256];
+  snprintf(b, sizeof b, "%d|%lld|%a|%d|%a|%a|%a|%a|%lld|%d|%d|%a|%d|%d|%d|%d", n_cond, (long long)c->nlines, mass,
+           cut->kind, cut->value, cut->cap, g->nu_min, g->dnu, (long long)g->n, o.precision, o.accumulate, o.weight,
+           o.count_regions, o.surrogate, shape, (int)c->core_nodes);
+  std::string key(b);
+  // the line fields (absent ones are passed to line preparation as null pointers)
+  const void *const bufs[] = {c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair, c->has_gself ? c->gself : nullptr,
+                              c->has_ncoll ? c->ncoll : nullptr, c->has_delta ? c->delta : nullptr,
+                              c->has_mass ? c->lmass : nullptr, c->has_weight ? c->lweight : nullptr,
+                              // per condition (a chunk's view of them)
+                              c->cond_host, c->cond_dev, c->cstats, c->cond_order,
+                              // records, maps, sums
+                              c->rec64, c->rec32, c->ext64, c->ckey, c->ckey32, c->core_rng, c->core_blk, c->tile_lo,
+                              c->tile_hi, c->kcore, c->kcore64, c->wingF, c->squeue, kappa};
+  for (const void *p : bufs) {
+    snprintf(b, sizeof b, "|%p", p);
+    key += b;
+  }
+  return key;
 }
 
 // The per-condition arrays as seen by a chunk of a batch: offset by the
