@@ -1662,8 +1662,8 @@ cudaError_t launch_kdist_bins(helk_ctx *c, const double *kappa, int64_t n, int n
 // The smallest value k_0 of a bin is factored out: T = e^{-k_0 m} S / N,
 // S = sum_j e^{-d_j}, d_j = (k_j - k_0) m >= 0, so S lies in [1, N] and each
 // term in (0, 1].  Terms with d_j >= 87 are below 2^-125 of S and left out
-// (for sorted values: every term from the first such j on, found by a binary
-// search); the rest are evaluated on the FP32 pipe as float-float pairs:
+// (whole blocks of values by the block's range); the rest are evaluated on the
+// FP32 pipe as float-float pairs:
 // k_j - k_0 is formed once per point in FP64 and kept as a pair D_j scaled
 // by the bin's 2^-F (F the exponent of the largest difference), d_j = D_j M
 // with M = m 2^F, and e^{-d} by a table-driven exponential (Tang 1989):
@@ -1948,9 +1948,9 @@ __device__ __forceinline__ float2 tr_poly(const float *a, int64_t stride, float 
   return make_float2(h, s.y - (h - s.x));
 }
 
-// A warp takes `per` (a power of two up to 32) column masses of a bin: the lanes
-// prepare one each (the FP64 work), then the warp runs through them, the lanes
-// sharing the bin's blocks.
+// A warp takes `per` (a power of two up to 32) column masses of a bin at a time: the
+// lanes prepare one each (the FP64 work), then the warp runs through them, the
+// lanes sharing the bin's blocks.
 __global__ void __launch_bounds__(TR_THREADS)
     k_trans_direct(const double *__restrict__ sorted, int64_t nb, int nm, const double *__restrict__ m,
                    const float2 *__restrict__ D, const TrBin *__restrict__ bins, const float *__restrict__ blk,
@@ -1965,81 +1965,83 @@ __global__ void __launch_bounds__(TR_THREADS)
   const int64_t nblk = tr_nblk(nb);
   const int used = (int)((nb - B.ju + TR_BLK - 1) / TR_BLK);
   const float *Bk = blk + (int64_t)b * TR_ROWS * nblk;
-  const int i = (blockIdx.y * (TR_THREADS / 32) + (threadIdx.x >> 5)) * per + lane;
-  if (i - lane >= nm) return;  // warp-uniform
-  const bool have = lane < per && i < nm;
-  const double mi = have ? m[i] : 0.0;
-  if (!B.ok) {  // the plain FP64 sum
-    for (int s = 0; s < per && i - lane + s < nm; ++s) {
-      const double ms = __shfl_sync(0xffffffffu, mi, s);
-      double t = 0.0;
-      for (int64_t j = lane; j < nb; j += 32) t += exp(-k[j] * ms);
-      t = warp_sum(t);
-      if (lane == 0) out[(int64_t)b * nm + i + s] = t / (double)nb;
+  const int64_t step = (int64_t)gridDim.y * (TR_THREADS / 32) * per;
+  for (int64_t i0 = ((int64_t)blockIdx.y * (TR_THREADS / 32) + (threadIdx.x >> 5)) * per; i0 < nm; i0 += step) {  // warp-uniform
+    const int64_t i = i0 + lane;
+    const bool have = lane < per && i < nm;
+    const double mi = have ? m[i] : 0.0;
+    if (!B.ok) {  // the plain FP64 sum
+      for (int s = 0; s < per && i0 + s < nm; ++s) {
+        const double ms = __shfl_sync(0xffffffffu, mi, s);
+        double t = 0.0;
+        for (int64_t j = lane; j < nb; j += 32) t += exp(-k[j] * ms);
+        t = warp_sum(t);
+        if (lane == 0) out[(int64_t)b * nm + i0 + s] = t / (double)nb;
+      }
+      continue;
     }
-    return;
-  }
-  const double E0 = exp(-(B.k0 * mi));  // 0: every term underflows, as e^{-k_0 m} does
-  const double Md = mi * B.scale;
-  const bool pairs = Md < 0x1p107;  // else every pair has d >= 128
-  const float2 M = split_pair(pairs ? Md : 0.0);
-  const uint32_t run = __ballot_sync(0xffffffffu, have && E0 > 0.0 && pairs);
-  float2 mine = make_float2(0.0f, 0.0f);
-  double pd = 0.0;
-  if (B.ju > B.jz) {  // tiny differences, FP64
-    for (int64_t j = B.jz; j < B.ju; ++j) {
-      const double d = (k[j] - B.k0) * mi;
-      if (d < TR_DMAX) pd += exp(-d);
+    const double E0 = exp(-(B.k0 * mi));  // 0: every term underflows, as e^{-k_0 m} does
+    const double Md = mi * B.scale;
+    const bool pairs = Md < 0x1p107;  // else every pair has d >= 128
+    const float2 M = split_pair(pairs ? Md : 0.0);
+    const uint32_t run = __ballot_sync(0xffffffffu, have && E0 > 0.0 && pairs);
+    float2 mine = make_float2(0.0f, 0.0f);
+    double pd = 0.0;
+    if (B.ju > B.jz) {  // tiny differences, FP64
+      for (int64_t j = B.jz; j < B.ju; ++j) {
+        const double d = (k[j] - B.k0) * mi;
+        if (d < TR_DMAX) pd += exp(-d);
+      }
     }
-  }
-  for (uint32_t left = run; left; left &= left - 1) {
-    const int s = __ffs(left) - 1;
-    const float2 Ms = make_float2(__shfl_sync(0xffffffffu, M.x, s), __shfl_sync(0xffffffffu, M.y, s));
-    float sh = 0.0f, sl = 0.0f, sf = 0.0f;
-    for (int q0 = 0; q0 < used; q0 += 32) {
-      const int q = q0 + lane;
-      float c = 0.0f, R = 0.0f;
-      if (q < used) {
-        c = Bk[q];
-        R = Bk[nblk + q];
-      }
-      const float low = isinf(R) ? 0.0f : (c - R) * Ms.x;
-      const bool use = q < used && low < (float)TR_DMAX;
-      const bool narrow = use && R * Ms.x <= 1.0f;
-      if (!__any_sync(0xffffffffu, use)) {
-        // later blocks hold larger values still
-        if (__all_sync(0xffffffffu, q >= used || !isinf(R))) break;
-      }
-      if (narrow) {
-        const float2 S = tr_poly(Bk + q, nblk, R, Ms);
-        const float2 d = ff_prod(make_float2(c, 0.0f), Ms);
-        tr_acc(sh, sl, ff_mul(ff_exp_neg(d.x, d.y, tab, L), S));
-      }
-      for (uint32_t wide = __ballot_sync(0xffffffffu, use && !narrow); wide; wide &= wide - 1) {
-        const int o = __ffs(wide) - 1;
-        const float lo = __shfl_sync(0xffffffffu, low, o);
-        const int64_t j = B.ju + (int64_t)(q0 + o) * TR_BLK + lane;
-        if (lo > TR_D32) {
-          const float d0 = j < nb ? Db[j].x * Ms.x : 1.0e3f, d1 = j + 32 < nb ? Db[j + 32].x * Ms.x : 1.0e3f;
-          if (d0 < (float)TR_DMAX) sf += expf(-d0);
-          if (d1 < (float)TR_DMAX) sf += expf(-d1);
-        } else {
-          const float2 far = make_float2(INFINITY, 0.0f);
-          const float2 d0 = j < nb ? ff_prod(Db[j], Ms) : far, d1 = j + 32 < nb ? ff_prod(Db[j + 32], Ms) : far;
-          const float2 e0 = ff_exp_neg(fminf(d0.x, 86.0f), d0.y, tab, L);
-          const float2 e1 = ff_exp_neg(fminf(d1.x, 86.0f), d1.y, tab, L);
-          if (d0.x < (float)TR_DMAX) tr_acc(sh, sl, e0);
-          if (d1.x < (float)TR_DMAX) tr_acc(sh, sl, e1);
+    for (uint32_t left = run; left; left &= left - 1) {
+      const int s = __ffs(left) - 1;
+      const float2 Ms = make_float2(__shfl_sync(0xffffffffu, M.x, s), __shfl_sync(0xffffffffu, M.y, s));
+      float sh = 0.0f, sl = 0.0f, sf = 0.0f;
+      for (int q0 = 0; q0 < used; q0 += 32) {
+        const int q = q0 + lane;
+        float c = 0.0f, R = 0.0f;
+        if (q < used) {
+          c = Bk[q];
+          R = Bk[nblk + q];
+        }
+        const float low = isinf(R) ? 0.0f : (c - R) * Ms.x;
+        const bool use = q < used && low < (float)TR_DMAX;
+        const bool narrow = use && R * Ms.x <= 1.0f;
+        if (!__any_sync(0xffffffffu, use)) {
+          // later blocks hold larger values still
+          if (__all_sync(0xffffffffu, q >= used || !isinf(R))) break;
+        }
+        if (narrow) {
+          const float2 S = tr_poly(Bk + q, nblk, R, Ms);
+          const float2 d = ff_prod(make_float2(c, 0.0f), Ms);
+          tr_acc(sh, sl, ff_mul(ff_exp_neg(d.x, d.y, tab, L), S));
+        }
+        for (uint32_t wide = __ballot_sync(0xffffffffu, use && !narrow); wide; wide &= wide - 1) {
+          const int o = __ffs(wide) - 1;
+          const float lo = __shfl_sync(0xffffffffu, low, o);
+          const int64_t j = B.ju + (int64_t)(q0 + o) * TR_BLK + lane;
+          if (lo > TR_D32) {
+            const float d0 = j < nb ? Db[j].x * Ms.x : 1.0e3f, d1 = j + 32 < nb ? Db[j + 32].x * Ms.x : 1.0e3f;
+            if (d0 < (float)TR_DMAX) sf += expf(-d0);
+            if (d1 < (float)TR_DMAX) sf += expf(-d1);
+          } else {
+            const float2 far = make_float2(INFINITY, 0.0f);
+            const float2 d0 = j < nb ? ff_prod(Db[j], Ms) : far, d1 = j + 32 < nb ? ff_prod(Db[j + 32], Ms) : far;
+            const float2 e0 = ff_exp_neg(fminf(d0.x, 86.0f), d0.y, tab, L);
+            const float2 e1 = ff_exp_neg(fminf(d1.x, 86.0f), d1.y, tab, L);
+            if (d0.x < (float)TR_DMAX) tr_acc(sh, sl, e0);
+            if (d1.x < (float)TR_DMAX) tr_acc(sh, sl, e1);
+          }
         }
       }
+      float2 t = make_float2(sh, sl + sf);
+      for (int o = 16; o > 0; o >>= 1) t = ff_add(t, shfl_xor_f2(t, o));
+      if (lane == s) mine = t;
     }
-    float2 t = make_float2(sh, sl + sf);
-    for (int o = 16; o > 0; o >>= 1) t = ff_add(t, shfl_xor_f2(t, o));
-    if (lane == s) mine = t;
-  }
-  if (have) {
-    const double t = (double)B.jz + pd + ((double)mine.x + (double)mine.y);
-    out[(int64_t)b * nm + i] = E0 > 0.0 ? E0 * t / (double)nb : 0.0;
+    if (have) {
+      const double t = (double)B.jz + pd + ((double)mine.x + (double)mine.y);
+      out[(int64_t)b * nm + i] = E0 > 0.0 ? E0 * t / (double)nb : 0.0;
+    }
   }
 }
 
@@ -2133,9 +2135,10 @@ __global__ void __launch_bounds__(TR_THREADS)
       if (lane == 0) blk[q * TRF_ROW + TR_ROWS] = fmaxf(lo, 0.0f);
     }
   __syncthreads();
-  const int part = lane & (P - 1), step = gridDim.y * (TR_THREADS / P);
-  for (int i0 = blockIdx.y * (TR_THREADS / P) + (threadIdx.x & ~31) / P; i0 < nm; i0 += step) {  // warp-uniform
-    const int i = i0 + lane / P;
+  const int part = lane & (P - 1);
+  const int64_t step = (int64_t)gridDim.y * (TR_THREADS / P);
+  for (int64_t i0 = (int64_t)blockIdx.y * (TR_THREADS / P) + (threadIdx.x & ~31) / P; i0 < nm; i0 += step) {  // warp-uniform
+    const int64_t i = i0 + lane / P;
     const bool have = i < nm;
     const double mi = have ? m[i] : 0.0;
     float sh = 0.0f, sl = 0.0f;
@@ -2259,8 +2262,9 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
         nb, D, bins, blk);
     // as many masses a warp (their FP64 exponentials cost one) as leave 16 warps an SM
     int per = 32;
-    while (per > 1 && (int64_t)nbins * ((nm + per - 1) / per) < 16ll * c->num_sms) per >>= 1;
-    dim3 grid(nbins, ((nm + per - 1) / per + wpc - 1) / wpc);
+    while (per > 1 && (int64_t)nbins * (((int64_t)nm + per - 1) / per) < 16ll * c->num_sms) per >>= 1;
+    const int64_t warps = ((int64_t)nm + per - 1) / per;
+    dim3 grid(nbins, (unsigned)std::min<int64_t>((warps + wpc - 1) / wpc, 65535));  // (the grid's limit in y)
     ++c->launches;
     k_trans_direct<<<grid, TR_THREADS, 0, c->stream>>>(sorted, nb, nm, m_dev, D, bins, blk, L, per, direct);
     e = cudaGetLastError();
