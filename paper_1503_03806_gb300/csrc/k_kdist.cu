@@ -1676,6 +1676,7 @@ cudaError_t launch_kdist_bins(helk_ctx *c, const double *kappa, int64_t n, int n
 // not sorted, finite and non-negative take the plain FP64 sum.
 constexpr int TR_THREADS = 256;
 constexpr double TR_DMAX = 87.0;  // e^-87 < 2^-125
+constexpr int TR_DMAX_HI = 0x4055C000;  // the high word of 87.0
 
 struct TrConsts {
   float l1, l2, l3;  // ln2/256 in three parts (l1 with 9 significant bits)
@@ -1831,6 +1832,7 @@ __global__ void __launch_bounds__(TR_THREADS)
 // are summed value by value, beyond d = 32 (1.3e-14 a term against a sum >= 1)
 // in plain FP32.
 constexpr int TR_BLK = 64;
+constexpr int TR_WARPS_SM = 24;  // see launch_transmission
 constexpr int TR_P = 18;        // coefficients
 constexpr int TR_PP = 11;       // of them pairs
 constexpr int TR_ROWS = 2 + 2 * TR_PP + (TR_P - TR_PP);  // floats a block: c, R, pairs (high then low), the rest
@@ -1974,7 +1976,12 @@ __global__ void __launch_bounds__(TR_THREADS)
       for (int s = 0; s < per && i0 + s < nm; ++s) {
         const double ms = __shfl_sync(0xffffffffu, mi, s);
         double t = 0.0;
-        for (int64_t j = lane; j < nb; j += 32) t += exp(-k[j] * ms);
+        // four exponentials side by side, then the rest
+        int64_t j = lane;
+        for (int64_t j0 = 0; j0 + 128 <= nb; j0 += 128, j += 128)
+          t += (exp(-k[j] * ms) + exp(-k[j + 32] * ms)) + (exp(-k[j + 64] * ms) + exp(-k[j + 96] * ms));
+#pragma unroll 1
+        for (; j < nb; j += 32) t += exp(-k[j] * ms);
         t = warp_sum(t);
         if (lane == 0) out[(int64_t)b * nm + i0 + s] = t / (double)nb;
       }
@@ -1991,14 +1998,15 @@ __global__ void __launch_bounds__(TR_THREADS)
       // Tiny differences, FP64, the lanes sharing them for one mass after the other: a
       // bin that spans many decades can consist of them, and few masses leave most
       // lanes without one of their own (1e5 values of 60 decades, 30 masses: 73.5 ms
-      // with a mass a lane).
+      // with a mass a lane, 2.5 ms so).
       for (uint32_t left = __ballot_sync(0xffffffffu, have && E0 > 0.0); left; left &= left - 1) {
         const int s = __ffs(left) - 1;
         const double ms = __shfl_sync(0xffffffffu, mi, s);
         double t = 0.0;
+#pragma unroll 2
         for (int64_t j = B.jz + lane; j < B.ju; j += 32) {
           const double d = (k[j] - B.k0) * ms;
-          if (d >= TR_DMAX) break;  // the values ascend
+          if (__double2hiint(d) >= TR_DMAX_HI) break;  // d >= 87 (the values ascend), off the FP64 unit
           t += exp(-d);
         }
         t = __shfl_sync(0xffffffffu, warp_sum(t), 0);
@@ -2272,11 +2280,16 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
     const int64_t nblk = tr_nblk(nb);
     k_trans_blocks<<<dim3(nbins, (unsigned)std::min<int64_t>((nblk + wpc - 1) / wpc, 64)), TR_THREADS, 0, c->stream>>>(
         nb, D, bins, blk);
-    // as many masses a warp (their FP64 exponentials cost one) as leave 16 warps an SM
+    // As many masses a warp (their FP64 exponentials cost one) as leave TR_WARPS_SM warps an
+    // SM, the same number for every warp of a bin: 32 to a warp and the rest to the last
+    // ones kept part of each SM idle where the sums are FP64 (300 unsorted bins of 10000
+    // values, 300 masses: 45.6 ms, 29.4 so; blocks 497 -> 445 us).  24 warps: 16 leave
+    // that case at 30.5.
     int per = 32;
-    while (per > 1 && (int64_t)nbins * (((int64_t)nm + per - 1) / per) < 16ll * c->num_sms) per >>= 1;
+    while (per > 1 && (int64_t)nbins * (((int64_t)nm + per - 1) / per) < (int64_t)TR_WARPS_SM * c->num_sms) per >>= 1;
     const int64_t warps = ((int64_t)nm + per - 1) / per;
     dim3 grid(nbins, (unsigned)std::min<int64_t>((warps + wpc - 1) / wpc, 65535));  // (the grid's limit in y)
+    per = (int)std::min<int64_t>(32, (nm + (int64_t)wpc * grid.y - 1) / ((int64_t)wpc * grid.y));
     ++c->launches;
     k_trans_direct<<<grid, TR_THREADS, 0, c->stream>>>(sorted, nb, nm, m_dev, D, bins, blk, L, per, direct);
     e = cudaGetLastError();
