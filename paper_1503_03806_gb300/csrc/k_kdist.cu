@@ -1776,51 +1776,6 @@ __device__ __forceinline__ float2 split_pair(double v) {
   return make_float2(h, (float)(v - (double)h));
 }
 
-// Per bin: k_0, the scale, the counts of equal and of tiny differences, and
-// the differences as scaled pairs D (one CTA per bin).
-__global__ void __launch_bounds__(TR_THREADS)
-    k_trans_prep(const double *__restrict__ sorted, int64_t nb, float2 *__restrict__ D, TrBin *__restrict__ bins) {
-  __shared__ int s_jz, s_ju;
-  const int b = blockIdx.x;
-  const double *k = sorted + (int64_t)b * nb;
-  const double k0 = k[0], kmax = k[nb - 1];
-  if (threadIdx.x == 0) {
-    s_jz = 0;
-    s_ju = 0;
-  }
-  __syncthreads();
-  bool bad = false;
-  for (int64_t j = threadIdx.x; j < nb; j += TR_THREADS) {
-    const double v = k[j];
-    bad |= !(v >= 0.0 && isfinite(v)) || (j > 0 && !(k[j - 1] <= v));
-  }
-  if (__syncthreads_or(bad)) {
-    if (threadIdx.x == 0) bins[b] = TrBin{k0, 1.0, 0, 0, 0, 0};
-    return;
-  }
-  const double dmax = kmax - k0;
-  const int F = dmax > 0.0 ? ilogb(dmax) : 0;
-  const double inv = ldexp(1.0, -F);
-  const double tiny = ldexp(1.0, F - 100);
-  int jz = 0, ju = 0;
-  for (int64_t j = threadIdx.x; j < nb; j += TR_THREADS) {
-    const double dj = k[j] - k0;
-    D[(int64_t)b * nb + j] = split_pair(dj * inv);
-    jz += dj == 0.0;
-    ju += dj == 0.0 || dj < tiny;  // (tiny is 0 when 2^(F-100) underflows)
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    jz += __shfl_down_sync(0xffffffffu, jz, o);
-    ju += __shfl_down_sync(0xffffffffu, ju, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&s_jz, jz);
-    atomicAdd(&s_ju, ju);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) bins[b] = TrBin{k0, ldexp(1.0, F), s_jz, s_ju, 1, 0};
-}
-
 // ---- blocks of neighbouring values --------------------------------------
 // The sorted differences of a bin vary slowly, so a block of TR_BLK of them is
 // summed at once for every column mass at which it is narrow: with c a value
@@ -1832,6 +1787,14 @@ __global__ void __launch_bounds__(TR_THREADS)
 // are summed value by value, beyond d = 32 (1.3e-14 a term against a sum >= 1)
 // in plain FP32.
 constexpr int TR_BLK = 64;
+// Coefficients cost a launch and about as much as the values of a few masses, so they
+// are made from TR_BLOCK_MASSES masses on, or for long bins when there are fewer
+// (bin, mass) pairs than SMs.  The kernel that prepares the bins makes them too where
+// that keeps every SM busy (TR_FUSED values or less, or a bin for each SM).  us,
+// value by value / coefficients: 300 bins of 1000 values, 4 masses 34 / 44, 12 masses
+// 48 / 48; 1 bin of 1e5, 1 mass 813 / 351; made apart / by the preparing kernel: 300
+// bins of 10000 at 30 masses 178 / 176, 10 bins 67 / 97.
+constexpr int TR_BLOCK_MASSES = 12, TR_FUSED = 2048;
 constexpr int TR_WARPS_SM = 24;  // see launch_transmission
 constexpr int TR_P = 18;        // coefficients
 constexpr int TR_PP = 11;       // of them pairs
@@ -1909,22 +1872,74 @@ __device__ __forceinline__ void tr_block(float2 d0, float2 d1, bool have0, bool 
   }
 }
 
-// Coefficients of a bin's blocks (from its first pair on), rows [TR_ROWS][nblk].
-__global__ void __launch_bounds__(TR_THREADS)
-    k_trans_blocks(int64_t nb, const float2 *__restrict__ D, const TrBin *__restrict__ bins, float *__restrict__ blk) {
-  const int b = blockIdx.x, lane = threadIdx.x & 31;
-  const TrBin B = bins[b];
-  if (!B.ok) return;
+// Coefficients of a bin's blocks (from its first pair ju on; part `part` of `parts` of
+// them), rows [TR_ROWS][nblk].
+__device__ __forceinline__ void tr_blocks(const float2 *Db, int64_t nb, int64_t ju, int part, int parts, float *blk) {
+  const int lane = threadIdx.x & 31;
   const int64_t nblk = tr_nblk(nb);
-  const float2 *Db = D + (int64_t)b * nb;
-  for (int64_t q = blockIdx.y * (TR_THREADS / 32) + (threadIdx.x >> 5); B.ju + q * TR_BLK < nb;
-       q += gridDim.y * (TR_THREADS / 32)) {
-    const int64_t j = B.ju + q * TR_BLK + lane;
+  for (int64_t q = part * (TR_THREADS / 32) + (threadIdx.x >> 5); ju + q * TR_BLK < nb;
+       q += parts * (TR_THREADS / 32)) {
+    const int64_t j = ju + q * TR_BLK + lane;
     const bool h0 = j < nb, h1 = j + 32 < nb;
     const float2 z = make_float2(0.0f, 0.0f);
-    tr_block(h0 ? Db[j] : z, h1 ? Db[j + 32] : z, h0, h1, (int)min((int64_t)TR_BLK, nb - B.ju - q * TR_BLK),
-             blk + (int64_t)b * TR_ROWS * nblk + q, nblk);
+    tr_block(h0 ? Db[j] : z, h1 ? Db[j + 32] : z, h0, h1, (int)min((int64_t)TR_BLK, nb - ju - q * TR_BLK), blk + q, nblk);
   }
+}
+
+__global__ void __launch_bounds__(TR_THREADS)
+    k_trans_blocks(int64_t nb, const float2 *__restrict__ D, const TrBin *__restrict__ bins, float *__restrict__ blk) {
+  const int b = blockIdx.x;
+  const TrBin B = bins[b];
+  if (B.ok) tr_blocks(D + (int64_t)b * nb, nb, B.ju, blockIdx.y, gridDim.y, blk + (int64_t)b * TR_ROWS * tr_nblk(nb));
+}
+
+// Per bin: k_0, the scale, the counts of equal and of tiny differences, and
+// the differences as scaled pairs D (one CTA per bin).  BLOCKS: also the coefficients
+// of its blocks.
+template <bool BLOCKS>
+__global__ void __launch_bounds__(TR_THREADS)
+    k_trans_prep(const double *__restrict__ sorted, int64_t nb, float2 *__restrict__ D, TrBin *__restrict__ bins,
+                 float *__restrict__ blk) {
+  __shared__ int s_jz, s_ju;
+  const int b = blockIdx.x;
+  const double *k = sorted + (int64_t)b * nb;
+  const double k0 = k[0], kmax = k[nb - 1];
+  if (threadIdx.x == 0) {
+    s_jz = 0;
+    s_ju = 0;
+  }
+  __syncthreads();
+  bool bad = false;
+  for (int64_t j = threadIdx.x; j < nb; j += TR_THREADS) {
+    const double v = k[j];
+    bad |= !(v >= 0.0 && isfinite(v)) || (j > 0 && !(k[j - 1] <= v));
+  }
+  if (__syncthreads_or(bad)) {
+    if (threadIdx.x == 0) bins[b] = TrBin{k0, 1.0, 0, 0, 0, 0};
+    return;
+  }
+  const double dmax = kmax - k0;
+  const int F = dmax > 0.0 ? ilogb(dmax) : 0;
+  const double inv = ldexp(1.0, -F);
+  const double tiny = ldexp(1.0, F - 100);
+  int jz = 0, ju = 0;
+  for (int64_t j = threadIdx.x; j < nb; j += TR_THREADS) {
+    const double dj = k[j] - k0;
+    D[(int64_t)b * nb + j] = split_pair(dj * inv);
+    jz += dj == 0.0;
+    ju += dj == 0.0 || dj < tiny;  // (tiny is 0 when 2^(F-100) underflows)
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    jz += __shfl_down_sync(0xffffffffu, jz, o);
+    ju += __shfl_down_sync(0xffffffffu, ju, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_jz, jz);
+    atomicAdd(&s_ju, ju);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) bins[b] = TrBin{k0, ldexp(1.0, F), s_jz, s_ju, 1, 0};
+  if (BLOCKS) tr_blocks(D + (int64_t)b * nb, nb, s_ju, 0, 1, blk + (int64_t)b * TR_ROWS * tr_nblk(nb));
 }
 
 // sum_p a_p (-z)^p of a block for z = R M (rows at a[row * stride])
@@ -2017,7 +2032,18 @@ __global__ void __launch_bounds__(TR_THREADS)
       const int s = __ffs(left) - 1;
       const float2 Ms = make_float2(__shfl_sync(0xffffffffu, M.x, s), __shfl_sync(0xffffffffu, M.y, s));
       float sh = 0.0f, sl = 0.0f, sf = 0.0f;
-      for (int q0 = 0; q0 < used; q0 += 32) {
+      if (!blk) {  // value by value, two a lane; the first of a pass is its smallest
+        for (int64_t j0 = B.ju; j0 < nb && Db[j0].x * Ms.x < (float)TR_DMAX; j0 += 64) {
+          const int64_t j = j0 + lane;
+          const float2 far = make_float2(INFINITY, 0.0f);
+          const float2 d0 = j < nb ? ff_prod(Db[j], Ms) : far, d1 = j + 32 < nb ? ff_prod(Db[j + 32], Ms) : far;
+          const float2 e0 = ff_exp_neg(fminf(d0.x, 86.0f), d0.y, tab, L);
+          const float2 e1 = ff_exp_neg(fminf(d1.x, 86.0f), d1.y, tab, L);
+          if (d0.x < (float)TR_DMAX) tr_acc(sh, sl, e0);
+          if (d1.x < (float)TR_DMAX) tr_acc(sh, sl, e1);
+        }
+      }
+      for (int q0 = 0; blk && q0 < used; q0 += 32) {
         const int q = q0 + lane;
         float c = 0.0f, R = 0.0f;
         if (q < used) {
@@ -2271,15 +2297,18 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
     float2 *D = reinterpret_cast<float2 *>(c->tr_pairs);
     TrBin *bins = reinterpret_cast<TrBin *>(c->tr_bins);
     ++c->launches;
-    k_trans_prep<<<nbins, TR_THREADS, 0, c->stream>>>(sorted, nb, D, bins);
+    const bool coefs = nm >= TR_BLOCK_MASSES || (nb > TR_FUSED && (int64_t)nbins * nm < c->num_sms);
+    const bool fused = coefs && (nb <= TR_FUSED || nbins >= c->num_sms);
+    float *blk = coefs ? reinterpret_cast<float *>(D + (int64_t)nbins * nb) : nullptr;
+    (fused ? k_trans_prep<true> : k_trans_prep<false>)<<<nbins, TR_THREADS, 0, c->stream>>>(sorted, nb, D, bins, blk);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    float *blk = reinterpret_cast<float *>(D + (int64_t)nbins * nb);
-    ++c->launches;
     const int wpc = TR_THREADS / 32;
-    const int64_t nblk = tr_nblk(nb);
-    k_trans_blocks<<<dim3(nbins, (unsigned)std::min<int64_t>((nblk + wpc - 1) / wpc, 64)), TR_THREADS, 0, c->stream>>>(
-        nb, D, bins, blk);
+    if (coefs && !fused) {
+      ++c->launches;
+      k_trans_blocks<<<dim3(nbins, (unsigned)std::min<int64_t>((tr_nblk(nb) + wpc - 1) / wpc, 64)), TR_THREADS, 0,
+                       c->stream>>>(nb, D, bins, blk);
+    }
     // As many masses a warp (their FP64 exponentials cost one) as leave TR_WARPS_SM warps an
     // SM, the same number for every warp of a bin: 32 to a warp and the rest to the last
     // ones kept part of each SM idle where the sums are FP64 (300 unsorted bins of 10000
