@@ -2106,18 +2106,18 @@ __device__ __forceinline__ double tr_kfit(const double *c, int ncheb, int j, int
 }
 
 // CTAs of one bin, one column mass to each group of P threads (a power of two up
-// to a warp; they share the blocks), the fit's ng values of k, their
-// pairs and the coefficients of blocks of `len` neighbouring points in shared
-// memory (k(g) is smooth in g, sorted or not).  A block whose spread is narrow for
-// a thread's mass is one exponential and a polynomial, any other point by point
-// (terms with d >= 87 skipped).  len is 16 while shared memory holds that; longer
-// blocks for the largest ng, past TR_BLK points without coefficients.
+// to a warp; they share the points), the fit's ng values of k and their
+// pairs in shared memory, and, if coefs, the coefficients of blocks of `len`
+// neighbouring points (k(g) is smooth in g, sorted or not).  A block whose spread is
+// narrow for a thread's mass is one exponential and a polynomial, any other point by
+// point (terms with d >= 87 skipped).  len is 16 while shared memory holds that;
+// longer blocks for the largest ng, past TR_BLK points without coefficients.
 constexpr int TRF_ROW = 36;  // floats a block: TR_ROWS, the smallest d, padding
 static_assert(TR_ROWS < TRF_ROW && TRF_ROW % 4 == 0, "block rows");
 
 __global__ void __launch_bounds__(TR_THREADS)
     k_trans_fit(const double *__restrict__ coef, int ncheb, int ng, int nm, const double *__restrict__ m,
-                TrConsts L, int P, int len, double *__restrict__ out) {
+                TrConsts L, int P, int len, bool coefs, double *__restrict__ out) {
   extern __shared__ __align__(16) double kfit[];  // ng values, ng pairs (a negative pair: FP64 term), the blocks
   float2 *Dg = reinterpret_cast<float2 *>(kfit + ng);
   float *blk = reinterpret_cast<float *>(kfit + 2 * ng);  // 16 ng bytes in: 16-byte aligned
@@ -2160,7 +2160,7 @@ __global__ void __launch_bounds__(TR_THREADS)
     }
   __syncthreads();
   const int nblk = (ng + len - 1) / len;
-  if (!bad)
+  if (coefs && !bad)
     for (int q = threadIdx.x >> 5; q < nblk; q += TR_THREADS / 32) {  // one warp a block
       const int j0 = q * len, n = min(len, ng - j0);
       float lo = INFINITY;
@@ -2199,7 +2199,16 @@ __global__ void __launch_bounds__(TR_THREADS)
         const double Md = mi * scale;
         const bool pairs = Md < 0x1p107;  // else every pair term has d >= 128
         const float2 M = split_pair(pairs ? Md : 0.0);
-        for (int q = part; q < nblk; q += P) {
+        for (int j = part; !coefs && j < ng; j += P) {
+          const float2 Dj = Dg[j];
+          if (Dj.x < 0.0f) {
+            pd += exp(-((kfit[j] - vmin) * mi));
+          } else if (pairs) {
+            const float2 d = ff_prod(Dj, M);
+            if (d.x < (float)TR_DMAX) tr_acc(sh, sl, ff_exp_neg(d.x, d.y, tab, L));
+          }
+        }
+        for (int q = part; coefs && q < nblk; q += P) {
           const float *bk = blk + q * TRF_ROW;
           const float R = bk[1], low = bk[TR_ROWS] * M.x;
           if (low >= (float)TR_DMAX) continue;
@@ -2325,15 +2334,25 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
     if (e != cudaSuccess) return e;
   }
   if (coef && fit) {
-    // threads that share a mass: as many as give every SM 512 threads; the values
-    // of k cost each CTA ng FP64 exponentials: as few CTAs a bin as leave two an SM
-    int P = 1;
-    while (P < 32 && (int64_t)nbins * nm * P < 512ll * c->num_sms) P <<= 1;
+    // Threads that share a mass: as many as fill half a CTA, give every SM 128 threads,
+    // or leave a thread 160 points while the CTA has work for it (each repeats the FP64
+    // exponential of its mass); no more than one to 16 points.  The values of k cost
+    // each CTA ng FP64 exponentials: as few CTAs a bin as leave two an SM.
+    int len = 16, P = 1;
+    while (P < 32 && P * len < ng &&
+           (2ll * nm * P <= TR_THREADS || (int64_t)nbins * nm * P < 128ll * c->num_sms ||
+            ((int64_t)nm * P <= 512 && ng > 160 * P)))
+      P <<= 1;
     const int most = (int)(((int64_t)nm * P + TR_THREADS - 1) / TR_THREADS);
     dim3 grid(nbins, std::min(most, std::max(1, (2 * c->num_sms + nbins - 1) / nbins)));
-    int len = 16;
+    // Coefficients where a CTA has masses enough to repay them (a warp a block).  us,
+    // 300 bins, without / with: 30 masses of 1000 points 107 / 122, 200 of 64 44 / 45, of
+    // 200 96 / 88, 1000 of 64 96 / 75, of 1000 838 / 395.
+    const int64_t share = nm / grid.y;
+    const bool coefs = share >= 100 && share * ng >= 16384;
     auto fit_smem = [&](int n) {
-      return (size_t)ng * (sizeof(double) + sizeof(float2)) + (size_t)((ng + n - 1) / n) * TRF_ROW * sizeof(float);
+      return (size_t)ng * (sizeof(double) + sizeof(float2)) +
+             (coefs ? (size_t)((ng + n - 1) / n) * TRF_ROW * sizeof(float) : 0);
     };
     while (len < 16384 && fit_smem(len) + 2304 > (size_t)c->max_smem_optin) len <<= 1;
     const size_t smem = fit_smem(len);
@@ -2343,7 +2362,7 @@ cudaError_t launch_transmission(helk_ctx *c, int nbins, int64_t nb, const double
         if (e != cudaSuccess) return e;
       }
       ++c->launches;
-      k_trans_fit<<<grid, TR_THREADS, smem, c->stream>>>(coef, ncheb, ng, nm, m_dev, L, P, len, fit);
+      k_trans_fit<<<grid, TR_THREADS, smem, c->stream>>>(coef, ncheb, ng, nm, m_dev, L, P, len, coefs, fit);
     } else {
       const size_t smem64 = (size_t)ng * sizeof(double);
       if (smem64 > 48 * 1024) {
