@@ -130,9 +130,11 @@ static __device__ __forceinline__ float core_rcp(float x) {
   return r;
 }
 
-// e^{-x^2}, with the rounding of x^2 made up for (0 below the normal range)
+// e^{-x^2}, with the rounding of x^2 made up for.  Below the normal range (x^2 from 87
+// to 100, the far end of an undamped line's core) it is a subnormal number, not 0:
+// the logarithms of the tables tell the two apart.
 static __device__ __forceinline__ float core_gauss(float x, float x2) {
-  if (x2 > 87.0f) return 0.0f;
+  if (x2 > 87.0f) return expf(-x2);
   int m;
   float lo;
   const float e = core_exp(-x2, m, lo);
