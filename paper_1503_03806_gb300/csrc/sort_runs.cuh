@@ -6,8 +6,10 @@
 
 namespace helk {
 
-// Upload: lists of at most this many ordered runs are merged, others sorted.
-constexpr int SORT_RUNS = 16;
+// Upload: lists of at most SORT_RUNS ordered runs are merged, others sorted; lists of
+// more than MERGE_SHORT lines if they have at most MERGE_RUNS_LONG runs.
+constexpr int SORT_RUNS = 16, MERGE_RUNS_LONG = 8;
+constexpr int64_t MERGE_SHORT = (int64_t)1 << 18;
 
 struct SortRuns {
   int n, end[SORT_RUNS + 1];
