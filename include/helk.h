@@ -192,7 +192,7 @@ helk_status helk_opacity(helk_ctx *ctx, double T, double P_atm,
  * pointer, tile shape) into a CUDA graph and replayed on later calls with the
  * same shape; only the condition values change between replays.  The
  * per-condition line records take 56 B (FP32 form) or 96 B (FP64 form; with
- * windows of fewer than 24 points to a side 64 B) per line, in the FP64 form
+ * windows of fewer than 24 points to a side or few lines 64 B) per line, in the FP64 form
  * also 8 B per grid point; when those of all n_cond conditions exceed the
  * record budget
  * (64 GiB unless set by helk_set_batch_budget), the conditions run in the

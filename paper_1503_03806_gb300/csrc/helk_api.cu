@@ -254,9 +254,15 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
   if (c->stats_host->unsorted) {
     HELK_TRY(cuda_check(c, launch_sort_lines(c, n, c->stats_host->unsorted, c->stats_host->run_end),
                         "sort lines"));
+    HELK_TRY(cuda_check(c, launch_list_cuts(c, n), "sort lines"));
+    HELK_TRY(cuda_check(c, cudaMemcpyAsync(c->stats_host->cuts, c->stats->cuts, sizeof c->stats->cuts,
+                                           cudaMemcpyDeviceToHost, c->stream),
+                        "sort lines"));
     HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "sort lines"));
   }
   c->nlines = n;
+  c->shape.n = n;
+  std::copy(c->stats_host->cuts, c->stats_host->cuts + LIST_CUTS + 1, c->shape.at);
   c->have_opacity = false;
   return HELK_OK;
 }
@@ -345,7 +351,7 @@ static bool wing_route(const helk_ctx *c, const helk_opts &o, const helk_cutoff 
   if (cut->kind == HELK_CUT_ABS) half = std::min(half, cut->value / g->dnu);
   if (cut->kind == HELK_CUT_LORENTZ) half = std::min(half, cut->cap / g->dnu);
   if (o.precision != HELK_PREC_F32_KAHAN) {
-    if (half < WING64_MIN_HALF) return false;
+    if (!wings_pay64(c->shape, g->nu_min, g->dnu, g->n, half)) return false;
   } else {
     const bool sparse = 2.0 * half * (double)c->nlines < WING32_MIN_LINES * (double)g->n;
     if (half < WING32_MIN_HALF || (sparse && g->n > (int64_t)c->num_sms * 512)) return false;
@@ -619,11 +625,11 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
 // reads or writes and that a later call may move (all of them: a list that grows and
 // shrinks again can move some and leave others where they were).
 static std::string batch_key(const helk_ctx *c, int n_cond, double mass, const helk_cutoff *cut,
-                             const helk_grid *g, const helk_opts &o, const double *kappa, int shape) {
+                             const helk_grid *g, const helk_opts &o, const double *kappa, int shape, bool wings) {
   char b[256];
-  snprintf(b, sizeof b, "%d|%lld|%a|%d|%a|%a|%a|%a|%lld|%d|%d|%a|%d|%d|%d|%d", n_cond, (long long)c->nlines, mass,
+  snprintf(b, sizeof b, "%d|%lld|%a|%d|%a|%a|%a|%a|%lld|%d|%d|%a|%d|%d|%d|%d|%d", n_cond, (long long)c->nlines, mass,
            cut->kind, cut->value, cut->cap, g->nu_min, g->dnu, (long long)g->n, o.precision, o.accumulate, o.weight,
-           o.count_regions, o.surrogate, shape, (int)c->core_nodes);
+           o.count_regions, o.surrogate, shape, (int)c->core_nodes, (int)wings);
   std::string key(b);
   // the line fields (absent ones are passed to line preparation as null pointers)
   const void *const bufs[] = {c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair, c->has_gself ? c->gself : nullptr,
@@ -746,7 +752,7 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
       // the chunk's view of the per-condition arrays (staging, parameters,
       // statistics, order): offset by its first condition, restored after
       const CondView view(c, k0);
-      const std::string key = batch_key(c, nk, mass, cut, g, o, kap, shape);
+      const std::string key = batch_key(c, nk, mass, cut, g, o, kap, shape, wg != nullptr);
       gx = find_graph(c, key);
       if (!gx) {
         cudaStream_t user = c->stream;

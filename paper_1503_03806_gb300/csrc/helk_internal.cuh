@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/helk.h"
+#include "route.cuh"
 #include "sort_runs.cuh"
 
 // Line-record budget of one chunk of helk_opacity_batch (64 GiB).
@@ -102,6 +103,7 @@ struct DevStats {
   int unsorted;                     // upload: descents of nu0, counted to SORT_RUNS or a few more
   unsigned int tile_counter;        // next (condition, tile) item of the persistent Voigt kernel
   int run_end[SORT_RUNS];           // upload: where the first of them are (in no order)
+  double cuts[LIST_CUTS + 1];       // upload: ListShape::at
 };
 
 // Core evaluations routed to the surrogate by the FP32 Voigt kernel: the
@@ -160,6 +162,7 @@ struct helk_ctx {
   int max_smem_optin = 0;
   // line list (sorted SoA)
   int64_t nlines = 0;
+  helk::ListShape shape{};  // of the uploaded list
   bool has_E = false, has_gself = false, has_ncoll = false, has_delta = false;
   bool has_mass = false, has_weight = false;
   double *nu0 = nullptr, *S0 = nullptr, *El = nullptr, *gair = nullptr,
@@ -360,6 +363,7 @@ __device__ __forceinline__ void tma_load_1d(uint32_t dst_smem, const void *src, 
 cudaError_t launch_validate_lines(helk_ctx *c, int64_t n);
 // descents, run_end: DevStats::unsorted and its run ends
 cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end);  // orders SoA by nu0
+cudaError_t launch_list_cuts(helk_ctx *c, int64_t n);  // DevStats::cuts of an ordered list
 // n_cond conditions: from c->cond_dev, or (n_cond == 1 and single != NULL)
 // the one condition passed by value.  Records of condition k start at
 // k * nlines; tile maps at k * ntiles.

@@ -18,12 +18,27 @@
 namespace helk {
 
 // -------------------------------------------------------- validation ---
+// DevStats::cuts by a CTA's first threads.
+__device__ __forceinline__ void list_cuts(int64_t n, const double *nu0, DevStats *st) {
+  if (threadIdx.x <= LIST_CUTS) st->cuts[threadIdx.x] = nu0[(n - 1) * threadIdx.x / LIST_CUTS];
+}
+__global__ void k_list_cuts(int64_t n, const double *__restrict__ nu0, DevStats *st) { list_cuts(n, nu0, st); }
+
+cudaError_t launch_list_cuts(helk_ctx *c, int64_t n) {
+  if (n <= 0) return cudaSuccess;
+  ++c->launches;
+  k_list_cuts<<<1, 96, 0, c->stream>>>(n, c->nu0, c->stats);
+  return cudaGetLastError();
+}
+
+// (of a list that is not ordered the cuts are taken again after it is)
 __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const double *__restrict__ S0,
                            const double *__restrict__ El, const double *__restrict__ gair,
                            const double *__restrict__ gself, const double *__restrict__ ncoll,
                            const double *__restrict__ delta, const double *__restrict__ lmass,
                            const double *__restrict__ lweight, DevStats *st) {
   int bad = 0;
+  if (blockIdx.x == 0) list_cuts(n, nu0, st);
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
        l += (int64_t)gridDim.x * blockDim.x) {
     double v = nu0[l];

@@ -1,0 +1,59 @@
+// route.cuh -- the rules by which an opacity call takes interpolated wings or the
+// point-by-point kernels (host side; shared by nothing else, so that a test can
+// compile it alone).
+#pragma once
+
+#include <stdint.h>
+
+#include <algorithm>
+
+namespace helk {
+
+// Centres of the ordered list at LIST_CUTS + 1 evenly spaced places ((n - 1) i /
+// LIST_CUTS), the first and the last line among them: how many lines lie where.
+constexpr int LIST_CUTS = 64;
+struct ListShape {
+  int64_t n;
+  double at[LIST_CUTS + 1];
+};
+
+// Lines below wavenumber x, between two cuts by interpolation.
+inline double lines_below(const ListShape &L, double x) {
+  if (L.n <= 0 || x <= L.at[0]) return 0.0;
+  if (x > L.at[LIST_CUTS]) return (double)L.n;
+  const int i = (int)(std::lower_bound(L.at, L.at + LIST_CUTS + 1, x) - L.at);  // at[i - 1] < x <= at[i]
+  const double f = (x - L.at[i - 1]) / (L.at[i] - L.at[i - 1]);
+  return ((double)(i - 1) + f) / LIST_CUTS * (double)L.n;
+}
+
+// Lines within `reach` points of a stretch of `points` grid points, the mean over
+// stretches at eight places of the grid.
+inline double lines_near(const ListShape &L, double nu_min, double dnu, int64_t n, double points, double reach) {
+  double sum = 0.0;
+  const double w = 0.5 * std::min(points, (double)n);
+  for (int k = 0; k < 8; ++k) {
+    const double mid = w + ((double)n - 2.0 * w) * (k + 0.5) / 8.0;
+    sum += lines_below(L, nu_min + (mid + w + reach) * dnu) - lines_below(L, nu_min + (mid - w - reach) * dnu);
+  }
+  return sum / 8.0;
+}
+
+// FP64 form.  Windows of `half` points to a side.  The wings' map, tree and core pass
+// cost the same for few lines (0.14 ns a point and ~20 us), the direct kernel a tile
+// of 2048 points some us a line that reaches it: the wings pay from about five lines
+// a tile on, on short grids, where the launches count, from about twenty.  us, wings /
+// direct:
+//   half a window of h points, 1e5 lines on 3e6 points   h = 24 2370 / 9110   64 3660 / 16000
+//   3e3 lines on 2e4 points                              h = 24   77 / 154
+//   3e6 points, lines a tile   2.3 (1e3 lines, h = 2500) 774 / 578    7 (1e4, h = 30) 749 / 1126
+//                              17 (1e3, h = 25000) 866 / 2084
+//   3e5 points                 2.3 (100, h = 2500) 175 / 121     7 (1e3, h = 30) 165 / 201
+//   3e4 points                 8.5 (100, h = 250) 62 / 42       23 (100, h = 2500) 84 / 85
+//   300 points, 10 lines 55 / 48, 100 lines 100 / 247
+constexpr double WING64_MIN_HALF = 24.0;
+inline bool wings_pay64(const ListShape &L, double nu_min, double dnu, int64_t n, double half) {
+  return half >= WING64_MIN_HALF &&
+         lines_near(L, nu_min, dnu, n, 2048.0, half) >= 5.0 + std::min(15.0, 4.0e5 / (double)n);
+}
+
+}  // namespace helk

@@ -36,20 +36,18 @@
 #include <vector>
 
 #include "helk_internal.cuh"
+#include "route.cuh"
 
 namespace helk {
 
-// Where the direct route is taken instead: narrow windows, and in the FP32 form few
-// lines to a point, on grids whose tiles give every SM work (the wings' map, far
-// sums and tree cost the same for few lines).  Opacity in ms, wings / direct,
-// half a window of h points:
-//   FP64, 1e5 lines on 3e6 points   h = 24 2.37 / 9.11   64 3.66 / 16.0
-//   FP64, 3e3 lines on 2e4 points   h = 24 0.077 / 0.154
-//   FP32, 1e5 lines on 3e6 points   h = 128 0.266 / 0.241   512 0.296 / 0.280
-//                                       768 (51 lines to a point) 0.301 / 0.306
-//   FP32, 1e6 lines on 3e6 points   h = 64 (43 lines to a point) 0.98 / 1.20
-//   FP32, 3e3 lines on 2e4 points   h = 64 (19 lines to a point) 0.040 / 0.063
-constexpr double WING64_MIN_HALF = 24.0, WING32_MIN_HALF = 64.0, WING32_MIN_LINES = 43.0;
+// Where the direct route is taken instead in the FP32 form (the FP64 form's rule is in
+// route.cuh): narrow windows, and few lines to a point on grids whose tiles give every
+// SM work.  Opacity in ms, wings / direct, half a window of h points:
+//   1e5 lines on 3e6 points   h = 128 0.266 / 0.241   512 0.296 / 0.280
+//                             768 (51 lines to a point) 0.301 / 0.306
+//   1e6 lines on 3e6 points   h = 64 (43 lines to a point) 0.98 / 1.20
+//   3e3 lines on 2e4 points   h = 64 (19 lines to a point) 0.040 / 0.063
+constexpr double WING32_MIN_HALF = 64.0, WING32_MIN_LINES = 43.0;
 constexpr int WG_S0 = 32;                   // points of a leaf
 constexpr int WG_LEVELS = 23;               // the coarsest panels have 2^27 points
 constexpr int WG_STAGES = 7;
