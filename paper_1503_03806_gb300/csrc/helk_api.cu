@@ -156,7 +156,9 @@ void helk_destroy(helk_ctx *c) {
   if (c->cond_dev) cudaFree(c->cond_dev);
   if (c->cstats) cudaFree(c->cstats);
   if (c->cond_order) cudaFree(c->cond_order);
+  if (c->cond_list) cudaFree(c->cond_list);
   if (c->cond_host) cudaFreeHost(c->cond_host);
+  if (c->cond_list_host) cudaFreeHost(c->cond_list_host);
   if (c->cstats_host) cudaFreeHost(c->cstats_host);
   if (c->cond_ev) cudaEventDestroy(c->cond_ev);
   for (auto &kv : c->graphs) cudaGraphExecDestroy(kv.second);
@@ -204,6 +206,14 @@ helk_status helk_sync(helk_ctx *c) {
   return HELK_OK;
 }
 
+// the double of an order key
+static double order_double(unsigned long long k) {
+  const unsigned long long bits = k >> 63 ? k & 0x7FFFFFFFFFFFFFFFull : ~k;
+  double v;
+  memcpy(&v, &bits, 8);
+  return v;
+}
+
 helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32_t on_device) {
   if (!c) return HELK_ERR_INVALID_ARG;
   c->err.clear();
@@ -240,7 +250,8 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
   c->has_delta = L->delta != nullptr;
   c->has_mass = L->mass != nullptr;
   c->has_weight = L->weight != nullptr;
-  HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->stats->bad_lines, 0, 2 * sizeof(int), c->stream),
+  HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->stats->bad_lines, 0,
+                                         sizeof(DevStats) - offsetof(DevStats, bad_lines), c->stream),
                       "lines_upload"));
   HELK_TRY(cuda_check(c, launch_validate_lines(c, n), "validate lines"));
   HELK_TRY(cuda_check(c, cudaMemcpyAsync(c->stats_host, c->stats, sizeof(DevStats),
@@ -254,13 +265,13 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
   if (c->stats_host->unsorted) {
     HELK_TRY(cuda_check(c, launch_sort_lines(c, n, c->stats_host->unsorted, c->stats_host->run_end),
                         "sort lines"));
-    HELK_TRY(cuda_check(c, launch_list_cuts(c, n), "sort lines"));
-    HELK_TRY(cuda_check(c, cudaMemcpyAsync(c->stats_host->cuts, c->stats->cuts, sizeof c->stats->cuts,
-                                           cudaMemcpyDeviceToHost, c->stream),
-                        "sort lines"));
     HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "sort lines"));
   }
   c->nlines = n;
+  c->gair_max = order_double(c->stats_host->gair_max);
+  c->gself_max = order_double(c->stats_host->gself_max);
+  c->ncoll_max = order_double(c->stats_host->ncoll_max);
+  c->ncoll_min = order_double(~c->stats_host->ncoll_min_inv);
   c->shape.n = n;
   std::copy(c->stats_host->cuts, c->stats_host->cuts + LIST_CUTS + 1, c->shape.at);
   c->have_opacity = false;
@@ -325,11 +336,15 @@ static helk_status ensure_conds(helk_ctx *c, int n_cond) {
   if (c->cond_dev) cudaFree(c->cond_dev);
   if (c->cstats) cudaFree(c->cstats);
   if (c->cond_order) cudaFree(c->cond_order);
+  if (c->cond_list) cudaFree(c->cond_list);
   if (c->cond_host) cudaFreeHost(c->cond_host);
+  if (c->cond_list_host) cudaFreeHost(c->cond_list_host);
   if (c->cstats_host) cudaFreeHost(c->cstats_host);
   c->cond_dev = nullptr;
   c->cstats = nullptr;
   c->cond_order = nullptr;
+  c->cond_list = nullptr;
+  c->cond_list_host = nullptr;
   c->cond_host = nullptr;
   c->cstats_host = nullptr;
   c->cond_cap = 0;
@@ -337,27 +352,43 @@ static helk_status ensure_conds(helk_ctx *c, int n_cond) {
   HELK_TRY(cuda_check(c, cudaMalloc((void **)&c->cond_dev, cap * sizeof(CondArgs)), "conditions"));
   HELK_TRY(cuda_check(c, cudaMalloc((void **)&c->cstats, cap * sizeof(CondStats)), "conditions"));
   HELK_TRY(cuda_check(c, cudaMalloc((void **)&c->cond_order, cap * sizeof(int)), "conditions"));
+  HELK_TRY(cuda_check(c, cudaMalloc((void **)&c->cond_list, cap * sizeof(int)), "conditions"));
+  HELK_TRY(cuda_check(c, cudaMallocHost((void **)&c->cond_list_host, cap * sizeof(int)), "conditions"));
   HELK_TRY(cuda_check(c, cudaMallocHost((void **)&c->cond_host, cap * sizeof(CondArgs)), "conditions"));
   HELK_TRY(cuda_check(c, cudaMallocHost((void **)&c->cstats_host, cap * sizeof(CondStats)), "conditions"));
   c->cond_cap = cap;
   return HELK_OK;
 }
 
-// Whether a call takes the interpolated-wings route, and its geometry.
-static bool wing_route(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g,
-                       WingGeom *out) {
-  if (o.count_regions) return false;
+// A bound on the half-width of a condition's windows, in points.  Lorentz cutoff: by
+// its cap, and, given the condition, by the list's largest width.
+static double max_half(const helk_cutoff *cut, const helk_grid *g) {
   double half = (double)g->n;
   if (cut->kind == HELK_CUT_ABS) half = std::min(half, cut->value / g->dnu);
   if (cut->kind == HELK_CUT_LORENTZ) half = std::min(half, cut->cap / g->dnu);
-  if (o.precision != HELK_PREC_F32_KAHAN) {
-    if (!wings_pay64(c->shape, g->nu_min, g->dnu, g->n, half)) return false;
-  } else {
-    const bool sparse = 2.0 * half * (double)c->nlines < WING32_MIN_LINES * (double)g->n;
-    if (half < WING32_MIN_HALF || (sparse && g->n > (int64_t)c->num_sms * 512)) return false;
-  }
-  *out = wing_geometry(g->n, half, c->num_sms);
-  return true;
+  return half;
+}
+static double cond_half(const helk_ctx *c, const helk_cutoff *cut, const helk_grid *g, double T, double P) {
+  const double half = max_half(cut, g);
+  if (cut->kind != HELK_CUT_LORENTZ) return half;
+  const double t = c->has_ncoll ? std::max(pow(T0 / T, c->ncoll_max), pow(T0 / T, c->ncoll_min)) : sqrt(T0 / T);
+  const double gl = t * 0.5 * P * (c->gair_max + (c->has_gself ? c->gself_max : c->gair_max));
+  return std::min(half, cut->value * gl / g->dnu);
+}
+
+// Whether a call takes the interpolated-wings route, and its geometry.  FP32 form: by
+// the call; its conditions share one route.
+static bool wing_route32(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g) {
+  if (o.count_regions) return false;
+  const double half = max_half(cut, g);
+  const bool sparse = 2.0 * half * (double)c->nlines < WING32_MIN_LINES * (double)g->n;
+  return half >= WING32_MIN_HALF && !(sparse && g->n > (int64_t)c->num_sms * 512);
+}
+// FP64 form: by the condition, so that one call and a batch agree.
+static bool wing_route64(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g, double T,
+                         double P) {
+  return !o.count_regions &&
+         wings_pay64(c->shape, g->nu_min, g->dnu, g->n, max_half(cut, g), cond_half(c, cut, g, T, P));
 }
 
 // Buffers for n_cond conditions of the current line list and tile shape (or
@@ -385,7 +416,7 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
     if (!c->join_ev)
       HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming), "core stream"));
   }
-  HELK_TRY(ensure_tiles(c, (wg ? (int64_t)wg->nmap : ntiles) * n_cond));
+  HELK_TRY(ensure_tiles(c, std::max(wg ? (int64_t)wg->nmap : 0, ntiles) * n_cond));
   if (wg)
     HELK_TRY(o.precision == HELK_PREC_F32_KAHAN ? ensure_wing32(c, n_cond, *wg) : ensure_wing64(c, n_cond, *wg));
   if (o.surrogate && !c->squeue) {
@@ -414,7 +445,7 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
 
 static CondArgs make_cond(const helk_ctx *c, double T, double P, double q_ratio, double mass) {
   const double vth = sqrt(2.0 * LN2 * KB * T / ((c->has_mass ? 1.0 : mass) * AMU)) / CLIGHT;
-  return CondArgs{T, P, q_ratio, sqrt(T0 / T), C2 / T0 - C2 / T, C2 / T, SQRTLN2 / vth, log(T0 / T)};
+  return CondArgs{T, P, q_ratio, sqrt(T0 / T), C2 / T0 - C2 / T, C2 / T, SQRTLN2 / vth, log(T0 / T), 0};
 }
 
 // Which core kernel (FP32 form): the one with nodes if a line of a condition can have
@@ -463,19 +494,19 @@ static int shape_points(int precision, int shape) {
 // The interpolated-wings route: candidate map, condition order, the far
 // kernel with the Algorithm 916 cores beside it on the side stream, then the
 // near kernel, which writes kappa.  FP64 form: the cores share the far
-// kernel's launch.
-static helk_status run_wings(helk_ctx *c, int n_cond, const helk_grid *g, const helk_opts &o, double *kappa,
-                             const WingGeom &wg) {
+// kernel's launch; list (device): the conditions, NULL for all.
+static helk_status run_wings(helk_ctx *c, int n_cond, const int *list, const helk_grid *g, const helk_opts &o,
+                             double *kappa, const WingGeom &wg) {
   if (o.precision != HELK_PREC_F32_KAHAN) {
-    HELK_TRY(cuda_check(c, launch_wingmap(c, n_cond, wg), "wing map"));
-    HELK_TRY(cuda_check(c, launch_wing_far64(c, n_cond, wg, *g), "voigt wings"));
-    return cuda_check(c, launch_wing_near64(c, n_cond, wg, *g, o, kappa), "voigt wings");
+    HELK_TRY(cuda_check(c, launch_wingmap(c, n_cond, list, wg), "wing map"));
+    HELK_TRY(cuda_check(c, launch_wing_far64(c, n_cond, list, wg, *g), "voigt wings"));
+    return cuda_check(c, launch_wing_near64(c, n_cond, list, wg, *g, o, kappa), "voigt wings");
   }
   HELK_TRY(cuda_check(c, launch_cond_order(c, n_cond), "condition order"));
   if (o.surrogate)
     HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->squeue->count, 0, sizeof(unsigned long long), c->stream), "voigt"));
   HELK_TRY(cuda_check(c, cudaEventRecord(c->fork_ev, c->stream), "voigt"));
-  HELK_TRY(cuda_check(c, launch_wingmap(c, n_cond, wg), "wing map"));
+  HELK_TRY(cuda_check(c, launch_wingmap(c, n_cond, nullptr, wg), "wing map"));
   HELK_TRY(cuda_check(c, launch_wing_far32(c, n_cond, wg), "voigt wings"));
   HELK_TRY(cuda_check(c, cudaStreamWaitEvent(c->side_stream, c->fork_ev, 0), "voigt cores"));
   HELK_TRY(cuda_check(c, launch_voigt_core(c, n_cond, *g, o), "voigt cores"));
@@ -488,10 +519,22 @@ static helk_status run_wings(helk_ctx *c, int n_cond, const helk_grid *g, const 
 
 // Tile map, condition order and the persistent Voigt kernel (for the FP32
 // form with its Algorithm 916 cores).  `shape`: the Voigt kernel's shape
-// code; `tile`: its points per CTA tile.
+// code; `tile`: its points per CTA tile.  The first n_wing conditions of
+// c->cond_list (all of them if n_wing == n_cond) take the wings of wg instead.
 static helk_status run_voigt(helk_ctx *c, int n_cond, const helk_grid *g, const helk_opts &o, double *kappa,
-                             int shape, int tile, int64_t ntiles, const WingGeom *wg) {
-  if (wg) return run_wings(c, n_cond, g, o, kappa, *wg);
+                             int shape, int tile, int64_t ntiles, const WingGeom *wg, int n_wing) {
+  if (n_wing == n_cond) return run_wings(c, n_cond, nullptr, g, o, kappa, *wg);
+  if (n_wing > 0) {  // FP64 form
+    HELK_TRY(run_wings(c, n_wing, c->cond_list, g, o, kappa, *wg));
+    HELK_TRY(cuda_check(c, launch_tilemap(c, n_cond, *g, tile, ntiles), "tilemap"));
+    HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->stats->tile_counter, 0, sizeof(unsigned int), c->stream),
+                        "tile counter"));
+    int *const order = c->cond_order;
+    c->cond_order = c->cond_list + n_wing;
+    const cudaError_t e = launch_voigt(c, n_cond - n_wing, *g, o, kappa, shape, ntiles);
+    c->cond_order = order;
+    return cuda_check(c, e, "voigt");
+  }
   HELK_TRY(cuda_check(c, launch_tilemap(c, n_cond, *g, tile, ntiles), "tilemap"));
   HELK_TRY(cuda_check(c, launch_cond_order(c, n_cond), "condition order"));
   HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->stats->tile_counter, 0, sizeof(unsigned int), c->stream),
@@ -533,17 +576,20 @@ helk_status helk_opacity(helk_ctx *c, double T, double P, double mass, const hel
   const int tile = shape_points(o.precision, shape);
   if (tile <= 0) return set_err(c, HELK_ERR_STATE, "opacity: no kernel shape");
   const int64_t ntiles = (g->n + tile - 1) / tile;
-  WingGeom geom;
-  const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
+  const bool wings =
+      o.precision == HELK_PREC_F32_KAHAN ? wing_route32(c, o, cut, g) : wing_route64(c, o, cut, g, T, P);
+  const WingGeom geom = wing_geometry(g->n, max_half(cut, g), c->num_sms);
+  const WingGeom *wg = wings ? &geom : nullptr;
   HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n, wg));
-  const CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
+  CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
+  one.wings = wings;
   choose_core_nodes(c, &one, 1, *g);
   stage_begin(c, HELK_STAGE_LINEPREP);
   HELK_TRY(prepare_lines(c, 1, &one, mass, cut, g, o, wg != nullptr));
   stage_end(c, HELK_STAGE_LINEPREP);
   if (c->nlines > 0) {
     stage_begin(c, HELK_STAGE_VOIGT);
-    HELK_TRY(run_voigt(c, 1, g, o, kappa, shape, tile, ntiles, wg));
+    HELK_TRY(run_voigt(c, 1, g, o, kappa, shape, tile, ntiles, wg, wings ? 1 : 0));
     stage_end(c, HELK_STAGE_VOIGT);
   } else if (!o.accumulate) {
     HELK_TRY(cuda_check(c, cudaMemsetAsync(kappa, 0, (size_t)g->n * 8, c->stream), "opacity"));
@@ -591,11 +637,11 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
   for (int i = 0; i < ncand && st == HELK_OK; ++i) {
     const int pts = std::max(1, shape_points(o.precision, cand[i]));
     const int64_t ntiles = (g->n + pts - 1) / pts;
-    st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles, nullptr);  // warm-up
+    st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles, nullptr, 0);  // warm-up
     float ms = 0.f;
     const int reps = 3;
     if (st == HELK_OK) st = cuda_check(c, cudaEventRecord(e0, c->stream), "autotune");
-    for (int r = 0; r < reps && st == HELK_OK; ++r) st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles, nullptr);
+    for (int r = 0; r < reps && st == HELK_OK; ++r) st = run_voigt(c, 1, g, o, c->kappa, cand[i], pts, ntiles, nullptr, 0);
     if (st == HELK_OK) st = cuda_check(c, cudaEventRecord(e1, c->stream), "autotune");
     if (st == HELK_OK) st = cuda_check(c, cudaEventSynchronize(e1), "autotune");
     if (st == HELK_OK) st = cuda_check(c, cudaEventElapsedTime(&ms, e0, e1), "autotune");
@@ -625,18 +671,18 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
 // reads or writes and that a later call may move (all of them: a list that grows and
 // shrinks again can move some and leave others where they were).
 static std::string batch_key(const helk_ctx *c, int n_cond, double mass, const helk_cutoff *cut,
-                             const helk_grid *g, const helk_opts &o, const double *kappa, int shape, bool wings) {
+                             const helk_grid *g, const helk_opts &o, const double *kappa, int shape, int n_wing) {
   char b[256];
   snprintf(b, sizeof b, "%d|%lld|%a|%d|%a|%a|%a|%a|%lld|%d|%d|%a|%d|%d|%d|%d|%d", n_cond, (long long)c->nlines, mass,
            cut->kind, cut->value, cut->cap, g->nu_min, g->dnu, (long long)g->n, o.precision, o.accumulate, o.weight,
-           o.count_regions, o.surrogate, shape, (int)c->core_nodes, (int)wings);
+           o.count_regions, o.surrogate, shape, (int)c->core_nodes, n_wing);
   std::string key(b);
   // the line fields (absent ones are passed to line preparation as null pointers)
   const void *const bufs[] = {c->nu0, c->S0, c->has_E ? c->El : nullptr, c->gair, c->has_gself ? c->gself : nullptr,
                               c->has_ncoll ? c->ncoll : nullptr, c->has_delta ? c->delta : nullptr,
                               c->has_mass ? c->lmass : nullptr, c->has_weight ? c->lweight : nullptr,
                               // per condition (a chunk's view of them)
-                              c->cond_host, c->cond_dev, c->cstats, c->cond_order,
+                              c->cond_host, c->cond_dev, c->cstats, c->cond_order, c->cond_list, c->cond_list_host,
                               // records, maps, sums
                               c->rec64, c->rec32, c->ext64, c->ckey, c->ckey32, c->core_rng, c->core_blk, c->tile_lo,
                               c->tile_hi, c->kcore, c->kcore64, c->wingF, c->squeue, kappa};
@@ -657,12 +703,16 @@ struct CondView {
     c->cond_dev += k0;
     c->cstats += k0;
     c->cond_order += k0;
+    c->cond_list += k0;
+    c->cond_list_host += k0;
   }
   ~CondView() {
     c->cond_host -= k0;
     c->cond_dev -= k0;
     c->cstats -= k0;
     c->cond_order -= k0;
+    c->cond_list -= k0;
+    c->cond_list_host -= k0;
   }
   CondView(const CondView &) = delete;
   CondView &operator=(const CondView &) = delete;
@@ -722,8 +772,12 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   // record budget (one chunk unless the list is very long), each chunk one
   // captured graph; the chunks share the record, tile-map and core buffers
   // and follow each other on the stream.
-  WingGeom geom;
-  const WingGeom *wg = wing_route(c, o, cut, g, &geom) ? &geom : nullptr;
+  const bool f64 = o.precision != HELK_PREC_F32_KAHAN;
+  const bool wings32 = !f64 && wing_route32(c, o, cut, g);
+  std::vector<char> wings(n_cond, wings32);
+  for (int k = 0; f64 && k < n_cond; ++k) wings[k] = wing_route64(c, o, cut, g, T[k], P[k]);
+  const WingGeom geom = wing_geometry(g->n, max_half(cut, g), c->num_sms);
+  const WingGeom *wg = std::count(wings.begin(), wings.end(), 1) > 0 ? &geom : nullptr;
   const int64_t rec_line =
       o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2))
                                          : (int64_t)(sizeof(LineRec64) + (wg ? sizeof(WingExt64) : 0));
@@ -740,8 +794,10 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   if (!c->cond_ev) HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->cond_ev, cudaEventDisableTiming), "graph"));
   // the previous batch must have read the staging buffer before it changes
   HELK_TRY(cuda_check(c, cudaEventSynchronize(c->cond_ev), "opacity_batch"));
-  for (int k = 0; k < n_cond; ++k)
+  for (int k = 0; k < n_cond; ++k) {
     c->cond_host[k] = make_cond(c, T[k], P[k], q_ratio ? q_ratio[k] : o.q_ratio, mass);
+    c->cond_host[k].wings = wings[k];
+  }
   choose_core_nodes(c, c->cond_host, n_cond, *g);
   stage_begin(c, HELK_STAGE_VOIGT);
   for (int j = 0; j < nchunk; ++j) {
@@ -752,7 +808,13 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
       // the chunk's view of the per-condition arrays (staging, parameters,
       // statistics, order): offset by its first condition, restored after
       const CondView view(c, k0);
-      const std::string key = batch_key(c, nk, mass, cut, g, o, kap, shape, wg != nullptr);
+      // its conditions (counted from its first) with wings, then the others
+      int n_wing = 0, rest = nk;
+      for (int k = nk - 1; k >= 0; --k)
+        if (!wings[k0 + k]) c->cond_list_host[--rest] = k;
+      for (int k = 0; k < nk; ++k)
+        if (wings[k0 + k]) c->cond_list_host[n_wing++] = k;
+      const std::string key = batch_key(c, nk, mass, cut, g, o, kap, shape, n_wing);
       gx = find_graph(c, key);
       if (!gx) {
         cudaStream_t user = c->stream;
@@ -764,8 +826,12 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
           st = cuda_check(c, cudaMemcpyAsync(c->cond_dev, c->cond_host, nk * sizeof(CondArgs),
                                              cudaMemcpyHostToDevice, c->stream),
                           "graph capture");
-          if (st == HELK_OK) st = prepare_lines(c, nk, nullptr, mass, cut, g, o, wg != nullptr);
-          if (st == HELK_OK) st = run_voigt(c, nk, g, o, kap, shape, tile, ntiles, wg);
+          if (st == HELK_OK && n_wing > 0 && n_wing < nk)
+            st = cuda_check(c, cudaMemcpyAsync(c->cond_list, c->cond_list_host, nk * sizeof(int),
+                                               cudaMemcpyHostToDevice, c->stream),
+                            "graph capture");
+          if (st == HELK_OK) st = prepare_lines(c, nk, nullptr, mass, cut, g, o, n_wing > 0);
+          if (st == HELK_OK) st = run_voigt(c, nk, g, o, kap, shape, tile, ntiles, wg, n_wing);
           const cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
           if (st == HELK_OK) st = cuda_check(c, e, "graph capture");
         }

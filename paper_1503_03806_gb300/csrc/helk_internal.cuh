@@ -104,6 +104,9 @@ struct DevStats {
   unsigned int tile_counter;        // next (condition, tile) item of the persistent Voigt kernel
   int run_end[SORT_RUNS];           // upload: where the first of them are (in no order)
   double cuts[LIST_CUTS + 1];       // upload: ListShape::at
+  // upload: order keys of the list's largest coefficients and extreme exponents (of
+  // the least its complement: every field starts at 0)
+  unsigned long long gair_max, gself_max, ncoll_max, ncoll_min_inv;
 };
 
 // Core evaluations routed to the surrogate by the FP32 Voigt kernel: the
@@ -125,6 +128,7 @@ struct CondArgs {
   // Gamma_D for the call's mass (1 amu where the lines carry masses)
   double tfac, kE, cT, kc;
   double lnT;  // ln(T0 / T)
+  int wings;   // FP64 form: the condition takes interpolated wings
 };
 
 // Per-condition results of line preparation and of the Voigt kernel.
@@ -163,6 +167,7 @@ struct helk_ctx {
   // line list (sorted SoA)
   int64_t nlines = 0;
   helk::ListShape shape{};  // of the uploaded list
+  double gair_max = 0.0, gself_max = 0.0, ncoll_max = 0.5, ncoll_min = 0.5;
   bool has_E = false, has_gself = false, has_ncoll = false, has_delta = false;
   bool has_mass = false, has_weight = false;
   double *nu0 = nullptr, *S0 = nullptr, *El = nullptr, *gair = nullptr,
@@ -207,6 +212,8 @@ struct helk_ctx {
   helk::CondArgs *cond_dev = nullptr, *cond_host = nullptr;  // host side pinned
   helk::CondStats *cstats = nullptr, *cstats_host = nullptr; // host side pinned
   int *cond_order = nullptr;
+  // a batch whose conditions take both FP64 routes: those with wings first
+  int *cond_list = nullptr, *cond_list_host = nullptr;  // host side pinned
   int cond_cap = 0;
   int last_ncond = 0;
   cudaEvent_t cond_ev = nullptr;   // completion of the last batch that read cond_host
@@ -362,13 +369,12 @@ __device__ __forceinline__ void tma_load_1d(uint32_t dst_smem, const void *src, 
 // k_lines.cu
 cudaError_t launch_validate_lines(helk_ctx *c, int64_t n);
 // descents, run_end: DevStats::unsorted and its run ends
-cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end);  // orders SoA by nu0
-cudaError_t launch_list_cuts(helk_ctx *c, int64_t n);  // DevStats::cuts of an ordered list
+cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end);  // orders SoA by nu0; stats_host->cuts
 // n_cond conditions: from c->cond_dev, or (n_cond == 1 and single != NULL)
 // the one condition passed by value.  Records of condition k start at
 // k * nlines; tile maps at k * ntiles.
 // The FP64 form's records.  wings: also the WingExt64 and the core reach
-// of the FP64 interpolated-wings route.
+// of the FP64 interpolated-wings route, of the conditions that take it.
 cudaError_t launch_lineprep(helk_ctx *c, int n_cond, const CondArgs *single, double mass,
                             const helk_cutoff &cut, const helk_grid &g, bool wings);
 // FP32 form: its records, in two steps (k_pack32 needs the largest strength)

@@ -18,27 +18,29 @@
 namespace helk {
 
 // -------------------------------------------------------- validation ---
-// DevStats::cuts by a CTA's first threads.
-__device__ __forceinline__ void list_cuts(int64_t n, const double *nu0, DevStats *st) {
-  if (threadIdx.x <= LIST_CUTS) st->cuts[threadIdx.x] = nu0[(n - 1) * threadIdx.x / LIST_CUTS];
+// Doubles as unsigned integers of the same order.
+__device__ __forceinline__ unsigned long long order_key(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b >> 63 ? ~b : b | 0x8000000000000000ull;
 }
-__global__ void k_list_cuts(int64_t n, const double *__restrict__ nu0, DevStats *st) { list_cuts(n, nu0, st); }
-
-cudaError_t launch_list_cuts(helk_ctx *c, int64_t n) {
-  if (n <= 0) return cudaSuccess;
-  ++c->launches;
-  k_list_cuts<<<1, 96, 0, c->stream>>>(n, c->nu0, c->stats);
-  return cudaGetLastError();
+// ListShape::at by a CTA's first threads.
+__device__ __forceinline__ void list_cuts(int64_t n, const double *nu0, double *cuts) {
+  if (threadIdx.x <= LIST_CUTS) cuts[threadIdx.x] = nu0[(n - 1) * threadIdx.x / LIST_CUTS];
+}
+// A maximum that most warps do not raise.
+__device__ __forceinline__ void raise_max(unsigned long long *at, unsigned long long v) {
+  if (v > *(volatile unsigned long long *)at) atomicMax(at, v);
 }
 
-// (of a list that is not ordered the cuts are taken again after it is)
+// (of a list that is not ordered the cuts are taken again when it is)
 __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const double *__restrict__ S0,
                            const double *__restrict__ El, const double *__restrict__ gair,
                            const double *__restrict__ gself, const double *__restrict__ ncoll,
                            const double *__restrict__ delta, const double *__restrict__ lmass,
                            const double *__restrict__ lweight, DevStats *st) {
   int bad = 0;
-  if (blockIdx.x == 0) list_cuts(n, nu0, st);
+  if (blockIdx.x == 0) list_cuts(n, nu0, st->cuts);
+  unsigned long long ga = 0, gs = 0, nmax = 0, nmin = 0;  // order keys; nmin: of the complement
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
        l += (int64_t)gridDim.x * blockDim.x) {
     double v = nu0[l];
@@ -51,12 +53,36 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
     if (lmass) ok = ok && isfinite(lmass[l]) && lmass[l] > 0.0;
     if (lweight) ok = ok && isfinite(lweight[l]) && lweight[l] >= 0.0;
     bad += !ok;
+    ga = max(ga, order_key(gair[l]));
+    if (gself) gs = max(gs, order_key(gself[l]));
+    if (ncoll) {
+      const unsigned long long k = order_key(ncoll[l]);
+      nmax = max(nmax, k);
+      nmin = max(nmin, ~k);
+    }
     if (l + 1 < n && nu0[l + 1] < v && *(volatile int *)&st->unsorted < SORT_RUNS) {
       const int q = atomicAdd(&st->unsorted, 1);
       if (q < SORT_RUNS) st->run_end[q] = (int)(l + 1);
     }
   }
   if (bad) atomicAdd(&st->bad_lines, bad);
+  // (of a list with bad values these mean nothing: it is refused)
+  for (int o = 16; o > 0; o >>= 1) {
+    ga = max(ga, __shfl_down_sync(0xffffffffu, ga, o));
+    if (gself) gs = max(gs, __shfl_down_sync(0xffffffffu, gs, o));
+    if (ncoll) {
+      nmax = max(nmax, __shfl_down_sync(0xffffffffu, nmax, o));
+      nmin = max(nmin, __shfl_down_sync(0xffffffffu, nmin, o));
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    raise_max(&st->gair_max, ga);
+    if (gself) raise_max(&st->gself_max, gs);
+    if (ncoll) {
+      raise_max(&st->ncoll_max, nmax);
+      raise_max(&st->ncoll_min_inv, nmin);
+    }
+  }
 }
 
 cudaError_t launch_validate_lines(helk_ctx *c, int64_t n) {
@@ -188,8 +214,7 @@ __global__ void k_line_keys(int64_t n, const double *__restrict__ nu0, unsigned 
        l += (int64_t)gridDim.x * blockDim.x) {
     double v = nu0[l];
     if (v == 0.0) v = 0.0;  // -0 -> +0
-    unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    keys[l] = (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+    keys[l] = order_key(v);
     vals[l] = (uint32_t)l;
   }
 }
@@ -216,7 +241,9 @@ __global__ void k_gather(int64_t n, const uint32_t *__restrict__ perm, GatherSet
     for (int f = 0; f < G.m; ++f) G.tmp[f][l] = G.field[f][p];
   }
 }
-__global__ void k_gather_back(int64_t n, GatherSet G) {
+// cuts: NULL, or where the cuts of the ordered list's centres go (its field 0)
+__global__ void k_gather_back(int64_t n, GatherSet G, double *cuts) {
+  if (cuts && blockIdx.x == 0) list_cuts(n, G.tmp[0], cuts);
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
        l += (int64_t)gridDim.x * blockDim.x)
     for (int f = 0; f < G.m; ++f) G.field[f][l] = G.tmp[f][l];
@@ -239,7 +266,8 @@ static cudaError_t reorder_fields(helk_ctx *c, int64_t n, const uint32_t *perm, 
     if (G.m == ntmp || (f == 9 && G.m > 0)) {
       c->launches += 2;
       k_gather<<<gb, 256, 0, c->stream>>>(n, perm, G);
-      k_gather_back<<<gb, 256, 0, c->stream>>>(n, G);
+      // the cuts straight to the pinned copy of the statistics that the upload waits for
+      k_gather_back<<<gb, 256, 0, c->stream>>>(n, G, G.field[0] == c->nu0 ? c->stats_host->cuts : nullptr);
       G.m = 0;
     }
   }
@@ -453,8 +481,10 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
     double ck = floor((v0 - A.nu_min) / A.dnu);
     if (ck < -4.0e15) ck = -4.0e15;
     if (ck > 4.0e15) ck = 4.0e15;
+    const int k32 = (int)min(max((long long)ck, -2147483647ll), 2147483647ll);
     if (cond == 0) ckey[l] = ck;
-    if (ext_all) {
+    if (cond == 0 && ckey32) ckey32[l] = k32;
+    if (ext_all && C.wings) {
       WingExt64 x;
       const double idnu = 1.0 / A.dnu, pos = (nu0p - A.nu_min) * idnu;
       const double cf = rint(pos), cc = fmin(fmax(cf, 0.0), (double)(A.ngrid - 1));
@@ -478,8 +508,6 @@ __global__ void k_lineprep(int64_t n, const double *__restrict__ nu0, const doub
       ext_all[(int64_t)cond * n + l] = x;
       // the core reach, as k_pack32 keeps it for the FP32 form
       const long long key = (long long)ck;
-      const int k32 = (int)min(max(key, -2147483647ll), 2147483647ll);
-      if (cond == 0) ckey32[l] = k32;
       const int clo = r.a2 >= R2_GH3 ? 1 : max(r.ilo, x.g3l + 1), chi = r.a2 >= R2_GH3 ? 0 : min(r.ihi, x.g3r - 1);
       int w1 = 0;
       if (clo <= chi) w1 = (int)min(max(key - clo, chi - key) + 1, 2000000000ll);

@@ -69,9 +69,9 @@ WingGeom wing_geometry(int64_t n, double half, int num_sms) {
 // One warp per group: its candidate lines, the contiguous range of the list
 // whose reference index lies within the condition's largest window half-width
 // of the group's points.
-__global__ void k_wingmap(int64_t nlines, const double *__restrict__ ckey, WingGeom G,
+__global__ void k_wingmap(int64_t nlines, const double *__restrict__ ckey, WingGeom G, const int *__restrict__ list,
                           const CondStats *__restrict__ cst, int32_t *__restrict__ lo, int32_t *__restrict__ hi) {
-  const int cond = blockIdx.y;
+  const int cond = list ? list[blockIdx.y] : blockIdx.y;
   const int m = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   if (m >= G.nmap) return;  // warp-uniform
   int k = 0;
@@ -92,10 +92,10 @@ __global__ void k_wingmap(int64_t nlines, const double *__restrict__ ckey, WingG
   }
 }
 
-cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const WingGeom &g) {
+cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const int *list, const WingGeom &g) {
   dim3 grid((unsigned)((g.nmap + 7) / 8), n_cond);
   ++c->launches;
-  k_wingmap<<<grid, 256, 0, c->stream>>>(c->nlines, c->ckey, g, c->cstats, c->tile_lo, c->tile_hi);
+  k_wingmap<<<grid, 256, 0, c->stream>>>(c->nlines, c->ckey, g, list, c->cstats, c->tile_lo, c->tile_hi);
   return cudaGetLastError();
 }
 

@@ -460,12 +460,12 @@ __global__ void __launch_bounds__(WG_THREADS, 2)
     k_wing_far64(const LineRec64 *__restrict__ rec_all, const WingExt64 *__restrict__ ext_all, int64_t nlines,
                  const int32_t *__restrict__ ckey32, const int32_t *__restrict__ lo_all,
                  const int32_t *__restrict__ hi_all, WingGeom G, double nu_min, double dnu,
-                 const CondStats *__restrict__ cst, const int *__restrict__ core_blk, const double *__restrict__ tab,
-                 double *__restrict__ F_all, double *__restrict__ kcore_all) {
+                 const int *__restrict__ list, const CondStats *__restrict__ cst, const int *__restrict__ core_blk,
+                 const double *__restrict__ tab, double *__restrict__ F_all, double *__restrict__ kcore_all) {
   __shared__ WingSmem64 S;
   __shared__ double fs[WG_WARPS][3][W64_P];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int cond = blockIdx.y;
+  const int cond = list ? list[blockIdx.y] : blockIdx.y;
   const LineRec64 *rec = rec_all + (int64_t)cond * nlines;
   const WingExt64 *ext = ext_all + (int64_t)cond * nlines;
   if ((int)blockIdx.x >= G.farblk) {
@@ -550,9 +550,10 @@ template <int NL>
 __global__ void __launch_bounds__(WG_THREADS, 3)
     k_wing_near64(const LineRec64 *__restrict__ rec_all, const WingExt64 *__restrict__ ext_all, int64_t nlines,
                   const int32_t *__restrict__ lo_all, const int32_t *__restrict__ hi_all, WingGeom G, double nu_min,
-                  double dnu, const CondStats *__restrict__ cst, const double *__restrict__ tab,
-                  const double *__restrict__ F_all, const double *__restrict__ kcore_all, double weight,
-                  int accumulate, double *__restrict__ kappa_all) {
+                  double dnu, const int *__restrict__ list, const CondStats *__restrict__ cst,
+                  const double *__restrict__ tab, const double *__restrict__ F_all,
+                  const double *__restrict__ kcore_all, double weight, int accumulate,
+                  double *__restrict__ kappa_all) {
   constexpr int s = NL * WG_S0, NH = NL / 2, NV = NL == 1 ? 3 : 9;
   __shared__ WingSmem64 S;
   __shared__ double fs[WG_WARPS][NV][W64_P];
@@ -560,7 +561,7 @@ __global__ void __launch_bounds__(WG_THREADS, 3)
   __shared__ uint32_t s_sub[WG_WARPS][S64_N][W64_WORDS];
   __shared__ double s_top[W64_P];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int cond = blockIdx.y;
+  const int cond = list ? list[blockIdx.y] : blockIdx.y;
   const int ngrid = G.ngrid;
   const int64_t gbase = (int64_t)blockIdx.x * 8 * s;
   const int top = wing_top(G, cst[cond].wmax);
@@ -811,22 +812,22 @@ helk_status ensure_wing64(helk_ctx *c, int n_cond, const WingGeom &g) {
   return st;
 }
 
-cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const WingGeom &g, const helk_grid &grid) {
+cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const int *list, const WingGeom &g, const helk_grid &grid) {
   ++c->launches;
   const int64_t blocks = g.farblk + (grid.n + WG_THREADS - 1) / WG_THREADS;
   k_wing_far64<<<dim3((unsigned)blocks, n_cond), WG_THREADS, 0, c->stream>>>(
-      c->rec64, c->ext64, c->nlines, c->ckey32, c->tile_lo, c->tile_hi, g, grid.nu_min, grid.dnu, c->cstats,
-      c->core_blk, c->wing_tab64, (double *)c->wingF, c->kcore64);
+      c->rec64, c->ext64, c->nlines, c->ckey32, c->tile_lo, c->tile_hi, g, grid.nu_min, grid.dnu, list,
+      c->cstats, c->core_blk, c->wing_tab64, (double *)c->wingF, c->kcore64);
   return cudaGetLastError();
 }
 
-cudaError_t launch_wing_near64(helk_ctx *c, int n_cond, const WingGeom &g, const helk_grid &grid, const helk_opts &o,
-                               double *kappa) {
+cudaError_t launch_wing_near64(helk_ctx *c, int n_cond, const int *list, const WingGeom &g, const helk_grid &grid,
+                               const helk_opts &o, double *kappa) {
   ++c->launches;
   auto near = g.lvl0 == 2 ? k_wing_near64<4> : k_wing_near64<1>;
   near<<<dim3((unsigned)g.groups[0], n_cond), WG_THREADS, 0, c->stream>>>(
-      c->rec64, c->ext64, c->nlines, c->tile_lo, c->tile_hi, g, grid.nu_min, grid.dnu, c->cstats, c->wing_tab64,
-      (const double *)c->wingF, c->kcore64, o.weight, o.accumulate, kappa);
+      c->rec64, c->ext64, c->nlines, c->tile_lo, c->tile_hi, g, grid.nu_min, grid.dnu, list, c->cstats,
+      c->wing_tab64, (const double *)c->wingF, c->kcore64, o.weight, o.accumulate, kappa);
   return cudaGetLastError();
 }
 

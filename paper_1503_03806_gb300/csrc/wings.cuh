@@ -86,8 +86,9 @@ __device__ __forceinline__ int wing_top(const WingGeom &g, long long wmax) {
 // host: the geometry for a grid of n points, windows of at most
 // `half` points on either side (a bound), on a GPU of num_sms SMs
 WingGeom wing_geometry(int64_t n, double half, int num_sms);
-// host: candidate line range of every group of every stage
-cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const WingGeom &g);
+// host: candidate line range of every group of every stage, for n_cond conditions:
+// those in `list` (device), or all if it is NULL
+cudaError_t launch_wingmap(helk_ctx *c, int n_cond, const int *list, const WingGeom &g);
 
 // k_wings.cu: the FP32 form
 helk_status ensure_wing32(helk_ctx *c, int n_cond, const WingGeom &g);
@@ -100,8 +101,8 @@ void wing_tables(int P, int PS, std::vector<double> &tab);
 
 // k_wings64.cu: the FP64 form (the far launch also takes the core sums)
 helk_status ensure_wing64(helk_ctx *c, int n_cond, const WingGeom &g);
-cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const WingGeom &g, const helk_grid &grid);
-cudaError_t launch_wing_near64(helk_ctx *c, int n_cond, const WingGeom &g, const helk_grid &grid, const helk_opts &o,
-                               double *kappa);
+cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const int *list, const WingGeom &g, const helk_grid &grid);
+cudaError_t launch_wing_near64(helk_ctx *c, int n_cond, const int *list, const WingGeom &g, const helk_grid &grid,
+                               const helk_opts &o, double *kappa);
 
 }  // namespace helk

@@ -24,8 +24,9 @@ extern "C" int cuts() { return helk::LIST_CUTS; }
 extern "C" double near(int64_t n, const double *at, double nu_min, double dnu, int64_t ng, double points, double reach) {
   return helk::lines_near(shape(n, at), nu_min, dnu, ng, points, reach);
 }
-extern "C" int pay64(int64_t n, const double *at, double nu_min, double dnu, int64_t ng, double half) {
-  return helk::wings_pay64(shape(n, at), nu_min, dnu, ng, half);
+extern "C" int pay64(int64_t n, const double *at, double nu_min, double dnu, int64_t ng, double half,
+                     double most) {
+  return helk::wings_pay64(shape(n, at), nu_min, dnu, ng, most, half);
 }
 """
 D, I = ctypes.c_double, ctypes.c_int64
@@ -76,13 +77,24 @@ def test_lines_near(lib, n, lo, hi):
 def test_measured_cases(lib, n, nlines, half, wings):
     nu = np.sort(np.random.default_rng(1).uniform(0.05, n * 0.01, nlines))
     a, p = at(lib, nu)
-    assert bool(lib.pay64(I(nlines), p, D(0.0), D(0.01), I(n), D(half))) == wings
+    assert bool(lib.pay64(I(nlines), p, D(0.0), D(0.01), I(n), D(half), D(half))) == wings
+
+
+@pytest.mark.parametrize("n,nlines,half,wings", [
+    (3_000_000, 100_000, 2.2e-4, False), (3_000_000, 1_000_000, 2.2e-4, False), (3_000_000, 100_000, 0.022, False),
+    (3_000_000, 1_000_000, 0.022, True), (3_000_000, 100_000, 0.22, True), (3_000_000, 100_000, 22.0, True),
+    (300_000, 10_000, 0.022, False), (300_000, 10_000, 0.22, True), (30_000, 1000, 0.022, False),
+    (30_000, 1000, 0.22, True), (30_000, 1000, 0.0, False)])
+def test_measured_pressures(lib, n, nlines, half, wings):
+    nu = np.sort(np.random.default_rng(1).uniform(0.05, n * 0.01, nlines))
+    a, p = at(lib, nu)
+    assert bool(lib.pay64(I(nlines), p, D(0.0), D(0.01), I(n), D(half), D(10000.0))) == wings
 
 
 def test_lines_elsewhere_do_not_count(lib):
     nu = np.sort(np.random.default_rng(1).uniform(0.05, 30000.0, 10_000))
     a, p = at(lib, nu)
-    assert not lib.pay64(I(10_000), p, D(10000.0), D(0.01), I(3000), D(100.0))
+    assert not lib.pay64(I(10_000), p, D(10000.0), D(0.01), I(3000), D(100.0), D(100.0))
     nu = np.sort(np.random.default_rng(1).uniform(20000.0, 30000.0, 1_000_000))
     a, p = at(lib, nu)
-    assert not lib.pay64(I(1_000_000), p, D(0.0), D(0.01), I(300_000), D(2500.0))
+    assert not lib.pay64(I(1_000_000), p, D(0.0), D(0.01), I(300_000), D(2500.0), D(2500.0))
