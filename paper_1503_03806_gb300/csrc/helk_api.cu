@@ -272,6 +272,7 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
   c->gself_max = order_double(c->stats_host->gself_max);
   c->ncoll_max = order_double(c->stats_host->ncoll_max);
   c->ncoll_min = order_double(~c->stats_host->ncoll_min_inv);
+  c->mass_min = order_double(~c->stats_host->mass_min_inv);
   c->shape.n = n;
   std::copy(c->stats_host->cuts, c->stats_host->cuts + LIST_CUTS + 1, c->shape.at);
   c->have_opacity = false;
@@ -448,13 +449,11 @@ static CondArgs make_cond(const helk_ctx *c, double T, double P, double q_ratio,
   return CondArgs{T, P, q_ratio, sqrt(T0 / T), C2 / T0 - C2 / T, C2 / T, SQRTLN2 / vth, log(T0 / T), 0};
 }
 
-// Which core kernel (FP32 form): the one with nodes if a line of a condition can have
-// beta <= CORE_NODE_BETA on the grid (a factor of 2 for centres beyond its end and
-// for shifts).  If none can, the plain kernel gives the same sums.
+// Which core kernel (FP32 form): the one with nodes if a line of a condition can use them.
 static void choose_core_nodes(helk_ctx *c, const CondArgs *conds, int n_cond, const helk_grid &g) {
-  const double top = std::max(fabs(g.nu_min), fabs(g.nu_min + g.dnu * (double)g.n));
-  c->core_nodes = c->has_mass;
-  for (int k = 0; k < n_cond; ++k) c->core_nodes |= g.dnu * conds[k].kc <= 2.0 * CORE_NODE_BETA * top;
+  c->core_nodes = false;
+  for (int k = 0; k < n_cond; ++k)
+    c->core_nodes |= core_nodes_possible(g.nu_min, g.dnu, g.n, conds[k].kc, c->has_mass ? c->mass_min : 1.0);
 }
 
 // Statistics reset and line preparation (and the FP32 records) of n_cond

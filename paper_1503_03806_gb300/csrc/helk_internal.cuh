@@ -106,7 +106,7 @@ struct DevStats {
   double cuts[LIST_CUTS + 1];       // upload: ListShape::at
   // upload: order keys of the list's largest coefficients and extreme exponents (of
   // the least its complement: every field starts at 0)
-  unsigned long long gair_max, gself_max, ncoll_max, ncoll_min_inv;
+  unsigned long long gair_max, gself_max, ncoll_max, ncoll_min_inv, mass_min_inv;
 };
 
 // Core evaluations routed to the surrogate by the FP32 Voigt kernel: the
@@ -167,7 +167,7 @@ struct helk_ctx {
   // line list (sorted SoA)
   int64_t nlines = 0;
   helk::ListShape shape{};  // of the uploaded list
-  double gair_max = 0.0, gself_max = 0.0, ncoll_max = 0.5, ncoll_min = 0.5;
+  double gair_max = 0.0, gself_max = 0.0, ncoll_max = 0.5, ncoll_min = 0.5, mass_min = 1.0;
   bool has_E = false, has_gself = false, has_ncoll = false, has_delta = false;
   bool has_mass = false, has_weight = false;
   double *nu0 = nullptr, *S0 = nullptr, *El = nullptr, *gair = nullptr,
@@ -403,8 +403,6 @@ cudaError_t launch_voigt(helk_ctx *c, int n_cond, const helk_grid &g, const helk
                          double *kappa, int shape, int64_t ntiles);
 // FP32 form: the Algorithm 916 cores that k_voigt_f32 leaves out, added into
 // kappa (launched after launch_voigt; no-op for the FP64 form).
-// largest beta of a line whose cores are taken through nodes
-constexpr double CORE_NODE_BETA = 0.3 / 16.0;
 cudaError_t launch_voigt_core(helk_ctx *c, int n_cond, const helk_grid &g, const helk_opts &o);
 cudaError_t launch_core_add(helk_ctx *c, int n_cond, const helk_grid &g, const helk_opts &o, double *kappa);
 // k_voigt64.cu: the FP64 form (called by the dispatch above) and the

@@ -40,7 +40,7 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
                            const double *__restrict__ lweight, DevStats *st) {
   int bad = 0;
   if (blockIdx.x == 0) list_cuts(n, nu0, st->cuts);
-  unsigned long long ga = 0, gs = 0, nmax = 0, nmin = 0;  // order keys; nmin: of the complement
+  unsigned long long ga = 0, gs = 0, nmax = 0, nmin = 0, mmin = 0;  // order keys; of the least their complements
   for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n;
        l += (int64_t)gridDim.x * blockDim.x) {
     double v = nu0[l];
@@ -60,6 +60,7 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
       nmax = max(nmax, k);
       nmin = max(nmin, ~k);
     }
+    if (lmass) mmin = max(mmin, ~order_key(lmass[l]));
     if (l + 1 < n && nu0[l + 1] < v && *(volatile int *)&st->unsorted < SORT_RUNS) {
       const int q = atomicAdd(&st->unsorted, 1);
       if (q < SORT_RUNS) st->run_end[q] = (int)(l + 1);
@@ -74,6 +75,7 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
       nmax = max(nmax, __shfl_down_sync(0xffffffffu, nmax, o));
       nmin = max(nmin, __shfl_down_sync(0xffffffffu, nmin, o));
     }
+    if (lmass) mmin = max(mmin, __shfl_down_sync(0xffffffffu, mmin, o));
   }
   if ((threadIdx.x & 31) == 0) {
     raise_max(&st->gair_max, ga);
@@ -82,6 +84,7 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
       raise_max(&st->ncoll_max, nmax);
       raise_max(&st->ncoll_min_inv, nmin);
     }
+    if (lmass) raise_max(&st->mass_min_inv, mmin);
   }
 }
 

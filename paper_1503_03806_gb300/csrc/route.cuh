@@ -1,11 +1,12 @@
 // route.cuh -- the rules by which an opacity call takes interpolated wings or the
-// point-by-point kernels (host side; shared by nothing else, so that a test can
-// compile it alone).
+// point-by-point kernels, and one core kernel or the other (host side; needs no other
+// header, so that a test can compile it alone).
 #pragma once
 
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 
 namespace helk {
 
@@ -57,6 +58,19 @@ constexpr double WING64_MIN_HALF = 24.0;
 inline bool wings_pay64(const ListShape &L, double nu_min, double dnu, int64_t n, double most, double half) {
   return most >= WING64_MIN_HALF && lines_near(L, nu_min, dnu, n, 2048.0, half) * std::min(1.0, 2.0 * half) >=
                                         5.0 + std::min(15.0, 4.0e5 / (double)n);
+}
+
+// FP32 form.  Largest beta (grid steps in Doppler units) of a line whose cores are
+// taken through nodes, and whether a line of a condition can have one as small: kc is
+// sqrt(ln2) nu / Gamma_D for the call's mass, or for 1 amu where the lines have masses,
+// of which mass_min is the smallest (beta grows with its root; pass 1 otherwise); a
+// factor of 2 for centres beyond the grid's end and for shifts.  If none can, the kernel
+// without nodes gives the same sums in less time (1e5 lines with masses, 3e6 points at
+// 0.01, 0.1 atm: 276 us a call, 289 with the other).
+constexpr double CORE_NODE_BETA = 0.3 / 16.0;
+inline bool core_nodes_possible(double nu_min, double dnu, int64_t n, double kc, double mass_min) {
+  const double top = std::max(std::fabs(nu_min), std::fabs(nu_min + dnu * (double)n));
+  return dnu * kc * std::sqrt(mass_min) <= 2.0 * CORE_NODE_BETA * top;
 }
 
 }  // namespace helk
