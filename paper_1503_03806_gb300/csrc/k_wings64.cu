@@ -455,7 +455,9 @@ __device__ __forceinline__ void core_points64(CoreLine64 (*s_line)[32], double (
 
 // ---------------------------------------------------------------- kernels --
 // The far kernel's CTAs (node sums of the coarser panels) first, then the core
-// sums, 256 points a CTA: one launch, so that they share the GPU.
+// sums, 256 points a CTA: one launch, so that they share the GPU.  LIST: the
+// conditions are those of `list` (without it the index is not kept in a register).
+template <bool LIST>
 __global__ void __launch_bounds__(WG_THREADS, 2)
     k_wing_far64(const LineRec64 *__restrict__ rec_all, const WingExt64 *__restrict__ ext_all, int64_t nlines,
                  const int32_t *__restrict__ ckey32, const int32_t *__restrict__ lo_all,
@@ -465,7 +467,7 @@ __global__ void __launch_bounds__(WG_THREADS, 2)
   __shared__ WingSmem64 S;
   __shared__ double fs[WG_WARPS][3][W64_P];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int cond = list ? list[blockIdx.y] : blockIdx.y;
+  const int cond = LIST ? list[blockIdx.y] : blockIdx.y;
   const LineRec64 *rec = rec_all + (int64_t)cond * nlines;
   const WingExt64 *ext = ext_all + (int64_t)cond * nlines;
   if ((int)blockIdx.x >= G.farblk) {
@@ -546,7 +548,7 @@ enum { S64_H = 0, S64_L = 2, S64_G1 = 6, S64_D = 10, S64_N = 14 };
 constexpr int W64_LEAF_MIN = 3;
 
 // NL: leaves of a warp's panel, 4 or 1 (WingGeom::lvl0 2 or 0).
-template <int NL>
+template <int NL, bool LIST>
 __global__ void __launch_bounds__(WG_THREADS, 3)
     k_wing_near64(const LineRec64 *__restrict__ rec_all, const WingExt64 *__restrict__ ext_all, int64_t nlines,
                   const int32_t *__restrict__ lo_all, const int32_t *__restrict__ hi_all, WingGeom G, double nu_min,
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(WG_THREADS, 3)
   __shared__ uint32_t s_sub[WG_WARPS][S64_N][W64_WORDS];
   __shared__ double s_top[W64_P];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int cond = list ? list[blockIdx.y] : blockIdx.y;
+  const int cond = LIST ? list[blockIdx.y] : blockIdx.y;
   const int ngrid = G.ngrid;
   const int64_t gbase = (int64_t)blockIdx.x * 8 * s;
   const int top = wing_top(G, cst[cond].wmax);
@@ -815,7 +817,8 @@ helk_status ensure_wing64(helk_ctx *c, int n_cond, const WingGeom &g) {
 cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const int *list, const WingGeom &g, const helk_grid &grid) {
   ++c->launches;
   const int64_t blocks = g.farblk + (grid.n + WG_THREADS - 1) / WG_THREADS;
-  k_wing_far64<<<dim3((unsigned)blocks, n_cond), WG_THREADS, 0, c->stream>>>(
+  auto far = list ? k_wing_far64<true> : k_wing_far64<false>;
+  far<<<dim3((unsigned)blocks, n_cond), WG_THREADS, 0, c->stream>>>(
       c->rec64, c->ext64, c->nlines, c->ckey32, c->tile_lo, c->tile_hi, g, grid.nu_min, grid.dnu, list,
       c->cstats, c->core_blk, c->wing_tab64, (double *)c->wingF, c->kcore64);
   return cudaGetLastError();
@@ -824,7 +827,8 @@ cudaError_t launch_wing_far64(helk_ctx *c, int n_cond, const int *list, const Wi
 cudaError_t launch_wing_near64(helk_ctx *c, int n_cond, const int *list, const WingGeom &g, const helk_grid &grid,
                                const helk_opts &o, double *kappa) {
   ++c->launches;
-  auto near = g.lvl0 == 2 ? k_wing_near64<4> : k_wing_near64<1>;
+  auto near = g.lvl0 == 2 ? (list ? k_wing_near64<4, true> : k_wing_near64<4, false>)
+                          : (list ? k_wing_near64<1, true> : k_wing_near64<1, false>);
   near<<<dim3((unsigned)g.groups[0], n_cond), WG_THREADS, 0, c->stream>>>(
       c->rec64, c->ext64, c->nlines, c->tile_lo, c->tile_hi, g, grid.nu_min, grid.dnu, list, c->cstats,
       c->wing_tab64, (const double *)c->wingF, c->kcore64, o.weight, o.accumulate, kappa);
