@@ -380,10 +380,7 @@ static double cond_half(const helk_ctx *c, const helk_cutoff *cut, const helk_gr
 // Whether a call takes the interpolated-wings route, and its geometry.  FP32 form: by
 // the call; its conditions share one route.
 static bool wing_route32(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g) {
-  if (o.count_regions) return false;
-  const double half = max_half(cut, g);
-  const bool sparse = 2.0 * half * (double)c->nlines < WING32_MIN_LINES * (double)g->n;
-  return half >= WING32_MIN_HALF && !(sparse && g->n > (int64_t)c->num_sms * 512);
+  return !o.count_regions && wings_pay32(c->shape, g->nu_min, g->dnu, g->n, max_half(cut, g), c->num_sms);
 }
 // FP64 form: by the condition, so that one call and a batch agree.
 static bool wing_route64(const helk_ctx *c, const helk_opts &o, const helk_cutoff *cut, const helk_grid *g, double T,

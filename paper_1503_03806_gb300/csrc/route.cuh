@@ -60,6 +60,23 @@ inline bool wings_pay64(const ListShape &L, double nu_min, double dnu, int64_t n
                                         5.0 + std::min(15.0, 4.0e5 / (double)n);
 }
 
+// FP32 form.  `most` as above; num_sms SMs.  By the lines that reach a tile of 2048
+// points, too: the direct kernel's time follows them, while the wings cost some 30 us
+// on short grids, 60 to 130 us on 3e6 points whatever the lines; between, grids whose
+// panels are the short ones (WingGeom::lvl0 0) take the longest to pay.  us, wings /
+// direct, at lines a tile (lines, half a window in points):
+//   3e3 points  30 (30, 2500) 47 / 39     85 (100, 250) 42 / 43    100 (100, 2500) 46 / 50
+//   3e4 points  23 (100, 2500) 46 / 39    85 (1e3, 250) 48 / 46    230 (1e3, 2500) 54 / 62
+//   3e5 points  70 (3e3, 2500) 73 / 55   170 (1e3, 25000) 72 / 61  235 (1e4, 2500) 82 / 80
+//              520 (3e3, 25000) 83 / 92  850 (1e5, 250) 133 / 200
+//   3e6 points  52 (3e3, 25000) 197 / 136 85 (1e5, 250) 278 / 252  119 (1e5, 768) 301 / 306
+//              173 (1e4, 25000) 218 / 265 235 (1e5, 2500) 325 / 406  725 (1e6, 64) 980 / 1200
+constexpr double WING32_MIN_HALF = 64.0;
+inline bool wings_pay32(const ListShape &L, double nu_min, double dnu, int64_t n, double most, int num_sms) {
+  const double lines = n <= (int64_t)512 * num_sms ? 100.0 : n < (int64_t)2048 * num_sms ? 200.0 : 120.0;
+  return most >= WING32_MIN_HALF && lines_near(L, nu_min, dnu, n, 2048.0, most) >= lines;
+}
+
 // FP32 form.  Largest beta (grid steps in Doppler units) of a line whose cores are
 // taken through nodes, and whether a line of a condition can have one as small: kc is
 // sqrt(ln2) nu / Gamma_D for the call's mass, or for 1 amu where the lines have masses,

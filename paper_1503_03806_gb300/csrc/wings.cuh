@@ -27,7 +27,8 @@
 // the next two.  A group scans its candidate lines once; lines taken at the
 // group's own level (lvl0 + 3k + 3) or coarser are dropped at once.  lvl0 is 2
 // (128 points a warp, 1024 a CTA), or 0 (32 and 256) on grids too short to give
-// every SM two CTAs of the former.
+// every SM two CTAs of the former.  Where the point-by-point kernels are taken instead:
+// route.cuh.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,18 +37,9 @@
 #include <vector>
 
 #include "helk_internal.cuh"
-#include "route.cuh"
 
 namespace helk {
 
-// Where the direct route is taken instead in the FP32 form (the FP64 form's rule is in
-// route.cuh): narrow windows, and few lines to a point on grids whose tiles give every
-// SM work.  Opacity in ms, wings / direct, half a window of h points:
-//   1e5 lines on 3e6 points   h = 128 0.266 / 0.241   512 0.296 / 0.280
-//                             768 (51 lines to a point) 0.301 / 0.306
-//   1e6 lines on 3e6 points   h = 64 (43 lines to a point) 0.98 / 1.20
-//   3e3 lines on 2e4 points   h = 64 (19 lines to a point) 0.040 / 0.063
-constexpr double WING32_MIN_HALF = 64.0, WING32_MIN_LINES = 43.0;
 constexpr int WG_S0 = 32;                   // points of a leaf
 constexpr int WG_LEVELS = 23;               // the coarsest panels have 2^27 points
 constexpr int WG_STAGES = 7;

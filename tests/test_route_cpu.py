@@ -1,6 +1,6 @@
 """The rules that choose between interpolated wings and point-by-point sums
 (route.cuh, compiled for the host): the number of lines near a stretch of the grid
-against a count, and the FP64 rule on the faster side of the measured cases that
+against a count, and each form's rule on the faster side of the measured cases that
 it states."""
 import ctypes
 import os
@@ -27,6 +27,9 @@ extern "C" double near(int64_t n, const double *at, double nu_min, double dnu, i
 extern "C" int pay64(int64_t n, const double *at, double nu_min, double dnu, int64_t ng, double half,
                      double most) {
   return helk::wings_pay64(shape(n, at), nu_min, dnu, ng, most, half);
+}
+extern "C" int pay32(int64_t n, const double *at, double nu_min, double dnu, int64_t ng, double most) {
+  return helk::wings_pay32(shape(n, at), nu_min, dnu, ng, most, 152);
 }
 """
 D, I = ctypes.c_double, ctypes.c_int64
@@ -89,6 +92,25 @@ def test_measured_pressures(lib, n, nlines, half, wings):
     nu = np.sort(np.random.default_rng(1).uniform(0.05, n * 0.01, nlines))
     a, p = at(lib, nu)
     assert bool(lib.pay64(I(nlines), p, D(0.0), D(0.01), I(n), D(half), D(10000.0))) == wings
+
+
+@pytest.mark.parametrize("n,nlines,half,wings", [
+    (3000, 10, 2500, False), (3000, 30, 2500, False), (3000, 1000, 250, True), (3000, 10_000, 63, False),
+    (30_000, 100, 2500, False), (30_000, 300, 25_000, True), (30_000, 1000, 2500, True), (30_000, 30, 25_000, False),
+    (300_000, 3000, 2500, False), (300_000, 1000, 25_000, False), (300_000, 3000, 25_000, True),
+    (300_000, 100_000, 250, True), (3_000_000, 3000, 25_000, False), (3_000_000, 100_000, 250, False),
+    (3_000_000, 10_000, 25_000, True), (3_000_000, 100_000, 2500, True), (3_000_000, 1_000_000, 64, True)])
+def test_measured_cases32(lib, n, nlines, half, wings):
+    nu = np.sort(np.random.default_rng(1).uniform(0.05, n * 0.01, nlines))
+    a, p = at(lib, nu)
+    assert bool(lib.pay32(I(nlines), p, D(0.0), D(0.01), I(n), D(half))) == wings
+
+
+def test_a_band_of_a_long_list32(lib):
+    for nlines, wings in ((10_000, False), (1_000_000, True)):
+        nu = np.sort(np.random.default_rng(1).uniform(0.05, 30000.0, nlines))
+        a, p = at(lib, nu)
+        assert bool(lib.pay32(I(nlines), p, D(10000.0), D(0.01), I(300_000), D(2500.0))) == wings
 
 
 def test_lines_elsewhere_do_not_count(lib):
