@@ -441,6 +441,17 @@ static helk_status ensure_call_buffers(helk_ctx *c, int n_cond, const helk_opts 
   return HELK_OK;
 }
 
+// The same for the route chosen.  Where there is no room for the FP64 wings' own buffers
+// (32 B a line, 8 B a point and a condition), the call takes the point-by-point kernels.
+static helk_status ensure_route_buffers(helk_ctx *c, int n_cond, const helk_opts &o, int64_t ntiles, int64_t ngrid,
+                                        const WingGeom &geom, bool &wings) {
+  const helk_status st = ensure_call_buffers(c, n_cond, o, ntiles, ngrid, wings ? &geom : nullptr);
+  if (st != HELK_ERR_OOM || !wings || o.precision == HELK_PREC_F32_KAHAN) return st;
+  c->err.clear();
+  wings = false;
+  return ensure_call_buffers(c, n_cond, o, ntiles, ngrid, nullptr);
+}
+
 static CondArgs make_cond(const helk_ctx *c, double T, double P, double q_ratio, double mass) {
   const double vth = sqrt(2.0 * LN2 * KB * T / ((c->has_mass ? 1.0 : mass) * AMU)) / CLIGHT;
   return CondArgs{T, P, q_ratio, sqrt(T0 / T), C2 / T0 - C2 / T, C2 / T, SQRTLN2 / vth, log(T0 / T), 0};
@@ -572,11 +583,10 @@ helk_status helk_opacity(helk_ctx *c, double T, double P, double mass, const hel
   const int tile = shape_points(o.precision, shape);
   if (tile <= 0) return set_err(c, HELK_ERR_STATE, "opacity: no kernel shape");
   const int64_t ntiles = (g->n + tile - 1) / tile;
-  const bool wings =
-      o.precision == HELK_PREC_F32_KAHAN ? wing_route32(c, o, cut, g) : wing_route64(c, o, cut, g, T, P);
+  bool wings = o.precision == HELK_PREC_F32_KAHAN ? wing_route32(c, o, cut, g) : wing_route64(c, o, cut, g, T, P);
   const WingGeom geom = wing_geometry(g->n, max_half(cut, g), c->num_sms);
+  HELK_TRY(ensure_route_buffers(c, 1, o, ntiles, g->n, geom, wings));
   const WingGeom *wg = wings ? &geom : nullptr;
-  HELK_TRY(ensure_call_buffers(c, 1, o, ntiles, g->n, wg));
   CondArgs one = make_cond(c, T, P, o.q_ratio, mass);
   one.wings = wings;
   choose_core_nodes(c, &one, 1, *g);
@@ -773,18 +783,20 @@ helk_status helk_opacity_batch(helk_ctx *c, int32_t n_cond, const double *T, con
   std::vector<char> wings(n_cond, wings32);
   for (int k = 0; f64 && k < n_cond; ++k) wings[k] = wing_route64(c, o, cut, g, T[k], P[k]);
   const WingGeom geom = wing_geometry(g->n, max_half(cut, g), c->num_sms);
-  const WingGeom *wg = std::count(wings.begin(), wings.end(), 1) > 0 ? &geom : nullptr;
+  bool any = std::count(wings.begin(), wings.end(), 1) > 0;
   const int64_t rec_line =
       o.precision == HELK_PREC_F32_KAHAN ? (int64_t)(sizeof(LineRec32) + sizeof(int2))
-                                         : (int64_t)(sizeof(LineRec64) + (wg ? sizeof(WingExt64) : 0));
+                                         : (int64_t)(sizeof(LineRec64) + (any ? sizeof(WingExt64) : 0));
   // the FP64 wings route also keeps a core sum a point
-  const int64_t rec_grid = wg && o.precision != HELK_PREC_F32_KAHAN ? g->n * 8 : 0;
+  const int64_t rec_grid = any && o.precision != HELK_PREC_F32_KAHAN ? g->n * 8 : 0;
   const int64_t per_cond = std::max<int64_t>(c->nlines, 1) * rec_line + rec_grid;
   const int gmax = (int)std::max<int64_t>(1, std::min<int64_t>(n_cond, c->batch_budget / per_cond));
   const int nchunk = (n_cond + gmax - 1) / gmax;
   const int chunk = (n_cond + nchunk - 1) / nchunk;
   HELK_TRY(ensure_conds(c, n_cond));
-  HELK_TRY(ensure_call_buffers(c, chunk, o, ntiles, g->n, wg));
+  HELK_TRY(ensure_route_buffers(c, chunk, o, ntiles, g->n, geom, any));
+  if (!any) std::fill(wings.begin(), wings.end(), 0);
+  const WingGeom *wg = any ? &geom : nullptr;
   if (!c->cap_stream)
     HELK_TRY(cuda_check(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "graph stream"));
   if (!c->cond_ev) HELK_TRY(cuda_check(c, cudaEventCreateWithFlags(&c->cond_ev, cudaEventDisableTiming), "graph"));
