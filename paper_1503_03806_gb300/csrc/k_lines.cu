@@ -599,7 +599,9 @@ __device__ __forceinline__ F2 f2_div(F2 a, F2 b) {
   const float rem = fmaf(-q, b.l, fmaf(-q, b.h, a.h) + a.l);
   return f2_norm(q, rem * r);
 }
-// v as a pair, from its bits (no FP64 instruction for 2^-70 < |v| < 2^127 and 0)
+// v as a pair, from its bits (no FP64 instruction for 2^-70 < |v| < 2^127 and 0); a v
+// past FP32's range as 2^100, far beyond what an exponential or a width takes, and
+// finite, so that its products are
 __device__ __forceinline__ F2 f2_of(double v) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
   const int e = (int)((hi >> 20) & 0x7FF) - 1023;
@@ -610,8 +612,9 @@ __device__ __forceinline__ F2 f2_of(double v) {
     return F2{h, sign ? -l : l};
   }
   if (e == -1023) return F2{0.0f, 0.0f};
+  if (e >= 127) return F2{__uint_as_float((hi & 0x80000000u) | 0x71800000u), 0.0f};
   const float h = (float)v;
-  return F2{h, e < 127 ? (float)(v - (double)h) : 0.0f};
+  return F2{h, (float)(v - (double)h)};
 }
 // v = (h + l) 2^e with 1 <= |h| < 2, from the bits (a normal v)
 __device__ __forceinline__ F2 f2_mant(double v, int &e) {
