@@ -43,21 +43,24 @@ inline double lines_near(const ListShape &L, double nu_min, double dnu, int64_t 
 // of a condition (under a Lorentz cutoff its windows may be much narrower).  The
 // wings' map, tree and core pass cost the same for few lines (0.14 ns a point and ~20
 // us), the direct kernel a tile of 2048 points some us a line that has a point of it:
-// the wings pay from about five lines a tile on, on short grids, where the launches
-// count, from about twenty.  us, wings / direct:
+// the wings pay from about six lines a tile on, on short grids, where the launches
+// count, from about thirty.  us, wings / direct:
 //   half a window of h points, 1e5 lines on 3e6 points   h = 24 2370 / 9110   64 3660 / 16000
 //   3e3 lines on 2e4 points                              h = 24   77 / 154
 //   3e6 points, lines a tile   2.3 (1e3 lines, h = 2500) 774 / 578    7 (1e4, h = 30) 749 / 1126
 //                              17 (1e3, h = 25000) 866 / 2084
 //   3e5 points                 2.3 (100, h = 2500) 175 / 121     7 (1e3, h = 30) 165 / 201
-//   3e4 points                 8.5 (100, h = 250) 62 / 42       23 (100, h = 2500) 84 / 85
+//   3e4 points                 8.5 (100, h = 250) 62 / 42       21 (300, h = 30) 68 / 61
+//                              23 (100, h = 2500) 84 / 85       85 (1e3, h = 250) 95 / 117
+//   3e3 points                 25 (30, h = 250) 61 / 51         85 (100, h = 250) 68 / 92
 //   300 points, 10 lines 55 / 48, 100 lines 100 / 247
 // Lorentz cutoff, 3e6 points, 1e5 lines (2 h of them have a point, 68 a tile)
 //   h = 0.0002 (1e-7 atm) 288 / 133    0.02 318 / 251    0.2 484 / 1031    22 1930 / 6570
 constexpr double WING64_MIN_HALF = 24.0;
 inline bool wings_pay64(const ListShape &L, double nu_min, double dnu, int64_t n, double most, double half) {
+  const double s = 1.4e5 / (double)n;
   return most >= WING64_MIN_HALF && lines_near(L, nu_min, dnu, n, 2048.0, half) * std::min(1.0, 2.0 * half) >=
-                                        5.0 + std::min(15.0, 4.0e5 / (double)n);
+                                        6.5 + std::min(25.0, s * s);
 }
 
 // FP32 form.  `most` as above; num_sms SMs.  By the lines that reach a tile of 2048

@@ -74,7 +74,8 @@ def test_lines_near(lib, n, lo, hi):
     (3_000_000, 1, 30, False), (3_000_000, 100, 25000, False), (3_000_000, 1000, 2500, False),
     (3_000_000, 1000, 25000, True), (3_000_000, 10_000, 30, True), (3_000_000, 100_000, 24, True),
     (3_000_000, 100_000, 23, False), (300_000, 100, 2500, False), (300_000, 1000, 30, True),
-    (300_000, 100, 25000, True), (30_000, 100, 250, False), (30_000, 10, 25000, False), (30_000, 100, 25000, True),
+    (300_000, 100, 25000, True), (30_000, 300, 30, False), (3000, 30, 250, False), (30_000, 1000, 250, True),
+    (30_000, 100, 250, False), (30_000, 10, 25000, False), (30_000, 100, 25000, True),
     (30_000, 10_000, 30, True), (3000, 10, 2500, False), (3000, 100, 250, True), (300, 10, 250, False),
     (300, 100, 30, True), (10_000, 300, 2000, True), (20_000, 3000, 24, True)])
 def test_measured_cases(lib, n, nlines, half, wings):
