@@ -206,9 +206,10 @@ helk_status helk_sync(helk_ctx *c) {
   return HELK_OK;
 }
 
-// the double of an order key
-static double order_double(unsigned long long k) {
-  const unsigned long long bits = k >> 63 ? k & 0x7FFFFFFFFFFFFFFFull : ~k;
+// A bound on the doubles whose high word has an order key: above (up) or below them.
+static double key_bound(unsigned k, bool up) {
+  const unsigned h = k & 0x80000000u ? k & 0x7FFFFFFFu : ~k;
+  const unsigned long long bits = (unsigned long long)h << 32 | (up == !(h >> 31) ? 0xFFFFFFFFu : 0u);
   double v;
   memcpy(&v, &bits, 8);
   return v;
@@ -268,11 +269,11 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
     HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "sort lines"));
   }
   c->nlines = n;
-  c->gair_max = order_double(c->stats_host->gair_max);
-  c->gself_max = order_double(c->stats_host->gself_max);
-  c->ncoll_max = order_double(c->stats_host->ncoll_max);
-  c->ncoll_min = order_double(~c->stats_host->ncoll_min_inv);
-  c->mass_min = order_double(~c->stats_host->mass_min_inv);
+  c->gair_max = key_bound(c->stats_host->gair_max, true);
+  c->gself_max = key_bound(c->stats_host->gself_max, true);
+  c->ncoll_max = key_bound(c->stats_host->ncoll_max, true);
+  c->ncoll_min = key_bound(~c->stats_host->ncoll_min_inv, false);
+  c->mass_min = key_bound(~c->stats_host->mass_min_inv, false);
   c->shape.n = n;
   std::copy(c->stats_host->cuts, c->stats_host->cuts + LIST_CUTS + 1, c->shape.at);
   c->have_opacity = false;

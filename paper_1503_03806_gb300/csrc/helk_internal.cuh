@@ -104,9 +104,9 @@ struct DevStats {
   unsigned int tile_counter;        // next (condition, tile) item of the persistent Voigt kernel
   int run_end[SORT_RUNS];           // upload: where the first of them are (in no order)
   double cuts[LIST_CUTS + 1];       // upload: ListShape::at
-  // upload: order keys of the list's largest coefficients and extreme exponents (of
-  // the least its complement: every field starts at 0)
-  unsigned long long gair_max, gself_max, ncoll_max, ncoll_min_inv, mass_min_inv;
+  // upload: order keys of the high words of the list's largest coefficients, extreme
+  // exponents and least mass (of the least the complement: every field starts at 0)
+  unsigned gair_max, gself_max, ncoll_max, ncoll_min_inv, mass_min_inv;
 };
 
 // Core evaluations routed to the surrogate by the FP32 Voigt kernel: the
@@ -167,7 +167,7 @@ struct helk_ctx {
   // line list (sorted SoA)
   int64_t nlines = 0;
   helk::ListShape shape{};  // of the uploaded list
-  double gair_max = 0.0, gself_max = 0.0, ncoll_max = 0.5, ncoll_min = 0.5, mass_min = 1.0;
+  double gair_max = 0.0, gself_max = 0.0, ncoll_max = 0.5, ncoll_min = 0.5, mass_min = 1.0;  // bounds, to 2^-20
   bool has_E = false, has_gself = false, has_ncoll = false, has_delta = false;
   bool has_mass = false, has_weight = false;
   double *nu0 = nullptr, *S0 = nullptr, *El = nullptr, *gair = nullptr,
