@@ -179,7 +179,8 @@ class Clocks:
 
 # The Voigt kernels' translation unit: the kernel file and the headers of
 # csrc/ it includes; the profile summaries record a hash of these sources.
-KERNEL_HEADERS = ("wings.cuh", "voigt_f32.cuh", "voigt_core.cuh", "voigt_common.cuh", "helk_internal.cuh")
+KERNEL_HEADERS = ("wings.cuh", "voigt_f32.cuh", "voigt_core.cuh", "voigt_common.cuh", "helk_internal.cuh",
+                  "route.cuh", "sort_runs.cuh")
 
 
 def kernel_source_hash(kernel_src):
@@ -420,8 +421,8 @@ def run_ours(args):
         e2e = {"value": world * r32["evals"] / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d,
                "d2h_bytes_per_step": d2h, "ms_per_step": e2e_s * 1e3}
 
-    # batched conditions: the 8 T x 8 P workload (1e6 lines) in one
-    # graph-captured persistent launch per call, k-tables of all 64 in one call
+    # batched conditions: the 8 T x 8 P workload (1e6 lines) in one captured
+    # graph per call, k-tables of all 64 in one call
     tpg = None
     if not args.no_tp_grid:
         wt = synth.WORKLOADS["tp_grid"]

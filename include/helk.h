@@ -192,15 +192,17 @@ helk_status helk_opacity(helk_ctx *ctx, double T, double P_atm,
  * pointer, tile shape) into a CUDA graph and replayed on later calls with the
  * same shape; only the condition values change between replays.  The
  * per-condition line records take 56 B (FP32 form) or 96 B (FP64 form; with
- * windows of fewer than 24 points to a side or few lines 64 B) per line, in the FP64 form
- * also 8 B per grid point; when those of all n_cond conditions exceed the
+ * windows of fewer than 24 points to a side or few lines 64 B) per line, in the
+ * FP64 form also 8 B per grid point; when those of all n_cond conditions exceed the
  * record budget
  * (64 GiB unless set by helk_set_batch_budget), the conditions run in the
  * fewest equal chunks that fit, each chunk its own captured graph, one after
  * the other on the stream (the context keeps
  * the 16 most recent graphs).  The results equal those of n_cond
- * helk_opacity calls bit for bit.  A call waits until the previous batch call
- * has read its conditions. */
+ * helk_opacity calls bit for bit (each condition takes the kernels that its own
+ * call takes; a call or chunk that finds no device memory for the FP64 form's
+ * interpolated wings goes point by point, to rounding the same).  A call waits
+ * until the previous batch call has read its conditions. */
 helk_status helk_opacity_batch(helk_ctx *ctx, int32_t n_cond, const double *T,
                                const double *P_atm, const double *q_ratio,
                                double mass_amu, const helk_cutoff *cut,
@@ -263,10 +265,12 @@ helk_status helk_kdist(helk_ctx *ctx, const double *kappa, int64_t n,
  * configuration of a precision's persistent Voigt kernel: the tile (grid
  * points per CTA tile), the warps per CTA and the candidate lines per
  * pipeline stage; it is named by a shape code (helk_tile_shape decodes it).
- * The shapes are those of the kernels that evaluate every point of a window;
- * calls without count_regions whose windows can reach 24 points to a side in
- * the FP64 form, or 64 and ~40 lines to a point in the FP32 form, interpolate
- * the wings and take no shape.
+ * The shapes are those of the kernels that evaluate every point of a window.
+ * Calls without count_regions interpolate the wings and take no shape where the
+ * cutoff allows windows of 24 points to a side (FP64 form) or 64 (FP32 form) and
+ * enough lines reach the grid: about 6 to 30 with a point of a stretch of 2048
+ * points in the FP64 form, 100 to 200 within reach of one in the FP32 form, the
+ * fewer the longer the grid.
  * Runs the line preparation of this condition once, then times every
  * candidate shape of opts->precision on it (three launches each, CUDA events
  * on the context stream) and keeps the fastest for later helk_opacity calls

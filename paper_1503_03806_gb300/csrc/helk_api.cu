@@ -670,10 +670,10 @@ helk_status helk_autotune(helk_ctx *c, double T, double P, double mass, const he
 
 // ---------------------------------------------------------------- batch --
 
-// Many (T, P) conditions in one persistent Voigt launch; the whole sequence
-// (condition upload from pinned staging, statistics reset, line preparation,
-// FP32 records, tile maps, condition order, Voigt kernel) is captured once
-// into a CUDA graph per call shape and replayed.
+// Many (T, P) conditions in one sequence of launches (condition upload from pinned
+// staging, statistics reset, line preparation, FP32 records, maps, condition order,
+// the kernels of the routes that the conditions take), captured once into a CUDA graph
+// per call shape and replayed.
 // The key of a captured sequence: its shape, and the address of every buffer that it
 // reads or writes and that a later call may move (all of them: a list that grows and
 // shrinks again can move some and leave others where they were).

@@ -1,6 +1,6 @@
 // k_voigt.cu -- the FP32 form of the line-tiled Voigt opacity kernel, which takes
-// every point of every window (narrow windows and counting calls; wings.cuh has the
-// route of the others, which shares the core kernel) (Sec. 2.3-2.4): FP32 profile evaluation on records with strengths scaled by
+// every point of every window (narrow windows, few lines and counting calls; wings.cuh
+// has the route of the others, which shares the core kernel) (Sec. 2.3-2.4): FP32 profile evaluation on records with strengths scaled by
 // 2^-E, Kahan-compensated FP32 accumulation per point, the result converted
 // to FP64 and rescaled at the flush; its Algorithm 916 cores in a separate
 // kernel that runs beside it on a second stream; the table of kernel shapes

@@ -1,6 +1,6 @@
 // k_voigt64.cu -- the FP64 form of the line-tiled Voigt opacity kernel, which takes
-// every point of every window (narrow windows and counting calls; wings.cuh has the
-// route of the others) (Sec. 2.3-2.4): FP64 throughout; u and r^2 use explicitly rounded
+// every point of every window (narrow windows, few lines and counting calls; wings.cuh
+// has the route of the others) (Sec. 2.3-2.4): FP64 throughout; u and r^2 use explicitly rounded
 // operations so that the method chosen per point matches the FP64 definition
 // bit for bit.
 //

@@ -293,7 +293,7 @@ class Context:
 
     def opacity_batch(self, T, P, mass, cut, grid, out=None, precision=HELK_PREC_F64, q_ratio=None,
                       accumulate=False, weight=1.0, count_regions=False, surrogate=False):
-        """n_cond conditions (T[k], P[k]) in one graph-captured persistent launch;
+        """n_cond conditions (T[k], P[k]) in one graph-captured sequence of launches;
         returns kappa as a (n_cond, n) float64 tensor."""
         torch = self.torch
         T = np.ascontiguousarray(T, dtype=np.float64)
