@@ -153,6 +153,8 @@ void helk_destroy(helk_ctx *c) {
   for (void *p : bufs)
     if (p) cudaFree(p);
   if (c->stats_host) cudaFreeHost(c->stats_host);
+  if (c->upload) cudaFree(c->upload);
+  if (c->upload_host) cudaFreeHost(c->upload_host);
   if (c->cond_dev) cudaFree(c->cond_dev);
   if (c->cstats) cudaFree(c->cstats);
   if (c->cond_order) cudaFree(c->cond_order);
@@ -223,6 +225,8 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
   if (n > 0 && (!L->nu0 || !L->S0 || !L->gamma_air))
     return set_err(c, HELK_ERR_INVALID_ARG, "lines_upload: nu0, S0 and gamma_air are required");
   HELK_TRY(bind_device(c));
+  if (!c->upload) HELK_TRY(cuda_check(c, cudaMalloc(&c->upload, sizeof(UploadStats)), "lines_upload"));
+  if (!c->upload_host) HELK_TRY(cuda_check(c, cudaMallocHost(&c->upload_host, sizeof(UploadStats)), "lines_upload"));
   const int64_t bytes = (n > 0 ? n : 1) * 8;
   double **dst[9] = {&c->nu0, &c->S0, &c->El, &c->gair, &c->gself, &c->ncoll, &c->delta, &c->lmass,
                      &c->lweight};
@@ -251,31 +255,29 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
   c->has_delta = L->delta != nullptr;
   c->has_mass = L->mass != nullptr;
   c->has_weight = L->weight != nullptr;
-  HELK_TRY(cuda_check(c, cudaMemsetAsync(&c->stats->bad_lines, 0,
-                                         sizeof(DevStats) - offsetof(DevStats, bad_lines), c->stream),
-                      "lines_upload"));
+  HELK_TRY(cuda_check(c, cudaMemsetAsync(c->upload, 0, sizeof(UploadStats), c->stream), "lines_upload"));
   HELK_TRY(cuda_check(c, launch_validate_lines(c, n), "validate lines"));
-  HELK_TRY(cuda_check(c, cudaMemcpyAsync(c->stats_host, c->stats, sizeof(DevStats),
+  HELK_TRY(cuda_check(c, cudaMemcpyAsync(c->upload_host, c->upload, sizeof(UploadStats),
                                          cudaMemcpyDeviceToHost, c->stream),
                       "lines_upload"));
   HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "lines_upload"));
-  if (c->stats_host->bad_lines)
+  if (c->upload_host->bad_lines)
     return set_err(c, HELK_ERR_INVALID_ARG,
-                   "lines_upload: " + std::to_string(c->stats_host->bad_lines) +
+                   "lines_upload: " + std::to_string(c->upload_host->bad_lines) +
                        " lines with non-finite or negative values");
-  if (c->stats_host->unsorted) {
-    HELK_TRY(cuda_check(c, launch_sort_lines(c, n, c->stats_host->unsorted, c->stats_host->run_end),
+  if (c->upload_host->unsorted) {
+    HELK_TRY(cuda_check(c, launch_sort_lines(c, n, c->upload_host->unsorted, c->upload_host->run_end),
                         "sort lines"));
     HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "sort lines"));
   }
   c->nlines = n;
-  c->gair_max = key_bound(c->stats_host->gair_max, true);
-  c->gself_max = key_bound(c->stats_host->gself_max, true);
-  c->ncoll_max = key_bound(c->stats_host->ncoll_max, true);
-  c->ncoll_min = key_bound(~c->stats_host->ncoll_min_inv, false);
-  c->mass_min = key_bound(~c->stats_host->mass_min_inv, false);
+  c->gair_max = key_bound(c->upload_host->gair_max, true);
+  c->gself_max = key_bound(c->upload_host->gself_max, true);
+  c->ncoll_max = key_bound(c->upload_host->ncoll_max, true);
+  c->ncoll_min = key_bound(~c->upload_host->ncoll_min_inv, false);
+  c->mass_min = key_bound(~c->upload_host->mass_min_inv, false);
   c->shape.n = n;
-  std::copy(c->stats_host->cuts, c->stats_host->cuts + LIST_CUTS + 1, c->shape.at);
+  std::copy(c->upload_host->cuts, c->upload_host->cuts + LIST_CUTS + 1, c->shape.at);
   c->have_opacity = false;
   return HELK_OK;
 }

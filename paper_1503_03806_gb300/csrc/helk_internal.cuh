@@ -96,16 +96,20 @@ struct __align__(16) LineRec32 {
 };
 static_assert(sizeof(LineRec32) == 48, "LineRec32 must be 48 bytes");
 
-// Device-side error flags and upload checks.
+// Device-side error flags.
 struct DevStats {
   int err_flags;                    // ERRF_*
-  int bad_lines;                    // validation failures at upload
-  int unsorted;                     // upload: descents of nu0, counted to SORT_RUNS or a few more
   unsigned int tile_counter;        // next (condition, tile) item of the persistent Voigt kernel
-  int run_end[SORT_RUNS];           // upload: where the first of them are (in no order)
-  double cuts[LIST_CUTS + 1];       // upload: ListShape::at
-  // upload: order keys of the high words of the list's largest coefficients, extreme
-  // exponents and least mass (of the least the complement: every field starts at 0)
+};
+
+// What an upload finds out about its list (every field starts at 0).
+struct UploadStats {
+  int bad_lines;                    // validation failures
+  int unsorted;                     // descents of nu0, counted to SORT_RUNS or a few more
+  int run_end[SORT_RUNS];           // where the first of them are (in no order)
+  double cuts[LIST_CUTS + 1];       // ListShape::at
+  // order keys of the high words of the list's largest coefficients, extreme exponents
+  // and least mass (of the least the complement)
   unsigned gair_max, gself_max, ncoll_max, ncoll_min_inv, mass_min_inv;
 };
 
@@ -207,6 +211,8 @@ struct helk_ctx {
   int64_t tile_cap = 0;
   helk::DevStats *stats = nullptr;      // device
   helk::DevStats *stats_host = nullptr; // pinned
+  // of the first upload on (a context that only trains allocates what it did)
+  helk::UploadStats *upload = nullptr, *upload_host = nullptr;  // host side pinned
   // conditions of the current call
   bool core_nodes = false;  // this call's choice of core kernel
   helk::CondArgs *cond_dev = nullptr, *cond_host = nullptr;  // host side pinned
@@ -368,8 +374,8 @@ __device__ __forceinline__ void tma_load_1d(uint32_t dst_smem, const void *src, 
 // ---------------------------------------------------------- launchers ---
 // k_lines.cu
 cudaError_t launch_validate_lines(helk_ctx *c, int64_t n);
-// descents, run_end: DevStats::unsorted and its run ends
-cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end);  // orders SoA by nu0; stats_host->cuts
+// descents, run_end: UploadStats::unsorted and its run ends
+cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *run_end);  // orders SoA by nu0; upload_host->cuts
 // n_cond conditions: from c->cond_dev, or (n_cond == 1 and single != NULL)
 // the one condition passed by value.  Records of condition k start at
 // k * nlines; tile maps at k * ntiles.

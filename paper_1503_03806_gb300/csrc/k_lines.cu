@@ -43,7 +43,7 @@ __global__ void k_validate(int64_t n, const double *__restrict__ nu0, const doub
                            const double *__restrict__ El, const double *__restrict__ gair,
                            const double *__restrict__ gself, const double *__restrict__ ncoll,
                            const double *__restrict__ delta, const double *__restrict__ lmass,
-                           const double *__restrict__ lweight, DevStats *st) {
+                           const double *__restrict__ lweight, UploadStats *st) {
   int bad = 0;
   if (blockIdx.x == 0) list_cuts(n, nu0, st->cuts);
   // order keys of high words (one operation a line and field: 1e7 ordered lines upload
@@ -96,7 +96,7 @@ cudaError_t launch_validate_lines(helk_ctx *c, int64_t n) {
                                             c->has_ncoll ? c->ncoll : nullptr,
                                             c->has_delta ? c->delta : nullptr,
                                             c->has_mass ? c->lmass : nullptr,
-                                            c->has_weight ? c->lweight : nullptr, c->stats);
+                                            c->has_weight ? c->lweight : nullptr, c->upload);
   return cudaGetLastError();
 }
 
@@ -268,7 +268,7 @@ static cudaError_t reorder_fields(helk_ctx *c, int64_t n, const uint32_t *perm, 
       c->launches += 2;
       k_gather<<<gb, 256, 0, c->stream>>>(n, perm, G);
       // the cuts straight to the pinned copy of the statistics that the upload waits for
-      k_gather_back<<<gb, 256, 0, c->stream>>>(n, G, G.field[0] == c->nu0 ? c->stats_host->cuts : nullptr);
+      k_gather_back<<<gb, 256, 0, c->stream>>>(n, G, G.field[0] == c->nu0 ? c->upload_host->cuts : nullptr);
       G.m = 0;
     }
   }
