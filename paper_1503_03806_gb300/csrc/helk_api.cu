@@ -271,11 +271,11 @@ helk_status helk_lines_upload(helk_ctx *c, const helk_lines *L, int64_t n, int32
     HELK_TRY(cuda_check(c, cudaStreamSynchronize(c->stream), "sort lines"));
   }
   c->nlines = n;
-  c->gair_max = key_bound(c->upload_host->gair_max, true);
-  c->gself_max = key_bound(c->upload_host->gself_max, true);
-  c->ncoll_max = key_bound(c->upload_host->ncoll_max, true);
-  c->ncoll_min = key_bound(~c->upload_host->ncoll_min_inv, false);
-  c->mass_min = key_bound(~c->upload_host->mass_min_inv, false);
+  c->gair_max = key_bound(c->upload_host->top[0], true);
+  c->gself_max = key_bound(c->upload_host->top[1], true);
+  c->ncoll_max = key_bound(c->upload_host->top[2], true);
+  c->ncoll_min = key_bound(~c->upload_host->top[3], false);
+  c->mass_min = key_bound(~c->upload_host->top[4], false);
   c->shape.n = n;
   std::copy(c->upload_host->cuts, c->upload_host->cuts + LIST_CUTS + 1, c->shape.at);
   c->have_opacity = false;

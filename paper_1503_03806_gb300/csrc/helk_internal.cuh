@@ -108,9 +108,9 @@ struct UploadStats {
   int unsorted;                     // descents of nu0, counted to SORT_RUNS or a few more
   int run_end[SORT_RUNS];           // where the first of them are (in no order)
   double cuts[LIST_CUTS + 1];       // ListShape::at
-  // order keys of the high words of the list's largest coefficients, extreme exponents
-  // and least mass (of the least the complement)
-  unsigned gair_max, gself_max, ncoll_max, ncoll_min_inv, mass_min_inv;
+  // order keys of the high words of the largest gamma_air, gamma_self and n_coll and of
+  // the least n_coll and mass (of the least the complement)
+  unsigned top[5];
 };
 
 // Core evaluations routed to the surrogate by the FP32 Voigt kernel: the
