@@ -284,11 +284,7 @@ cudaError_t launch_sort_lines(helk_ctx *c, int64_t n, int descents, const int *r
   const int nblk = (int)((n + RS_TILE - 1) / RS_TILE);
   // scratch: 2 key arrays, 2 value arrays, counts, one double array
   int64_t need = 2 * n * 8 + 2 * n * 4 + (int64_t)256 * nblk * 4 + n * 8 + 64;
-  // A merge's time grows with the number of runs, the radix passes' does not: from 9 runs
-  // on only short lists are merged.  Upload in us, merged / sorted: 2e5 lines, 16 runs 317
-  // / 389; 2e6 lines, 4 runs 733 / 1440, 16 runs 2294 / 1465; 1e7 lines, 4 runs 3440 / 6920,
-  // 16 runs 12410 / 6920.
-  const bool merge = descents < MERGE_RUNS_LONG || (descents < SORT_RUNS && n <= MERGE_SHORT);
+  const bool merge = merge_pays(n, descents + 1);
   if (merge) need = (int64_t)GATHER_FIELDS * n * 8 + n * 4;
   helk_status st = ensure_buf(c, &c->tmp, &c->tmp_cap, need, "line sort scratch");
   if (st != HELK_OK) return cudaErrorMemoryAllocation;
